@@ -48,10 +48,14 @@ struct PruneWorkspace {
     unsigned long long *counters;                            // [8]: 0 near-tie groups, 1 lbs swaps, 2 near-ties of the sort, 3 of the swaps
     double *objective;                                       // [4]: after gns, after lbs, identity order
     double *sorted_mean;                                     // [C] channel means in rank order
+    unsigned long long *kept;                                // [C] retained sums of |W| per position of an order
+    double *base[3];                                         // [C/4] group values: after gns, after lbs, identity order
     uint16_t *wt;                                            // [C][ldt] |W| bits, channel-major
+    uint16_t *wb;                                            // [nblocks][No][stride] |W| bits, gathered per shuffle block
+    uint8_t *irregular;                                      // [nblocks][No] the row needs fp64 products in the block shuffle
     double *table;                                           // [nblocks][64][4][256]
-    double *base;                                            // [C/4]
-    long ldt;
+    long ldt;                                                // No rounded up to 8
+    int stride;                                              // lbs_block rounded up to 8
     int splits;
     size_t total_bytes;
 };

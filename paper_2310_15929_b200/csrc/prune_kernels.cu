@@ -9,12 +9,17 @@
 
 #include <math.h>
 
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <mutex>
+#include <type_traits>
+
+#include "spgemm_device.cuh"
+
 namespace esp {
 
 namespace {
-
-constexpr int kLbsMax = 256;       // widest local-shuffle block
-constexpr int kLbsGroups = kLbsMax / 4;
 
 __device__ __forceinline__ double half_bits_abs_to_double(uint16_t h) {
     return (double)__half2float(__ushort_as_half((unsigned short)(h & 0x7FFFu)));
@@ -355,34 +360,88 @@ __global__ void entropy_score_kernel(int C, int T, int bins, const unsigned int 
 }
 
 // --------------------------------------------------------------------------------------------------
-// K3: exact column sums of |W| (units of 2^-24) -> mean of the metric per channel (for the global shuffle).
+// K3: exact column sums of |W| (units of 2^-24) -> mean of the metric per channel (for the global shuffle), and / or the exact
+// retained sums A_q of every group of 4 consecutive positions of an order (Eq. 5; theta NULL = the identity, read in the same
+// 16-byte pieces).  The two share the pass over W.
 // --------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) colabs_kernel(const __half *__restrict__ W, int No, int C, long ldw,
-                                                     int rows_per_split, unsigned long long *__restrict__ colsum) {
+template <bool COLSUM, bool GROUPS>
+__global__ void __launch_bounds__(256) colabs_kernel(const __half *__restrict__ W, int No, int C, long ldw, int rows_per_split,
+                                                     const double *__restrict__ score, const int32_t *__restrict__ theta,
+                                                     unsigned long long *__restrict__ colsum, unsigned long long *__restrict__ kept) {
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int c0 = (blockIdx.x * 32 + tx) * 8;
     const int r_begin = blockIdx.y * rows_per_split;
     const int r_end = min(No, r_begin + rows_per_split);
-    long long acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    long long acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, top[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (c0 < C) {
-        for (int r = r_begin + ty; r < r_end; r += 8) {
-            uint4 v = __ldg(reinterpret_cast<const uint4 *>(W + (long)r * ldw + c0));
-            const uint16_t *h = reinterpret_cast<const uint16_t *>(&v);
+        int ch[8];
+        double sc[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc[k] += half_bits_abs_fixed(h[k]);
+        for (int k = 0; k < 8; ++k) {
+            ch[k] = GROUPS && theta ? theta[c0 + k] : c0 + k;
+            sc[k] = GROUPS ? score[ch[k]] : 0.0;
         }
+        auto load = [&](int r) -> uint4 {
+            const uint16_t *row = reinterpret_cast<const uint16_t *>(W) + (long)r * ldw;
+            if (!(GROUPS && theta)) return __ldg(reinterpret_cast<const uint4 *>(row + c0));
+            uint32_t w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) w[k] = __ldg(row + ch[2 * k]) | ((uint32_t)__ldg(row + ch[2 * k + 1]) << 16);
+            return make_uint4(w[0], w[1], w[2], w[3]);
+        };
+        auto add_row = [&](const uint4 &v) {
+            const uint16_t *h = reinterpret_cast<const uint16_t *>(&v);
+            long long f[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                f[k] = half_bits_abs_fixed(h[k]);
+                if (COLSUM) acc[k] += f[k];
+            }
+            if constexpr (GROUPS) {
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    double xi[4];
+                    int ahead[4] = {0, 0, 0, 0};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) xi[k] = __dmul_rn(half_bits_abs_to_double(h[4 * g + k]), sc[4 * g + k]);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (q != k) ahead[k] += (xi[q] > xi[k] || (xi[q] == xi[k] && q < k)) ? 1 : 0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (ahead[k] < 2) top[4 * g + k] += f[4 * g + k];
+                }
+            }
+        };
+        // four rows in flight per thread
+        int r = r_begin + ty;
+        for (; r + 24 < r_end; r += 32) {
+            uint4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = load(r + 8 * u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) add_row(v[u]);
+        }
+        for (; r < r_end; r += 8) add_row(load(r));
     }
     __shared__ long long s_acc[8][256 + 1];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s_acc[ty][tx * 8 + k] = acc[k];
-    __syncthreads();
     const int c = blockIdx.x * 256 + threadIdx.x;
-    if (c < C) {
-        long long a = 0;
+    auto reduce = [&](const long long (&v)[8], unsigned long long *out) {
+        __syncthreads();
 #pragma unroll
-        for (int y = 0; y < 8; ++y) a += s_acc[y][threadIdx.x];
-        atomicAdd(&colsum[c], (unsigned long long)a);      // integer: order-independent
-    }
+        for (int k = 0; k < 8; ++k) s_acc[ty][tx * 8 + k] = v[k];
+        __syncthreads();
+        if (c < C) {
+            long long a = 0;
+#pragma unroll
+            for (int y = 0; y < 8; ++y) a += s_acc[y][threadIdx.x];
+            atomicAdd(&out[c], (unsigned long long)a);         // integer: order-independent
+        }
+    };
+    if constexpr (COLSUM) reduce(acc, colsum);
+    if constexpr (GROUPS) reduce(top, kept);
 }
 
 __global__ void mean_metric_kernel(int C, int No, const unsigned long long *__restrict__ colsum,
@@ -442,421 +501,43 @@ __global__ void __launch_bounds__(256) gns_near_tie_kernel(int C, const double *
 
 // --------------------------------------------------------------------------------------------------
 // K5: local block shuffle (Algorithm 1 lines 3-14).
-// Wt[c][j] = |W[j,c]| bits, channel-major and zero-padded to ldt rows, so a channel's column is contiguous.
 // --------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) abs_transpose_kernel(const __half *__restrict__ W, int No, int C, long ldw,
-                                                            uint16_t *__restrict__ Wt, long ldt) {
-    __shared__ uint16_t tile[32][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int c_base = blockIdx.x * 32, r_base = blockIdx.y * 32;
-    const uint16_t *Wb = reinterpret_cast<const uint16_t *>(W);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int r = r_base + ty + i * 8, c = c_base + tx;
-        tile[ty + i * 8][tx] = (r < No && c < C) ? (uint16_t)(Wb[(long)r * ldw + c] & 0x7FFFu) : (uint16_t)0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int c = c_base + ty + i * 8, r = r_base + tx;
-        if (c < C && r < ldt) Wt[(long)c * ldt + r] = tile[tx][ty + i * 8];
-    }
-}
+#include "lbs_kernels.cuh"
 
-// Retained metric sum of one group of 4 channels over all rows (Eq. 5 restricted to the group), computed
-// by one warp.  Every lane returns the value.
-//   kept(j,k): slot k is among the 2 largest xi[j,.] = |w| * s (ties: lower slot)
-//   A_k = sum_j kept(j,k) |w_jk| exactly;  V = ((s0*a0 + s1*a1) + s2*a2) + s3*a3
-__device__ double group_value_warp(const uint16_t *__restrict__ Wt, long ldt, const double *__restrict__ score,
-                                   int c0, int c1, int c2, int c3) {
-    const int lane = threadIdx.x & 31;
-    const int ch[4] = {c0, c1, c2, c3};
-    double sc[4];
-    long long A[4] = {0, 0, 0, 0};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sc[k] = score[ch[k]];
-    for (long j = lane * 8; j < ldt; j += 256) {
-        uint4 v[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const uint4 *>(Wt + (long)ch[k] * ldt + j);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            uint16_t h[4];
-            double xi[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                h[k] = reinterpret_cast<const uint16_t *>(&v[k])[e];
-                xi[k] = __dmul_rn(half_bits_abs_to_double(h[k]), sc[k]);
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                int ahead = 0;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (q == k) continue;
-                    ahead += (xi[q] > xi[k] || (xi[q] == xi[k] && q < k)) ? 1 : 0;
-                }
-                if (ahead < 2) A[k] += half_bits_abs_fixed(h[k]);
-            }
-        }
-    }
+// base[g] = V(g) from the retained sums of its four positions (theta NULL = the identity order).
+__global__ void __launch_bounds__(256) group_values_kernel(const unsigned long long *__restrict__ kept, const double *__restrict__ score,
+                                                           const int32_t *__restrict__ theta, int G, double *__restrict__ base) {
+    const int g = blockIdx.x * 256 + threadIdx.x;
+    if (g >= G) return;
+    unsigned long long A[4];
+    double s[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) A[k] += __shfl_xor_sync(0xFFFFFFFFu, A[k], off);
+        A[k] = kept[4 * g + k];
+        s[k] = score[theta ? theta[4 * g + k] : 4 * g + k];
     }
-    double t0 = __dmul_rn(sc[0], __dmul_rn(__ll2double_rn(A[0]), 0x1p-24));
-    double t1 = __dmul_rn(sc[1], __dmul_rn(__ll2double_rn(A[1]), 0x1p-24));
-    double t2 = __dmul_rn(sc[2], __dmul_rn(__ll2double_rn(A[2]), 0x1p-24));
-    double t3 = __dmul_rn(sc[3], __dmul_rn(__ll2double_rn(A[3]), 0x1p-24));
-    return __dadd_rn(__dadd_rn(__dadd_rn(t0, t1), t2), t3);
+    base[g] = lbs_group_value(A, s);
 }
 
-// --------------------------------------------------------------------------------------------------
-// V(group with slot k replaced by candidate x) for all candidates x of a block, without re-ranking four columns
-// per row and candidate.  With the three fixed slots ordered f1, f2, f3 by the metric (ties: lower slot), the
-// candidate is kept exactly when it is ahead of f2; f1 is always kept, f2 is kept exactly when the candidate is not,
-// f3 never.  So per row only f2's slot and |w| matter: phase 1 stores them (4 bytes per row, shared memory) and the
-// exact sums B_q of |w_q| over rows where q is f1 or f2; phase 2 (one warp per candidate) needs one multiply and one
-// compare per row and candidate:  A_x = sum kept |w_x|,  A_q = B_q - sum [q is f2 and x kept] |w_q|.
-// The kept sets, the exact integer sums and the order of the four multiplies and three adds are those of
-// group_value_warp, so the values are bit-identical to it.
-// --------------------------------------------------------------------------------------------------
-__device__ __forceinline__ bool metric_ahead(double xa, int sa, double xb, int sb) { return xa > xb || (xa == xb && sa < sb); }
-
-// Phase 1, whole CTA.  ch[4]: the group's channels; k: the slot to be replaced.  pk[j] = f2 slot << 16 | |w_f2| bits.
-// s_B[4] (shared, zeroed by the caller before the preceding barrier) receives B_q.
-__device__ void lbs_slot_prepare(const uint16_t *__restrict__ Wt, long ldt, const double *__restrict__ score,
-                                 const int (&ch)[4], int k, uint32_t *__restrict__ pk, unsigned long long *s_B) {
-    double sc[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) sc[q] = score[ch[q]];
-    long long B[4] = {0, 0, 0, 0};
-    for (long j = (long)threadIdx.x * 8; j < ldt; j += (long)blockDim.x * 8) {
-        uint4 v[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (q != k) v[q] = *reinterpret_cast<const uint4 *>(Wt + (long)ch[q] * ldt + j);
-        uint32_t out[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            uint16_t h[4];
-            double xi[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                h[q] = (q != k) ? reinterpret_cast<const uint16_t *>(&v[q])[e] : (uint16_t)0;
-                xi[q] = __dmul_rn(half_bits_abs_to_double(h[q]), sc[q]);
-            }
-            // rank of each fixed slot among the three fixed ones
-            int f1 = -1, f2 = -1;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (q == k) continue;
-                int ahead = 0;
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    if (r != k && r != q) ahead += metric_ahead(xi[r], r, xi[q], q) ? 1 : 0;
-                if (ahead == 0) f1 = q;
-                if (ahead == 1) f2 = q;
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q == f1 || q == f2) B[q] += half_bits_abs_fixed(h[q]);
-            uint16_t hf2 = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q == f2) hf2 = h[q];
-            out[e] = ((uint32_t)f2 << 16) | hf2;
-        }
-        *reinterpret_cast<uint4 *>(pk + j) = make_uint4(out[0], out[1], out[2], out[3]);
-        *reinterpret_cast<uint4 *>(pk + j + 4) = make_uint4(out[4], out[5], out[6], out[7]);
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) B[q] += __shfl_xor_sync(0xFFFFFFFFu, B[q], off);
-        if ((threadIdx.x & 31) == 0 && B[q]) atomicAdd(&s_B[q], (unsigned long long)B[q]);   // integers: order-free
-    }
-}
-
-// Phase 2, one warp: the value for candidate channel cx in slot k.  Every lane returns it.
-__device__ double lbs_slot_candidate(const uint16_t *__restrict__ Wt, long ldt, const double (&sc_fixed)[4], int k, int cx,
-                                     double sx, const uint32_t *__restrict__ pk, const unsigned long long *s_B) {
-    const int lane = threadIdx.x & 31;
-    // Per-lane sums of |w| are kept as doubles: every term is a multiple of 2^-24 below 2^16 and a lane adds fewer than
-    // 2^11 of them, so every partial sum is a multiple of 2^-24 below 2^27 -- 51 bits, exact in fp64 -- and equals the
-    // integer sum of group_value_warp once scaled by 2^24.  (One conversion and one predicated add per term instead of the
-    // shifts, selects and 64-bit adds of the integer form: this loop is bound by instruction issue.)
-    double Ax = 0.0, D0 = 0.0, D1 = 0.0, D2 = 0.0, D3 = 0.0;
-    const uint16_t *col = Wt + (long)cx * ldt;
-    // The decision "is the candidate ahead of f2" is the fp64 comparison of |w_x| * s_x with |w_f2| * s_f2.  Its fp32 image
-    // (exact |w|, scores rounded once, one rounded multiply: each product within 2^-23 relative of its fp64 counterpart)
-    // decides it whenever the two products differ by more than 2^-21 of the larger: then the fp64 products differ the same
-    // way.  Only the rows that are closer (ties, zero padding) take the fp64 multiplies.
-    const float sx32 = (float)sx;
-    const float s32[4] = {(float)sc_fixed[0], (float)sc_fixed[1], (float)sc_fixed[2], (float)sc_fixed[3]};
-    auto rows8 = [&](const uint4 &vx, long j) {
-        const uint4 p0 = *reinterpret_cast<const uint4 *>(pk + j);
-        const uint4 p1 = *reinterpret_cast<const uint4 *>(pk + j + 4);
-        const uint32_t pkv[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const uint16_t hx = reinterpret_cast<const uint16_t *>(&vx)[e];
-            const uint32_t rec = pkv[e];
-            const uint16_t hf = (uint16_t)(rec & 0xFFFFu);
-            const bool f2_odd = (rec & 0x10000u) != 0, f2_high = (rec & 0x20000u) != 0;
-            const float wx = __half2float(__ushort_as_half(hx));           // (hx, hf hold magnitudes: the sign bit is clear)
-            const float wf = __half2float(__ushort_as_half(hf));
-            const float sf32 = f2_high ? (f2_odd ? s32[3] : s32[2]) : (f2_odd ? s32[1] : s32[0]);
-            const float px = wx * sx32, pf = wf * sf32;
-            const float big = fmaxf(fabsf(px), fabsf(pf));                 // (scores may be negative when the caller supplies them)
-            const float diff = px - pf;
-            bool kept = diff > 0.f;
-            // undecided in fp32: closer than the margin, or so small that fp32 products lose relative accuracy
-            if (!(fabsf(diff) > big * 0x1p-21f && big >= 0x1p-100f)) {
-                const int f2 = (int)(rec >> 16);
-                const double sf = f2 == 0 ? sc_fixed[0] : f2 == 1 ? sc_fixed[1] : f2 == 2 ? sc_fixed[2] : sc_fixed[3];
-                const double xx = __dmul_rn(half_bits_abs_to_double(hx), sx);
-                const double xf = __dmul_rn(half_bits_abs_to_double(hf), sf);
-                kept = metric_ahead(xx, k, xf, f2);
-            }
-            if (kept) {
-                const double wfd = (double)wf;
-                Ax = __dadd_rn(Ax, (double)wx);
-                if (f2_high) { if (f2_odd) D3 = __dadd_rn(D3, wfd); else D2 = __dadd_rn(D2, wfd); }
-                else { if (f2_odd) D1 = __dadd_rn(D1, wfd); else D0 = __dadd_rn(D0, wfd); }
-            }
-        }
-    };
-    // the column comes from L2: four 16-byte loads per lane are in flight before the first is used
-    long j = lane * 8;
-    for (; j + 3 * 256 < ldt; j += 4 * 256) {
-        uint4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldg(reinterpret_cast<const uint4 *>(col + j + u * 256));
-#pragma unroll
-        for (int u = 0; u < 4; ++u) rows8(v[u], j + u * 256);
-    }
-    for (; j < ldt; j += 256) rows8(__ldg(reinterpret_cast<const uint4 *>(col + j)), j);
-    long long Axi = __double2ll_rn(__dmul_rn(Ax, 0x1p24));                  // exact: see above
-    long long D[4] = {__double2ll_rn(__dmul_rn(D0, 0x1p24)), __double2ll_rn(__dmul_rn(D1, 0x1p24)),
-                      __double2ll_rn(__dmul_rn(D2, 0x1p24)), __double2ll_rn(__dmul_rn(D3, 0x1p24))};
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        Axi += __shfl_xor_sync(0xFFFFFFFFu, Axi, off);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) D[q] += __shfl_xor_sync(0xFFFFFFFFu, D[q], off);
-    }
-    double t[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const long long A = (q == k) ? Axi : (long long)s_B[q] - D[q];
-        const double sq = (q == k) ? sx : sc_fixed[q];
-        t[q] = __dmul_rn(sq, __dmul_rn(__ll2double_rn(A), 0x1p-24));
-    }
-    return __dadd_rn(__dadd_rn(__dadd_rn(t[0], t[1]), t[2]), t[3]);
-}
-
-// table[b][g][slot][x] = V(group g of block b with its slot replaced by block channel x); base[G] = V(g).
-// grid (nblocks * 64 * 4): one CTA per (block, group, slot); block 256 (8 warps); dynamic shared memory ldt * 4 bytes.
-__global__ void __launch_bounds__(256, 4) lbs_table_kernel(const uint16_t *__restrict__ Wt, long ldt,
-                                                        const double *__restrict__ score,
-                                                        const int32_t *__restrict__ theta0, int C, int lbs_block,
-                                                        double *__restrict__ table, double *__restrict__ base) {
-    extern __shared__ uint32_t s_pk[];
-    __shared__ unsigned long long s_B[4];
-    const int slot = blockIdx.x & 3;
-    const int g = (blockIdx.x >> 2) % kLbsGroups, b = (blockIdx.x >> 2) / kLbsGroups;
-    const int p0 = b * lbs_block;
-    const int m = min(lbs_block, C - p0);
-    if (g * 4 >= m) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int grp[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) grp[k] = theta0[p0 + g * 4 + k];
-    if (threadIdx.x < 4) s_B[threadIdx.x] = 0;
-    __syncthreads();
-    lbs_slot_prepare(Wt, ldt, score, grp, slot, s_pk, s_B);
-    __syncthreads();
-    double sc[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sc[k] = score[grp[k]];
-    double *tb = table + (((long)b * kLbsGroups + g) * 4 + slot) * kLbsMax;
-    for (int x = warp; x < m; x += 8) {
-        const int cx = theta0[p0 + x];
-        const double v = lbs_slot_candidate(Wt, ldt, sc, slot, cx, score[cx], s_pk, s_B);
-        if (lane == 0) tb[x] = v;
-    }
-    if (slot == 0 && warp == 0) {
-        double v = group_value_warp(Wt, ldt, score, grp[0], grp[1], grp[2], grp[3]);
-        if (lane == 0) base[p0 / 4 + g] = v;
-    }
-}
-
-// (Two CTAs per SM, at 64 registers per thread with a few spills: one cluster of eight occupies eight SMs whatever its
-// CTAs need, only 15 such clusters fit 148 SMs, and a weight has 32 to 86 blocks -- the second CTA per SM halves the number
-// of waves, and the LLaMA-65B-shaped layer's producer went from 3.4 to 2.1 s.)
-// One cluster of 8 CTAs per block of positions: repeat { best cross-group swap by table lookup; apply if gain > 0;
-// refresh the two touched groups }.  Every CTA takes the same decision from the same table (no exchange needed), then
-// refreshes one of the 2 groups x 4 slots of table rows; a cluster barrier publishes the rows before the next
-// decision.  grid (nblocks * 8), cluster (8), block 512, dynamic shared memory ldt * 4 bytes.
-constexpr int kLbsCluster = 8;
-__global__ void __launch_bounds__(512, 2) lbs_greedy_kernel(const uint16_t *__restrict__ Wt, long ldt,
-                                                          const double *__restrict__ score,
-                                                          const int32_t *__restrict__ theta0, int C, int lbs_block,
-                                                          int max_swaps, double *__restrict__ table,
-                                                          double *__restrict__ base, int32_t *__restrict__ theta,
-                                                          unsigned long long *__restrict__ counters) {
-    extern __shared__ uint32_t s_pk[];
-    const int b = blockIdx.x / kLbsCluster;
-    const int unit = blockIdx.x % kLbsCluster;                  // rank in the cluster: which (group, slot) this CTA refreshes
-    const int p0 = b * lbs_block;
-    const int m = min(lbs_block, C - p0);
-    const int G = m / 4;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    __shared__ int pos2x[kLbsMax];
-    __shared__ int chan[kLbsMax];
-    __shared__ double s_base[kLbsGroups];
-    __shared__ double red_gain[16], red_second[16];
-    __shared__ int red_idx[16];
-    __shared__ int decision;      // linear pair index i*256+j, or -1 to stop
-    __shared__ unsigned long long s_B[4];
-    double *tb = table + (long)b * kLbsGroups * 4 * kLbsMax;
-    if (tid < m) { pos2x[tid] = tid; chan[tid] = theta0[p0 + tid]; }
-    if (tid < G) s_base[tid] = base[p0 / 4 + tid];
-    __syncthreads();
-    int swaps = 0;
-    int near_swaps = 0;                                        // kept by thread 0 only
-    for (;;) {
-        double best = -INFINITY, second = -INFINITY;           // second: largest gain once one instance of the best is set aside
-        int best_e = 0x7FFFFFFF;
-        if (max_swaps <= 0 || swaps < max_swaps) {
-            for (int e = tid; e < kLbsMax * kLbsMax; e += 512) {
-                const int i = e >> 8, j = e & 255;
-                if (j <= i || j >= m || (i >> 2) == (j >> 2)) continue;
-                const int gi = i >> 2, si = i & 3, gj = j >> 2, sj = j & 3;
-                // rows of the table are rewritten by other CTAs of the cluster: read them from L2, never from this SM's L1
-                double after = __dadd_rn(__ldcg(&tb[(gi * 4 + si) * kLbsMax + pos2x[j]]), __ldcg(&tb[(gj * 4 + sj) * kLbsMax + pos2x[i]]));
-                double gain = __dsub_rn(after, __dadd_rn(s_base[gi], s_base[gj]));
-                if (gain > best || (gain == best && e < best_e)) { second = fmax(second, best); best = gain; best_e = e; }
-                else second = fmax(second, gain);
-            }
-        }
-        // merging two (best, second) pairs: the larger best wins (ties: smaller pair index), the loser's best competes
-        // with both seconds -- the result is the second-largest of the union whatever the order of merging
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            double og = __shfl_xor_sync(0xFFFFFFFFu, best, off);
-            double os = __shfl_xor_sync(0xFFFFFFFFu, second, off);
-            int oe = __shfl_xor_sync(0xFFFFFFFFu, best_e, off);
-            second = fmax(fmax(second, os), fmin(best, og));
-            if (og > best || (og == best && oe < best_e)) { best = og; best_e = oe; }
-        }
-        if (lane == 0) { red_gain[warp] = best; red_second[warp] = second; red_idx[warp] = best_e; }
+// Eq. 5 objectives: the group values summed in group order, one order per CTA (base0, base1, base2 -> out[0..2]).  The additions are
+// one serial chain by definition; the values are brought into shared memory first, so that the chain waits on nothing else (one
+// thread reading them from L2 took 40 us for 1024 groups, this 8).
+__global__ void __launch_bounds__(256) objective_kernel(int G, const double *__restrict__ base0, const double *__restrict__ base1,
+                                                        const double *__restrict__ base2, double *__restrict__ out) {
+    __shared__ double s[2048];
+    const double *base = blockIdx.x == 0 ? base0 : blockIdx.x == 1 ? base1 : base2;
+    double t = 0.0;
+    for (int g0 = 0; g0 < G; g0 += 2048) {
+        const int n = min(2048, G - g0);
         __syncthreads();
-        if (warp == 0) {
-            best = lane < 16 ? red_gain[lane] : -INFINITY;
-            second = lane < 16 ? red_second[lane] : -INFINITY;
-            best_e = lane < 16 ? red_idx[lane] : 0x7FFFFFFF;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                double og = __shfl_xor_sync(0xFFFFFFFFu, best, off);
-                double os = __shfl_xor_sync(0xFFFFFFFFu, second, off);
-                int oe = __shfl_xor_sync(0xFFFFFFFFu, best_e, off);
-                second = fmax(fmax(second, os), fmin(best, og));
-                if (og > best || (og == best && oe < best_e)) { best = og; best_e = oe; }
-            }
-            if (lane == 0) {
-                decision = (best > 0.0) ? best_e : -1;
-                // an applied swap whose runner-up is within 1e-6 relative: counted, not acted on
-                if (best > 0.0 && second > -INFINITY && __dsub_rn(best, second) < __dmul_rn(1e-6, fabs(best))) ++near_swaps;
-            }
-        }
+        for (int i = threadIdx.x; i < n; i += 256) s[i] = base[g0 + i];
         __syncthreads();
-        const int d = decision;
-        if (d < 0) break;
-        const int bi = d >> 8, bj = d & 255;
-        if (tid == 0) { int t = pos2x[bi]; pos2x[bi] = pos2x[bj]; pos2x[bj] = t; }
-        ++swaps;
-        __syncthreads();
-        // Refresh.  Row (g, slot) of the table holds the values of group g with that slot replaced by each candidate, so it
-        // depends on g's OTHER three channels only: of the eight rows of the two touched groups, the two rows of the swapped
-        // slots themselves stay as they are, six need new values.  Their candidates are dealt in quarters, three of the 24
-        // quarters to each of the cluster's eight CTAs (a CTA prepares the per-row records of each row it has a share of);
-        // units 0 and 4 also recompute the base value of one group each.
-        {
-            if ((unit == 0 || unit == 4) && warp == 0) {
-                const int g = unit == 0 ? (bi >> 2) : (bj >> 2);
-                double v = group_value_warp(Wt, ldt, score, chan[pos2x[g * 4]], chan[pos2x[g * 4 + 1]], chan[pos2x[g * 4 + 2]],
-                                            chan[pos2x[g * 4 + 3]]);
-                if (lane == 0) base[p0 / 4 + g] = v;
-            }
-            const int quarter_size = (m + 3) >> 2;
-            int prepared = -1;
-            for (int qq = 3 * unit; qq < 3 * unit + 3; ++qq) {
-                const int row = qq >> 2, quarter = qq & 3, which = row / 3;
-                int slot = row - 3 * which;                      // the (row mod 3)-th slot other than the swapped one
-                if (slot >= ((which ? bj : bi) & 3)) ++slot;
-                const int g = (which ? bj : bi) >> 2;
-                int ch[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) ch[k] = chan[pos2x[g * 4 + k]];
-                double sc[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) sc[k] = score[ch[k]];
-                if (row != prepared) {
-                    __syncthreads();                             // the previous row's records are no longer being read
-                    if (tid < 4) s_B[tid] = 0;
-                    __syncthreads();
-                    lbs_slot_prepare(Wt, ldt, score, ch, slot, s_pk, s_B);
-                    __syncthreads();
-                    prepared = row;
-                }
-                const int x_end = min(m, (quarter + 1) * quarter_size);
-                for (int x = quarter * quarter_size + warp; x < x_end; x += 16) {
-                    const int cx = chan[x];
-                    const double v = lbs_slot_candidate(Wt, ldt, sc, slot, cx, score[cx], s_pk, s_B);
-                    if (lane == 0) tb[(g * 4 + slot) * kLbsMax + x] = v;
-                }
-            }
+        if (threadIdx.x == 0) {
+#pragma unroll 16
+            for (int i = 0; i < n; ++i) t = __dadd_rn(t, s[i]);
         }
-        __threadfence();
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        if (tid < 2) {                                          // the two refreshed base values, written by units 0 and 4
-            const int g = tid == 0 ? (bi >> 2) : (bj >> 2);
-            s_base[g] = *reinterpret_cast<volatile double *>(base + p0 / 4 + g);
-        }
-        __syncthreads();
     }
-    if (unit != 0) return;
-    if (tid < m) theta[p0 + tid] = chan[pos2x[tid]];
-    if (tid < G) base[p0 / 4 + tid] = s_base[tid];
-    if (tid == 0 && swaps) atomicAdd(&counters[1], (unsigned long long)swaps);
-    if (tid == 0 && near_swaps) atomicAdd(&counters[3], (unsigned long long)near_swaps);
-}
-
-// Sum of the group values in group order (Eq. 5 objective), one thread: deterministic.
-__global__ void objective_kernel(int G, const double *__restrict__ base, double *__restrict__ out) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double t = 0.0;
-        for (int g = 0; g < G; ++g) t = __dadd_rn(t, base[g]);
-        *out = t;
-    }
-}
-
-// base[g] = V(g) under theta for every group (the objective of an order that the block shuffle does not produce itself).
-__global__ void __launch_bounds__(256) group_values_kernel(const uint16_t *__restrict__ Wt, long ldt,
-                                                           const double *__restrict__ score,
-                                                           const int32_t *__restrict__ theta, int G,
-                                                           double *__restrict__ base) {
-    const int g = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (g >= G) return;
-    int c[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) c[k] = theta ? theta[4 * g + k] : 4 * g + k;      // NULL: the identity order
-    double v = group_value_warp(Wt, ldt, score, c[0], c[1], c[2], c[3]);
-    if ((threadIdx.x & 31) == 0) base[g] = v;
+    if (threadIdx.x == 0) out[blockIdx.x] = t;
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -1100,11 +781,17 @@ PruneWorkspace carve_prune_workspace(void *ws, int No, int C, int T, const esp_p
     w.counters = (unsigned long long *)take(sizeof(unsigned long long) * 8);
     w.objective = (double *)take(sizeof(double) * 4);
     w.sorted_mean = (double *)take(sizeof(double) * C);
-    w.ldt = (long)align_up((size_t)No, 256);
-    w.wt = (uint16_t *)take(sizeof(uint16_t) * (size_t)C * w.ldt);
-    int nblocks = ceil_div(C, o.lbs_block > 0 ? o.lbs_block : kLbsMax);
-    w.table = (double *)take(sizeof(double) * (size_t)nblocks * kLbsGroups * 4 * kLbsMax);
-    w.base = (double *)take(sizeof(double) * (size_t)(C / 4 + 1));
+    w.kept = (unsigned long long *)take(sizeof(unsigned long long) * C);
+    for (double *&base : w.base) base = (double *)take(sizeof(double) * (size_t)(C / 4 + 1));
+    if (o.use_lbs) {
+        const int nblocks = ceil_div(C, o.lbs_block);
+        w.ldt = (long)align_up((size_t)No, 8);
+        w.stride = (int)align_up((size_t)o.lbs_block, 8);
+        w.wt = (uint16_t *)take(sizeof(uint16_t) * (size_t)C * w.ldt);
+        w.wb = (uint16_t *)take(sizeof(uint16_t) * (size_t)nblocks * No * w.stride);
+        w.irregular = (uint8_t *)take((size_t)nblocks * No);
+        w.table = (double *)take(sizeof(double) * (size_t)nblocks * kLbsGroups * 4 * kLbsMax);
+    }
     w.total_bytes = off;
     return w;
 }
@@ -1215,13 +902,19 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
     if (chan_entropy) ESP_CUDA_OK(cudaMemcpyAsync(chan_entropy, w.entropy, sizeof(double) * C, cudaMemcpyDeviceToDevice, stream));
     if (chan_score) ESP_CUDA_OK(cudaMemcpyAsync(chan_score, w.score, sizeof(double) * C, cudaMemcpyDeviceToDevice, stream));
 
-    // K3 + K4
-    if (o.use_gns && !o.perm_override) {
-        ESP_CUDA_OK(cudaMemsetAsync(w.colsum, 0, sizeof(unsigned long long) * C, stream));
-        const int wsplits = pick_splits(No, ceil_div(C, 256), di.sm_count);
-        colabs_kernel<<<dim3(ceil_div(C, 256), wsplits), 256, 0, stream>>>(W, No, C, ldw, ceil_div(No, wsplits), w.colsum);
-        mean_metric_kernel<<<cblocks, cthreads, 0, stream>>>(C, No, w.colsum, w.score, w.mean);
-    }
+    // K3 + K4: the column sums for the global shuffle and, when objectives are asked for, the retained sums under the identity
+    const int G = C / 4;
+    const bool gns = o.use_gns && !o.perm_override;
+    const int wsplits = pick_splits(No, ceil_div(C, 256), di.sm_count);
+    const dim3 wgrid(ceil_div(C, 256), wsplits);
+    const int wrows = ceil_div(No, wsplits);
+    if (gns) ESP_CUDA_OK(cudaMemsetAsync(w.colsum, 0, sizeof(unsigned long long) * C, stream));
+    if (stats) ESP_CUDA_OK(cudaMemsetAsync(w.kept, 0, sizeof(unsigned long long) * C, stream));
+    if (gns && stats) colabs_kernel<true, true><<<wgrid, 256, 0, stream>>>(W, No, C, ldw, wrows, w.score, nullptr, w.colsum, w.kept);
+    else if (gns) colabs_kernel<true, false><<<wgrid, 256, 0, stream>>>(W, No, C, ldw, wrows, w.score, nullptr, w.colsum, w.kept);
+    else if (stats) colabs_kernel<false, true><<<wgrid, 256, 0, stream>>>(W, No, C, ldw, wrows, w.score, nullptr, w.colsum, w.kept);
+    if (gns) mean_metric_kernel<<<cblocks, cthreads, 0, stream>>>(C, No, w.colsum, w.score, w.mean);
+    if (stats) group_values_kernel<<<ceil_div(G, 256), 256, 0, stream>>>(w.kept, w.score, nullptr, G, w.base[2]);
     int32_t *theta0 = (o.use_lbs || stats) ? w.theta0 : perm;
     if (o.perm_override)
         ESP_CUDA_OK(cudaMemcpyAsync(theta0, o.perm_override, sizeof(int32_t) * C, cudaMemcpyDeviceToDevice, stream));
@@ -1232,45 +925,34 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
     ESP_CUDA_OK(cudaGetLastError());
 
     // K5
-    const int G = C / 4;
-    if (o.use_lbs || stats) {
-        abs_transpose_kernel<<<dim3(ceil_div(C, 32), ceil_div(w.ldt, 32)), 256, 0, stream>>>(W, No, C, ldw, w.wt, w.ldt);
-    }
-    if (stats) {                             // Eq. 5 under the identity order (w.base is rewritten below)
-        group_values_kernel<<<ceil_div(G, 8), 256, 0, stream>>>(w.wt, w.ldt, w.score, nullptr, G, w.base);
-        objective_kernel<<<1, 32, 0, stream>>>(G, w.base, w.objective + 2);
-    }
     if (o.use_lbs) {
         const int nblocks = ceil_div(C, o.lbs_block);
-        const size_t pk_smem = (size_t)w.ldt * sizeof(uint32_t);          // per-row f2 record of one (group, slot)
-        if (pk_smem > (size_t)di.max_smem_optin - 8192) return ESP_ERR_UNSUPPORTED;   // No beyond ~56000 rows
-        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pk_smem));
-        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pk_smem));
-        lbs_table_kernel<<<nblocks * kLbsGroups * 4, 256, pk_smem, stream>>>(w.wt, w.ldt, w.score, w.theta0, C, o.lbs_block,
-                                                                            w.table, w.base);
-        if (stats) objective_kernel<<<1, 32, 0, stream>>>(G, w.base, w.objective);
-        {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(nblocks * kLbsCluster);
-            cfg.blockDim = dim3(512);
-            cfg.dynamicSmemBytes = pk_smem;
-            cfg.stream = stream;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = kLbsCluster;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_greedy_kernel, (const uint16_t *)w.wt, w.ldt, (const double *)w.score,
-                                           (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, w.base, perm,
-                                           w.counters));
-        }
-        if (stats) objective_kernel<<<1, 32, 0, stream>>>(G, w.base, w.objective + 1);
+        const size_t row_bytes = sizeof(uint16_t) * (size_t)C;
+        // rows per CTA: about 96 KB of shared memory (two CTAs per SM), and a grid of two CTAs per SM at least
+        int gather_rows = (int)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / row_bytes));
+        gather_rows = std::max(1, std::min(gather_rows, No / (2 * std::max(1, di.sm_count))));
+        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(row_bytes * gather_rows)));
+        lbs_gather_kernel<<<ceil_div(No, gather_rows), 256, row_bytes * gather_rows, stream>>>(W, No, C, ldw, w.score, w.theta0, o.lbs_block, w.stride,
+                                                                                               nblocks, gather_rows, w.wb, w.irregular);
+        lbs_transpose_kernel<<<dim3(ceil_div(C, 64), ceil_div(No, 64)), 256, 0, stream>>>(W, No, C, ldw, w.wt, w.ldt);
+        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LbsTableSmem)));
+        lbs_table_kernel<<<nblocks * kLbsGroups, kTableThreads, sizeof(LbsTableSmem), stream>>>(w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score,
+                                                                                                w.theta0, C, o.lbs_block, w.table, w.base[0]);
+        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbs_greedy_smem(kGreedyMinCluster)));
+        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        const int nc = lbs_cluster_size(nblocks, No, di.device);
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr;
+        lbs_greedy_config(cfg, attr, nblocks, nc, stream);
+        ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, (const uint8_t *)w.irregular, No,
+                                       w.stride, (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table,
+                                       (const double *)w.base[0], w.base[1], perm, w.counters, nc));
+        if (stats) objective_kernel<<<3, 256, 0, stream>>>(G, w.base[0], w.base[1], w.base[2], w.objective);
     } else if (stats) {
-        group_values_kernel<<<ceil_div(G, 8), 256, 0, stream>>>(w.wt, w.ldt, w.score, w.theta0, G, w.base);
-        objective_kernel<<<1, 32, 0, stream>>>(G, w.base, w.objective);
-        ESP_CUDA_OK(cudaMemcpyAsync(w.objective + 1, w.objective, sizeof(double), cudaMemcpyDeviceToDevice, stream));
+        ESP_CUDA_OK(cudaMemsetAsync(w.kept, 0, sizeof(unsigned long long) * C, stream));
+        colabs_kernel<false, true><<<wgrid, 256, 0, stream>>>(W, No, C, ldw, wrows, w.score, w.theta0, w.colsum, w.kept);
+        group_values_kernel<<<ceil_div(G, 256), 256, 0, stream>>>(w.kept, w.score, w.theta0, G, w.base[0]);
+        objective_kernel<<<3, 256, 0, stream>>>(G, w.base[0], w.base[0], w.base[2], w.objective);
         ESP_CUDA_OK(cudaMemcpyAsync(perm, w.theta0, sizeof(int32_t) * C, cudaMemcpyDeviceToDevice, stream));
     }
     ESP_CUDA_OK(cudaGetLastError());

@@ -98,6 +98,43 @@ def test_block_shuffle_tall_weights_bit_exact(No, C, block, cap):
     assert ref.lbs.swaps_total > 0
 
 
+@pytest.mark.parametrize("kind", ["equal_scores", "zero_scores", "negative_scores", "large_weights", "ties_in_some_rows"])
+@pytest.mark.parametrize("No,C,block,cap", [(40, 264, 256, 0), (1100, 256, 256, 5), (67, 48, 12, 0)])
+def test_block_shuffle_rows_that_fp32_cannot_decide(kind, No, C, block, cap):
+    """The block shuffle's fp64 path: rows with equal products (settled by position), rows with |w| >= 0.5, blocks with scores
+    that are zero or negative -- all rows of a weight or a few among regular ones, in slices shorter and longer than a chunk."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8100 + No)
+    W = (g0.standard_normal((No, C)) * (1.5 if kind == "large_weights" else 0.02)).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(C)
+    if kind == "equal_scores":
+        s[:] = 2.5
+    elif kind == "zero_scores":
+        s[::5] = 0.0
+    elif kind == "negative_scores":
+        s[::7] *= -1.0
+    elif kind == "ties_in_some_rows":
+        s[1::2] = s[::2]
+        W[::6, 1::2] = W[::6, ::2]
+        W[3::6, ::3] = 0.0
+    ref = orc.metric_prune(W, None, 1.0, score=s, lbs_block=block, lbs_max_swaps=cap)
+    g = GpuPrune(W, None, 1.0, score=s, lbs_block=block, lbs_max_swaps=cap)
+    assert_identical_to_oracle(g, ref)
+
+
+@pytest.mark.parametrize("No", [1, 3, 192 * 16, 192 * 16 + 1, 1024 * 16 + 5])
+def test_block_shuffle_row_slices(No):
+    """Rows dealt to the CTAs of one block's cluster: fewer rows than CTAs, slices at the edge between the two row loops,
+    slices of more than one chunk."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8200 + No)
+    W = (g0.standard_normal((No, 64)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(64)
+    ref = orc.metric_prune(W, None, 1.0, score=s, lbs_max_swaps=6)
+    g = GpuPrune(W, None, 1.0, score=s, lbs_max_swaps=6)
+    assert_identical_to_oracle(g, ref)
+
+
 def test_llama7b_q_projection_full_size_block_shuffle():
     """Workload 1's q projection whole (4096 x 4096, 16 shuffle blocks, Student-t rows): global shuffle, block shuffle
     capped at 4 swaps per block on both sides (the oracle's table alone is 4.3e9 row evaluations), selection and
