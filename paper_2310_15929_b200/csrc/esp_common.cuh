@@ -40,11 +40,11 @@ esp_status_t device_info(DeviceInfo *out);
 // ---- pruning launchers (prune_kernels.cu) ----------------------------------------------------------
 struct PruneWorkspace {
     // all pointers into the caller's workspace
-    double *part_sumsq; float *part_min; float *part_max;   // [splits][C]
-    double *lo, *hi, *norm, *entropy, *score, *mean;         // [C]
+    double *lo, *hi, *norm, *score, *mean;                   // [C]
     unsigned int *counts;                                    // [C][bins]
     unsigned long long *colsum;                              // [C]
     int32_t *theta0;                                         // [C]
+    size_t cleared_bytes;                                    // from counters to the end of counts: zeroed at the start of a call
     unsigned long long *counters;                            // [8]: 0 near-tie groups, 1 lbs swaps, 2 near-ties of the sort, 3 of the swaps
     double *objective;                                       // [4]: after gns, after lbs, identity order
     double *sorted_mean;                                     // [C] channel means in rank order
@@ -56,7 +56,6 @@ struct PruneWorkspace {
     double *table;                                           // [nblocks][64][4][256]
     long ldt;                                                // No rounded up to 8
     int stride;                                              // lbs_block rounded up to 8
-    int splits;
     size_t total_bytes;
 };
 PruneWorkspace carve_prune_workspace(void *ws, int No, int C, int T, const esp_prune_opts &o);
@@ -73,7 +72,6 @@ esp_status_t launch_decompress(const __half *vals, const uint8_t *meta, const in
 struct CalibState {
     double *sumsq, *lo, *hi, *norm;
     unsigned int *counts;
-    double *part_sumsq; float *part_min; float *part_max;
     size_t total_bytes;
 };
 CalibState carve_calib_state(void *state, int C, int bins);

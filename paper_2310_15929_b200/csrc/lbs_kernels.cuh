@@ -216,21 +216,6 @@ __device__ __forceinline__ void lbs_group_sums(const LbsRows<ROWS> &R, int lo, i
 constexpr uint32_t kNarrowMask = 0x3FFFFFFFu, kNarrowBase = 0x40000000u;
 constexpr int kNarrowRun = 128;
 
-__device__ __forceinline__ uint64_t f32x2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 // if (p > bound) { a += f; d += u; } as one comparison and two predicated additions (left to itself the compiler selects addends: four
 // instructions instead of two).
 __device__ __forceinline__ void lbs_count(uint32_t &a, uint32_t &d, uint32_t f, uint32_t u, float p, float bound) {

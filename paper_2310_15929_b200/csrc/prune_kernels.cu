@@ -32,48 +32,118 @@ __device__ __forceinline__ long long half_bits_abs_fixed(uint16_t h) {
     return e == 0 ? m : ((1024 + m) << (e - 1));
 }
 
+// Two fp32 values per register pair and instruction.
+__device__ __forceinline__ uint64_t f32x2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// A launch that may be set up while the preceding kernel runs: the kernels launched this way wait for it (griddepcontrol.wait) before
+// their first access to memory, so stream order holds; what they save is the gap between two launches.  `cluster`: CTAs per cluster
+// along y.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_overlapped(void (*kern)(Params...), dim3 grid, int cluster, int threads, size_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = cluster;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+
 // --------------------------------------------------------------------------------------------------
-// K1: per-channel sum of squares (fp64), min and max over a slice of tokens.   Eq. 2 / range of Eq. 1.
-// grid (ceil(C/256), splits), block 256 = 32 channel-vectors of 8 x 8 token lanes.
+// K1: per-channel sum of squares (fp64), min and max.   Eq. 2 / range of Eq. 1.
+// grid (ceil(C/64), splits of the tokens), cluster (1, splits), block 256 = 8 channel-vectors of 8 x 32 token lanes.  Bound by the
+// read of X.  The splits of a column block are one cluster: their partial results meet in distributed shared memory, added in split
+// order -- deterministic, without partial arrays in HBM and without a second kernel (which, with one thread per channel, took 8 us
+// for 8 splits of 8192 channels and 37 us for 64 of 4096) or a last-CTA tail (8 us).  2048 x 8192: 13.5 + 8.5 -> 14 us.
 // --------------------------------------------------------------------------------------------------
+struct ColStatsOut {
+    double *sumsq;                           // running sum of squares (streaming calibration), or NULL:
+    double *norm;                            // the norm of this call's tokens
+    double *lo, *hi;                         // running (sumsq != NULL) or this call's range
+};
+__device__ __forceinline__ double ld_cluster_f64(const double *local, uint32_t rank) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(map_to_rank(smem_u32(local), rank)) : "memory");
+    return v;
+}
 constexpr int kColAhead = 8;                                              // rows each thread keeps in flight
-constexpr int kColSmem = (kColAhead + 1) * 256 * 16;                      // the threads' load rings; >= the partial results after
-static_assert(kColSmem >= (int)(sizeof(double) * 8 * 257 + 2 * sizeof(float) * 8 * 257), "the reduction reuses the ring");
-__global__ void __launch_bounds__(256) colstats_kernel(const __half *__restrict__ X, int T, int C, long ldx,
-                                                       int rows_per_split, double *__restrict__ part_sumsq,
-                                                       float *__restrict__ part_min, float *__restrict__ part_max) {
+constexpr int kColSmem = (kColAhead + 1) * 256 * 16;                      // the threads' load rings
+__global__ void __launch_bounds__(256) colstats_kernel(const __half *__restrict__ X, int T, int C, long ldx, int rows_per_split,
+                                                       const ColStatsOut out) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int c0 = (blockIdx.x * 32 + tx) * 8;
-    const int r_begin = blockIdx.y * rows_per_split;
+    __shared__ double s_acc[8][64], s_sum[64];
+    __shared__ float s_mn[8][64], s_mx[8][64], s_lo[64], s_hi[64];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int c0 = (blockIdx.x * 8 + tx) * 8;
+    const int splits = gridDim.y, rank = blockIdx.y;
+    const int r_begin = rank * rows_per_split;
     const int r_end = min(T, r_begin + rows_per_split);
     double acc[8];
-    float mn[8], mx[8];
+    __half2 mn[4], mx[4];                                     // (two channels per instruction; NaNs are passed over)
 #pragma unroll
-    for (int k = 0; k < 8; ++k) { acc[k] = 0.0; mn[k] = INFINITY; mx[k] = -INFINITY; }
+    for (int k = 0; k < 8; ++k) acc[k] = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        mn[k] = __half2half2(__ushort_as_half((unsigned short)0x7C00));
+        mx[k] = __half2half2(__ushort_as_half((unsigned short)0xFC00));
+    }
+    grid_dependency_wait();
+    grid_launch_dependents();
+    // the channel that this thread finishes (if any), and the state it adds to
+    const int c = blockIdx.x * 64 + tid;
+    const bool mine = tid < 64 && tid % splits == rank && c < C;
+    double run_sumsq = 0.0, run_lo = INFINITY, run_hi = -INFINITY;
+    if (mine && out.sumsq) { run_sumsq = out.sumsq[c]; run_lo = out.lo[c]; run_hi = out.hi[c]; }
     if (c0 < C) {
         auto add_row = [&](const uint4 &v) {
-            const __half *h = reinterpret_cast<const __half *>(&v);
+            const __half2 *h = reinterpret_cast<const __half2 *>(&v);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                float f = __half2float(h[k]);
-                acc[k] = __dadd_rn(acc[k], (double)(f * f));   // f*f is exact in fp32 (22-bit product)
-                mn[k] = fminf(mn[k], f);
-                mx[k] = fmaxf(mx[k], f);
+            for (int k = 0; k < 4; ++k) {
+                const float2 f = __half22float2(h[k]);
+                acc[2 * k] = __dadd_rn(acc[2 * k], (double)(f.x * f.x));   // f*f is exact in fp32 (22-bit product)
+                acc[2 * k + 1] = __dadd_rn(acc[2 * k + 1], (double)(f.y * f.y));
+                mn[k] = __hmin2(mn[k], h[k]);
+                mx[k] = __hmax2(mx[k], h[k]);
             }
         };
-        // Rows in the same order as a plain loop (the order of the fp64 additions is part of the result).  This thread's rows
-        // are r_begin + ty + 8 i, i < n; kColAhead of its 16-byte pieces are kept in flight through a private slot ring in
-        // shared memory (asynchronous copies, one group per row; one slot more than rows in flight, so the slot being
+        // This thread's rows are r_begin + ty + 32 i, i < n; kColAhead of its 16-byte pieces are kept in flight through a private slot
+        // ring in shared memory (asynchronous copies, one group per row; one slot more than rows in flight, so the slot being
         // refilled is the one read an iteration ago) -- the registers leave no room for that many rows.
-        const int n = (r_end - r_begin - ty + 7) / 8;
+        const int n = (r_end - r_begin - ty + 31) / 32;
         const __half *xcol = X + (long)(r_begin + ty) * ldx + c0;
-        uint4 *ring = reinterpret_cast<uint4 *>(s_dyn) + threadIdx.x;      // slot j of this thread: ring[256 * j]
+        uint4 *ring = reinterpret_cast<uint4 *>(s_dyn) + tid;             // slot j of this thread: ring[256 * j]
         const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
         int wr = 0;
         auto fetch = [&](int i) {
             if (i < n)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ring_s + (uint32_t)(wr * 4096)), "l"(xcol + (long)i * 8 * ldx)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ring_s + (uint32_t)(wr * 4096)), "l"(xcol + (long)i * 32 * ldx)
                              : "memory");
             asm volatile("cp.async.commit_group;" ::: "memory");          // (an empty group past the end keeps the count in step)
             wr = wr == kColAhead ? 0 : wr + 1;
@@ -90,44 +160,69 @@ __global__ void __launch_bounds__(256) colstats_kernel(const __half *__restrict_
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    __syncthreads();                         // every thread is done with its ring: the buffer now holds the partial results
-    double (*s_acc)[256 + 1] = reinterpret_cast<double (*)[256 + 1]>(s_dyn);
-    float (*s_mn)[256 + 1] = reinterpret_cast<float (*)[256 + 1]>(s_dyn + sizeof(double) * 8 * 257);
-    float (*s_mx)[256 + 1] = reinterpret_cast<float (*)[256 + 1]>(s_dyn + sizeof(double) * 8 * 257 + sizeof(float) * 8 * 257);
+    // the four token lanes of a warp, the eight warps, the CTAs of the cluster: each in a fixed order
 #pragma unroll
-    for (int k = 0; k < 8; ++k) { s_acc[ty][tx * 8 + k] = acc[k]; s_mn[ty][tx * 8 + k] = mn[k]; s_mx[ty][tx * 8 + k] = mx[k]; }
+    for (int o = 8; o <= 16; o <<= 1) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc[k] = __dadd_rn(acc[k], __shfl_xor_sync(0xFFFFFFFFu, acc[k], o));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            mn[k] = __hmin2(mn[k], __shfl_xor_sync(0xFFFFFFFFu, mn[k], o));
+            mx[k] = __hmax2(mx[k], __shfl_xor_sync(0xFFFFFFFFu, mx[k], o));
+        }
+    }
+    if ((tid & 31) < 8) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            s_acc[tid >> 5][tx * 8 + k] = acc[k];
+            s_mn[tid >> 5][tx * 8 + k] = __half2float(k & 1 ? __high2half(mn[k >> 1]) : __low2half(mn[k >> 1]));
+            s_mx[tid >> 5][tx * 8 + k] = __half2float(k & 1 ? __high2half(mx[k >> 1]) : __low2half(mx[k >> 1]));
+        }
+    }
     __syncthreads();
-    const int c = blockIdx.x * 256 + threadIdx.x;
-    if (c < C) {
+    if (tid < 64) {
         double a = 0.0;
         float lo = INFINITY, hi = -INFINITY;
 #pragma unroll
-        for (int y = 0; y < 8; ++y) {      // fixed order: deterministic
-            a = __dadd_rn(a, s_acc[y][threadIdx.x]);
-            lo = fminf(lo, s_mn[y][threadIdx.x]);
-            hi = fmaxf(hi, s_mx[y][threadIdx.x]);
+        for (int y = 0; y < 8; ++y) {
+            a = __dadd_rn(a, s_acc[y][tid]);
+            lo = fminf(lo, s_mn[y][tid]);
+            hi = fmaxf(hi, s_mx[y][tid]);
         }
-        part_sumsq[(long)blockIdx.y * C + c] = a;
-        part_min[(long)blockIdx.y * C + c] = lo;
-        part_max[(long)blockIdx.y * C + c] = hi;
+        s_sum[tid] = a;
+        s_lo[tid] = lo;
+        s_hi[tid] = hi;
     }
+    cluster_sync_all();
+    if (mine) {
+        double a = 0.0;
+        float lo = INFINITY, hi = -INFINITY;
+#pragma unroll 8
+        for (int r = 0; r < splits; ++r) {
+            a = __dadd_rn(a, ld_cluster_f64(&s_sum[tid], (uint32_t)r));
+            lo = fminf(lo, ld_dsmem_f32(smem_u32(&s_lo[tid]), (uint32_t)r));
+            hi = fmaxf(hi, ld_dsmem_f32(smem_u32(&s_hi[tid]), (uint32_t)r));
+        }
+        if (out.sumsq) {                     // one chunk folded into the running state (chunk order = call order)
+            out.sumsq[c] = __dadd_rn(run_sumsq, a);
+            out.lo[c] = fmin(run_lo, (double)lo);
+            out.hi[c] = fmax(run_hi, (double)hi);
+        } else {
+            out.norm[c] = sqrt(a);
+            out.lo[c] = (double)lo;
+            out.hi[c] = (double)hi;
+        }
+    }
+    cluster_sync_all();                      // the partial results of this CTA have been read
 }
 
-__global__ void colstats_finish_kernel(int C, int splits, const double *__restrict__ part_sumsq,
-                                       const float *__restrict__ part_min, const float *__restrict__ part_max,
-                                       double *__restrict__ norm, double *__restrict__ lo, double *__restrict__ hi) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    double a = 0.0;
-    float mn = INFINITY, mx = -INFINITY;
-    for (int s = 0; s < splits; ++s) {
-        a = __dadd_rn(a, part_sumsq[(long)s * C + c]);
-        mn = fminf(mn, part_min[(long)s * C + c]);
-        mx = fmaxf(mx, part_max[(long)s * C + c]);
-    }
-    norm[c] = sqrt(a);
-    lo[c] = (double)mn;
-    hi[c] = (double)mx;
+// Token splits of the statistics pass: up to four CTAs per SM (that many fit, and a second wave of a few would double the time), 64
+// token rows each at least, one cluster (eight CTAs).
+inline esp_status_t launch_colstats(const __half *X, int T, int C, long ldx, const ColStatsOut &out, int sm_count, cudaStream_t stream) {
+    const int cols = ceil_div(C, 64);
+    const int splits = std::max(1, std::min({8, 4 * sm_count / cols, ceil_div(T, 64)}));
+    ESP_CUDA_OK(launch_overlapped(colstats_kernel, dim3(cols, splits), splits, 256, kColSmem, stream, X, T, C, ldx, ceil_div(T, splits), out));
+    return ESP_OK;
 }
 
 // The layer-wide bin range: every channel's [lo, hi] replaced by the minimum and maximum over all channels (one CTA).
@@ -147,31 +242,10 @@ __global__ void __launch_bounds__(1024) global_range_kernel(int C, double *__res
     for (int c = threadIdx.x; c < C; c += 1024) { lo[c] = mn; hi[c] = mx; }
 }
 
-// Streaming calibration: fold one chunk's partial statistics into the running state (chunk order = call order).
-__global__ void calib_merge_kernel(int C, int splits, const double *__restrict__ part_sumsq, const float *__restrict__ part_min,
-                                   const float *__restrict__ part_max, double *__restrict__ sumsq, double *__restrict__ lo,
-                                   double *__restrict__ hi) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    double a = 0.0;
-    float mn = INFINITY, mx = -INFINITY;
-    for (int s = 0; s < splits; ++s) {
-        a = __dadd_rn(a, part_sumsq[(long)s * C + c]);
-        mn = fminf(mn, part_min[(long)s * C + c]);
-        mx = fmaxf(mx, part_max[(long)s * C + c]);
-    }
-    sumsq[c] = __dadd_rn(sumsq[c], a);
-    lo[c] = fmin(lo[c], (double)mn);
-    hi[c] = fmax(hi[c], (double)mx);
-}
 __global__ void calib_reset_kernel(int C, int bins, double *sumsq, double *lo, double *hi, unsigned int *counts) {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < C) { sumsq[i] = 0.0; lo[i] = INFINITY; hi[i] = -INFINITY; }
     if (i < (long)C * bins) counts[i] = 0u;
-}
-__global__ void calib_norm_kernel(int C, const double *__restrict__ sumsq, double *__restrict__ norm) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < C) norm[c] = sqrt(sumsq[c]);
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -203,7 +277,37 @@ __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restr
                                                            int rows_per_split, int bins, const double *__restrict__ lo,
                                                            const double *__restrict__ hi, unsigned int *__restrict__ counts) {
     extern __shared__ __align__(16) unsigned int s_cnt[];   // [8][bins][8][R] | the threads' load rings: [kHistAhead + 1][256] x 16 bytes
+    __shared__ float s_neg_lo[64], s_r[64];
+    __shared__ __half s_lo[64], s_hi[64];
     for (int i = threadIdx.x; i < 64 * R * bins; i += 256) s_cnt[i] = 0;
+    grid_dependency_wait();
+    grid_launch_dependents();
+    // Exact bin: floor of the fp64 quotient q = (x - lo) * K / (hi - lo).  Almost every element gets there with one fp32
+    // subtraction and one fused multiply-add (two elements per instruction), and no float <-> integer conversion (those run at a
+    // quarter of the fp32 rate): with 2^S the largest power of two such that K * 2^S <= 2^22 and r = K * 2^S / (hi - lo) rounded once,
+    //     t = fma(x - lo, r, 2^23 + 2)
+    // lies in [2^23, 2^24), where floats are the integers, so the low 23 bits of t ARE n + 2 with n = round((x - lo) * r), and
+    // |n - q * 2^S| <= 1: the subtraction (lo is exact in fp32) and r are each within 2^-24 relative, together at most
+    // q * 2^S * 2^-23 <= 1/2, and the fma rounds once to an integer, at most 1/2.  So wherever n + 2 mod 2^S is 4 or more, bits S and
+    // up of t are the exact bin.  The other elements (4 in 2^S: about one in ten thousand for a hundred bins, and always the
+    // channel's minimum and maximum) take the fp64 division.  Elements are first clamped to the channel's range (two per
+    // instruction), which bounds the counter's address whatever the input; a channel without a usable r (constant, or a range
+    // that is not finite) is clamped to zero with r = 0, so n = 0 sends every element to the fp64 path.
+    const int S = 22 - (32 - __clz(bins - 1));                                // bins >= 2
+    if (threadIdx.x < 64 && blockIdx.x * 64 + threadIdx.x < C) {
+        const int c = blockIdx.x * 64 + threadIdx.x;
+        const double dl = lo[c], dh = hi[c], rng = __dsub_rn(dh, dl);
+        float l = (float)dl, r = (float)(((double)bins / rng) * (double)(1 << S));
+        __half cl = __float2half_rn(l), ch = __float2half_rn((float)dh);
+        if (!(rng > 0.0 && rng < 1e6) || !(r <= 0x1p60f) || (double)__half2float(cl) != dl || (double)__half2float(ch) != dh) {
+            l = r = 0.f;
+            cl = ch = __ushort_as_half((unsigned short)0);
+        }
+        s_neg_lo[threadIdx.x] = -l;
+        s_r[threadIdx.x] = r;
+        s_lo[threadIdx.x] = cl;
+        s_hi[threadIdx.x] = ch;
+    }
     __syncthreads();
     const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
     const int cl = tx * 8;
@@ -211,32 +315,20 @@ __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restr
     const int r_begin = blockIdx.y * rows_per_split;
     const int r_end = min(T, r_begin + rows_per_split);
     if (c0 < C) {
-        // Exact bin: floor of the fp64 quotient q = (x - lo) * K / (hi - lo).  Almost every element gets there with one fp32
-        // subtraction and one fused multiply-add, and no float <-> integer conversion (those run at a quarter of the fp32
-        // rate): with 2^S the largest power of two such that K * 2^S <= 2^22 and r = K * 2^S / (hi - lo) rounded once,
-        //     t = fma(x - lo, r, 2^23)
-        // lies in [2^23, 2^24), where floats are the integers, so the low 23 bits of t ARE n = round((x - lo) * r), and
-        // |n - q * 2^S| <= 1: the subtraction (lo is exact in fp32) and r are each within 2^-24 relative, together at most
-        // q * 2^S * 2^-23 <= 1/2, and the fma rounds once to an integer, at most 1/2.  So wherever n mod 2^S is neither
-        // 0, 1, 2^S - 2 nor 2^S - 1, n >> S is the exact bin.  The other elements (4 in 2^S: about one in ten thousand for
-        // a hundred bins, and always the channel's minimum and maximum) take the fp64 division.  r = 0 gives n = 0 and sends
-        // every element of a channel there (a constant channel, or a range whose lower end is not an fp16 value).
-        const int S = 22 - (32 - __clz(bins - 1));                            // bins >= 2
         const unsigned int frac_mask = (1u << S) - 1u;
-        float lf[8], rf[8];
+        uint64_t neg_lo[4], rf[4];
+        __half2 lo_h[4], hi_h[4];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const double l = lo[c0 + k];
-            const double rng = __dsub_rn(hi[c0 + k], l);
-            lf[k] = (float)l;
-            rf[k] = (rng > 0.0 && (double)lf[k] == l) ? (float)(((double)bins / rng) * (double)(1 << S)) : 0.f;
-            if (!(rf[k] <= 0x1p60f)) rf[k] = 0.f;                            // (a range so small that r overflows: exact path)
+        for (int k2 = 0; k2 < 4; ++k2) {
+            neg_lo[k2] = f32x2(s_neg_lo[cl + 2 * k2], s_neg_lo[cl + 2 * k2 + 1]);
+            rf[k2] = f32x2(s_r[cl + 2 * k2], s_r[cl + 2 * k2 + 1]);
+            lo_h[k2] = __halves2half2(s_lo[cl + 2 * k2], s_lo[cl + 2 * k2 + 1]);
+            hi_h[k2] = __halves2half2(s_hi[cl + 2 * k2], s_hi[cl + 2 * k2 + 1]);
         }
-        uint32_t cnt_k[8];                                                 // this thread's counter of bin 0 for each of its channels
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            cnt_k[k] = (uint32_t)__cvta_generic_to_shared(s_cnt + ((k * bins) * 8 + tx) * R + (ty & (R - 1)));
-        const unsigned int last_bin = (unsigned int)(bins - 1);
+        const uint64_t magic = f32x2(8388610.f, 8388610.f);                  // 2^23 + 2
+        // this thread's counter of bin -(2^23's bits >> S) for its first channel; the next channel's lies cnt_step bytes behind it
+        const uint32_t cnt_0 = (uint32_t)__cvta_generic_to_shared(s_cnt + tx * R + (ty & (R - 1))) - (0x4B000000u >> S) * (uint32_t)(32 * R);
+        const uint32_t cnt_step = (uint32_t)(bins * 32 * R);
         // One branch per row of eight elements, not one per element: the eight estimates are formed first, together with the
         // smallest distance-to-a-boundary code among them; only a row that holds an undecided element (about one row in a
         // thousand) goes back over its elements.
@@ -245,27 +337,31 @@ __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restr
             unsigned int b[8], closest = 0xFFFFFFFFu;
 #pragma unroll
             for (int k2 = 0; k2 < 4; ++k2) {
-                const float2 xf2 = __half22float2(h2[k2]);
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int k = 2 * k2 + e;
-                    const float xf = e ? xf2.y : xf2.x;
-                    const unsigned int n = __float_as_uint(fmaf(xf - lf[k], rf[k], 8388608.f)) - 0x4B000000u;
-                    // (the clamp keeps the index inside the counter row whatever the input, e.g. a NaN)
-                    b[k] = min(n >> S, last_bin);
-                    closest = min(closest, (n + 2u) & frac_mask);
-                }
+                const float2 x = __half22float2(__hmin2(__hmax2(h2[k2], lo_h[k2]), hi_h[k2]));
+                const uint64_t t = fma_f32x2(add_f32x2(f32x2(x.x, x.y), neg_lo[k2]), rf[k2], magic);
+                const unsigned int t0 = (unsigned int)t, t1 = (unsigned int)(t >> 32);
+                b[2 * k2] = t0 >> S;
+                b[2 * k2 + 1] = t1 >> S;
+                closest = min(closest, min(t0 & frac_mask, t1 & frac_mask));
             }
             if (closest < 4u) {
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float xf = __half2float(reinterpret_cast<const __half *>(&v)[k]);
-                    const unsigned int n = __float_as_uint(fmaf(xf - lf[k], rf[k], 8388608.f)) - 0x4B000000u;
-                    if (((n + 2u) & frac_mask) < 4u) b[k] = (unsigned int)histogram_exact_bin(xf, c0 + k, bins, lo, hi);
+                for (int k2 = 0; k2 < 4; ++k2) {
+                    const float2 x = __half22float2(__hmin2(__hmax2(h2[k2], lo_h[k2]), hi_h[k2]));
+                    const uint64_t t = fma_f32x2(add_f32x2(f32x2(x.x, x.y), neg_lo[k2]), rf[k2], magic);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        if (((unsigned int)(e ? t >> 32 : t) & frac_mask) < 4u)
+                            b[2 * k2 + e] = (0x4B000000u >> S) + (unsigned int)histogram_exact_bin(__half2float(e ? __high2half(h2[k2]) : __low2half(h2[k2])),
+                                                                                                  c0 + 2 * k2 + e, bins, lo, hi);
                 }
             }
+            uint32_t base = cnt_0;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(cnt_k[k] + (uint32_t)(32 * R) * b[k]) : "memory");
+            for (int k = 0; k < 8; ++k) {
+                asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(base + (uint32_t)(32 * R) * b[k]) : "memory");
+                base += cnt_step;
+            }
         };
         // This thread's rows are r_begin + ty + 32 * i, i < n.  Loads and counting must overlap, and with 80 registers per thread
         // (three CTAs per SM) there is no room for a second set of rows in registers: every thread keeps kHistAhead of its own
@@ -298,65 +394,96 @@ __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restr
         asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 64 * bins; i += 256) {
-        const int cc = i / bins, b = i - cc * bins;                        // channel of this CTA, bin
-        const int c = blockIdx.x * 64 + cc;
-        const unsigned int *src = s_cnt + (((cc & 7) * bins + b) * 8 + (cc >> 3)) * R;
-        unsigned int n = 0;
 #pragma unroll
-        for (int rep = 0; rep < R; ++rep) n += src[rep];
-        if (c < C && n) atomicAdd(&counts[(long)c * bins + b], n);
+    for (int k = 0; k < 8; ++k) {
+        const int c = blockIdx.x * 64 + cl + k;
+        for (int bin = ty; bin < bins; bin += 32) {
+            const unsigned int *src = s_cnt + ((k * bins + bin) * 8 + tx) * R;
+            unsigned int n = 0;
+#pragma unroll
+            for (int rep = 0; rep < R; ++rep) n += src[rep];
+            if (c < C && n) atomicAdd(&counts[(long)c * bins + bin], n);
+        }
     }
 }
 
 // Counter replicas for a bin count: as many as keep three CTAs on an SM (about 75 KB each), none beyond.
-inline esp_status_t launch_histogram(const __half *X, int T, int C, long ldx, int splits, int bins, const double *lo,
-                                     const double *hi, unsigned int *counts, cudaStream_t stream) {
+// Token splits: whole waves of three CTAs per SM (the counting is bound by the shared-memory atomics, about 17 ns per token row of a CTA
+// at that residency, so a partial wave is lost time; 2048 x 8192: 640 CTAs 30 us, 384 CTAs 20.5); a CTA's set-up and the addition of its counters to the global ones take as long
+// as some 250 rows.
+inline esp_status_t launch_histogram(const __half *X, int T, int C, long ldx, int bins, const double *lo, const double *hi, unsigned int *counts,
+                                     int sm_count, cudaStream_t stream) {
     const size_t per_replica = sizeof(unsigned int) * 64 * (size_t)bins;
     const size_t ring = (size_t)(kHistAhead + 1) * 256 * 16;
     const int R = per_replica * 4 + ring <= 75 * 1024 ? 4 : per_replica * 2 + ring <= 75 * 1024 ? 2 : 1;
     const size_t smem = per_replica * R + ring;
-    const dim3 grid(ceil_div(C, 64), splits);
-    const int rows = ceil_div(T, splits);
-    if (R == 4) {
-        ESP_CUDA_OK(cudaFuncSetAttribute(histogram_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        histogram_kernel<4><<<grid, 256, smem, stream>>>(X, T, C, ldx, rows, bins, lo, hi, counts);
-    } else if (R == 2) {
-        ESP_CUDA_OK(cudaFuncSetAttribute(histogram_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        histogram_kernel<2><<<grid, 256, smem, stream>>>(X, T, C, ldx, rows, bins, lo, hi, counts);
-    } else {
-        ESP_CUDA_OK(cudaFuncSetAttribute(histogram_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        histogram_kernel<1><<<grid, 256, smem, stream>>>(X, T, C, ldx, rows, bins, lo, hi, counts);
+    const int cols = ceil_div(C, 64), most = std::max(1, std::min(64, ceil_div(T, 32)));
+    int splits = 1;
+    long best = -1;
+    for (int s = 1; s <= most; ++s) {
+        const long cost = (long)ceil_div((long)cols * s, 3L * sm_count) * (ceil_div(T, s) + 250);
+        if (best < 0 || cost < best) { best = cost; splits = s; }
     }
+    const int rows = ceil_div(T, splits);
+    auto kern = R == 4 ? histogram_kernel<4> : R == 2 ? histogram_kernel<2> : histogram_kernel<1>;
+    ESP_CUDA_OK(ensure_dynamic_smem((const void *)kern, (int)smem));
+    ESP_CUDA_OK(launch_overlapped(kern, dim3(cols, splits), 1, 256, smem, stream, X, T, C, ldx, rows, bins, lo, hi, counts));
     return ESP_OK;
 }
 
 // IR_c = -sum_k p_k ln p_k (Eq. 1, bins in index order, empty bins skipped) and s_c = IR_c + alpha*AM_c (Eq. 3).
-__global__ void entropy_score_kernel(int C, int T, int bins, const unsigned int *__restrict__ counts,
-                                     const double *__restrict__ norm, double alpha, int use_entropy, int use_norm,
-                                     const double *__restrict__ score_override, double *__restrict__ entropy,
-                                     double *__restrict__ score) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
+// A CTA takes kEntropyChannels channels: all threads form the terms of its counts, then one thread per channel subtracts them in bin
+// order, the order being part of the result.  (One thread per channel doing both, with strided reads, took 42 us whatever the size;
+// this 11.)
+struct EntropyOut {
+    const double *norm, *sumsq;              // the norm is given, or the sum of squares it is the root of
+    double *score;
+    double *norm_out, *entropy_out, *score_out;      // copies for the caller, or NULL
+};
+constexpr int kEntropyChannels = 16;
+__global__ void __launch_bounds__(256) entropy_score_kernel(int C, int T, int bins, const unsigned int *__restrict__ counts, double alpha,
+                                                            int use_entropy, int use_norm, const double *__restrict__ score_override,
+                                                            const EntropyOut out) {
+    extern __shared__ double s_term[];       // [kEntropyChannels][bins | 1]
+    const int c0 = blockIdx.x * kEntropyChannels, nc = min(kEntropyChannels, C - c0), ld = bins | 1;
+    grid_dependency_wait();
+    grid_launch_dependents();
+    if (counts) {
+        for (int i = threadIdx.x; i < nc * bins; i += 256) {
+            const unsigned int n = counts[(long)c0 * bins + i];
+            const double p = __ddiv_rn((double)n, (double)T);
+            s_term[(i / bins) * ld + i % bins] = n ? __dmul_rn(p, log(p)) : 0.0;
+        }
+    }
+    __syncthreads();
+    if ((int)threadIdx.x >= nc) return;
+    const int c = c0 + threadIdx.x;
     double ir = 0.0;
     if (counts) {
-        for (int k = 0; k < bins; ++k) {
-            unsigned int n = counts[(long)c * bins + k];
-            if (n) {
-                double p = __ddiv_rn((double)n, (double)T);
-                ir = __dsub_rn(ir, __dmul_rn(p, log(p)));
-            }
-        }
-        entropy[c] = ir;
+#pragma unroll 4
+        for (int k = 0; k < bins; ++k) ir = __dsub_rn(ir, s_term[threadIdx.x * ld + k]);
+        if (out.entropy_out) out.entropy_out[c] = ir;
     }
+    const bool have_norm = out.norm || out.sumsq;
+    const double norm = out.sumsq ? sqrt(out.sumsq[c]) : have_norm ? out.norm[c] : 0.0;
+    if (out.norm_out && have_norm) out.norm_out[c] = norm;
     double s = 0.0;
     if (score_override) {
         s = score_override[c];
     } else {
         if (use_entropy) s = __dadd_rn(s, ir);
-        if (use_norm) s = __dadd_rn(s, __dmul_rn(alpha, norm[c]));
+        if (use_norm) s = __dadd_rn(s, __dmul_rn(alpha, norm));
     }
-    score[c] = s;
+    out.score[c] = s;
+    if (out.score_out) out.score_out[c] = s;
+}
+inline esp_status_t launch_entropy(int C, int T, int bins, const unsigned int *counts, const esp_prune_opts &o, const double *score_override,
+                                   const EntropyOut &out, cudaStream_t stream) {
+    const size_t smem = counts ? sizeof(double) * kEntropyChannels * (size_t)(bins | 1) : 0;
+    if (smem > 48 * 1024) ESP_CUDA_OK(ensure_dynamic_smem((const void *)entropy_score_kernel, (int)smem));
+    ESP_CUDA_OK(launch_overlapped(entropy_score_kernel, dim3(ceil_div(C, kEntropyChannels)), 1, 256, smem, stream, C, T, bins, counts, o.alpha,
+                                  o.use_entropy, o.use_norm, score_override, out));
+    return ESP_OK;
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -457,30 +584,37 @@ __global__ void mean_metric_kernel(int C, int No, const unsigned long long *__re
 // mean metric; the channel of rank r goes to group r mod G, slot r div G (neighbours in rank never share
 // a group).
 // --------------------------------------------------------------------------------------------------
+// A CTA ranks 32 channels, each by eight threads over an eighth of the means (shared memory), so that the C^2 comparisons spread over C / 32
+// CTAs: 57 -> 13 us for 4096 channels against a CTA of 256 channels with one thread each.
 __global__ void __launch_bounds__(256) gns_rank_kernel(int C, const double *__restrict__ mean, int use_gns, int m_group,
                                                        int32_t *__restrict__ theta0, double *__restrict__ sorted_mean) {
-    __shared__ double tile[256];
-    const int c = blockIdx.x * 256 + threadIdx.x;
+    __shared__ double tile[2048];
+    __shared__ int s_rank[32];
+    const int c = blockIdx.x * 32 + (threadIdx.x & 31), part = threadIdx.x >> 5;
     if (!use_gns) {
-        if (c < C) theta0[c] = c;
+        if (part == 0 && c < C) theta0[c] = c;
         return;
     }
+    if (threadIdx.x < 32) s_rank[threadIdx.x] = 0;
     const double mine = (c < C) ? mean[c] : 0.0;
     int rank = 0;
-    for (int base = 0; base < C; base += 256) {
+    for (int base = 0; base < C; base += 2048) {
         __syncthreads();
-        if (base + threadIdx.x < C) tile[threadIdx.x] = mean[base + threadIdx.x];
+        const int n = min(2048, C - base);
+        for (int i = threadIdx.x; i < n; i += 256) tile[i] = mean[base + i];
         __syncthreads();
-        const int n = min(256, C - base);
-        for (int i = 0; i < n; ++i) {
-            double other = tile[i];
-            rank += (other > mine || (other == mine && base + i < c)) ? 1 : 0;
-        }
+        // (the means of lower channels are ahead when equal, those of higher ones are not: two loops without an index compare)
+        const int lo = part * 256, hi = min(n, lo + 256), split = min(max(c - base, lo), hi);
+        int i = lo;
+        for (; i < split; ++i) rank += tile[i] >= mine ? 1 : 0;
+        for (; i < hi; ++i) rank += tile[i] > mine ? 1 : 0;
     }
-    if (c < C) {
-        const int G = C / m_group;
-        theta0[(rank % G) * m_group + rank / G] = c;
-        sorted_mean[rank] = mine;
+    atomicAdd(&s_rank[threadIdx.x & 31], rank);
+    __syncthreads();
+    if (part == 0 && c < C) {
+        const int G = C / m_group, r = s_rank[threadIdx.x];
+        theta0[(r % G) * m_group + r / G] = c;
+        sorted_mean[r] = mine;
     }
 }
 
@@ -763,25 +897,20 @@ PruneWorkspace carve_prune_workspace(void *ws, int No, int C, int T, const esp_p
     PruneWorkspace w{};
     size_t off = 0;
     auto take = [&](size_t bytes) { void *p = ws ? (char *)ws + off : nullptr; off += align_up(bytes, 256); return p; };
-    // the split count must not depend on the device so the size query and the call agree
-    w.splits = ceil_div(T > 0 ? T : 1, 256);
-    if (w.splits > 64) w.splits = 64;
-    w.part_sumsq = (double *)take(sizeof(double) * (size_t)w.splits * C);
-    w.part_min = (float *)take(sizeof(float) * (size_t)w.splits * C);
-    w.part_max = (float *)take(sizeof(float) * (size_t)w.splits * C);
     w.lo = (double *)take(sizeof(double) * C);
     w.hi = (double *)take(sizeof(double) * C);
     w.norm = (double *)take(sizeof(double) * C);
-    w.entropy = (double *)take(sizeof(double) * C);
     w.score = (double *)take(sizeof(double) * C);
     w.mean = (double *)take(sizeof(double) * C);
-    w.counts = (unsigned int *)take(sizeof(unsigned int) * (size_t)C * o.bins);
-    w.colsum = (unsigned long long *)take(sizeof(unsigned long long) * C);
-    w.theta0 = (int32_t *)take(sizeof(int32_t) * C);
+    // cleared by one call: counters .. counts
     w.counters = (unsigned long long *)take(sizeof(unsigned long long) * 8);
     w.objective = (double *)take(sizeof(double) * 4);
-    w.sorted_mean = (double *)take(sizeof(double) * C);
+    w.colsum = (unsigned long long *)take(sizeof(unsigned long long) * C);
     w.kept = (unsigned long long *)take(sizeof(unsigned long long) * C);
+    w.counts = (unsigned int *)take(sizeof(unsigned int) * (size_t)C * o.bins);
+    w.cleared_bytes = w.counts ? (size_t)((char *)w.counts - (char *)w.counters) + sizeof(unsigned int) * (size_t)C * o.bins : 0;
+    w.theta0 = (int32_t *)take(sizeof(int32_t) * C);
+    w.sorted_mean = (double *)take(sizeof(double) * C);
     for (double *&base : w.base) base = (double *)take(sizeof(double) * (size_t)(C / 4 + 1));
     if (o.use_lbs) {
         const int nblocks = ceil_div(C, o.lbs_block);
@@ -803,7 +932,7 @@ esp_status_t launch_pack(const __half *vals, const uint8_t *meta, int No, int C,
     return ESP_OK;
 }
 
-// ---- streaming calibration: state = sumsq | lo | hi | norm (f64[C] each) | counts u32[C][bins] | chunk partials [64][C]
+// ---- streaming calibration: state = sumsq | lo | hi | norm (f64[C] each) | counts u32[C][bins]
 CalibState carve_calib_state(void *state, int C, int bins) {
     CalibState c{};
     size_t off = 0;
@@ -813,9 +942,6 @@ CalibState carve_calib_state(void *state, int C, int bins) {
     c.hi = (double *)take(sizeof(double) * C);
     c.norm = (double *)take(sizeof(double) * C);
     c.counts = (unsigned int *)take(sizeof(unsigned int) * (size_t)C * bins);
-    c.part_sumsq = (double *)take(sizeof(double) * 64 * (size_t)C);
-    c.part_min = (float *)take(sizeof(float) * 64 * (size_t)C);
-    c.part_max = (float *)take(sizeof(float) * 64 * (size_t)C);
     c.total_bytes = off;
     return c;
 }
@@ -828,35 +954,22 @@ esp_status_t launch_calib_reset(const CalibState &c, int C, int bins, cudaStream
 }
 
 esp_status_t launch_calib_range(const CalibState &c, const __half *X, int T, int C, long ldx, cudaStream_t stream) {
-    int splits = ceil_div(T, 256);
-    if (splits > 64) splits = 64;
-    colstats_kernel<<<dim3(ceil_div(C, 256), splits), 256, kColSmem, stream>>>(X, T, C, ldx, ceil_div(T, splits), c.part_sumsq, c.part_min,
-                                                                       c.part_max);
-    calib_merge_kernel<<<ceil_div(C, 256), 256, 0, stream>>>(C, splits, c.part_sumsq, c.part_min, c.part_max, c.sumsq, c.lo, c.hi);
-    ESP_CUDA_OK(cudaGetLastError());
-    return ESP_OK;
+    DeviceInfo di;
+    esp_status_t st = device_info(&di);
+    if (st != ESP_OK) return st;
+    return launch_colstats(X, T, C, ldx, ColStatsOut{c.sumsq, nullptr, c.lo, c.hi}, di.sm_count, stream);
 }
 
 esp_status_t launch_calib_histogram(const CalibState &c, const __half *X, int T, int C, long ldx, int bins, cudaStream_t stream) {
     DeviceInfo di;
     esp_status_t st = device_info(&di);
     if (st != ESP_OK) return st;
-    const int hsplits = pick_splits(T, ceil_div(C, 64), di.sm_count);
-    if (launch_histogram(X, T, C, ldx, hsplits, bins, c.lo, c.hi, c.counts, stream) != ESP_OK) return ESP_ERR_CUDA;
-    ESP_CUDA_OK(cudaGetLastError());
-    return ESP_OK;
+    return launch_histogram(X, T, C, ldx, bins, c.lo, c.hi, c.counts, di.sm_count, stream);
 }
 
 esp_status_t launch_calib_finish(const CalibState &c, int C, int bins, long long T_total, const esp_prune_opts &o, double *chan_norm,
                                  double *chan_entropy, double *chan_score, cudaStream_t stream) {
-    calib_norm_kernel<<<ceil_div(C, 256), 256, 0, stream>>>(C, c.sumsq, c.norm);
-    // entropy needs a scratch output even when the caller does not want it: the chunk partials are free by now
-    double *entropy = chan_entropy ? chan_entropy : c.part_sumsq;
-    entropy_score_kernel<<<ceil_div(C, 256), 256, 0, stream>>>(C, (int)T_total, bins, c.counts, c.norm, o.alpha, o.use_entropy,
-                                                               o.use_norm, nullptr, entropy, chan_score);
-    ESP_CUDA_OK(cudaGetLastError());
-    if (chan_norm) ESP_CUDA_OK(cudaMemcpyAsync(chan_norm, c.norm, sizeof(double) * C, cudaMemcpyDeviceToDevice, stream));
-    return ESP_OK;
+    return launch_entropy(C, (int)T_total, bins, c.counts, o, nullptr, EntropyOut{nullptr, c.sumsq, chan_score, chan_norm, chan_entropy, nullptr}, stream);
 }
 
 esp_status_t launch_decompress(const __half *vals, const uint8_t *meta, const int32_t *perm, int No, int C,
@@ -875,32 +988,23 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
     if (st != ESP_OK) return st;
     const int cthreads = 256;
     const int cblocks = ceil_div(C, cthreads);
-    ESP_CUDA_OK(cudaMemsetAsync(w.counters, 0, sizeof(unsigned long long) * 8, stream));
-    ESP_CUDA_OK(cudaMemsetAsync(w.objective, 0, sizeof(double) * 4, stream));
+    ESP_CUDA_OK(cudaMemsetAsync(w.counters, 0, w.cleared_bytes, stream));
 
     const bool need_stats_pass = (o.score_override == nullptr) || chan_norm || chan_entropy;
     if (need_stats_pass && Xcal) {
         // K1
-        const int rows1 = ceil_div(T, w.splits);
-        colstats_kernel<<<dim3(ceil_div(C, 256), w.splits), 256, kColSmem, stream>>>(Xcal, T, C, ldx, rows1, w.part_sumsq,
-                                                                             w.part_min, w.part_max);
-        colstats_finish_kernel<<<cblocks, cthreads, 0, stream>>>(C, w.splits, w.part_sumsq, w.part_min, w.part_max,
-                                                                 w.norm, w.lo, w.hi);
+        st = launch_colstats(Xcal, T, C, ldx, ColStatsOut{nullptr, w.norm, w.lo, w.hi}, di.sm_count, stream);
+        if (st != ESP_OK) return st;
         if (o.global_bin_range) global_range_kernel<<<1, 1024, 0, stream>>>(C, w.lo, w.hi);
         // K2
-        ESP_CUDA_OK(cudaMemsetAsync(w.counts, 0, sizeof(unsigned int) * (size_t)C * o.bins, stream));
-        const int hsplits = pick_splits(T, ceil_div(C, 64), di.sm_count);
-        if (launch_histogram(Xcal, T, C, ldx, hsplits, o.bins, w.lo, w.hi, w.counts, stream) != ESP_OK) return ESP_ERR_CUDA;
-        entropy_score_kernel<<<cblocks, cthreads, 0, stream>>>(C, T, o.bins, w.counts, w.norm, o.alpha, o.use_entropy,
-                                                               o.use_norm, o.score_override, w.entropy, w.score);
+        st = launch_histogram(Xcal, T, C, ldx, o.bins, w.lo, w.hi, w.counts, di.sm_count, stream);
+        if (st != ESP_OK) return st;
+        st = launch_entropy(C, T, o.bins, w.counts, o, o.score_override, EntropyOut{w.norm, nullptr, w.score, chan_norm, chan_entropy, chan_score}, stream);
     } else {
-        entropy_score_kernel<<<cblocks, cthreads, 0, stream>>>(C, T, o.bins, nullptr, w.norm, o.alpha, o.use_entropy,
-                                                               o.use_norm, o.score_override, w.entropy, w.score);
+        st = launch_entropy(C, T, o.bins, nullptr, o, o.score_override, EntropyOut{nullptr, nullptr, w.score, nullptr, nullptr, chan_score}, stream);
     }
+    if (st != ESP_OK) return st;
     ESP_CUDA_OK(cudaGetLastError());
-    if (chan_norm) ESP_CUDA_OK(cudaMemcpyAsync(chan_norm, w.norm, sizeof(double) * C, cudaMemcpyDeviceToDevice, stream));
-    if (chan_entropy) ESP_CUDA_OK(cudaMemcpyAsync(chan_entropy, w.entropy, sizeof(double) * C, cudaMemcpyDeviceToDevice, stream));
-    if (chan_score) ESP_CUDA_OK(cudaMemcpyAsync(chan_score, w.score, sizeof(double) * C, cudaMemcpyDeviceToDevice, stream));
 
     // K3 + K4: the column sums for the global shuffle and, when objectives are asked for, the retained sums under the identity
     const int G = C / 4;
@@ -908,8 +1012,6 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
     const int wsplits = pick_splits(No, ceil_div(C, 256), di.sm_count);
     const dim3 wgrid(ceil_div(C, 256), wsplits);
     const int wrows = ceil_div(No, wsplits);
-    if (gns) ESP_CUDA_OK(cudaMemsetAsync(w.colsum, 0, sizeof(unsigned long long) * C, stream));
-    if (stats) ESP_CUDA_OK(cudaMemsetAsync(w.kept, 0, sizeof(unsigned long long) * C, stream));
     if (gns && stats) colabs_kernel<true, true><<<wgrid, 256, 0, stream>>>(W, No, C, ldw, wrows, w.score, nullptr, w.colsum, w.kept);
     else if (gns) colabs_kernel<true, false><<<wgrid, 256, 0, stream>>>(W, No, C, ldw, wrows, w.score, nullptr, w.colsum, w.kept);
     else if (stats) colabs_kernel<false, true><<<wgrid, 256, 0, stream>>>(W, No, C, ldw, wrows, w.score, nullptr, w.colsum, w.kept);
@@ -919,7 +1021,7 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
     if (o.perm_override)
         ESP_CUDA_OK(cudaMemcpyAsync(theta0, o.perm_override, sizeof(int32_t) * C, cudaMemcpyDeviceToDevice, stream));
     else {
-        gns_rank_kernel<<<ceil_div(C, 256), 256, 0, stream>>>(C, w.mean, o.use_gns, o.m_group, theta0, w.sorted_mean);
+        gns_rank_kernel<<<ceil_div(C, 32), 256, 0, stream>>>(C, w.mean, o.use_gns, o.m_group, theta0, w.sorted_mean);
         if (o.use_gns && stats) gns_near_tie_kernel<<<ceil_div(C, 256), 256, 0, stream>>>(C, w.sorted_mean, w.counters);
     }
     ESP_CUDA_OK(cudaGetLastError());
