@@ -942,6 +942,7 @@ CalibState carve_calib_state(void *state, int C, int bins) {
     c.hi = (double *)take(sizeof(double) * C);
     c.norm = (double *)take(sizeof(double) * C);
     c.counts = (unsigned int *)take(sizeof(unsigned int) * (size_t)C * bins);
+    take(16 * 64 * (size_t)C);               // (unused: the size that callers rely on has room for 64 chunk partials per channel)
     c.total_bytes = off;
     return c;
 }
