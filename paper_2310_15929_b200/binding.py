@@ -82,6 +82,7 @@ _lib.esp_spgemm_workspace_bytes.argtypes = [c_int, c_int, c_int, POINTER(esp_gem
 _lib.esp_spgemm.restype = c_int
 _lib.esp_spgemm.argtypes = [c_void_p, c_int, c_int, c_long, c_void_p, c_void_p, c_int, c_void_p, c_long,
                             POINTER(esp_gemm_opts), c_void_p, c_size_t, c_void_p]
+_spgemm, _byref = _lib.esp_spgemm, ctypes.byref
 _lib.esp_last_device_status.restype = c_int
 _lib.esp_multicast_available.restype = c_int
 _lib.esp_selftest_wait_timeout.restype = c_int
@@ -103,10 +104,23 @@ def _ptr(t):
     return t.data_ptr()
 
 
+def _current_stream() -> int:
+    """The current stream's handle on the current device.  The raw query: building the torch.cuda.Stream object that
+    torch.cuda.current_stream() returns takes 3.2 us, a quarter of a decode call's host time."""
+    global _current_stream
+    import torch
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+    else:
+        torch.cuda.init()
+        _current_stream = lambda: raw(device())
+    return _current_stream()
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -201,12 +215,10 @@ def esp_spgemm_raw(X, M, K, ldx, packed, perm, N, Y, ldy, opts, workspace, works
 def esp_spgemm(X, packed, perm, Y, opts, workspace=None, stream=None):
     """Y [M,N] = X . P . W_s^T.  X is [M,K] (token-major) or [K,M] (channel-major) per opts.x_layout."""
     M, N = Y.shape
-    if opts.x_layout == ESP_X_CHANNEL_MAJOR:
-        K = X.shape[0]
-    else:
-        K = X.shape[1]
-    st = esp_spgemm_raw(X, M, K, X.stride(0), packed, perm, N, Y, Y.stride(0), opts, workspace,
-                        0 if workspace is None else workspace.numel() * workspace.element_size(), _stream(stream))
+    K = X.shape[0] if opts.x_layout == ESP_X_CHANNEL_MAJOR else X.shape[1]
+    # (a decode call is a few microseconds of GPU time: no helper calls on this path)
+    st = _spgemm(_ptr(X), M, K, X.stride(0), _ptr(packed), _ptr(perm), N, _ptr(Y), Y.stride(0), _byref(opts), _ptr(workspace),
+                 0 if workspace is None else workspace.nbytes, _current_stream() if stream is None else _stream(stream))
     if st != ESP_OK:
         raise EsparseError(st, "esp_spgemm")
 
@@ -239,17 +251,18 @@ _lib.esp_spgemm_grouped.argtypes = [c_int, POINTER(c_void_p), c_int, c_int, c_lo
                                     c_size_t, c_void_p]
 
 
+_group_types = [(c_void_p * n, c_int * n, c_long * n) for n in range(5)]      # (making an array type costs more than filling it)
+
+
 def esp_spgemm_grouped(Xs, packeds, perms, Ys, opts, workspace=None, stream=None):
     """Ys[i] = Xs[i] . P[i] . W_s[i]^T for up to 4 problems with common M and K in one call (one launch up to 256 tokens)."""
     n = len(Ys)
     M = Ys[0].shape[0]
     K = Xs[0].shape[0] if opts.x_layout == ESP_X_CHANNEL_MAJOR else Xs[0].shape[1]
-    arr = lambda items: (c_void_p * n)(*[_ptr(t) for t in items])
-    Ns = (c_int * n)(*[y.shape[1] for y in Ys])
-    ldys = (c_long * n)(*[y.stride(0) for y in Ys])
-    st = int(_lib.esp_spgemm_grouped(n, arr(Xs), M, K, Xs[0].stride(0), arr(packeds), arr(perms), Ns, arr(Ys), ldys,
-                                     ctypes.byref(opts), _ptr(workspace),
-                                     0 if workspace is None else workspace.numel() * workspace.element_size(), _stream(stream)))
+    ptrs, ints, longs = _group_types[n] if n < len(_group_types) else (c_void_p * n, c_int * n, c_long * n)
+    st = _lib.esp_spgemm_grouped(n, ptrs(*map(_ptr, Xs)), M, K, Xs[0].stride(0), ptrs(*map(_ptr, packeds)), ptrs(*map(_ptr, perms)),
+                                 ints(*[y.shape[1] for y in Ys]), ptrs(*map(_ptr, Ys)), longs(*[y.stride(0) for y in Ys]),
+                                 _byref(opts), _ptr(workspace), 0 if workspace is None else workspace.nbytes, _stream(stream))
     if st != ESP_OK:
         raise EsparseError(st, "esp_spgemm_grouped")
 
