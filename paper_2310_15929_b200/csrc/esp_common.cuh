@@ -87,6 +87,7 @@ struct GemmPlan {
     int token_tile;    // MMA N
     int split_k;       // cluster size along K
     int stages;
+    int x_mode, x_area;    // streaming kernel: how token-major X reaches it, and the shared memory that takes per CTA
 };
 esp_status_t plan_gemm(int M, int N, int K, const esp_gemm_opts &o, size_t workspace_bytes, GemmPlan *plan);
 size_t gemm_workspace_bytes(int M, int K, const esp_gemm_opts &o);        // everything any plan could use

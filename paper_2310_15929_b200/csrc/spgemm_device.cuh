@@ -56,6 +56,7 @@ struct GemmParams {
     const uint32_t *xflags;  // one word per image: 1 once it is complete
     const __half *bias;      // [N] added to every token row before the activation, or NULL
     int act;                 // ESP_ACT_*
+    int x_mode, x_area;      // streaming kernel: how token-major X reaches it, shared-memory bytes per CTA for that (0, 0: X is channel-major)
     int raster_panel;        // pair kernel: token tiles per panel of the cluster -> tile map (0 / 1 = row by row)
 };
 

@@ -456,6 +456,14 @@ __global__ void __launch_bounds__(192) spgemm_tma_kernel(const GemmParams p, con
 // 4096 x 4096 at 128 tokens: owners pulling the rows from their peers with remote loads took 8.4 us for 64 KB per CTA;
 // element-wise pushes for slice counts that are not a power of two took 10 us at 32 tokens.  The 16-byte pushes take
 // about 1.5 us.)
+//
+// Token-major X without a transposing launch in front of the product (whose 3 us lie on the path from one layer's output to the next
+// one's input, and which costs the host 2 us):
+//   kXDirect, one or two tokens  a producer thread loads its channel's elements of each stage straight from X, kXAhead stages ahead;
+//   kXCluster, small weights     the cluster's slices together span all channels: each CTA reads ITS contiguous range of channels of
+//                                the tile's tokens (16-byte loads along the channels), transposes it in registers into an area in
+//                                shared memory [8-token chunk][channel][16 bytes], and a stage's permuted channel rows are fetched from
+//                                whichever CTA of the cluster holds the channel, 16 bytes at a time, kXAhead stages ahead.
 // grid (feature tiles, token tiles, split_k), cluster (1,1,split_k), block 192:
 //   warp 0 lane 0  weight-tile producer        warp 1  tensor-memory allocation; lane 0: tcgen05.cp + sparse MMAs
 //   warps 2..5     X row producers, then epilogue (one quarter of the accumulator lanes each)
@@ -482,14 +490,20 @@ __host__ __device__ inline int stream_cnt4(int bn, int split) { return (((bn + s
 // Pushed partials at one owner: [sender][group of 4 rows][128 features][4 rows] fp32.
 inline size_t stream_push_bytes(int bn, int split) { return split > 1 ? (size_t)split * stream_cnt4(bn, split) * 512 : 0; }
 inline size_t stream_recv_bytes(int bn, int split) { return bn <= 32 ? stream_push_bytes(bn, split) : 0; }   // beside the ring
-inline size_t stream_smem_bytes(int bn, int stages, int split) {
+// Token-major X: how the kernel gets it (see the comment above).
+constexpr int kXChannelMajor = 0, kXDirect = 1, kXCluster = 2;
+constexpr int kXDirectTokens = 2, kXAreaMax = 48 * 1024;
+inline int stream_x_area_bytes(int bn, int M, int k_tiles_per_split) { return k_tiles_per_split * kTileK * 16 * (((M < bn ? M : bn) + 7) / 8); }
+inline size_t stream_smem_bytes(int bn, int stages, int split, int x_area) {
     size_t ring = (size_t)stages * (kTileBytes + 256 * bn);
     if (bn > 32 && ring < stream_push_bytes(bn, split)) ring = stream_push_bytes(bn, split);   // wide tiles receive into the ring
-    return ring + stream_recv_bytes(bn, split) + kPermRing * 512 + 512 + 1024;
+    return ring + stream_recv_bytes(bn, split) + (size_t)x_area + kPermRing * 512 + 512 + 1024;
 }
 
-template <int BN>
-__global__ void __launch_bounds__(StreamCfg<BN>::kThreads) spgemm_stream_kernel(const GemmGroup grp, const int stages) {
+// XMODE: kernels of their own, so that the registers of the token-major producers cost the channel-major form no residency.
+template <int BN, int XMODE>
+__global__ void __launch_bounds__(StreamCfg<BN>::kThreads, XMODE == kXChannelMajor ? 1 : 4) spgemm_stream_kernel(const GemmGroup grp, const int stages) {
+    constexpr bool TM = XMODE != kXChannelMajor, xcluster = XMODE == kXCluster;
     using L = StreamCfg<BN>;
     // this CTA's problem: selected with constant indices so that the parameters stay in registers
     GemmParams p = grp.p[0];
@@ -508,7 +522,8 @@ __global__ void __launch_bounds__(StreamCfg<BN>::kThreads) spgemm_stream_kernel(
     uint32_t ring_bytes = (uint32_t)stages * L::kStage;
     if (!L::kEarlyPush && ring_bytes < push_bytes) ring_bytes = push_bytes;
     const uint32_t recv_off = L::kEarlyPush ? ring_bytes : 0u;
-    const uint32_t perm_off = ring_bytes + (L::kEarlyPush ? push_bytes : 0u);
+    const uint32_t xarea_off = ring_bytes + (L::kEarlyPush ? push_bytes : 0u);
+    const uint32_t perm_off = xarea_off + (xcluster ? (uint32_t)p.x_area : 0u);
     const uint32_t bar_off = perm_off + kPermRing * 512;
     const uint32_t bar_base = sbase + bar_off;
     auto full = [&](int s) { return bar_base + 8u * s; };
@@ -531,7 +546,8 @@ __global__ void __launch_bounds__(StreamCfg<BN>::kThreads) spgemm_stream_kernel(
     // block -- BN < 64: token tile --, channel step) into the workspace; a stage's X is then one bulk copy per token
     // block instead of 16-byte row copies from every producer thread (which are limited to one 32-byte sector per clock
     // per SM).
-    const bool imaged = p.ximg != nullptr;
+    const bool imaged = !TM && p.ximg != nullptr;
+    const int slice_ch = p.k_tiles_per_split * kTileK;                // channels per slice: channel c is held by rank c / slice_ch
     const uint32_t rank = (split > 1) ? cluster_ctarank() : 0u;
     const int owned = max(0, min(cnt4, BN - (int)rank * cnt4));      // rows of this tile that this CTA finishes
 
@@ -571,16 +587,19 @@ __global__ void __launch_bounds__(StreamCfg<BN>::kThreads) spgemm_stream_kernel(
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    if (split > 1) cluster_arrive();       // every CTA of the cluster is running and has its barriers set up
+    if (split > 1 && !(xcluster && warp >= 2)) cluster_arrive();       // every CTA of the cluster is running and has its barriers set up
     grid_launch_dependents();
 
-    // Cluster barrier protocol (split > 1): phase A = "every CTA has its barriers set up" (arrived above); wide tiles add
-    // phase B = "every CTA's MMAs are done with the ring".  Every thread takes part in every phase, whatever happened to it.
+    // Cluster barrier protocol (split > 1): phase A = "every CTA has its barriers set up" (arrived above; with token-major X also "its
+    // channels are in the X area", arrived by the producers, where the cluster shares X); wide tiles add phase B = "every CTA's MMAs are done with the ring",
+    // shared X phase Z = "this CTA reads no other's X area any more" (waited for before the exit).  Every thread takes part in
+    // every phase, whatever happened to it.
     if (warp == 0) {
         // (later weight tiles are issued by the X producer warps below, right after they have seen the stage's `empty`)
         if (split > 1) {
             cluster_wait();
             if (!L::kEarlyPush) { cluster_arrive(); cluster_wait(); }
+            if (xcluster) cluster_arrive();
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -611,6 +630,7 @@ __global__ void __launch_bounds__(StreamCfg<BN>::kThreads) spgemm_stream_kernel(
         if (split > 1) {
             cluster_wait();
             if (!L::kEarlyPush) { cluster_arrive(); cluster_wait(); }
+            if (xcluster) cluster_arrive();
         }
     } else {
         // ---- X producers: thread g copies the 16-byte pieces e = g, g + 128, ... of the stage's 128 rows
@@ -653,6 +673,114 @@ __global__ void __launch_bounds__(StreamCfg<BN>::kThreads) spgemm_stream_kernel(
                 }
             }
             if (nk == 0) grid_dependency_wait();                      // (no flag to see: wait for the stream order itself)
+        } else if constexpr (TM) {
+            // ---- token-major X: this slice's channels into the X area, then a stage's rows from the cluster's areas
+            const int chunks = (min(p.M, BN) + 7) >> 3;               // 8-token chunks of the tile that exist
+            const int own_ch = nk * kTileK, area_ch = slice_ch;
+            uint8_t *area = smem + xarea_off;
+            // chunks beyond them: zero in every ring slot, once
+            if (chunks < L::kChunks) {
+                for (int i = g; i < stages * 128 * (L::kChunks - chunks); i += L::kProd) {
+                    const int s = i / (128 * (L::kChunks - chunks)), q = i - s * (128 * (L::kChunks - chunks));
+                    const int r = q & 127, cc = chunks + (q >> 7);
+                    const int cs = cc ^ ((r >> L::kSwzShift) & (L::kChunks - 1));
+                    *reinterpret_cast<uint4 *>(smem + s * L::kStage + kTileBytes + r * L::kRowBytes + (cs << 4)) = make_uint4(0u, 0u, 0u, 0u);
+                }
+            }
+            grid_dependency_wait();                                   // X may come from the preceding kernel
+            if constexpr (xcluster) {
+            for (int i = g; i < (own_ch >> 3) * chunks; i += L::kProd) {
+                const int blk = i % (own_ch >> 3), cc = i / (own_ch >> 3);
+                const int c = kt_begin * kTileK + blk * 8, t0 = tok0 + cc * 8;
+                uint4 v[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    v[t] = make_uint4(0u, 0u, 0u, 0u);
+                    if (c < p.K && t0 + t < p.M) v[t] = __ldg(reinterpret_cast<const uint4 *>(xb + (long)(t0 + t) * p.ldx + c));
+                }
+                // 8 x 8 transposition; channel 8 b + e goes to place 8 b + (e ^ (b & 7)), so that neighbouring threads meet different banks
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t sel = (e & 1) ? 0x7632u : 0x5410u;
+                    uint32_t w[8], o[4];
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) w[t] = (e >> 1) == 0 ? v[t].x : (e >> 1) == 1 ? v[t].y : (e >> 1) == 2 ? v[t].z : v[t].w;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) o[j] = __byte_perm(w[2 * j], w[2 * j + 1], sel);
+                    *reinterpret_cast<uint4 *>(area + ((size_t)cc * area_ch + blk * 8 + (e ^ (blk & 7))) * 16) = make_uint4(o[0], o[1], o[2], o[3]);
+                }
+            }
+            __syncwarp();
+            if (split > 1) { cluster_arrive(); cluster_wait(); }      // phase A
+            else asm volatile("bar.sync 1, %0;" ::"n"(L::kProd) : "memory");
+            }
+            const uint32_t area_s = sbase + xarea_off;
+            const bool ring_over = nk > kPermRing;                    // (g < 128 = every producer of these tiles)
+            static_assert(L::kProd == 128, "one channel row per producer");
+            constexpr int kXAhead = XMODE == kXDirect ? 8 : BN == 16 ? 2 : 1;
+            static_assert(kPermRing >= 2 * kXAhead, "ring of permutation entries");
+            constexpr int kRegs = XMODE == kXDirect ? 1 : L::kChunks;
+            uint4 ahead[kXAhead][kRegs];                              // (direct: word t = the element of token t)
+            auto fetch = [&](int it, uint4 (&v)[kRegs]) {
+#pragma unroll
+                for (int cc = 0; cc < kRegs; ++cc) v[cc] = make_uint4(0u, 0u, 0u, 0u);
+                // (a thread reads and writes its own entries of the permutation ring only)
+                const int ch = it < nk ? perm_s[(it % kPermRing) * 128 + g] : -1;
+                if (ch < 0) return;
+                if constexpr (XMODE == kXDirect) {
+                    const uint16_t *x = xb + ch;
+                    v[0].x = __ldg(x);
+                    if (p.M > 1) v[0].y = __ldg(x + p.ldx);
+                } else {
+                    const int owner = ch / slice_ch, local = ch - owner * slice_ch;
+                    const uint32_t at = area_s + (uint32_t)((local ^ ((local >> 3) & 7)) * 16);
+                    const uint32_t remote = split > 1 ? map_to_rank(at, (uint32_t)owner) : at;
+#pragma unroll
+                    for (int cc = 0; cc < L::kChunks; ++cc)
+                        if (cc < chunks)
+                            asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                         : "=r"(v[cc].x), "=r"(v[cc].y), "=r"(v[cc].z), "=r"(v[cc].w)
+                                         : "r"(remote + (uint32_t)(cc * area_ch * 16))
+                                         : "memory");
+                }
+            };
+#pragma unroll
+            for (int u = 0; u < kXAhead; ++u) fetch(u, ahead[u]);
+            for (int it0 = 0; it0 < nk; it0 += kXAhead) {
+#pragma unroll
+                for (int u = 0; u < kXAhead; ++u) {
+                    const int it = it0 + u;
+                    if (it >= nk) break;
+                    const int s = it % stages;
+                    const uint32_t ph = (uint32_t)(it / stages) & 1u;
+                    if (alive && !mbar_wait(empty(s), ph ^ 1u, abort_flag)) alive = false;
+                    if (alive) {
+                        uint8_t *xs = smem + s * L::kStage + kTileBytes + g * L::kRowBytes;
+                        if constexpr (XMODE == kXDirect) {
+                            const uint4 e = ahead[u][0];
+                            *reinterpret_cast<uint4 *>(xs + (((g >> L::kSwzShift) & (L::kChunks - 1)) << 4)) = make_uint4(e.x | (e.y << 16), 0u, 0u, 0u);
+                        } else {
+#pragma unroll
+                            for (int cc = 0; cc < L::kChunks; ++cc)
+                                if (cc < chunks) *reinterpret_cast<uint4 *>(xs + ((cc ^ ((g >> L::kSwzShift) & (L::kChunks - 1))) << 4)) = ahead[u][cc];
+                        }
+                        fence_async_smem();                           // generic-proxy writes -> read by the MMA
+                        mbar_arrive(full(s));
+                        if (it >= prefetch && lane == 0 && (warp - 2) == (s & 3)) {      // weight tile beyond the start-up ones, as below
+                            mbar_arrive_expect_tx(full(s), kTileBytes);
+                            bulk_load(sbase + s * L::kStage, w_src + (long)it * kTileBytes, kTileBytes, full(s));
+                        }
+                    }
+                    if (ring_over) {                                  // the entry of stage it is used up: that of kPermRing stages on
+                        if (it > 0) perm_s[((it - 1) % kPermRing) * 128 + g] = refill;
+                        const int kpos = (kt_begin + it + kPermRing) * kTileK + g;
+                        refill = (it + kPermRing < nk && kpos < p.K) ? (p.perm ? __ldg(p.perm + kpos) : kpos) : -1;
+                    }
+                    fetch(it + kXAhead, ahead[u]);
+                }
+            }
+            __syncwarp();
+            if (xcluster && split > 1) cluster_arrive();              // phase Z (waited for at the end)
         } else {
         grid_dependency_wait();                                       // X may come from the preceding kernel
         for (int it = 0; it < nk; ++it) {
@@ -772,7 +900,7 @@ __global__ void __launch_bounds__(StreamCfg<BN>::kThreads) spgemm_stream_kernel(
             const int cgrp = (warp - 2) >> 2;
             const bool ok = __all_sync(0xFFFFFFFFu, alive && (nk == 0 || mbar_wait(accum_bar, 0, abort_flag)));   // warp-uniform
             tc_fence_after();
-            cluster_wait();                                          // phase A: every CTA of the cluster has its barriers
+            if (!xcluster) cluster_wait();                           // phase A: every CTA of the cluster has its barriers
             if (!L::kEarlyPush) { cluster_arrive(); cluster_wait(); }   // phase B: every CTA's MMAs are done with the ring
             const int groups = cnt4 >> 2;                            // 4-row groups per owner
 #pragma unroll 1
@@ -819,6 +947,7 @@ __global__ void __launch_bounds__(StreamCfg<BN>::kThreads) spgemm_stream_kernel(
             }
         }
     }
+    if (xcluster && split > 1) cluster_wait();                        // phase Z
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
@@ -894,11 +1023,21 @@ esp_status_t launch_xtile_narrow(const GemmParams &p, uint8_t *img, uint32_t *fl
     return ESP_OK;
 }
 
+// The kernel for these parameters.
+template <int BN>
+auto stream_kernel_for(int x_mode) {
+    if constexpr (BN == 16)
+        if (x_mode == kXDirect) return spgemm_stream_kernel<BN, kXDirect>;
+    if constexpr (BN <= 32)
+        if (x_mode == kXCluster) return spgemm_stream_kernel<BN, kXCluster>;
+    return spgemm_stream_kernel<BN, kXChannelMajor>;
+}
+
 template <int BN>
 esp_status_t launch_stream(const GemmParams &p, int f_tiles, int t_tiles, int split, int stages, bool dependent,
                            cudaStream_t stream) {
-    auto kern = spgemm_stream_kernel<BN>;
-    const size_t smem = stream_smem_bytes(BN, stages, split);
+    auto kern = stream_kernel_for<BN>(p.x_mode);
+    const size_t smem = stream_smem_bytes(BN, stages, split, p.x_area);
     ESP_CUDA_OK(ensure_dynamic_smem((const void *)kern, (int)smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(f_tiles, t_tiles, split);
@@ -925,8 +1064,8 @@ esp_status_t launch_stream(const GemmParams &p, int f_tiles, int t_tiles, int sp
 // The same launch for a group of problems (feature tiles concatenated along grid.x).
 template <int BN>
 esp_status_t launch_stream_group(const GemmGroup &grp, int t_tiles, int split, int stages, bool dependent, cudaStream_t stream) {
-    auto kern = spgemm_stream_kernel<BN>;
-    const size_t smem = stream_smem_bytes(BN, stages, split);
+    auto kern = stream_kernel_for<BN>(grp.p[0].x_mode);
+    const size_t smem = stream_smem_bytes(BN, stages, split, grp.p[0].x_area);
     ESP_CUDA_OK(ensure_dynamic_smem((const void *)kern, (int)smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grp.ft_start[grp.count], t_tiles, split);
@@ -948,9 +1087,9 @@ esp_status_t launch_stream_group(const GemmGroup &grp, int t_tiles, int split, i
 
 // Clusters of `split` CTAs of the streaming kernel that can be resident at once on this device.
 template <int BN>
-int stream_cluster_capacity(int split, int stages) {
-    auto kern = spgemm_stream_kernel<BN>;
-    const size_t smem = stream_smem_bytes(BN, stages, split);
+int stream_cluster_capacity(int split, int stages, int x_mode, int x_area) {
+    auto kern = stream_kernel_for<BN>(x_mode);
+    const size_t smem = stream_smem_bytes(BN, stages, split, x_area);
     if (ensure_dynamic_smem((const void *)kern, (int)smem) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1, 1, split);
@@ -1126,22 +1265,22 @@ size_t gemm_workspace_bytes(int M, int K, const esp_gemm_opts &o) {
 }
 
 // Resident capacity (in CTAs) of the streaming kernel for one configuration, cached per process.
-static int stream_capacity_ctas(int bn, int split, int stages) {
+static int stream_capacity_ctas(int bn, int split, int stages, int x_mode, int x_area) {
     static std::mutex mu;
     static std::map<long, int> cache;
     int dev = 0;
     cudaGetDevice(&dev);
-    const long key = (((long)dev * 512 + bn) * 16 + split) * 16 + stages;
+    const long key = (((((long)dev * 512 + bn) * 16 + split) * 16 + stages) * 4 + x_mode) * 65536 + x_area;
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     int clusters = 0;
     switch (bn) {
-        case 16: clusters = stream_cluster_capacity<16>(split, stages); break;
-        case 32: clusters = stream_cluster_capacity<32>(split, stages); break;
-        case 64: clusters = stream_cluster_capacity<64>(split, stages); break;
-        case 128: clusters = stream_cluster_capacity<128>(split, stages); break;
-        case 256: clusters = stream_cluster_capacity<256>(split, stages); break;
+        case 16: clusters = stream_cluster_capacity<16>(split, stages, x_mode, x_area); break;
+        case 32: clusters = stream_cluster_capacity<32>(split, stages, x_mode, x_area); break;
+        case 64: clusters = stream_cluster_capacity<64>(split, stages, x_mode, x_area); break;
+        case 128: clusters = stream_cluster_capacity<128>(split, stages, x_mode, x_area); break;
+        case 256: clusters = stream_cluster_capacity<256>(split, stages, x_mode, x_area); break;
         default: break;
     }
     cache[key] = clusters * split;
@@ -1154,6 +1293,8 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
     esp_status_t st = device_info(&di);
     if (st != ESP_OK) return st;
     GemmPlan g;
+    g.x_mode = kXChannelMajor;
+    g.x_area = 0;
     const int k_tiles = ceil_div(K, kTileK);
     const int f_tiles = ceil_div(N, kTileFeat);
     const bool channel_major_available = (o.x_layout == ESP_X_CHANNEL_MAJOR) || have_workspace;
@@ -1281,7 +1422,21 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
             if (wanted != 0 && split != wanted) continue;
             if (!no_empty_slice(split)) continue;
             const int kts = ceil_div(k_tiles, split);
-            const size_t fixed = stream_recv_bytes(bn, split) + kPermRing * 512 + 512 + 1024;
+            // token-major X without a transposing launch: up to two tokens straight from X (4096 x 11008, us per call: 14.6 -> 13.0 at
+            // one token, 14.6 -> 15.4 at two; 22016 x 8192: 37.2 -> 34.9 and 35.5; at four tokens the element loads cost more than the
+            // launch, 14.7 -> 22.8), through the cluster where the weight is
+            // small (its start is longer, but the call saves a launch: 512 x 512 at 128 tokens 8.7 -> 6.2, 2048 x 2048 at 16 tokens 8.1 ->
+            // 7.0, at 32 tokens 8.2 -> 8.9; 4096 x 4096 at 16 tokens 9.2 -> 11.7)
+            int x_mode = kXChannelMajor, x_area = 0;
+            if (g.kernel == ESP_KERNEL_STREAM && o.x_layout == ESP_X_TOKEN_MAJOR) {
+                const long weight = (long)N * K;
+                if (bn == 16 && (M == 1 || (M <= kXDirectTokens && K <= 8192))) x_mode = kXDirect;
+                else if (bn <= 32 && weight <= (M <= 16 ? 4500000L : 1200000L) && stream_x_area_bytes(bn, M, kts) <= kXAreaMax) {
+                    x_mode = kXCluster;
+                    x_area = stream_x_area_bytes(bn, M, kts);
+                }
+            }
+            const size_t fixed = stream_recv_bytes(bn, split) + (size_t)x_area + kPermRing * 512 + 512 + 1024;
             int last_stages = -1;
             for (int r = 1; r <= 4; ++r) {
                 const size_t budget = (size_t)di.max_smem_optin / r - (r > 1 ? 1024 : 0);
@@ -1295,7 +1450,7 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
                 if (stages > kts) stages = kts < 2 ? 2 : kts;
                 if (stages == last_stages) continue;
                 last_stages = stages;
-                const int cap = stream_capacity_ctas(bn, split, stages);
+                const int cap = stream_capacity_ctas(bn, split, stages, x_mode, x_area);
                 if (cap <= 0) continue;
                 const long ctas = tiles * split;
                 const long waves = (ctas + cap - 1) / cap;
@@ -1310,12 +1465,12 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
                 // (not when every CTA has an SM of its own anyway: a deeper ring is then free, measured 16.0 -> 12.6 us on
                 // 4096 x 4096 at 64 tokens)
                 if (o.static_weights && o.pipeline_stages == 0 && ctas > di.sm_count &&
-                    2 * (stream_smem_bytes(bn, stages, split) + 1024) > (size_t)di.max_smem_optin)
+                    2 * (stream_smem_bytes(bn, stages, split, x_area) + 1024) > (size_t)di.max_smem_optin)
                     cost += 3.0;
                 if (log_plans())
                     fprintf(stderr, "esparse plan M=%d N=%d K=%d tile=%d: split=%d stages=%d capacity=%d ctas=%ld waves=%ld cost=%.2f\n", M, N, K,
                             bn, split, stages, cap, ctas, waves, cost);
-                if (cost < best_cost) { best_cost = cost; best_split = split; best_stages = stages; }
+                if (cost < best_cost) { best_cost = cost; best_split = split; best_stages = stages; g.x_mode = x_mode; g.x_area = x_area; }
             }
         }
         if (best_split == 0) return ESP_ERR_UNSUPPORTED;
@@ -1444,6 +1599,8 @@ esp_status_t launch_spgemm(const __half *X, int M, int K, long ldx, const void *
     p.ximg = nullptr;
     p.xflags = nullptr;
     p.raster_panel = 0;
+    p.x_mode = plan.x_mode;
+    p.x_area = plan.x_area;
     const int f_tiles = ceil_div(N, kTileFeat), t_tiles = ceil_div(M, plan.token_tile);
     const bool quad_form = plan.kernel == ESP_KERNEL_QUAD_TILED || plan.kernel == ESP_KERNEL_QUAD_MULTICAST;
     if (plan.kernel == ESP_KERNEL_PAIR || plan.kernel == ESP_KERNEL_PAIR_TILED || quad_form || plan.kernel == ESP_KERNEL_PAIR_PERSIST) {
@@ -1460,7 +1617,7 @@ esp_status_t launch_spgemm(const __half *X, int M, int K, long ldx, const void *
         }
     }
     if (plan.kernel != ESP_KERNEL_GATHER) {
-        if (!p.x_channel_major && plan.kernel != ESP_KERNEL_PAIR_TILED &&
+        if (!p.x_channel_major && plan.x_mode == kXChannelMajor && plan.kernel != ESP_KERNEL_PAIR_TILED &&
             !(plan.kernel == ESP_KERNEL_STREAM_IMAGES && plan.token_tile >= 64)) {
             // token-major input: transposed (not permuted) copy into the caller's workspace
             const long ldt = transposed_ld(M);
@@ -1590,9 +1747,11 @@ esp_status_t launch_spgemm_group(int count, const void *const *X, int M, int K, 
         p.ximg = nullptr;
         p.xflags = nullptr;
         p.raster_panel = 0;
+        p.x_mode = plan.x_mode;
+    p.x_area = plan.x_area;
         grp.ft_start[i] = ft;
         if (i < count) {
-            if (o.x_layout != ESP_X_CHANNEL_MAJOR) {      // token-major: a transposed copy per distinct input, one after the other
+            if (o.x_layout != ESP_X_CHANNEL_MAJOR && plan.x_mode == kXChannelMajor) {      // token-major: a transposed copy per distinct input, one after the other
                 const long ldt = transposed_ld(M);
                 int first = i;
                 for (int e = 0; e < i; ++e)

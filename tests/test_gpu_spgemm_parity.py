@@ -610,6 +610,26 @@ def test_grouped_products_in_one_call(M, channel_major):
         check(q["Y"].cpu().numpy(), ref_product(q["X"], q["vals"], q["meta"], q["theta"]))
 
 
+@pytest.mark.parametrize("M,N,K,splits", [(1, 200, 8, (1,)), (1, 130, 2320, (1, 3, 8)), (2, 128, 1032, (1, 5)),                       # straight from X
+                                          (3, 200, 8, (1,)), (8, 130, 1160, (1, 3, 8)), (9, 256, 2320, (1, 4)), (16, 128, 264, (2,)),  # the cluster's
+                                          (17, 130, 1032, (2, 7)), (33, 200, 520, (1, 4)), (129, 256, 648, (0, 3))])
+def test_token_major_input_without_a_transposed_copy(M, N, K, splits):
+    """The streaming kernel's two token-major forms: one token and two, few steps and more than the permutation ring holds;
+    8-token chunks full and ragged, slices of unequal length, several token tiles.  Same bits as the channel-major form in the
+    same tile and slices."""
+    from tests.gpu_util import pack_on_gpu, spgemm
+    vals, meta, theta = pruned(7100 + M + K, N, K)
+    X = (np.random.default_rng(M + K).standard_normal((M, K))).astype(np.float16)
+    packed = pack_on_gpu(vals, meta)
+    Yref = ref_product(X, vals, meta, theta)
+    for split in splits:
+        tile = 16 if M <= 16 or M > 64 else 32
+        kw = dict(split_k=split, token_tile=tile, static_weights=1)
+        Y = spgemm(X, packed, theta, N, **kw)
+        check(Y, Yref)
+        assert np.array_equal(Y, spgemm(X, packed, theta, N, channel_major=True, kernel=4, **kw))
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
