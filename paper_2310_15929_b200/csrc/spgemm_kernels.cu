@@ -501,8 +501,9 @@ inline size_t stream_smem_bytes(int bn, int stages, int split, int x_area) {
 }
 
 // XMODE: kernels of their own, so that the registers of the token-major producers cost the channel-major form no residency.
+// (At least 1152 threads per SM for that one, 56 registers: two CTAs of 576 threads share an SM, six of 192.)
 template <int BN, int XMODE>
-__global__ void __launch_bounds__(StreamCfg<BN>::kThreads, XMODE == kXChannelMajor ? 1 : 4) spgemm_stream_kernel(const GemmGroup grp, const int stages) {
+__global__ void __launch_bounds__(StreamCfg<BN>::kThreads, XMODE == kXChannelMajor ? 1152 / StreamCfg<BN>::kThreads : 4) spgemm_stream_kernel(const GemmGroup grp, const int stages) {
     constexpr bool TM = XMODE != kXChannelMajor, xcluster = XMODE == kXCluster;
     using L = StreamCfg<BN>;
     // this CTA's problem: selected with constant indices so that the parameters stay in registers
