@@ -313,14 +313,13 @@ esp_status_t esp_spgemm_tune(const void *X, int M, int K, long ldx, const void *
     std::vector<Cand> cands;
     cands.push_back({opts->force_kernel, opts->token_tile, opts->split_k, opts->pipeline_stages});
     if (M > 64) {
-        for (int tile : {240, 224, 192, 128}) {
+        for (int tile : {256, 240, 224, 192, 128}) {
             if (tile > 128 && M <= 128) continue;
-            for (int split = 1; split <= (tile == 128 ? 4 : 1); ++split) {      // K-slices: 128-token tiles only
+            for (int split = 1; split <= (tile == 128 || tile == 256 ? 4 : 1); ++split) {      // K-slices: 128- and 256-token tiles
                 cands.push_back({ESP_KERNEL_PAIR_TILED, tile, split, 0});
                 cands.push_back({ESP_KERNEL_PAIR, tile, split, 0});
             }
         }
-        cands.push_back({ESP_KERNEL_PAIR, 256, 1, 0});
         if (M > 256)
             for (int tile : {240, 224, 192}) cands.push_back({ESP_KERNEL_PAIR_PERSIST, tile, 1, 0});      // never planned, sometimes ahead
     }

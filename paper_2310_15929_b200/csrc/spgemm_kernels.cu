@@ -1249,6 +1249,7 @@ static size_t ximg_bytes(int M, int K, int tn) {
         case 128: return xtile_bytes<128>(M, K);
         case 192: return xtile_bytes<192>(M, K);
         case 224: return xtile_bytes<224>(M, K);
+        case 256: return xtile_bytes<256>(M, K);
         default: return xtile_bytes<240>(M, K);
     }
 }
@@ -1259,7 +1260,7 @@ size_t gemm_workspace_bytes(int M, int K, const esp_gemm_opts &o) {
                                o.force_kernel == ESP_KERNEL_PAIR_PERSIST || o.force_kernel == ESP_KERNEL_QUAD_MULTICAST;
     if (pair_possible) {
         size_t img = 0;
-        for (int tn : {128, 192, 224, 240}) img = std::max(img, ximg_bytes(M, K, tn));
+        for (int tn : {128, 192, 224, 240, 256}) img = std::max(img, ximg_bytes(M, K, tn));
         n += img;
     }
     return n;
@@ -1287,6 +1288,42 @@ static int stream_capacity_ctas(int bn, int split, int stages, int x_mode, int x
     cache[key] = clusters * split;
     return clusters * split;
 }
+
+// Clusters of 2 x split CTAs of the pair kernel that the device holds at once, asked once per device.
+static int pair_cluster_capacity(int device, int split) {
+    static std::mutex mu;
+    static std::map<int, int> cache;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find(device * 16 + split);
+    if (it != cache.end()) return it->second;
+    auto kern = spgemm_pair_kernel<1, 256, true>;
+    const int smem = PairCfg<1, 256>::kTotal;
+    int n = 0;
+    if (2 * split <= 8 && ensure_dynamic_smem((const void *)kern, smem) == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        cfg.gridDim = dim3(2, 1, split);
+        cfg.blockDim = dim3(kPairThreads);
+        cfg.dynamicSmemBytes = smem;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = split;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    }
+    if (log_plans()) fprintf(stderr, "esparse pair clusters of %d CTAs: %d fit\n", 2 * split, n);
+    return cache[device * 16 + split] = n;
+}
+
+// Token tiles of the pair kernel: features (in 128-feature tiles) x tokens of a pair's tile, time of a 128-channel step, and of the rest
+// of a wave (start, ring fill, epilogue).  Measured, one wave of 16 to 86 steps, tiled form: 256 features x 256 tokens 19.5 us at 16 steps,
+// 28.4 at 32, 60 at 86; 512 x 128 the same area in 21.6, 31 and 66 (its MMAs are half as wide, so the weight operand is read from
+// shared memory twice as often: the MMA thread is busy 850 to 1000 of a step's 1130 clocks); the widest cover 1.9 times the
+// area in 1.4 times the time and win once the grid fills whole waves.
+struct PairTile { int tokens, feature_tiles; double step_us, fixed_us; };
+static const PairTile kPairTiles[] = {{240, 4, 0.83, 13.0}, {224, 4, 0.82, 12.5}, {192, 4, 0.80, 12.0}, {256, 2, 0.585, 9.7}, {128, 4, 0.66, 10.5}};
 
 static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts &o, size_t workspace_bytes, GemmPlan *plan) {
     const bool have_workspace = workspace_bytes >= transpose_bytes(M, K, o) && (workspace_bytes > 0 || o.x_layout == ESP_X_CHANNEL_MAJOR);
@@ -1331,7 +1368,7 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
             if (images_room && bn == 0 && o.split_k <= 8 && M > 16 && M <= 256) {
                 const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
                 if (!pair) {
-                    const bool pays = M <= 32 ? weight >= 200000000L : M <= 64 ? (f_tiles >= 64 || weight >= 64000000L) : M <= 128 ? weight >= 40000000L : weight >= 16000000L;
+                    const bool pays = M <= 32 ? weight >= 200000000L : M <= 64 ? ((f_tiles >= 64 && weight >= 40000000L) || weight >= 64000000L) : M <= 128 ? weight >= 40000000L : weight >= 16000000L;
                     // (up to 32 tokens: 32-token images -- 36864 x 9216 at 32 tokens 67.5 -> 64.3 us, 9216 x 36864 76 -> 70)
                     if (pays) { g.kernel = ESP_KERNEL_STREAM_IMAGES; bn = M <= 32 ? 32 : (M > 128 && weight >= 64000000L) ? 128 : 64; }
                 } else if (M > 128 && o.split_k == 0 && weight >= 80000000L && per_wave / pairs128 >= 2) {
@@ -1344,47 +1381,49 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
     const bool wide_only = g.kernel == ESP_KERNEL_QUAD_TILED || g.kernel == ESP_KERNEL_PAIR_PERSIST ||
                            g.kernel == ESP_KERNEL_QUAD_MULTICAST;                                      // no 128-token form
     if (g.kernel == ESP_KERNEL_PAIR || g.kernel == ESP_KERNEL_PAIR_TILED || wide_only) {
-        const long f_pairs = ceil_div(f_tiles, 4), per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
-        if (bn == 0) {
-            // cost ~ waves of clusters x time of one wave, in clocks: a channel step costs its MMAs (8 x TN/2 clocks) and its
-            // 36 KB of weights + X tile (64-token blocks: 16 KB for TN = 128, else 32 KB) at the ~70 B/clk an SM pulls from
-            // L2.  Wide tiles win once the grid fills the machine; a grid of less than one wave runs faster on narrow ones.
-            double best = -1.0;
-            for (int tn : {240, 224, 192, 128}) {
-                if (tn == 128 && wide_only) continue;
-                const long clusters = f_pairs * ceil_div(M, tn);
-                const double mma = 4.0 * tn, copy = (36864.0 + (tn > 128 ? 32768.0 : 16384.0)) / 70.0;
-                // per wave: the channel steps (both terms show in the measured step time), an epilogue that grows with the
-                // tile (about ten steps' worth at 240 tokens) and a fixed set-up.  Waves: a grid of up to two waves runs as
-                // whole waves (equal tiles end together); over many waves the clusters drift apart and the last, partial wave
-                // costs less and less of a whole one (measured at 4.4 waves: already closer to the fractional count).
-                const double w = (double)clusters / (double)per_wave, whole = (double)ceil_div(clusters, per_wave);
+        const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
+        const bool requested = bn != 0;
+        int split = 1;
+        double best = -1.0;
+        for (const PairTile &t : kPairTiles) {
+            if (requested ? t.tokens != bn : (wide_only && (t.tokens == 128 || t.tokens == 256))) continue;
+            // waves x time of one wave.  Waves: a grid of up to two waves runs as whole waves (equal tiles end together); over many
+            // waves the clusters drift apart and the last, partial wave costs less and less of a whole one.
+            // K-slices (128- and 256-token tiles: the pushed partial rows of all slices must fit the ring), each of at least four
+            // channel steps: a cluster of 2 x split CTAs, of which far fewer fit the GPU (two slices: 33 on 148 SMs), and about
+            // 10 us for the reduction.  Beyond 256 tokens two slices at most: three ran far slower (4096 x 11008 at 384 tokens 70
+            // against 50 us).
+            const long pairs = (long)ceil_div(f_tiles, t.feature_tiles) * ceil_div(M, t.tokens);
+            const bool sliced = t.tokens == 128 || t.tokens == 256;
+            int most = sliced ? (M > 256 ? 2 : 4) : 1;
+            int wanted = o.split_k;
+            if (wanted > 0) {
+                if (!sliced && wanted > 1) continue;
+                while (wanted > 1 && (k_tiles / wanted < 4 || (long)ceil_div(k_tiles, wanted) * (wanted - 1) >= k_tiles)) --wanted;
+                most = wanted;
+            }
+            for (int sp = wanted > 0 ? wanted : 1; sp <= most; ++sp) {
+                if (sp > 1 && wanted == 0 && (k_tiles / sp < 4 || (long)ceil_div(k_tiles, sp) * (sp - 1) >= k_tiles)) continue;
+                const long cap = std::max<long>(1, sp == 1 ? per_wave : pair_cluster_capacity(di.device, sp));
+                if (sp > 1 && wanted == 0 && pairs > cap) continue;
+                const double w = (double)pairs / (double)cap, whole = (double)ceil_div(pairs, cap);
                 const double waves = w <= 2.0 ? whole : w + (whole - w) * (2.0 / w);
-                const double cost = waves * (0.5 * (mma + copy) * k_tiles + 40.0 * tn + 2000.0);
-                if (best < 0.0 || cost < best) { best = cost; bn = tn; }
+                const double cost = waves * (t.step_us * ceil_div(k_tiles, sp) + t.fixed_us) + (sp > 1 ? 10.0 : 0.0);
+                if (log_plans()) fprintf(stderr, "esparse plan M=%d N=%d K=%d pair tile=%d split=%d pairs=%ld waves=%.2f cost=%.1f\n", M, N, K, t.tokens, sp, pairs, waves, cost);
+                if (best < 0.0 || cost < best) { best = cost; bn = t.tokens; split = sp; }
             }
         }
-        if (bn != 128 && bn != 192 && bn != 224 && bn != 240 && bn != 256) return ESP_ERR_INVALID_ARG;
-        // K-slices (128-token tiles only: the pushed partial rows of all slices must fit the ring): as many as fill one
-        // wave of pairs, each slice keeping at least four channel steps
-        int split = 1;
-        if (bn == 128) {
-            const long pairs = f_pairs * ceil_div(M, 128);
-            // (beyond 256 tokens two slices at most: three ran far slower than two -- 4096 x 4096 at 384 tokens 46 against
-            // 30 us, 4096 x 11008 at 384 tokens 70 against 50 -- and four no faster)
-            split = o.split_k > 0 ? o.split_k : (int)std::min<long>(M > 256 ? 2 : 4, std::max<long>(1, per_wave / pairs));
-            while (split > 1 && (k_tiles / split < 4 || (long)ceil_div(k_tiles, split) * (split - 1) >= k_tiles)) --split;
-        } else if (o.split_k > 1) {
-            return ESP_ERR_INVALID_ARG;
-        }
+        if (best < 0.0) return ESP_ERR_INVALID_ARG;
         // the tiled form needs room for the X images behind the transposed copy; without it the gather form runs.  Up to
         // 128 tokens the gather form is taken anyway: one launch instead of two, and X is small.
-        const bool room = bn != 256 && workspace_bytes >= transpose_bytes(M, K, o) + ximg_bytes(M, K, bn);
+        // (on a large weight the gather's row copies cost more than that launch: 22016 x 8192 at 100 tokens 76 -> 61 us)
+        const bool room = workspace_bytes >= transpose_bytes(M, K, o) + ximg_bytes(M, K, bn);
         if ((g.kernel == ESP_KERNEL_PAIR_TILED || wide_only) && !room) return ESP_ERR_WORKSPACE;
         if (wide_only && (bn == 128 || bn == 256)) return ESP_ERR_INVALID_ARG;
         // (129..256 tokens in one K-slice: the tiled form too -- 11008 x 4096 at 256 tokens 37.4 -> 33.4 us, 13824 x 5120
         // 47.2 -> 41.6; with K-slices the gather form stays ahead there)
-        if (g.kernel == ESP_KERNEL_PAIR && o.force_kernel == ESP_KERNEL_AUTO && room && (M > 256 || (M > 128 && split == 1)))
+        if (g.kernel == ESP_KERNEL_PAIR && o.force_kernel == ESP_KERNEL_AUTO && room &&
+            (M > 256 || (split == 1 && (M > 128 || (long)N * K >= 80000000L)) || bn == 256))
             g.kernel = ESP_KERNEL_PAIR_TILED;
         g.token_tile = bn;
         g.split_k = split;
@@ -1559,9 +1598,9 @@ esp_status_t launch_tiled_form(GemmParams &p, const GemmPlan &plan, const uint16
     p.xflags = flags;
     esp_status_t st = x_tm ? launch_xtile_tm<TN>(p, x_tm, ldx_tm, img, flags, dependent, stream) : launch_xtile<TN>(p, img, flags, dependent, stream);
     if (st != ESP_OK) return st;
-    if constexpr (TN == 128) {
+    if constexpr (TN == 128 || TN == 256) {
         if (plan.kernel != ESP_KERNEL_PAIR_TILED) return ESP_ERR_INVALID_ARG;
-        return launch_pair<2, 128, true>(p, true, stream, plan.split_k);
+        return launch_pair<TN == 128 ? 2 : 1, TN, true>(p, true, stream, plan.split_k);
     } else {
         switch (plan.kernel) {
             case ESP_KERNEL_QUAD_TILED: return launch_quad<TN>(p, true, stream);
@@ -1643,6 +1682,7 @@ esp_status_t launch_spgemm(const __half *X, int M, int K, long ldx, const void *
                 case 192: return launch_tiled_form<192>(p, plan, x_tm, ldx, img, dependent, stream, di.sm_count);
                 case 224: return launch_tiled_form<224>(p, plan, x_tm, ldx, img, dependent, stream, di.sm_count);
                 case 240: return launch_tiled_form<240>(p, plan, x_tm, ldx, img, dependent, stream, di.sm_count);
+                case 256: return launch_tiled_form<256>(p, plan, x_tm, ldx, img, dependent, stream, di.sm_count);
                 default: return ESP_ERR_INVALID_ARG;
             }
         }
@@ -1652,7 +1692,7 @@ esp_status_t launch_spgemm(const __half *X, int M, int K, long ldx, const void *
                 case 192: return launch_pair<2, 192>(p, dependent, stream);
                 case 224: return launch_pair<2, 224>(p, dependent, stream);
                 case 240: return launch_pair<2, 240>(p, dependent, stream);
-                case 256: return launch_pair<1, 256>(p, dependent, stream);
+                case 256: return launch_pair<1, 256>(p, dependent, stream, plan.split_k);
                 default: return ESP_ERR_INVALID_ARG;
             }
         }

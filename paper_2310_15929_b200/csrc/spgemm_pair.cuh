@@ -142,11 +142,19 @@ __device__ __forceinline__ void dsmem_copy(uint32_t dst_cluster, uint32_t src_ct
 constexpr int kPairProducers = 512;                  // X producer threads (warps 2..17)
 constexpr int kPairThreads = 64 + kPairProducers;
 
-template <int NA, int TN>
-struct PairCfg {
+// One X operand image: half a token tile x 128 channels.
+template <int TN>
+struct XImage {
     static constexpr int kHalf = TN / 2;                              // tokens of X each CTA stages
     static constexpr int kTokBlocks = (kHalf + 63) / 64;              // 64-token blocks of 128 rows x 128 bytes
     static constexpr int kXStage = kTokBlocks * 16384;
+};
+
+template <int NA, int TN>
+struct PairCfg : XImage<TN> {
+    using XImage<TN>::kHalf;
+    using XImage<TN>::kTokBlocks;
+    using XImage<TN>::kXStage;
     static constexpr int kWStage = NA * kTileBytes;
     static constexpr int kStage = kWStage + kXStage;                  // a multiple of 1024
     static constexpr int kStagesFit = (227 * 1024 - 512 - 1024) / kStage;
@@ -171,7 +179,7 @@ template <int TN>
 __global__ void __launch_bounds__(256) xtile_kernel(const uint16_t *__restrict__ X, long ldx, int M, int K,
                                                     const int32_t *__restrict__ perm, uint8_t *__restrict__ img,
                                                     uint32_t *__restrict__ flags, int k_tiles) {
-    using L = PairCfg<2, TN>;
+    using L = XImage<TN>;
     const int h = blockIdx.x, kt = blockIdx.y;
     const int tok_cta = (h >> 1) * TN + (h & 1) * L::kHalf;
     uint8_t *dst = img + ((size_t)h * k_tiles + kt) * L::kXStage;
@@ -243,7 +251,7 @@ template <int TN>
 __global__ void __launch_bounds__(256) xtile_tm_kernel(const uint16_t *__restrict__ X, long ldx, int M, int K,
                                                        const int32_t *__restrict__ inv, uint8_t *__restrict__ img,
                                                        uint32_t *__restrict__ flags, uint32_t *__restrict__ counts, int k_tiles) {
-    using L = PairCfg<2, TN>;
+    using L = XImage<TN>;
     __shared__ uint32_t s[64][33];           // [channel][token pair], one word of padding per row
     __shared__ int s_last;
     const int h = blockIdx.x, tb = blockIdx.y, c0 = blockIdx.z * 64;
@@ -838,7 +846,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) spgemm_pair_kernel(const Gemm
 
 template <int TN>
 size_t xtile_image_bytes(int M, int K) {
-    return (size_t)2 * ((M + TN - 1) / TN) * ((K + kTileK - 1) / kTileK) * PairCfg<2, TN>::kXStage;
+    return (size_t)2 * ((M + TN - 1) / TN) * ((K + kTileK - 1) / kTileK) * XImage<TN>::kXStage;
 }
 template <int TN>
 size_t xtile_flag_bytes(int M, int K) {
@@ -854,7 +862,7 @@ size_t xtile_bytes(int M, int K) {           // images | one flag word per image
 template <int TN>
 esp_status_t launch_xtile_tm(const GemmParams &p, const uint16_t *X_tm, long ldx_tm, uint8_t *img, uint32_t *flags,
                              bool dependent, cudaStream_t stream) {
-    using L = PairCfg<2, TN>;
+    using L = XImage<TN>;
     const int n_h = 2 * ((p.M + TN - 1) / TN), n_flags = n_h * p.k_tiles;
     int32_t *inv = reinterpret_cast<int32_t *>(reinterpret_cast<uint8_t *>(flags) + xtile_flag_bytes<TN>(p.M, p.K));
     uint32_t *counts = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(inv) + align_up((size_t)p.K * 4, 256));

@@ -630,6 +630,23 @@ def test_token_major_input_without_a_transposed_copy(M, N, K, splits):
         assert np.array_equal(Y, spgemm(X, packed, theta, N, channel_major=True, kernel=4, **kw))
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 128, 136), (130, 300, 1160), (256, 256, 2184), (300, 1000, 648), (513, 640, 520)])
+def test_tiled_256_by_256_pair_kernel(M, N, K):
+    """The pair kernel's 256-feature x 256-token tile from X images: ragged tokens, a last pair with one feature tile or two, fewer
+    channel steps than ring slots and more, K-slices of unequal length, both layouts and output types; same bits as its gather form."""
+    from tests.gpu_util import pack_on_gpu, spgemm
+    vals, meta, theta = pruned(7300 + M + K, N, K)
+    X = (np.random.default_rng(M + K).standard_normal((M, K))).astype(np.float16)
+    packed = pack_on_gpu(vals, meta)
+    Yref = ref_product(X, vals, meta, theta)
+    for split in (1, 2, 3, 4):
+        kw = dict(token_tile=256, split_k=split, channel_major=True)
+        Y = spgemm(X, packed, theta, N, kernel=6, **kw)
+        check(Y, Yref)
+        assert np.array_equal(Y, spgemm(X, packed, theta, N, kernel=5, **kw))
+    check(spgemm(X, packed, theta, N, kernel=6, token_tile=256, out_f32=True, static_weights=1), Yref, True)
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
