@@ -1325,6 +1325,43 @@ static int pair_cluster_capacity(int device, int split) {
 struct PairTile { int tokens, feature_tiles; double step_us, fixed_us; };
 static const PairTile kPairTiles[] = {{240, 4, 0.83, 13.0}, {224, 4, 0.82, 12.5}, {192, 4, 0.80, 12.0}, {256, 2, 0.585, 9.7}, {128, 4, 0.66, 10.5}};
 
+// The pair kernel's tile and K-slices of least time (us, as measured) for these sizes; *tile != 0 and split_k != 0 are requests.
+static double best_pair_tile(int M, int f_tiles, int k_tiles, int split_k, bool wide_only, const DeviceInfo &di, int *tile, int *split) {
+    const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
+    const bool requested = *tile != 0;
+    const int request = *tile;
+    double best = -1.0;
+    for (const PairTile &t : kPairTiles) {
+        if (requested ? t.tokens != request : (wide_only && (t.tokens == 128 || t.tokens == 256))) continue;
+        // waves x time of one wave.  Waves: a grid of up to two waves runs as whole waves (equal tiles end together); over many
+        // waves the clusters drift apart and the last, partial wave costs less and less of a whole one.
+        // K-slices (128- and 256-token tiles: the pushed partial rows of all slices must fit the ring), each of at least four
+        // channel steps: a cluster of 2 x split CTAs, of which far fewer fit the GPU (two slices: 33 on 148 SMs), and about
+        // 10 us for the reduction.  Beyond 256 tokens two slices at most: three ran far slower (4096 x 11008 at 384 tokens 70
+        // against 50 us).
+        const long pairs = (long)ceil_div(f_tiles, t.feature_tiles) * ceil_div(M, t.tokens);
+        const bool sliced = t.tokens == 128 || t.tokens == 256;
+        int most = sliced ? (M > 256 ? 2 : 4) : 1;
+        int wanted = split_k;
+        if (wanted > 0) {
+            if (!sliced && wanted > 1) continue;
+            while (wanted > 1 && (k_tiles / wanted < 4 || (long)ceil_div(k_tiles, wanted) * (wanted - 1) >= k_tiles)) --wanted;
+            most = wanted;
+        }
+        for (int sp = wanted > 0 ? wanted : 1; sp <= most; ++sp) {
+            if (sp > 1 && wanted == 0 && (k_tiles / sp < 4 || (long)ceil_div(k_tiles, sp) * (sp - 1) >= k_tiles)) continue;
+            const long cap = std::max<long>(1, sp == 1 ? per_wave : pair_cluster_capacity(di.device, sp));
+            if (sp > 1 && wanted == 0 && pairs > cap) continue;
+            const double w = (double)pairs / (double)cap, whole = (double)ceil_div(pairs, cap);
+            const double waves = w <= 2.0 ? whole : w + (whole - w) * (2.0 / w);
+            const double cost = waves * (t.step_us * ceil_div(k_tiles, sp) + t.fixed_us) + (sp > 1 ? 10.0 : 0.0);
+            if (log_plans()) fprintf(stderr, "esparse plan M=%d f_tiles=%d k_tiles=%d pair tile=%d split=%d pairs=%ld waves=%.2f cost=%.1f\n", M, f_tiles, k_tiles, t.tokens, sp, pairs, waves, cost);
+            if (best < 0.0 || cost < best) { best = cost; *tile = t.tokens; *split = sp; }
+        }
+    }
+    return best;
+}
+
 static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts &o, size_t workspace_bytes, GemmPlan *plan) {
     const bool have_workspace = workspace_bytes >= transpose_bytes(M, K, o) && (workspace_bytes > 0 || o.x_layout == ESP_X_CHANNEL_MAJOR);
     DeviceInfo di;
@@ -1370,7 +1407,18 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
                 if (!pair) {
                     const bool pays = M <= 32 ? weight >= 200000000L : M <= 64 ? ((f_tiles >= 64 && weight >= 40000000L) || weight >= 64000000L) : M <= 128 ? weight >= 40000000L : weight >= 16000000L;
                     // (up to 32 tokens: 32-token images -- 36864 x 9216 at 32 tokens 67.5 -> 64.3 us, 9216 x 36864 76 -> 70)
-                    if (pays) { g.kernel = ESP_KERNEL_STREAM_IMAGES; bn = M <= 32 ? 32 : (M > 128 && weight >= 64000000L) ? 128 : 64; }
+                    if (pays) {
+                        bn = M <= 32 ? 32 : (M > 128 && weight >= 64000000L) ? 128 : 64;
+                        g.kernel = ESP_KERNEL_STREAM_IMAGES;
+                        // beyond 128 tokens that kernel is bound by what all its CTAs pull from L2, about 9 TB/s: long weights go to the
+                        // pair kernel's K-slices, whose larger tiles pull less (4096 x 11008 at 200 tokens: 41.5 -> 40.0 us)
+                        int tile = 0, sp = 1;
+                        const double bytes = (double)f_tiles * ceil_div(M, bn) * k_tiles * (kTileBytes + 256.0 * bn);
+                        if (M > 128 && o.split_k == 0 && best_pair_tile(M, f_tiles, k_tiles, 0, false, di, &tile, &sp) < bytes / 9e6 - 2.0) {
+                            g.kernel = ESP_KERNEL_PAIR;
+                            bn = 0;
+                        }
+                    }
                 } else if (M > 128 && o.split_k == 0 && weight >= 80000000L && per_wave / pairs128 >= 2) {
                     g.kernel = ESP_KERNEL_STREAM_IMAGES;
                     bn = 128;
@@ -1381,39 +1429,8 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
     const bool wide_only = g.kernel == ESP_KERNEL_QUAD_TILED || g.kernel == ESP_KERNEL_PAIR_PERSIST ||
                            g.kernel == ESP_KERNEL_QUAD_MULTICAST;                                      // no 128-token form
     if (g.kernel == ESP_KERNEL_PAIR || g.kernel == ESP_KERNEL_PAIR_TILED || wide_only) {
-        const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
-        const bool requested = bn != 0;
         int split = 1;
-        double best = -1.0;
-        for (const PairTile &t : kPairTiles) {
-            if (requested ? t.tokens != bn : (wide_only && (t.tokens == 128 || t.tokens == 256))) continue;
-            // waves x time of one wave.  Waves: a grid of up to two waves runs as whole waves (equal tiles end together); over many
-            // waves the clusters drift apart and the last, partial wave costs less and less of a whole one.
-            // K-slices (128- and 256-token tiles: the pushed partial rows of all slices must fit the ring), each of at least four
-            // channel steps: a cluster of 2 x split CTAs, of which far fewer fit the GPU (two slices: 33 on 148 SMs), and about
-            // 10 us for the reduction.  Beyond 256 tokens two slices at most: three ran far slower (4096 x 11008 at 384 tokens 70
-            // against 50 us).
-            const long pairs = (long)ceil_div(f_tiles, t.feature_tiles) * ceil_div(M, t.tokens);
-            const bool sliced = t.tokens == 128 || t.tokens == 256;
-            int most = sliced ? (M > 256 ? 2 : 4) : 1;
-            int wanted = o.split_k;
-            if (wanted > 0) {
-                if (!sliced && wanted > 1) continue;
-                while (wanted > 1 && (k_tiles / wanted < 4 || (long)ceil_div(k_tiles, wanted) * (wanted - 1) >= k_tiles)) --wanted;
-                most = wanted;
-            }
-            for (int sp = wanted > 0 ? wanted : 1; sp <= most; ++sp) {
-                if (sp > 1 && wanted == 0 && (k_tiles / sp < 4 || (long)ceil_div(k_tiles, sp) * (sp - 1) >= k_tiles)) continue;
-                const long cap = std::max<long>(1, sp == 1 ? per_wave : pair_cluster_capacity(di.device, sp));
-                if (sp > 1 && wanted == 0 && pairs > cap) continue;
-                const double w = (double)pairs / (double)cap, whole = (double)ceil_div(pairs, cap);
-                const double waves = w <= 2.0 ? whole : w + (whole - w) * (2.0 / w);
-                const double cost = waves * (t.step_us * ceil_div(k_tiles, sp) + t.fixed_us) + (sp > 1 ? 10.0 : 0.0);
-                if (log_plans()) fprintf(stderr, "esparse plan M=%d N=%d K=%d pair tile=%d split=%d pairs=%ld waves=%.2f cost=%.1f\n", M, N, K, t.tokens, sp, pairs, waves, cost);
-                if (best < 0.0 || cost < best) { best = cost; bn = t.tokens; split = sp; }
-            }
-        }
-        if (best < 0.0) return ESP_ERR_INVALID_ARG;
+        if (best_pair_tile(M, f_tiles, k_tiles, o.split_k, wide_only, di, &bn, &split) < 0.0) return ESP_ERR_INVALID_ARG;
         // the tiled form needs room for the X images behind the transposed copy; without it the gather form runs.  Up to
         // 128 tokens the gather form is taken anyway: one launch instead of two, and X is small.
         // (on a large weight the gather's row copies cost more than that launch: 22016 x 8192 at 100 tokens 76 -> 61 us)
