@@ -647,6 +647,36 @@ def test_tiled_256_by_256_pair_kernel(M, N, K):
     check(spgemm(X, packed, theta, N, kernel=6, token_tile=256, out_f32=True, static_weights=1), Yref, True)
 
 
+@pytest.mark.parametrize("N,stride,shift", [(129, 129, 0), (254, 254, 0), (200, 201, 0), (384, 391, 8), (255, 260, 8), (250, 256, 0)])
+@pytest.mark.parametrize("kernel,tile", [(5, 128), (6, 192), (6, 256)])
+def test_pair_kernel_rows_without_alignment(kernel, tile, N, stride, shift):
+    """Output rows whose stride is no multiple of 16 bytes, at either parity: right values, same bits as on aligned rows, and nothing
+    written beside them."""
+    import torch
+    from paper_2310_15929_b200 import binding as b
+    from tests.gpu_util import pack_on_gpu
+    dev = torch.device("cuda:0")
+    M, K = 277, 520
+    vals, meta, theta = pruned(7900 + N, N, K)
+    X = (np.random.default_rng(N).standard_normal((M, K))).astype(np.float16)
+    Yref = ref_product(X, vals, meta, theta)
+    packed = pack_on_gpu(vals, meta)
+    Xt, perm = torch.from_numpy(X).to(dev), torch.from_numpy(theta).to(dev)
+    for dtype in (torch.float16, torch.float32):
+        o = b.esp_gemm_opts_default()
+        o.force_kernel, o.token_tile, o.out_dtype = kernel, tile, int(dtype == torch.float32)
+        ws = torch.empty(max(16, b.esp_spgemm_workspace_bytes(M, N, K, o)), dtype=torch.uint8, device=dev)
+        whole = torch.full((M, 392), 77.0, dtype=dtype, device=dev)            # aligned rows
+        b.esp_spgemm(Xt, packed, perm, whole[:, :N], o, ws)
+        buf = torch.full((M * stride + shift,), 77.0, dtype=dtype, device=dev)
+        Y = buf[shift:].view(M, stride)[:, :N]
+        b.esp_spgemm(Xt, packed, perm, Y, o, ws)
+        check(Y.cpu().numpy(), Yref, dtype == torch.float32)
+        assert torch.equal(Y, whole[:, :N])
+        assert bool((buf[:shift] == 77).all()) and bool((buf[shift:].view(M, stride)[:, N:] == 77).all())
+        assert bool((whole[:, N:] == 77).all())
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
