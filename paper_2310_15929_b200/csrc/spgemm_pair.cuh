@@ -756,31 +756,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) spgemm_pair_kernel(const Gemm
                 }
                 return;
             }
-            // Rows of Y without 16-byte alignment: a warp per row, its lanes on consecutive 32-bit words.  (One thread per 16 bytes,
-            // as above, would store element by element, each store of a warp touching 32 sectors: 17037 x 784 at 2008 tokens
-            // 176 us against 95, and 80 at 17040; 4811 x 2840 at 3687 tokens 137 against 96, and 89 at 4816.)
-            const int rows = ok ? min(TN, p.M - tok0) : 0;
-#pragma unroll 2
-            for (int row = g >> 5; row < rows; row += kPairProducers / 32) {
-                OutT *dst = yo + (long)(tok0 + row) * p.ldy;
-                const OutT *src = reinterpret_cast<const OutT *>(area) + row * 128;
-                if constexpr (sizeof(OutT) == 4) {
-#pragma unroll
-                    for (int f = lane; f < 128; f += 32)
-                        if (f < f_valid) dst[f] = src[f];
-                } else {
-                    const uint32_t *words = reinterpret_cast<const uint32_t *>(src);
-                    const uint32_t odd = (uint32_t)((reinterpret_cast<uintptr_t>(dst) >> 1) & 1u);   // element 0 in the upper half of a word of Y
-                    const int n_words = (f_valid - (int)odd) >> 1;
-#pragma unroll
-                    for (int i = lane; i < 64; i += 32) {
-                        const uint32_t w = __funnelshift_r(words[i], words[min(i + 1, 63)], 16u * odd);
-                        if (i < n_words) reinterpret_cast<uint32_t *>(dst + odd)[i] = w;
-                    }
-                    if (lane == 0 && odd) dst[0] = src[0];
-                    if (lane == 1 && (int)odd + 2 * n_words < f_valid) dst[f_valid - 1] = src[f_valid - 1];
-                }
-            }
+            store_unaligned_rows(yo + (long)tok0 * p.ldy, p.ldy, reinterpret_cast<const OutT *>(area), f_valid, ok ? min(TN, p.M - tok0) : 0, g >> 5,
+                                 kPairProducers / 32, lane);
         };
         if (split > 1) {
             // ---- K-slices: the pairs of the cluster hold partial sums of the same tile.  Its token rows are dealt to the

@@ -648,8 +648,8 @@ def test_tiled_256_by_256_pair_kernel(M, N, K):
 
 
 @pytest.mark.parametrize("N,stride,shift", [(129, 129, 0), (254, 254, 0), (200, 201, 0), (384, 391, 8), (255, 260, 8), (250, 256, 0)])
-@pytest.mark.parametrize("kernel,tile", [(5, 128), (6, 192), (6, 256)])
-def test_pair_kernel_rows_without_alignment(kernel, tile, N, stride, shift):
+@pytest.mark.parametrize("kernel,tile", [(4, 16), (4, 64), (4, 256), (5, 128), (6, 192), (6, 256), (10, 128)])
+def test_output_rows_without_alignment(kernel, tile, N, stride, shift):
     """Output rows whose stride is no multiple of 16 bytes, at either parity: right values, same bits as on aligned rows, and nothing
     written beside them."""
     import torch
@@ -664,7 +664,7 @@ def test_pair_kernel_rows_without_alignment(kernel, tile, N, stride, shift):
     Xt, perm = torch.from_numpy(X).to(dev), torch.from_numpy(theta).to(dev)
     for dtype in (torch.float16, torch.float32):
         o = b.esp_gemm_opts_default()
-        o.force_kernel, o.token_tile, o.out_dtype = kernel, tile, int(dtype == torch.float32)
+        o.force_kernel, o.token_tile, o.split_k, o.out_dtype = kernel, tile, 1, int(dtype == torch.float32)
         ws = torch.empty(max(16, b.esp_spgemm_workspace_bytes(M, N, K, o)), dtype=torch.uint8, device=dev)
         whole = torch.full((M, 392), 77.0, dtype=dtype, device=dev)            # aligned rows
         b.esp_spgemm(Xt, packed, perm, whole[:, :N], o, ws)
