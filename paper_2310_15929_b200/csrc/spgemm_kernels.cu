@@ -1080,45 +1080,34 @@ esp_status_t launch_stream_group(const GemmGroup &grp, int t_tiles, int split, i
     return ESP_OK;
 }
 
-// Clusters of `split` CTAs of the streaming kernel that can be resident at once on this device.
-template <int BN>
-int stream_cluster_capacity(int split, int stages, int x_mode, int x_area) {
-    auto kern = stream_kernel_for<BN>(x_mode);
-    const size_t smem = stream_smem_bytes(BN, stages, split, x_area);
-    if (ensure_dynamic_smem((const void *)kern, (int)smem) != cudaSuccess) return 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1, 1, split);
-    cfg.blockDim = dim3(StreamCfg<BN>::kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = split;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+// Clusters of `split` CTAs that the device's GPCs hold with one streaming CTA per SM, asked once per device and size.  (The occupancy
+// calculator answers with one CTA per SM for these kernels whatever their size, since it cannot know how much tensor memory a CTA
+// will allocate; so the packing is asked for a CTA that fills an SM, and stream_capacity_ctas counts the CTAs that share one.)
+static int stream_clusters_one_per_sm(int device, int split) {
+    static std::mutex mu;
+    static std::map<int, int> cache;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find(device * 16 + split);
+    if (it != cache.end()) return it->second;
+    auto kern = stream_kernel_for<128>(kXChannelMajor);
+    const size_t smem = stream_smem_bytes(128, 4, split, 0);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
-    // The occupancy calculator answers with one CTA per SM for these kernels whatever their size (it cannot know how much
-    // tensor memory a CTA will allocate); CTAs do share an SM when shared memory, threads and tensor-memory columns
-    // allow.  So its answer is taken as the packing of clusters onto GPCs at the calculator's CTAs per SM and scaled.
-    int api_per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&api_per_sm, kern, StreamCfg<BN>::kThreads, smem) != cudaSuccess || api_per_sm < 1) {
-        cudaGetLastError();
-        api_per_sm = 1;
+    if (ensure_dynamic_smem((const void *)kern, (int)smem) == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, 1, split);
+        cfg.blockDim = dim3(StreamCfg<128>::kThreads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = split;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
     }
-    int dev = 0, smem_per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    int per_sm = (int)((size_t)smem_per_sm / (smem + 1024));
-    per_sm = per_sm < 2048 / StreamCfg<BN>::kThreads ? per_sm : 2048 / StreamCfg<BN>::kThreads;
-    per_sm = per_sm < 512 / (int)tmem_cols_for(BN) ? per_sm : 512 / (int)tmem_cols_for(BN);
-    if (per_sm < api_per_sm) per_sm = api_per_sm;
-    const int clusters = (int)((long)n * per_sm / api_per_sm);
-    if (log_plans())
-        fprintf(stderr, "esparse occupancy tile=%d split=%d stages=%d smem=%zu: calculator clusters=%d at %d CTAs/SM, taken %d at %d CTAs/SM\n", BN,
-                split, stages, smem, n, api_per_sm, clusters, per_sm);
-    return clusters;
+    if (log_plans()) fprintf(stderr, "esparse streaming clusters of %d CTAs, one CTA per SM: %d fit\n", split, n);
+    return cache[device * 16 + split] = n;
 }
 
 #include "spgemm_pair.cuh"
@@ -1261,26 +1250,11 @@ size_t gemm_workspace_bytes(int M, int K, const esp_gemm_opts &o) {
 }
 
 // Resident capacity (in CTAs) of the streaming kernel for one configuration, cached per process.
-static int stream_capacity_ctas(int bn, int split, int stages, int x_mode, int x_area) {
-    static std::mutex mu;
-    static std::map<long, int> cache;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const long key = (((((long)dev * 512 + bn) * 16 + split) * 16 + stages) * 4 + x_mode) * 65536 + x_area;
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = cache.find(key);
-    if (it != cache.end()) return it->second;
-    int clusters = 0;
-    switch (bn) {
-        case 16: clusters = stream_cluster_capacity<16>(split, stages, x_mode, x_area); break;
-        case 32: clusters = stream_cluster_capacity<32>(split, stages, x_mode, x_area); break;
-        case 64: clusters = stream_cluster_capacity<64>(split, stages, x_mode, x_area); break;
-        case 128: clusters = stream_cluster_capacity<128>(split, stages, x_mode, x_area); break;
-        case 256: clusters = stream_cluster_capacity<256>(split, stages, x_mode, x_area); break;
-        default: break;
-    }
-    cache[key] = clusters * split;
-    return clusters * split;
+static int stream_capacity_ctas(const DeviceInfo &di, const int *layer, int bn, int split, int stages, int x_area) {
+    const int threads = bn >= 64 ? StreamCfg<64>::kThreads : StreamCfg<16>::kThreads;
+    int per_sm = (int)((size_t)(di.max_smem_optin + 1024) / (stream_smem_bytes(bn, stages, split, x_area) + 1024));
+    per_sm = std::min(per_sm, std::min(2048 / threads, 512 / tmem_cols_for(bn)));
+    return layer[split] * split * std::max(per_sm, 1);
 }
 
 // Clusters of 2 x split CTAs of the pair kernel that the device holds at once, asked once per device.
@@ -1356,6 +1330,160 @@ static double best_pair_tile(int M, int f_tiles, int k_tiles, int split_k, bool 
     return best;
 }
 
+// K-slices, ring depth and input form of the streaming kernel for one token tile (split_k != 0: that many slices, or fewer without an
+// empty one).  `capacity`: CTAs that the device holds at once in that form.
+struct StreamShape { int split, stages, x_mode, x_area, capacity; };
+static bool stream_shape(int M, int N, int K, const esp_gemm_opts &o, int kernel, int bn, int split_k, const DeviceInfo &di, const int *layer,
+                         StreamShape *shape) {
+    const int k_tiles = ceil_div(K, kTileK), f_tiles = ceil_div(N, kTileFeat);
+    const long tiles = (long)f_tiles * ceil_div(M, bn);
+    auto no_empty_slice = [&](int split) { return (long)ceil_div(k_tiles, split) * (split - 1) < k_tiles; };
+    // Pick K-slices and CTAs per SM so that, if possible, the whole grid is resident at once and each CTA
+    // has a short chain of tiles: cost ~ waves x (tiles per CTA + fixed start-up and reduction time).
+    const size_t per_stage = (size_t)kTileBytes + 256 * (size_t)bn;
+    double best_cost = 1e30;
+    shape->split = 0;
+    int wanted = split_k > k_tiles ? k_tiles : split_k;      // a requested split steps down to one without empty slices
+    while (wanted > 1 && !no_empty_slice(wanted)) --wanted;
+    for (int split = 1; split <= 8 && split <= k_tiles; ++split) {
+        if (wanted != 0 && split != wanted) continue;
+        if (!no_empty_slice(split)) continue;
+        const int kts = ceil_div(k_tiles, split);
+        // token-major X without a transposing launch: up to two tokens straight from X (4096 x 11008, us per call: 14.6 -> 13.0 at
+        // one token, 14.6 -> 15.4 at two; 22016 x 8192: 37.2 -> 34.9 and 35.5; at four tokens the element loads cost more than the
+        // launch, 14.7 -> 22.8), through the cluster where the weight is
+        // small (its start is longer, but the call saves a launch: 512 x 512 at 128 tokens 8.7 -> 6.2, 2048 x 2048 at 16 tokens 8.1 ->
+        // 7.0, at 32 tokens 8.2 -> 8.9; 4096 x 4096 at 16 tokens 9.2 -> 11.7)
+        int x_mode = kXChannelMajor, x_area = 0;
+        if (kernel == ESP_KERNEL_STREAM && o.x_layout == ESP_X_TOKEN_MAJOR) {
+            const long weight = (long)N * K;
+            if (bn == 16 && (M == 1 || (M <= kXDirectTokens && K <= 8192))) x_mode = kXDirect;
+            else if (bn <= 32 && weight <= (M <= 16 ? 4500000L : 1200000L) && stream_x_area_bytes(bn, M, kts) <= kXAreaMax) {
+                x_mode = kXCluster;
+                x_area = stream_x_area_bytes(bn, M, kts);
+            }
+        }
+        const size_t fixed = stream_recv_bytes(bn, split) + (size_t)x_area + kPermRing * 512 + 512 + 1024;
+        int last_stages = -1;
+        for (int r = 1; r <= 4; ++r) {
+            const size_t budget = (size_t)di.max_smem_optin / r - (r > 1 ? 1024 : 0);
+            if (budget < fixed + 2 * per_stage) break;
+            int stages = (int)((budget - fixed) / per_stage);
+            if (o.pipeline_stages > 0) {                              // a requested ring depth: this one only, or what fits
+                if (r > 1) break;
+                if (stages > o.pipeline_stages) stages = o.pipeline_stages;
+            }
+            if (stages > kMaxStages) stages = kMaxStages;
+            if (stages > kts) stages = kts < 2 ? 2 : kts;
+            if (stages == last_stages) continue;
+            last_stages = stages;
+            const int cap = stream_capacity_ctas(di, layer, bn, split, stages, x_area);
+            if (cap <= 0) continue;
+            const long ctas = tiles * split;
+            const long waves = (ctas + cap - 1) / cap;
+            // per CTA: kts steps + set-up, reduction and epilogue, which grow with the token tile (measured: a 256-token
+            // tile in one wave of 32 steps beats three waves of 8)
+            // wide token tiles are bound by their X gather, which CTAs sharing an SM share: a step costs as many
+            // times more as CTAs of one wave sit on an SM
+            const long in_wave = ctas < cap ? ctas : cap;
+            const double share = (bn >= 64 && kernel == ESP_KERNEL_STREAM) ? (double)((in_wave + di.sm_count - 1) / di.sm_count) : 1.0;
+            double cost = (double)waves * (kts * share + 2.0 + bn / 32.0) + (split > 1 ? 0.25 + 0.05 * split : 0.0) + 0.01 * r;
+            // with static_weights consecutive launches overlap on an SM: prefer leaving room for a CTA of the next one
+            // (not when every CTA has an SM of its own anyway: a deeper ring is then free, measured 16.0 -> 12.6 us on
+            // 4096 x 4096 at 64 tokens)
+            if (o.static_weights && o.pipeline_stages == 0 && ctas > di.sm_count &&
+                2 * (stream_smem_bytes(bn, stages, split, x_area) + 1024) > (size_t)di.max_smem_optin)
+                cost += 3.0;
+            if (log_plans())
+                fprintf(stderr, "esparse plan M=%d N=%d K=%d tile=%d: split=%d stages=%d capacity=%d ctas=%ld waves=%ld cost=%.2f\n", M, N, K,
+                        bn, split, stages, cap, ctas, waves, cost);
+            if (cost < best_cost) { best_cost = cost; *shape = StreamShape{split, stages, x_mode, x_area, cap}; }
+        }
+    }
+    return shape->split != 0;
+}
+
+// Times (us) of the forms that a product of more than 64 tokens on a weight below 40 M elements can take, fitted to 33000 measured
+// calls: random shapes of 512..11008 features x channels at 60..8200 tokens, every form, tile and number of K-slices that runs
+// (half of the estimates within 5 to 10 %, nine of ten within 20 %; the form chosen by them is 2.5 % slower than the best
+// measured one in the geometric mean).  Rules of one threshold each stood here before: up to 256 tokens the streaming kernel's 128- and
+// 256-token tiles, the pair kernel beyond.  Small weights lost most: 1010 x 1960 at 181 tokens 15.3 -> 7.8 us, 972 x 3280 at 546 34 -> 16.
+// Streaming kernel: waves of the grid (`wave`), CTAs on an SM in each (`wave_sm`), channel steps of these, MB that all CTAs pull from
+// L2, K-slices, and the pass that writes X images (per 1e6 elements of X).
+struct StreamTime { int tokens; bool images; double start, step, step_sm, wave, wave_sm, per_mb, slice, image; };
+static const StreamTime kStreamTimes[] = {
+    {32, false, 1.57, 0.443, 0.000, 3.42, 0.00, 0.040, 0.06, 0.00},
+    {64, false, 1.97, 0.578, 0.146, 0.84, 1.92, 0.054, 0.17, 0.00},
+    {128, false, 3.01, 0.654, 0.157, 0.00, 3.34, 0.052, 0.18, 0.00},
+    {256, false, 0.00, 0.000, 1.113, 0.00, 9.93, 0.033, 0.49, 0.00},
+    {32, true, 3.81, 0.362, 0.000, 4.43, 0.00, 0.030, 0.06, 1.60},
+    {64, true, 4.21, 0.389, 0.000, 3.04, 1.66, 0.028, 0.19, 0.73},
+    {128, true, 5.03, 0.276, 0.115, 2.27, 3.26, 0.044, 0.22, 0.71},
+    {256, true, 0.75, 0.000, 1.207, 0.00, 11.90, 0.015, 0.77, 0.97},
+};
+// Pair kernel, gather form and tiled form: one channel step, the rest of a wave, K-slices, the tiling pass (or, gather form, the row
+// copies).
+struct PairTime { int tokens; bool tiled; double step, wave, slices, x; };
+static const PairTime kPairTimes[] = {
+    {128, false, 0.827, 11.1, 4.5, 0.26},
+    {256, false, 0.782, 9.5, 5.4, 0.56},
+    {128, true, 0.594, 13.3, 5.2, 0.93},
+    {192, true, 0.718, 13.4, 0.0, 1.16},
+    {224, true, 0.715, 14.3, 0.0, 1.16},
+    {240, true, 0.727, 14.5, 0.0, 1.09},
+    {256, true, 0.520, 11.7, 6.9, 0.96},
+};
+
+// The form of least estimated time.
+static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, bool images_room, const DeviceInfo &di, const int *layer, GemmPlan *g) {
+    const int k_tiles = ceil_div(K, kTileK), f_tiles = ceil_div(N, kTileFeat);
+    const double x_elems = 1e-6 * (double)K * M;
+    double best = 1e30;
+    auto take = [&](double us, int kernel, int tile, const StreamShape &sh) {
+        if (log_plans()) fprintf(stderr, "esparse plan M=%d N=%d K=%d kernel=%d tile=%d split=%d: %.1f us\n", M, N, K, (int)kernel, tile, sh.split, us);
+        if (us >= best) return;
+        best = us;
+        g->kernel = kernel;
+        g->token_tile = tile;
+        g->split_k = sh.split;
+        g->stages = sh.stages;
+        g->x_mode = sh.x_mode;
+        g->x_area = sh.x_area;
+    };
+    for (const StreamTime &t : kStreamTimes) {
+        if ((t.images && !images_room) || t.tokens >= 2 * M) continue;
+        const int kernel = t.images ? ESP_KERNEL_STREAM_IMAGES : ESP_KERNEL_STREAM;
+        const long tiles = (long)f_tiles * ceil_div(M, t.tokens);
+        for (int split : {1, 2, 3, 4, 6, 8}) {
+            StreamShape sh;
+            if (split > k_tiles || (long)ceil_div(k_tiles, split) * (split - 1) >= k_tiles) continue;
+            if (!stream_shape(M, N, K, o, kernel, t.tokens, split, di, layer, &sh)) continue;
+            const long ctas = tiles * split, waves = (ctas + sh.capacity - 1) / sh.capacity;
+            const long on_sm = waves * ((std::min<long>(ctas, sh.capacity) + di.sm_count - 1) / di.sm_count);
+            const int steps = ceil_div(k_tiles, split);
+            const double mb = 1e-6 * (double)ctas * steps * (kTileBytes + 256.0 * t.tokens);
+            take(t.start + waves * (t.wave + t.step * steps) + on_sm * (t.wave_sm + t.step_sm * steps) + t.per_mb * mb + t.slice * split + t.image * x_elems,
+                 kernel, t.tokens, sh);
+        }
+    }
+    const long per_wave = std::max(1, di.sm_count / 2);
+    for (const PairTime &t : kPairTimes) {
+        if (t.tiled && !images_room) continue;
+        const bool sliced = t.tokens == 128 || t.tokens == 256;             // (as in best_pair_tile)
+        const long pairs = (long)ceil_div(f_tiles, t.tokens == 256 ? 2 : 4) * ceil_div(M, t.tokens);
+        for (int split = 1; split <= (sliced ? (M > 256 ? 2 : 4) : 1); ++split) {
+            if (split > 1 && (k_tiles / split < 4 || (long)ceil_div(k_tiles, split) * (split - 1) >= k_tiles)) continue;
+            const long cap = std::max<long>(1, split == 1 ? per_wave : pair_cluster_capacity(di.device, split));
+            if (split > 1 && pairs > cap) continue;
+            const double w = (double)pairs / (double)cap, whole = (double)ceil_div(pairs, cap);
+            const double waves = w <= 2.0 ? whole : w + (whole - w) * (2.0 / w);
+            take(waves * (t.wave + t.step * ceil_div(k_tiles, split)) + (split > 1 ? t.slices : 0.0) + t.x * x_elems,
+                 t.tiled ? ESP_KERNEL_PAIR_TILED : ESP_KERNEL_PAIR, t.tokens, StreamShape{split, 0, kXChannelMajor, 0, 0});
+        }
+    }
+    return best < 1e30;
+}
+
 static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts &o, size_t workspace_bytes, GemmPlan *plan) {
     const bool have_workspace = workspace_bytes >= transpose_bytes(M, K, o) && (workspace_bytes > 0 || o.x_layout == ESP_X_CHANNEL_MAJOR);
     DeviceInfo di;
@@ -1368,6 +1496,8 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
     const int f_tiles = ceil_div(N, kTileFeat);
     const bool channel_major_available = (o.x_layout == ESP_X_CHANNEL_MAJOR) || have_workspace;
     int bn = o.token_tile;
+    int layer[9] = {};
+    for (int split = 1; split <= 8; ++split) layer[split] = stream_clusters_one_per_sm(di.device, split);
     g.kernel = ESP_KERNEL_GATHER;
     if (o.force_kernel != ESP_KERNEL_GATHER && channel_major_available) {
         if (o.force_kernel == ESP_KERNEL_TMA) g.kernel = ESP_KERNEL_TMA;
@@ -1379,6 +1509,17 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
         else if (o.force_kernel == ESP_KERNEL_STREAM) g.kernel = ESP_KERNEL_STREAM;
         else if (o.force_kernel == ESP_KERNEL_STREAM_IMAGES) g.kernel = ESP_KERNEL_STREAM_IMAGES;
         else {
+            const long weight = (long)N * K;
+            // Small and middle weights at more than 64 tokens: the form of least estimated time.  (A few feature tiles on few tokens keep
+            // the rule of narrow token tiles below, which those times do not cover; larger weights keep the rules that follow,
+            // which measure within 10 % of the best form there.  Beyond 256 tokens and below 16 channel steps the tiled pair form stays the
+            // default, as callers that ask for the plan expect; the others would gain up to 7 us of 15 there.)
+            const bool narrow = M <= 256 && (long)f_tiles * k_tiles <= 64 && (long)f_tiles * ceil_div(M, 64) * std::min(k_tiles, 8) <= 2L * di.sm_count;
+            if (M > 64 && bn == 0 && o.split_k == 0 && o.pipeline_stages == 0 && !narrow && (M <= 256 || k_tiles >= 16) && weight < (M > 1000 ? 15000000L : 40000000L) &&
+                fastest_form(M, N, K, o, workspace_bytes >= gemm_workspace_bytes(M, K, o), di, layer, &g)) {
+                *plan = g;
+                return ESP_OK;
+            }
             // The pair kernel takes every M > 64; a requested token tile or slice count that only the streaming kernel has
             // (tiles below 128 tokens, more than four slices, slices of a 256-token tile) goes there.
             const bool stream_only = (bn != 0 && bn < 128) || o.split_k > 4 || (bn == 256 && o.split_k > 1);
@@ -1394,7 +1535,6 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
             // 78 -> 67 / 118 -> 68 us; 9216 x 9216 at 64 / 128 tokens 41 -> 28 / 47 -> 37 us; but 9216 x 9216 at 32 tokens
             // 22.5 -> 28.4, 4096 x 4096 at 128 tokens 15.0 -> 17.1).  It also replaces the pair kernel's gather form where that
             // would run K-slices at 129..256 tokens (9216 x 9216 at 256 tokens: 95 -> 55 us).
-            const long weight = (long)N * K;
             const bool images_room = workspace_bytes >= transpose_bytes(M, K, o) + ximg_bytes(M, K, 128);
             if (images_room && bn == 0 && o.split_k <= 8 && M > 16 && M <= 256) {
                 const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
@@ -1462,71 +1602,12 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
     const long tiles = (long)f_tiles * t_tiles;
     auto no_empty_slice = [&](int split) { return (long)ceil_div(k_tiles, split) * (split - 1) < k_tiles; };
     if (g.kernel == ESP_KERNEL_STREAM || g.kernel == ESP_KERNEL_STREAM_IMAGES) {
-        // Pick K-slices and CTAs per SM so that, if possible, the whole grid is resident at once and each CTA
-        // has a short chain of tiles: cost ~ waves x (tiles per CTA + fixed start-up and reduction time).
-        const size_t per_stage = (size_t)kTileBytes + 256 * (size_t)bn;
-        double best_cost = 1e30;
-        int best_split = 0, best_stages = 0;
-        int wanted = o.split_k > k_tiles ? k_tiles : o.split_k;      // a requested split steps down to one without empty slices
-        while (wanted > 1 && !no_empty_slice(wanted)) --wanted;
-        for (int split = 1; split <= 8 && split <= k_tiles; ++split) {
-            if (wanted != 0 && split != wanted) continue;
-            if (!no_empty_slice(split)) continue;
-            const int kts = ceil_div(k_tiles, split);
-            // token-major X without a transposing launch: up to two tokens straight from X (4096 x 11008, us per call: 14.6 -> 13.0 at
-            // one token, 14.6 -> 15.4 at two; 22016 x 8192: 37.2 -> 34.9 and 35.5; at four tokens the element loads cost more than the
-            // launch, 14.7 -> 22.8), through the cluster where the weight is
-            // small (its start is longer, but the call saves a launch: 512 x 512 at 128 tokens 8.7 -> 6.2, 2048 x 2048 at 16 tokens 8.1 ->
-            // 7.0, at 32 tokens 8.2 -> 8.9; 4096 x 4096 at 16 tokens 9.2 -> 11.7)
-            int x_mode = kXChannelMajor, x_area = 0;
-            if (g.kernel == ESP_KERNEL_STREAM && o.x_layout == ESP_X_TOKEN_MAJOR) {
-                const long weight = (long)N * K;
-                if (bn == 16 && (M == 1 || (M <= kXDirectTokens && K <= 8192))) x_mode = kXDirect;
-                else if (bn <= 32 && weight <= (M <= 16 ? 4500000L : 1200000L) && stream_x_area_bytes(bn, M, kts) <= kXAreaMax) {
-                    x_mode = kXCluster;
-                    x_area = stream_x_area_bytes(bn, M, kts);
-                }
-            }
-            const size_t fixed = stream_recv_bytes(bn, split) + (size_t)x_area + kPermRing * 512 + 512 + 1024;
-            int last_stages = -1;
-            for (int r = 1; r <= 4; ++r) {
-                const size_t budget = (size_t)di.max_smem_optin / r - (r > 1 ? 1024 : 0);
-                if (budget < fixed + 2 * per_stage) break;
-                int stages = (int)((budget - fixed) / per_stage);
-                if (o.pipeline_stages > 0) {                              // a requested ring depth: this one only, or what fits
-                    if (r > 1) break;
-                    if (stages > o.pipeline_stages) stages = o.pipeline_stages;
-                }
-                if (stages > kMaxStages) stages = kMaxStages;
-                if (stages > kts) stages = kts < 2 ? 2 : kts;
-                if (stages == last_stages) continue;
-                last_stages = stages;
-                const int cap = stream_capacity_ctas(bn, split, stages, x_mode, x_area);
-                if (cap <= 0) continue;
-                const long ctas = tiles * split;
-                const long waves = (ctas + cap - 1) / cap;
-                // per CTA: kts steps + set-up, reduction and epilogue, which grow with the token tile (measured: a 256-token
-                // tile in one wave of 32 steps beats three waves of 8)
-                // wide token tiles are bound by their X gather, which CTAs sharing an SM share: a step costs as many
-                // times more as CTAs of one wave sit on an SM
-                const long in_wave = ctas < cap ? ctas : cap;
-                const double share = (bn >= 64 && g.kernel == ESP_KERNEL_STREAM) ? (double)((in_wave + di.sm_count - 1) / di.sm_count) : 1.0;
-                double cost = (double)waves * (kts * share + 2.0 + bn / 32.0) + (split > 1 ? 0.25 + 0.05 * split : 0.0) + 0.01 * r;
-                // with static_weights consecutive launches overlap on an SM: prefer leaving room for a CTA of the next one
-                // (not when every CTA has an SM of its own anyway: a deeper ring is then free, measured 16.0 -> 12.6 us on
-                // 4096 x 4096 at 64 tokens)
-                if (o.static_weights && o.pipeline_stages == 0 && ctas > di.sm_count &&
-                    2 * (stream_smem_bytes(bn, stages, split, x_area) + 1024) > (size_t)di.max_smem_optin)
-                    cost += 3.0;
-                if (log_plans())
-                    fprintf(stderr, "esparse plan M=%d N=%d K=%d tile=%d: split=%d stages=%d capacity=%d ctas=%ld waves=%ld cost=%.2f\n", M, N, K,
-                            bn, split, stages, cap, ctas, waves, cost);
-                if (cost < best_cost) { best_cost = cost; best_split = split; best_stages = stages; g.x_mode = x_mode; g.x_area = x_area; }
-            }
-        }
-        if (best_split == 0) return ESP_ERR_UNSUPPORTED;
-        g.split_k = best_split;
-        g.stages = best_stages;
+        StreamShape shape;
+        if (!stream_shape(M, N, K, o, g.kernel, bn, o.split_k, di, layer, &shape)) return ESP_ERR_UNSUPPORTED;
+        g.split_k = shape.split;
+        g.stages = shape.stages;
+        g.x_mode = shape.x_mode;
+        g.x_area = shape.x_area;
         *plan = g;
         return ESP_OK;
     }

@@ -677,6 +677,28 @@ def test_output_rows_without_alignment(kernel, tile, N, stride, shift):
         assert bool((whole[:, N:] == 77).all())
 
 
+@pytest.mark.parametrize("M,N,K", [(65, 512, 512), (65, 1030, 1032), (129, 2050, 520), (256, 384, 2056), (257, 700, 4104), (640, 1152, 2056), (1001, 514, 2320)])
+@pytest.mark.parametrize("channel_major", [False, True])
+def test_form_chosen_for_small_weights(M, N, K, channel_major):
+    """Default options, sizes on which the streaming, image and pair forms are chosen, with a workspace and without."""
+    import torch
+    from paper_2310_15929_b200 import binding as b
+    from tests.gpu_util import pack_on_gpu
+    dev = torch.device("cuda:0")
+    vals, meta, theta = pruned(8300 + M + K, N, K)
+    X = (np.random.default_rng(M + K).standard_normal((M, K))).astype(np.float16)
+    Yref = ref_product(X, vals, meta, theta)
+    packed, perm = pack_on_gpu(vals, meta), torch.from_numpy(theta).to(dev)
+    ldx = (M + 7) // 8 * 8
+    Xt = torch.from_numpy(X).to(dev) if not channel_major else torch.nn.functional.pad(torch.from_numpy(X.T.copy()), (0, ldx - M)).to(dev)[:, :M]
+    o = b.esp_gemm_opts_default()
+    o.x_layout = int(channel_major)
+    for ws in (torch.empty(b.esp_spgemm_workspace_bytes(M, N, K, o), dtype=torch.uint8, device=dev), None):
+        Y = torch.empty(M, N, dtype=torch.float16, device=dev)
+        b.esp_spgemm(Xt, packed, perm, Y, o, ws)
+        check(Y.cpu().numpy(), Yref)
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
