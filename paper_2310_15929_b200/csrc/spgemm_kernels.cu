@@ -501,9 +501,11 @@ inline size_t stream_smem_bytes(int bn, int stages, int split, int x_area) {
 }
 
 // XMODE: kernels of their own, so that the registers of the token-major producers cost the channel-major form no residency.
-// (At least 1152 threads per SM for that one, 56 registers: two CTAs of 576 threads share an SM, six of 192.)
+// (Registers: two CTAs of 576 threads share an SM, 56 each; a 256-token tile has an SM to itself; of the narrow tiles, whose shared memory lets
+// two to four CTAs share one, four and three.  Bounded to 56 as well, a narrow tile's X loop lost up to 10 %: 4096 x 4096 at 16 tokens,
+// device-bound, 6.9 -> 6.45 us, 2208 x 6528 at 37 tokens 10.4 -> 9.7.)
 template <int BN, int XMODE>
-__global__ void __launch_bounds__(StreamCfg<BN>::kThreads, XMODE == kXChannelMajor ? 1152 / StreamCfg<BN>::kThreads : 4) spgemm_stream_kernel(const GemmGroup grp, const int stages) {
+__global__ void __launch_bounds__(StreamCfg<BN>::kThreads, BN == 256 ? 1 : BN >= 64 ? 2 : XMODE == kXChannelMajor ? 4 : 3) spgemm_stream_kernel(const GemmGroup grp, const int stages) {
     constexpr bool TM = XMODE != kXChannelMajor, xcluster = XMODE == kXCluster;
     using L = StreamCfg<BN>;
     // this CTA's problem: selected with constant indices so that the parameters stay in registers
