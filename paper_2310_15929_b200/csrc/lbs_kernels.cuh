@@ -23,7 +23,7 @@
 //
 // Measured against one comparison and two fp64 additions per (row, candidate, slot) with a warp per candidate (about 29 instructions
 // each): table of a 4096 x 4096 weight 6.94 -> 0.92 ms, greedy kernel 67.7 -> 9.3 ms; 13824 x 5120: 29.1 -> 3.8 ms and 223 -> 24.6 ms;
-// 512 x 512 (two blocks): 15.6 -> 3.0 ms.
+// 512 x 512 (two blocks): 15.6 -> 2.6 ms.
 
 constexpr int kLbsMax = 256;       // widest local-shuffle block
 constexpr int kLbsGroups = kLbsMax / 4;
@@ -35,9 +35,20 @@ struct LbsRec {                    // one row of one group: the slots ranked sec
     float p2, p3;                  // their products
     uint32_t u2, u3;               // their |w|: integers of 2^-24, in an irregular row fp16 bits
 };
+// A short slice's regular rows (lbs_thin): per live slot the product to beat, and what the candidate then displaces from each of the
+// three other slots (one of them, zero from the rest).
+constexpr int kThinRows = 192;
+template <int NS>
+struct __align__(16) LbsThinRec {
+    float bound[NS];
+    uint32_t u[NS][3];
+};
 template <int ROWS>
 struct LbsRows {                   // the rows of a chunk as one group sees them, sorted by class
-    LbsRec rec[ROWS];
+    union {
+        LbsRec rec[ROWS];
+        struct { LbsThinRec<4> thin[kThinRows]; LbsRec thin_irregular[kThinRows]; };
+    };
     uint16_t row[ROWS];
     uint16_t h1[ROWS];             // |w| bits of the slot ranked first
     uint8_t order[ROWS];           // rank order
@@ -126,11 +137,11 @@ __device__ __forceinline__ int lbs_classify(const uint16_t (&h)[4], const LbsGro
 
 // Sorted records of NG groups over `nrows` <= ROWS rows.  Wt: the channel-major copy at the chunk's first row, so that the lanes of a
 // warp read consecutive rows of a channel (from the gathered rows, 32 lanes would touch 32 lines per slot).  A thread keeps its
-// records in registers from the count to the scatter.  `thin`: regular rows stay one class (see lbs_each) and the group sums of all
+// records in registers from the count to the scatter.  `thin`: regular rows stay one class (see lbs_thin) and the group sums of all
 // rows are added here; else those of the irregular ones.  The class counters are zero on entry and on return.
-template <int NG, int ROWS, int THREADS>
+template <int NG, int ROWS, int THREADS, int NS>
 __device__ __forceinline__ void lbs_prepare(const uint16_t *__restrict__ Wt, long ldt, const uint8_t *__restrict__ irregular, int nrows,
-                                            const LbsGroup *grp, bool thin, LbsRows<ROWS> *rows, uint32_t *sums) {
+                                            const LbsGroup *grp, const int *skip, bool thin, LbsRows<ROWS> *rows, uint32_t *sums) {
     constexpr int kPer = NG * ROWS / THREADS;
     static_assert(kPer * THREADS == NG * ROWS && kPer <= 4, "rows per thread");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -185,7 +196,22 @@ __device__ __forceinline__ void lbs_prepare(const uint16_t *__restrict__ Wt, lon
         const int i = tid + u * THREADS;
         if (i < total) {
             const int g = NG > 1 && i >= nrows ? 1 : 0, at = rows[g].off[(where[u] >> 8) & 0xFF] + (where[u] >> 16);
-            rows[g].rec[at] = rec[u];
+            if (!thin) rows[g].rec[at] = rec[u];
+            else if (irr[u]) rows[g].thin_irregular[at - rows[g].off[kLbsIrregular]] = rec[u];
+            else {
+                int p1, p2, p3, p4;
+                lbs_order_slots(where[u] & 0xFF, p1, p2, p3, p4);
+                LbsThinRec<NS> &t = reinterpret_cast<LbsThinRec<NS> *>(rows[g].thin)[at];
+#pragma unroll
+                for (int l = 0; l < NS; ++l) {
+                    const int k = NS == 4 ? l : l + (l >= skip[g] ? 1 : 0);
+                    const bool top = k == p1 || k == p2;
+                    const int f2 = top ? p3 : p2;
+                    t.bound[l] = top ? rec[u].p3 : rec[u].p2;
+#pragma unroll
+                    for (int o = 0; o < 3; ++o) t.u[l][o] = o + (o >= k ? 1 : 0) == f2 ? (top ? rec[u].u3 : rec[u].u2) : 0u;
+                }
+            }
             rows[g].row[at] = (uint16_t)(i - g * nrows);
             rows[g].h1[at] = h1[u];
             rows[g].order[at] = (uint8_t)where[u];
@@ -316,115 +342,167 @@ __device__ __forceinline__ void lbs_regular(const uint16_t *__restrict__ Wb, int
     }
 }
 
-// ---- The rows [lo, hi) one by one, one candidate per lane (x; a group's candidates in eight warps), the per-slot totals in registers, a
-// branch on the row's rank order.  For irregular rows (fp64 products, 64-bit sums), and for the regular rows of a short slice, where a
-// class would change every few rows and what that costs above would be most of the time.
-template <int P1, int P2, int P3, int P4, typename Acc>
-__device__ __forceinline__ void lbs_add(Acc (&kept)[4], Acc (&displaced)[4][4], Acc f, Acc u2, Acc u3, bool gt2, bool eq2, bool gt3, bool eq3) {
+// ---- One candidate per lane (x; a group's candidates in eight warps), the per-slot totals in registers.
+// The regular rows of a short slice, where a class would change every few rows and what that costs above would be most of the time:
+// four predicated additions per live slot, whatever the row's rank order -- no branch (a jump by rank order took 550 clocks a row, most of
+// them fetching instructions).
+template <int NS, int ROWS>
+__device__ __forceinline__ void lbs_thin(const uint16_t *__restrict__ Wb, int stride, const LbsRows<ROWS> &R, int nrows, int x, int skip,
+                                         const float *s32, uint32_t *cells) {
+    using Cells = LbsCells<NS>;
+    const bool on = x < stride;
+    const float sx = s32[x];
+    const uint16_t *wl = Wb + x;
+    const LbsThinRec<NS> *recs = reinterpret_cast<const LbsThinRec<NS> *>(R.thin);
+    uint32_t kept[NS], displaced[NS][3];
+#pragma unroll
+    for (int l = 0; l < NS; ++l) kept[l] = displaced[l][0] = displaced[l][1] = displaced[l][2] = 0u;
+    constexpr int kBatch = 8;                                     // this many rows' weights at once, the next ones on their way meanwhile
+    uint16_t cur[kBatch], next[kBatch];
+    auto load = [&](int q) {
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) next[u] = on && q + u < nrows ? __ldg(wl + (uint32_t)R.row[q + u] * (uint32_t)stride) : (uint16_t)0;
+    };
+    load(0);
+#pragma unroll 1
+    for (int q0 = 0; q0 < nrows; q0 += kBatch) {
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) cur[u] = next[u];
+        load(q0 + kBatch);
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            if (q0 + u >= nrows) break;
+            const LbsThinRec<NS> rec = recs[q0 + u];
+            const float w = __half2float(__ushort_as_half(cur[u])), p = w * sx;
+            const uint32_t f = __float_as_uint(fmaf(w, 4.f, 2.f)) - kNarrowBase;
+#pragma unroll
+            for (int l = 0; l < NS; ++l)
+                asm("{\n\t.reg .pred p;\n\tsetp.gt.f32 p, %8, %9;\n\t@p add.u32 %0, %0, %4;\n\t@p add.u32 %1, %1, %5;\n\t@p add.u32 %2, %2, %6;\n\t"
+                    "@p add.u32 %3, %3, %7;\n\t}"
+                    : "+r"(kept[l]), "+r"(displaced[l][0]), "+r"(displaced[l][1]), "+r"(displaced[l][2])
+                    : "r"(f), "r"(rec.u[l][0]), "r"(rec.u[l][1]), "r"(rec.u[l][2]), "f"(p), "f"(rec.bound[l]));
+        }
+    }
+    // (16 returning additions in flight before their carries are looked at)
+    uint32_t *cell = cells + (x & 7) * 32 + (x >> 3);
+    uint32_t old[NS][4];
+#pragma unroll
+    for (int l = 0; l < NS; ++l) {
+        old[l][3] = atomicAdd(cell + l * kLbsMax, kept[l]);
+#pragma unroll
+        for (int o = 0; o < 3; ++o) old[l][o] = atomicAdd(cell + (NS + 3 * l + o) * kLbsMax, displaced[l][o]);
+    }
+#pragma unroll
+    for (int l = 0; l < NS; ++l) {
+        if (old[l][3] + kept[l] < kept[l]) atomicAdd(cell + l * kLbsMax + Cells::kWords, 1u);
+#pragma unroll
+        for (int o = 0; o < 3; ++o)
+            if (old[l][o] + displaced[l][o] < displaced[l][o]) atomicAdd(cell + (NS + 3 * l + o) * kLbsMax + Cells::kWords, 1u);
+    }
+}
+
+// Irregular rows [lo, hi): fp64 products, 64-bit sums, a branch on the row's rank order.
+template <int P1, int P2, int P3, int P4>
+__device__ __forceinline__ void lbs_add(unsigned long long (&kept)[4], unsigned long long (&displaced)[4][4], unsigned long long f, unsigned long long u2,
+                                        unsigned long long u3, bool gt2, bool eq2, bool gt3, bool eq3) {
     if (gt3 || (eq3 && P1 < P3)) { kept[P1] += f; displaced[P1][P3] += u3; }
     if (gt3 || (eq3 && P2 < P3)) { kept[P2] += f; displaced[P2][P3] += u3; }
     if (gt2 || (eq2 && P3 < P2)) { kept[P3] += f; displaced[P3][P2] += u2; }
     if (gt2 || (eq2 && P4 < P2)) { kept[P4] += f; displaced[P4][P2] += u2; }
 }
-template <bool EXACT, int NS, int ROWS>
-__device__ __forceinline__ void lbs_each(const uint16_t *__restrict__ Wb, int stride, const LbsRows<ROWS> &R, int lo, int hi, int x, const LbsGroup &grp,
-                                         int skip, const float *s32, const double *s64, uint32_t *cells) {
+template <int NS, int ROWS>
+__device__ __forceinline__ void lbs_exact(const uint16_t *__restrict__ Wb, int stride, const LbsRows<ROWS> &R, const LbsRec *recs, int lo, int hi, int x,
+                                          const LbsGroup &grp, int skip, const double *s64, uint32_t *cells) {
     using Cells = LbsCells<NS>;
-    using Acc = typename std::conditional<EXACT, unsigned long long, uint32_t>::type;
     const bool on = x < stride;
-    const float sx32 = s32[x];
-    const double sx64 = s64[x];
+    const double sx = s64[x];
     const uint16_t *wl = Wb + x;
-    Acc kept[4] = {0, 0, 0, 0}, displaced[4][4] = {};
-    constexpr int kBatch = EXACT ? 2 : 8;                         // this many rows' weights at once, the next ones on their way meanwhile
-    uint16_t cur[kBatch], next[kBatch];
-    auto load = [&](int q) {
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) next[u] = on && q + u < hi ? __ldg(wl + (uint32_t)R.row[q + u] * (uint32_t)stride) : (uint16_t)0;
-    };
-    load(lo);
+    unsigned long long kept[4] = {0, 0, 0, 0}, displaced[4][4] = {};
+    auto load = [&](int q) -> uint16_t { return on && q < hi ? __ldg(wl + (uint32_t)R.row[q] * (uint32_t)stride) : (uint16_t)0; };
+    uint16_t n0 = load(lo), n1 = load(lo + 1), n2 = load(lo + 2);  // the next rows' weights on their way
 #pragma unroll 1
-    for (int q0 = lo; q0 < hi; q0 += kBatch) {
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) cur[u] = next[u];
-        load(q0 + kBatch);
-#pragma unroll 1
-        for (int u = 0; u < kBatch && q0 + u < hi; ++u) {
-            const int q = q0 + u, order = R.order[q];
-            const LbsRec rec = R.rec[q];
-            const uint16_t hx = cur[0];
-#pragma unroll
-            for (int i = 0; i + 1 < kBatch; ++i) cur[i] = cur[i + 1];
-            Acc f, u2, u3;
-            bool gt2, gt3, eq2 = false, eq3 = false;
-            if constexpr (EXACT) {
-                int p1, p2, p3, p4;
-                lbs_order_slots(order, p1, p2, p3, p4);
-                const double xx = __dmul_rn(half_bits_abs_to_double(hx), sx64);
-                const double x2 = __dmul_rn(half_bits_abs_to_double((uint16_t)rec.u2), grp.s[p2]), x3 = __dmul_rn(half_bits_abs_to_double((uint16_t)rec.u3), grp.s[p3]);
-                gt2 = xx > x2; eq2 = xx == x2; gt3 = xx > x3; eq3 = xx == x3;
-                f = (Acc)half_bits_abs_fixed(hx);
-                u2 = (Acc)half_bits_abs_fixed((uint16_t)rec.u2);
-                u3 = (Acc)half_bits_abs_fixed((uint16_t)rec.u3);
-            } else {
-                const float w = __half2float(__ushort_as_half(hx)), p = w * sx32;
-                gt2 = p > rec.p2; gt3 = p > rec.p3;
-                f = __float_as_uint(fmaf(w, 4.f, 2.f)) - kNarrowBase;
-                u2 = rec.u2; u3 = rec.u3;
-            }
+    for (int q = lo; q < hi; ++q) {
+        const uint16_t hx = n0;
+        n0 = n1;
+        n1 = n2;
+        n2 = load(q + 3);
+        const int order = R.order[q];
+        const LbsRec rec = recs[q - lo];
+        int p1, p2, p3, p4;
+        lbs_order_slots(order, p1, p2, p3, p4);
+        const double xx = __dmul_rn(half_bits_abs_to_double(hx), sx);
+        const double x2 = __dmul_rn(half_bits_abs_to_double((uint16_t)rec.u2), grp.s[p2]), x3 = __dmul_rn(half_bits_abs_to_double((uint16_t)rec.u3), grp.s[p3]);
+        const bool gt2 = xx > x2, eq2 = xx == x2, gt3 = xx > x3, eq3 = xx == x3;
+        const unsigned long long f = (unsigned long long)half_bits_abs_fixed(hx), u2 = (unsigned long long)half_bits_abs_fixed((uint16_t)rec.u2),
+                                 u3 = (unsigned long long)half_bits_abs_fixed((uint16_t)rec.u3);
 #define ESP_ORDER(N, P1, P2, P3, P4) case N: lbs_add<P1, P2, P3, P4>(kept, displaced, f, u2, u3, gt2, eq2, gt3, eq3); break;
-            switch (order) {
-                ESP_ORDER(0, 0, 1, 2, 3) ESP_ORDER(1, 0, 1, 3, 2) ESP_ORDER(2, 0, 2, 1, 3) ESP_ORDER(3, 0, 2, 3, 1) ESP_ORDER(4, 0, 3, 1, 2) ESP_ORDER(5, 0, 3, 2, 1)
-                ESP_ORDER(6, 1, 0, 2, 3) ESP_ORDER(7, 1, 0, 3, 2) ESP_ORDER(8, 1, 2, 0, 3) ESP_ORDER(9, 1, 2, 3, 0) ESP_ORDER(10, 1, 3, 0, 2) ESP_ORDER(11, 1, 3, 2, 0)
-                ESP_ORDER(12, 2, 0, 1, 3) ESP_ORDER(13, 2, 0, 3, 1) ESP_ORDER(14, 2, 1, 0, 3) ESP_ORDER(15, 2, 1, 3, 0) ESP_ORDER(16, 2, 3, 0, 1) ESP_ORDER(17, 2, 3, 1, 0)
-                ESP_ORDER(18, 3, 0, 1, 2) ESP_ORDER(19, 3, 0, 2, 1) ESP_ORDER(20, 3, 1, 0, 2) ESP_ORDER(21, 3, 1, 2, 0) ESP_ORDER(22, 3, 2, 0, 1) ESP_ORDER(23, 3, 2, 1, 0)
-                default: break;
-            }
-#undef ESP_ORDER
+        switch (order) {
+            ESP_ORDER(0, 0, 1, 2, 3) ESP_ORDER(1, 0, 1, 3, 2) ESP_ORDER(2, 0, 2, 1, 3) ESP_ORDER(3, 0, 2, 3, 1) ESP_ORDER(4, 0, 3, 1, 2) ESP_ORDER(5, 0, 3, 2, 1)
+            ESP_ORDER(6, 1, 0, 2, 3) ESP_ORDER(7, 1, 0, 3, 2) ESP_ORDER(8, 1, 2, 0, 3) ESP_ORDER(9, 1, 2, 3, 0) ESP_ORDER(10, 1, 3, 0, 2) ESP_ORDER(11, 1, 3, 2, 0)
+            ESP_ORDER(12, 2, 0, 1, 3) ESP_ORDER(13, 2, 0, 3, 1) ESP_ORDER(14, 2, 1, 0, 3) ESP_ORDER(15, 2, 1, 3, 0) ESP_ORDER(16, 2, 3, 0, 1) ESP_ORDER(17, 2, 3, 1, 0)
+            ESP_ORDER(18, 3, 0, 1, 2) ESP_ORDER(19, 3, 0, 2, 1) ESP_ORDER(20, 3, 1, 0, 2) ESP_ORDER(21, 3, 1, 2, 0) ESP_ORDER(22, 3, 2, 0, 1) ESP_ORDER(23, 3, 2, 1, 0)
+            default: break;
         }
+#undef ESP_ORDER
     }
     const int at = (x & 7) * 32 + (x >> 3);
+    uint32_t old[4][4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if (k == skip) continue;
-        lbs_add64(cells + Cells::kept(k, skip) * kLbsMax + at, Cells::kWords, kept[k]);
 #pragma unroll
         for (int o = 0; o < 4; ++o)
-            if (o != k) lbs_add64(cells + Cells::displaced(k, o, skip) * kLbsMax + at, Cells::kWords, displaced[k][o]);
+            old[k][o] = atomicAdd(cells + (o == k ? Cells::kept(k, skip) : Cells::displaced(k, o, skip)) * kLbsMax + at, (uint32_t)(o == k ? kept[k] : displaced[k][o]));
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (k == skip) continue;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            const unsigned long long v = o == k ? kept[k] : displaced[k][o];
+            const uint32_t up = (uint32_t)(v >> 32) + (old[k][o] + (uint32_t)v < (uint32_t)v ? 1u : 0u);
+            if (up) atomicAdd(cells + (o == k ? Cells::kept(k, skip) : Cells::displaced(k, o, skip)) * kLbsMax + Cells::kWords + at, up);
+        }
     }
 }
 
 // One chunk of rows, NG groups, into the cells and sums.
-constexpr int kThinRows = 192;
 template <int NG, int ROWS, int THREADS, int NS>
 __device__ __forceinline__ void lbs_chunk(const uint16_t *__restrict__ Wb, int stride, const uint16_t *__restrict__ Wt, long ldt,
                                           const uint8_t *__restrict__ irregular, int nrows, const LbsGroup *grp, const int *skip, LbsRows<ROWS> *rows,
                                           const float *s32, const double *s64, uint4 *ring, uint32_t *cells, uint32_t *sums) {
     constexpr int kWarps = THREADS / 32;
     static_assert(kWarps == 8 * NG, "a group's candidates in eight warps");
-    static_assert(NG * ROWS <= kNarrowRun * kWarps && kThinRows * (1 << 23) < (1ll << 32), "32-bit sums");
+    static_assert(NG * ROWS <= kNarrowRun * kWarps && kThinRows * (1ll << 23) < (1ll << 32), "32-bit sums");
+    static_assert(sizeof(LbsThinRec<4>) * kThinRows + sizeof(LbsRec) * kThinRows <= sizeof(LbsRec) * ROWS, "records of a short slice");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool thin = nrows <= kThinRows;
-    lbs_prepare<NG, ROWS, THREADS>(Wt, ldt, irregular, nrows, grp, thin, rows, sums);
+    lbs_prepare<NG, ROWS, THREADS, NS>(Wt, ldt, irregular, nrows, grp, skip, thin, rows, sums);
     const int mine = warp >> 3, x = lane * 8 + (warp & 7);        // group and candidate of this lane in the loops over single rows
     uint32_t *cells_mine = cells + mine * 2 * LbsCells<NS>::kWords;
     const LbsRows<ROWS> &R = rows[mine];
     const int regular = R.off[kLbsIrregular];
-    if (thin) {
-        lbs_each<false, NS>(Wb, stride, R, 0, regular, x, grp[mine], skip[mine], s32, s64, cells_mine);
-    } else {
-        // every warp an equal run of the groups' sorted regular rows, all candidates
-        const int n0 = rows[0].off[kLbsIrregular], total = n0 + (NG > 1 ? rows[NG - 1].off[kLbsIrregular] : 0);
-        const int seg = (total + kWarps - 1) / kWarps, first = warp * seg, last = min(total, first + seg);
+    // (half of the warps take the irregular rows first: that loop waits on memory and branches, the other fills the issue slots)
 #pragma unroll 1
-        for (int g = 0; g < NG; ++g) {
-            const int base = g == 0 ? 0 : n0, lo = max(first - base, 0), hi = min(last - base, rows[g].off[kLbsIrregular]);
-            if (lo < hi)
-                lbs_regular<NS>(Wb, stride, rows[g], lo, hi, skip[g], s32, ring + warp * kRing * 32, cells + g * 2 * LbsCells<NS>::kWords,
-                                sums + g * 2 * kLbsGroupSums);
+    for (int turn = 0; turn < 2; ++turn) {
+        if ((turn ^ warp) & 1) {
+            if (regular < nrows)
+                lbs_exact<NS>(Wb, stride, R, thin ? R.thin_irregular : R.rec + regular, regular, nrows, x, grp[mine], skip[mine], s64, cells_mine);
+        } else if (thin) {
+            lbs_thin<NS>(Wb, stride, R, regular, x, skip[mine], s32, cells_mine);
+        } else {
+            // every warp an equal run of the groups' sorted regular rows, all candidates
+            const int n0 = rows[0].off[kLbsIrregular], total = n0 + (NG > 1 ? rows[NG - 1].off[kLbsIrregular] : 0);
+            const int seg = (total + kWarps - 1) / kWarps, first = warp * seg, last = min(total, first + seg);
+#pragma unroll 1
+            for (int g = 0; g < NG; ++g) {
+                const int base = g == 0 ? 0 : n0, lo = max(first - base, 0), hi = min(last - base, rows[g].off[kLbsIrregular]);
+                if (lo < hi)
+                    lbs_regular<NS>(Wb, stride, rows[g], lo, hi, skip[g], s32, ring + warp * kRing * 32, cells + g * 2 * LbsCells<NS>::kWords,
+                                    sums + g * 2 * kLbsGroupSums);
+            }
         }
     }
-    if (regular < nrows) lbs_each<true, NS>(Wb, stride, R, regular, nrows, x, grp[mine], skip[mine], s32, s64, cells_mine);
     __syncthreads();
 }
 
@@ -711,13 +789,19 @@ __device__ __forceinline__ void st_remote_s32(uint32_t remote_addr, int v) {
 __device__ __forceinline__ unsigned long long lbs_cluster_cell(const uint32_t *cell, int n, int nc) {
     const uint32_t at = smem_u32(cell);
     unsigned long long v = 0;
-#pragma unroll 4
-    for (int c = 0; c < nc; ++c) {
-        const uint32_t remote = map_to_rank(at, (uint32_t)c);
-        uint32_t lo, hi;
-        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(lo) : "r"(remote));
-        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(hi) : "r"(remote + 4u * (uint32_t)n));
-        v += ((unsigned long long)hi << 32) | lo;
+    for (int c0 = 0; c0 < nc; c0 += 8) {     // (sixteen loads in flight)
+        uint32_t lo[8], hi[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            lo[c] = hi[c] = 0u;
+            if (c0 + c < nc) {
+                const uint32_t remote = map_to_rank(at, (uint32_t)(c0 + c));
+                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(lo[c]) : "r"(remote));
+                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(hi[c]) : "r"(remote + 4u * (uint32_t)n));
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v += ((unsigned long long)hi[c] << 32) | lo[c];
     }
     return v;
 }
