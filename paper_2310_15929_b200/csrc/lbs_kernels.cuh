@@ -22,7 +22,7 @@
 //  * |w| < 0.5 becomes an integer of 2^-24 with one fp32 fma, so the sums are 32-bit adds.
 //
 // Measured against one comparison and two fp64 additions per (row, candidate, slot) with a warp per candidate (about 29 instructions
-// each): table of a 4096 x 4096 weight 6.94 -> 0.92 ms, greedy kernel 67.7 -> 9.3 ms; 13824 x 5120: 29.1 -> 3.8 ms and 223 -> 24.6 ms;
+// each): table of a 4096 x 4096 weight 6.94 -> 0.92 ms, greedy kernel 67.7 -> 8.7 ms; 13824 x 5120: 29.1 -> 3.8 ms and 223 -> 24.4 ms;
 // 512 x 512 (two blocks): 15.6 -> 2.6 ms.
 
 constexpr int kLbsMax = 256;       // widest local-shuffle block
@@ -37,7 +37,7 @@ struct LbsRec {                    // one row of one group: the slots ranked sec
 };
 // A short slice's regular rows (lbs_thin): per live slot the product to beat, and what the candidate then displaces from each of the
 // three other slots (one of them, zero from the rest).
-constexpr int kThinRows = 192;
+constexpr int kThinRows = 192, kThinBatch = 16;
 template <int NS>
 struct __align__(16) LbsThinRec {
     float bound[NS];
@@ -47,7 +47,7 @@ template <int ROWS>
 struct LbsRows {                   // the rows of a chunk as one group sees them, sorted by class
     union {
         LbsRec rec[ROWS];
-        struct { LbsThinRec<4> thin[kThinRows]; LbsRec thin_irregular[kThinRows]; };
+        struct { LbsThinRec<4> thin[kThinRows + kThinBatch]; LbsRec thin_irregular[kThinRows]; };
     };
     uint16_t row[ROWS];
     uint16_t h1[ROWS];             // |w| bits of the slot ranked first
@@ -217,6 +217,17 @@ __device__ __forceinline__ void lbs_prepare(const uint16_t *__restrict__ Wt, lon
             rows[g].order[at] = (uint8_t)where[u];
         }
     }
+    if (thin && warp < NG) {                                      // the last batch is filled up
+        const int at = rows[warp].off[kLbsIrregular] + lane;
+        if (lane < kThinBatch) {
+            LbsThinRec<NS> &t = reinterpret_cast<LbsThinRec<NS> *>(rows[warp].thin)[at];
+#pragma unroll
+            for (int l = 0; l < NS; ++l) {
+                t.bound[l] = INFINITY;
+                t.u[l][0] = t.u[l][1] = t.u[l][2] = 0u;
+            }
+        }
+    }
     __syncthreads();
 }
 
@@ -241,6 +252,13 @@ __device__ __forceinline__ void lbs_group_sums(const LbsRows<ROWS> &R, int lo, i
 // values below 2^23) however many were added, and an addend costs one fma.
 constexpr uint32_t kNarrowMask = 0x3FFFFFFFu, kNarrowBase = 0x40000000u;
 constexpr int kNarrowRun = 128;
+constexpr int kClassRows = 4;      // what the end of a class costs a warp, in rows
+// Rows taken at once: equal chunks, and no more than leave every warp's run at 128 rows (see lbs_chunk).
+__host__ __device__ constexpr int lbs_chunk_limit(int capacity) { return capacity - kClassRows * kLbsIrregular; }
+__device__ __forceinline__ int lbs_chunk_rows(int n, int capacity) {
+    const int chunks = max(1, (n + lbs_chunk_limit(capacity) - 1) / lbs_chunk_limit(capacity));
+    return max(8, ((n + chunks - 1) / chunks + 7) & ~7);
+}
 
 // if (p > bound) { a += f; d += u; } as one comparison and two predicated additions (left to itself the compiler selects addends: four
 // instructions instead of two).
@@ -357,7 +375,7 @@ __device__ __forceinline__ void lbs_thin(const uint16_t *__restrict__ Wb, int st
     uint32_t kept[NS], displaced[NS][3];
 #pragma unroll
     for (int l = 0; l < NS; ++l) kept[l] = displaced[l][0] = displaced[l][1] = displaced[l][2] = 0u;
-    constexpr int kBatch = 8;                                     // this many rows' weights at once, the next ones on their way meanwhile
+    constexpr int kBatch = kThinBatch;                            // this many rows' weights at once, the next ones on their way meanwhile
     uint16_t cur[kBatch], next[kBatch];
     auto load = [&](int q) {
 #pragma unroll
@@ -371,8 +389,7 @@ __device__ __forceinline__ void lbs_thin(const uint16_t *__restrict__ Wb, int st
         load(q0 + kBatch);
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
-            if (q0 + u >= nrows) break;
-            const LbsThinRec<NS> rec = recs[q0 + u];
+            const LbsThinRec<NS> rec = recs[q0 + u];             // (beyond the last row: nothing is ahead of its bound)
             const float w = __half2float(__ushort_as_half(cur[u])), p = w * sx;
             const uint32_t f = __float_as_uint(fmaf(w, 4.f, 2.f)) - kNarrowBase;
 #pragma unroll
@@ -473,8 +490,8 @@ __device__ __forceinline__ void lbs_chunk(const uint16_t *__restrict__ Wb, int s
                                           const float *s32, const double *s64, uint4 *ring, uint32_t *cells, uint32_t *sums) {
     constexpr int kWarps = THREADS / 32;
     static_assert(kWarps == 8 * NG, "a group's candidates in eight warps");
-    static_assert(NG * ROWS <= kNarrowRun * kWarps && kThinRows * (1ll << 23) < (1ll << 32), "32-bit sums");
-    static_assert(sizeof(LbsThinRec<4>) * kThinRows + sizeof(LbsRec) * kThinRows <= sizeof(LbsRec) * ROWS, "records of a short slice");
+    static_assert(NG * (lbs_chunk_limit(ROWS) + kClassRows * kLbsIrregular) <= kNarrowRun * kWarps && kThinRows * (1ll << 23) < (1ll << 32), "32-bit sums");
+    static_assert(sizeof(LbsThinRec<4>) * (kThinRows + kThinBatch) + sizeof(LbsRec) * kThinRows <= sizeof(LbsRec) * ROWS, "records of a short slice");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool thin = nrows <= kThinRows;
     lbs_prepare<NG, ROWS, THREADS, NS>(Wt, ldt, irregular, nrows, grp, skip, thin, rows, sums);
@@ -491,12 +508,29 @@ __device__ __forceinline__ void lbs_chunk(const uint16_t *__restrict__ Wb, int s
         } else if (thin) {
             lbs_thin<NS>(Wb, stride, R, regular, x, skip[mine], s32, cells_mine);
         } else {
-            // every warp an equal run of the groups' sorted regular rows, all candidates
-            const int n0 = rows[0].off[kLbsIrregular], total = n0 + (NG > 1 ? rows[NG - 1].off[kLbsIrregular] : 0);
-            const int seg = (total + kWarps - 1) / kWarps, first = warp * seg, last = min(total, first + seg);
+            // every warp a run of the groups' sorted regular rows, all candidates: equal shares of rows + kClassRows for every class that
+            // has rows (a class ends with its sums going to the cells).  Equal numbers of rows leave the warps whose run crosses the
+            // small classes far behind: a quarter of a swap was spent waiting for them (4096 x 4096 10.7 -> 10.1 ms, 3584 x 1224 5.63 -> 5.01 ms).
+            int regular_rows[NG], at[NG + 1];                     // (cost before each group)
+            uint32_t classes[NG];
+            at[0] = 0;
+#pragma unroll
+            for (int g = 0; g < NG; ++g) {
+                regular_rows[g] = rows[g].off[kLbsIrregular];
+                classes[g] = __ballot_sync(0xFFFFFFFFu, lane < kLbsIrregular && rows[g].off[lane + 1] > rows[g].off[lane]);
+                at[g + 1] = at[g] + regular_rows[g] + kClassRows * __popc(classes[g]);
+            }
 #pragma unroll 1
             for (int g = 0; g < NG; ++g) {
-                const int base = g == 0 ? 0 : n0, lo = max(first - base, 0), hi = min(last - base, rows[g].off[kLbsIrregular]);
+                const int start = rows[g].off[lane] + kClassRows * __popc(classes[g] & ((1u << lane) - 1u));     // cost before class `lane`
+                auto place = [&](int cost) {                      // the sorted place that this much cost reaches
+                    cost = max(0, min(at[NG], cost) - at[g]);
+                    const uint32_t begun = classes[g] & __ballot_sync(0xFFFFFFFFu, start <= cost);
+                    if (begun == 0u) return 0;
+                    const int c = 31 - __clz(begun);
+                    return min(rows[g].off[c] + max(0, cost - __shfl_sync(0xFFFFFFFFu, start, c) - kClassRows), rows[g].off[c + 1]);
+                };
+                const int lo = place(at[NG] * warp / kWarps), hi = warp == kWarps - 1 ? regular_rows[g] : place(at[NG] * (warp + 1) / kWarps);
                 if (lo < hi)
                     lbs_regular<NS>(Wb, stride, rows[g], lo, hi, skip[g], s32, ring + warp * kRing * 32, cells + g * 2 * LbsCells<NS>::kWords,
                                     sums + g * 2 * kLbsGroupSums);
@@ -699,8 +733,9 @@ __global__ void __launch_bounds__(kTableThreads, 2) lbs_table_kernel(const uint1
     __syncthreads();
     const uint16_t *Wblk = Wb + (size_t)b * No * stride;
     const uint8_t *iblk = irregular + (size_t)b * No;
-    for (int r0 = 0; r0 < No; r0 += kTableRows)
-        lbs_chunk<1, kTableRows, kTableThreads, 4>(Wblk + (size_t)r0 * stride, stride, Wt + r0, ldt, iblk + r0, min(kTableRows, No - r0), &S.grp, &S.skip,
+    const int chunk_rows = lbs_chunk_rows(No, kTableRows);
+    for (int r0 = 0; r0 < No; r0 += chunk_rows)
+        lbs_chunk<1, kTableRows, kTableThreads, 4>(Wblk + (size_t)r0 * stride, stride, Wt + r0, ldt, iblk + r0, min(chunk_rows, No - r0), &S.grp, &S.skip,
                                                    &S.rows, S.s32, S.s64, S.ring, S.cells, S.sums);
     if (tid < kLbsGroupSums) S.total[tid] = lbs_cell(S.sums + tid, kLbsGroupSums);
     __syncthreads();
@@ -829,7 +864,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
     for (int x = tid; x < m; x += kGreedyThreads) { S.pos2x[x] = x; S.chan[x] = theta0[p0 + x]; }
     for (int g = tid; g < G; g += kGreedyThreads) S.base[g] = base0[p0 / 4 + g];
     lbs_load_scores(score, theta0, p0, m, S.s64, S.s32);          // (ends with a barrier: everything above is visible)
-    const int per_cta = (No + nc - 1) / nc, row0 = min(No, rank * per_cta), nrows_all = min(No, row0 + per_cta) - row0;
+    const int per_cta = (No + nc - 1) / nc, row0 = min(No, rank * per_cta), nrows_all = min(No, row0 + per_cta) - row0, chunk_rows = lbs_chunk_rows(nrows_all, kGreedyRows);
     const uint16_t *Wblk = Wb + ((size_t)b * No + row0) * stride;
     const uint8_t *iblk = irregular + (size_t)b * No + row0;
 
@@ -913,8 +948,8 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
         if (tid == 0) { S.pos2x[bi] = xj; S.pos2x[bj] = xi; }
         // Row (g, slot) of the table holds g with that slot replaced, so it depends on g's OTHER three channels: the rows of the two
         // swapped slots stay as they are (but for the channel that left them, which was no candidate before).
-        for (int r0 = 0; r0 < nrows_all; r0 += kGreedyRows)
-            lbs_chunk<2, kGreedyRows, kGreedyThreads, 3>(Wblk + (size_t)r0 * stride, stride, Wt + row0 + r0, ldt, iblk + r0, min(kGreedyRows, nrows_all - r0),
+        for (int r0 = 0; r0 < nrows_all; r0 += chunk_rows)
+            lbs_chunk<2, kGreedyRows, kGreedyThreads, 3>(Wblk + (size_t)r0 * stride, stride, Wt + row0 + r0, ldt, iblk + r0, min(chunk_rows, nrows_all - r0),
                                                          S.grp, S.skip, S.rows, S.s32, S.s64, S.ring, &S.cells[0][0], &S.sums[0][0]);
         cluster_arrive();
         cluster_wait();                                           // the sums of every CTA are complete
@@ -922,9 +957,10 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
         const int share = ((kEntries + nc - 1) / nc + 31) & ~31, e0 = rank * share;
         unsigned long long *part = reinterpret_cast<unsigned long long *>(S.rows);      // [4 sums][share]: the sorted rows are used up
         static_assert(sizeof(S.rows[0].rec) >= 4 * 8 * (kEntries / kGreedyMinCluster), "room for the largest share, counters untouched");
-        if (tid < 2 * kLbsGroupSums)
-            S.total[tid / kLbsGroupSums][tid % kLbsGroupSums] =
-                lbs_cluster_cell(&S.sums[tid / kLbsGroupSums][tid % kLbsGroupSums], kLbsGroupSums, nc);
+        if (tid >= kGreedyThreads - 2 * kLbsGroupSums) {          // (the last warp: the fewest entries below are its own)
+            const int t = tid - (kGreedyThreads - 2 * kLbsGroupSums);
+            S.total[t / kLbsGroupSums][t % kLbsGroupSums] = lbs_cluster_cell(&S.sums[t / kLbsGroupSums][t % kLbsGroupSums], kLbsGroupSums, nc);
+        }
         for (int t = tid; t < 4 * share; t += kGreedyThreads) {
             const int sel = t / share, e = e0 + t - sel * share;
             if (e < kEntries) {
