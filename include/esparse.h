@@ -180,14 +180,16 @@ enum { ESP_KERNEL_AUTO = 0,
                                     unit's row gather (correct, but that unit retires such gathers too
                                     slowly to feed the MMA; kept for comparison)                        */
        ESP_KERNEL_STREAM = 4,    /* channel-major X rows streamed by asynchronous 16-byte copies, weight
-                                    tiles by bulk copies; every token count (default up to 256 tokens,
-                                    except where the pair kernel below is faster)                       */
+                                    tiles by bulk copies; every token count (default up to 64 tokens
+                                    and wherever it is estimated fastest beyond); small problems read
+                                    token-major X themselves, without a transposing launch               */
        ESP_KERNEL_PAIR = 5,      /* large M: two SMs share one 512-feature x token_tile MMA tile
-                                    (token_tile 240 by default; 128, 192, 224 or 256 on request); X rows
-                                    are gathered through the permutation by 16-byte copies              */
+                                    (token_tile 128, 192, 224 or 240; 256: 256 features; K-slices with
+                                    128 and 256); X rows are gathered through the permutation by
+                                    16-byte copies                                                       */
        ESP_KERNEL_PAIR_TILED = 6,/* the same tile, fed by bulk copies: a pass over X first writes the
                                     permuted, swizzled operand images into the workspace (default for
-                                    more than 256 tokens when the workspace has room; token_tile 128..240) */
+                                    most sizes beyond 256 tokens when the workspace has room; same tiles) */
        ESP_KERNEL_QUAD_TILED = 7,/* ESP_KERNEL_PAIR_TILED with two such tiles (same features, neighbouring
                                     token tiles) per cluster of four SMs: every weight tile is fetched once per
                                     cluster and handed to the other pair through distributed shared memory
@@ -202,7 +204,7 @@ enum { ESP_KERNEL_AUTO = 0,
                                     ESP_KERNEL_PAIR_TILED: a pass over X writes the permuted, swizzled operand images of every
                                     (token block, channel step) into the workspace and a stage's X is one bulk copy per
                                     block instead of 16-byte row copies; same results bit for bit; needs the workspace
-                                    (default for 17..256 tokens on large weights)                        */
+                                    (default where it is estimated fastest, and on large weights)        */
        ESP_KERNEL_QUAD_MULTICAST = 9 };/* the cluster of ESP_KERNEL_QUAD_TILED with every weight tile delivered to
                                     both pairs by ONE tiled load (cluster multicast of the tensor memory unit) instead
                                     of a hand-over: token_tile 192, 224 or 240, same results bit for bit.  Its kernel
