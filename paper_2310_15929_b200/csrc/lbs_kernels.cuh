@@ -879,7 +879,10 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
             gr[j - i - 1] = (i >> 2) == (j >> 2) ? -INFINITY : __dsub_rn(after, __dadd_rn(S.base[i >> 2], S.base[j >> 2]));
         }
     }
-    __syncthreads();
+    // (a barrier of the cluster, not of the CTA: the first exchange below stores into the shared memory of the other CTAs, which have to be
+    // running by then)
+    cluster_arrive();
+    cluster_wait();
     int swaps = 0, near_swaps = 0;
     for (;;) {
         double best = -INFINITY, second = -INFINITY;              // second: largest gain once one instance of the best is set aside

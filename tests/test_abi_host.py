@@ -211,3 +211,14 @@ def test_cluster_multicast_loads_live_only_in_the_companion_source():
     if os.path.exists(MC_SOURCE):
         assert load_with_multicast.search(open(MC_SOURCE).read())
         assert b.esp_multicast_available() == os.path.exists(MC_LIB_PATH)
+
+
+def test_block_shuffle_clusters_meet_before_their_first_remote_store():
+    """Another CTA's shared memory may only be accessed once that CTA is known to run: in the greedy kernel's source, a wait on
+    the cluster barrier stands before the first store into (or load from) a peer, outside of any branch or loop."""
+    csrc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2310_15929_b200", "csrc")
+    text = open(os.path.join(csrc, "lbs_kernels.cuh")).read()
+    body = text[text.index("lbs_greedy_kernel("):]
+    body = body[:body.index("\n}\n")]
+    first_remote = min(body.index(name) for name in ("st_remote_f64(", "st_remote_s32(", "lbs_cluster_cell("))
+    assert re.search(r"^    cluster_arrive\(\);\n    cluster_wait\(\);$", body[:first_remote], re.M)

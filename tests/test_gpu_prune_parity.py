@@ -135,6 +135,20 @@ def test_block_shuffle_row_slices(No):
     assert_identical_to_oracle(g, ref)
 
 
+@pytest.mark.parametrize("block", [4, 8, 60, 64])
+@pytest.mark.parametrize("No,C", [(33, 8), (48, 64), (300, 264)])
+def test_block_shuffle_narrow_blocks(No, C, block):
+    """Narrow blocks, whose clusters come to their first exchange of winners with next to no set-up: a single group (no pair
+    at all), two groups, a width that is no power of two, a ragged last block."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8300 + No)
+    W = (g0.standard_normal((No, C)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(C)
+    ref = orc.metric_prune(W, None, 1.0, score=s, lbs_block=block)
+    g = GpuPrune(W, None, 1.0, score=s, lbs_block=block)
+    assert_identical_to_oracle(g, ref)
+
+
 def test_llama7b_q_projection_full_size_block_shuffle():
     """Workload 1's q projection whole (4096 x 4096, 16 shuffle blocks, Student-t rows): global shuffle, block shuffle
     capped at 4 swaps per block on both sides (the oracle's table alone is 4.3e9 row evaluations), selection and
