@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(256) entropy_score_kernel(int C, int T, int bi
 inline esp_status_t launch_entropy(int C, int T, int bins, const unsigned int *counts, const esp_prune_opts &o, const double *score_override,
                                    const EntropyOut &out, cudaStream_t stream) {
     const size_t smem = counts ? sizeof(double) * kEntropyChannels * (size_t)(bins | 1) : 0;
-    if (smem > 48 * 1024) ESP_CUDA_OK(ensure_dynamic_smem((const void *)entropy_score_kernel, (int)smem));
+    ESP_CUDA_OK(ensure_dynamic_smem((const void *)entropy_score_kernel, (int)smem));
     ESP_CUDA_OK(launch_overlapped(entropy_score_kernel, dim3(ceil_div(C, kEntropyChannels)), 1, 256, smem, stream, C, T, bins, counts, o.alpha,
                                   o.use_entropy, o.use_norm, score_override, out));
     return ESP_OK;
@@ -1034,14 +1034,14 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
         // rows per CTA: about 96 KB of shared memory (two CTAs per SM), and a grid of two CTAs per SM at least
         int gather_rows = (int)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / row_bytes));
         gather_rows = std::max(1, std::min(gather_rows, No / (2 * std::max(1, di.sm_count))));
-        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(row_bytes * gather_rows)));
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_gather_kernel, (int)(row_bytes * gather_rows)));
         lbs_gather_kernel<<<ceil_div(No, gather_rows), 256, row_bytes * gather_rows, stream>>>(W, No, C, ldw, w.score, w.theta0, o.lbs_block, w.stride,
                                                                                                nblocks, gather_rows, w.wb, w.irregular);
         lbs_transpose_kernel<<<dim3(ceil_div(C, 64), ceil_div(No, 64)), 256, 0, stream>>>(W, No, C, ldw, w.wt, w.ldt);
-        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LbsTableSmem)));
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_table_kernel, (int)sizeof(LbsTableSmem)));
         lbs_table_kernel<<<nblocks * kLbsGroups, kTableThreads, sizeof(LbsTableSmem), stream>>>(w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score,
                                                                                                 w.theta0, C, o.lbs_block, w.table, w.base[0]);
-        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbs_greedy_smem(kGreedyMinCluster)));
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_greedy_kernel, (int)lbs_greedy_smem(kGreedyMinCluster)));
         ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         const int nc = lbs_cluster_size(nblocks, No, di.device);
         cudaLaunchConfig_t cfg;
@@ -1066,9 +1066,9 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
     // (and no more than leave the grid two CTAs per SM)
     int sel_rows = (int)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / row_smem));
     sel_rows = std::max(1, std::min(sel_rows, No / (2 * std::max(1, di.sm_count))));
-    ESP_CUDA_OK(cudaFuncSetAttribute(select_compress_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(row_smem * sel_rows)));
+    ESP_CUDA_OK(ensure_dynamic_smem((const void *)select_compress_kernel, (int)(row_smem * sel_rows)));
     if (o.m_group == 8) {
-        ESP_CUDA_OK(cudaFuncSetAttribute(select_compress_48_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem));
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)select_compress_48_kernel, (int)row_smem));
         select_compress_48_kernel<<<No, 256, row_smem, stream>>>(W, No, C, ldw, w.score, perm, vals, meta, w.counters);
     } else
         select_compress_kernel<<<ceil_div(No, sel_rows), 256, row_smem * sel_rows, stream>>>(W, No, C, ldw, w.score, perm, vals, meta,

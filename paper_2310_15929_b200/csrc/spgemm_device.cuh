@@ -17,23 +17,26 @@ constexpr uint32_t kSpinLimit = 1u << 22;
 // Host-side caches of what a repeated call would otherwise redo (a decode call is a few microseconds of GPU time: the
 // host must not take longer).  All thread-local: no lock on the call path.
 //
-// The opt-in shared-memory size of a kernel sticks to the function: it is raised once per kernel, device and size.
+// The opt-in shared-memory size belongs to the kernel for the whole process, and setting it can lower it: a size that one thread raised
+// for its launches and another set to the smaller one of its own would fail the first thread's next launch.  So every caller sets
+// the same size, the most that the kernel can be given, once per thread, kernel and device.
 inline cudaError_t ensure_dynamic_smem(const void *kern, int bytes) {
-    struct Entry { const void *kern; int dev, bytes; };
+    struct Entry { const void *kern; int dev, most; };
     thread_local Entry cache[96];
     thread_local int n = 0;
     int dev = 0;
     cudaGetDevice(&dev);
     for (int i = 0; i < n; ++i)
-        if (cache[i].kern == kern && cache[i].dev == dev) {
-            if (cache[i].bytes >= bytes) return cudaSuccess;
-            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-            if (e == cudaSuccess) cache[i].bytes = bytes;
-            return e;
-        }
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && n < 96) cache[n++] = Entry{kern, dev, bytes};
-    return e;
+        if (cache[i].kern == kern && cache[i].dev == dev) return bytes <= cache[i].most ? cudaSuccess : cudaErrorInvalidValue;
+    int most = 0;
+    cudaFuncAttributes attr;
+    cudaError_t e = cudaFuncGetAttributes(&attr, kern);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    most -= (int)attr.sharedSizeBytes;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess && n < 96) cache[n++] = Entry{kern, dev, most};
+    return e == cudaSuccess && bytes > most ? cudaErrorInvalidValue : e;
 }
 inline bool log_plans() {
     static const bool on = getenv("ESP_LOG") != nullptr;

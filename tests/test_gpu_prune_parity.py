@@ -319,6 +319,45 @@ def test_global_bin_range_variant(No, C, T):
     assert_identical_to_oracle(g, ref)
 
 
+@pytest.mark.parametrize("what", ["histogram", "product"])
+def test_shared_memory_size_is_not_lowered_by_another_thread(what):
+    """The size of dynamic shared memory that a kernel may be launched with belongs to the process: a thread that launches a kernel
+    with much, another that launches it with little, and the first one again."""
+    import threading
+    from tests.gpu_util import calibrate_in_chunks, pack_on_gpu, spgemm
+    g0 = np.random.default_rng(31)
+    X = g0.standard_normal((100, 512)).astype(np.float16)
+    if what == "histogram":
+        def call(much):
+            bins = 512 if much else 300
+            assert np.array_equal(calibrate_in_chunks([X], 0.1, bins=bins)[3], orc.channel_histogram(X, bins))
+    else:
+        W = (g0.standard_normal((128, 512)) * 0.02).astype(np.float16)
+        ref = orc.metric_prune(W, None, 1.0, score=np.ones(512), use_lbs=False)
+        packed = pack_on_gpu(ref.vals, ref.meta)
+        want = orc.product(X, ref.vals, ref.meta, ref.theta)
+        def call(much):
+            Y = spgemm(X, packed, ref.theta, 128, channel_major=True, kernel=4, token_tile=64, split_k=1, pipeline_stages=4 if much else 2)
+            assert np.linalg.norm(Y - want) < 1e-3 * np.linalg.norm(want)
+    errors, turn = [], [threading.Event() for _ in range(4)]
+
+    def steps(mine):
+        for i in mine:
+            turn[i].wait(60)
+            try:
+                call(i != 1)
+            except Exception as e:                            # (a failed assertion is reported below, by the test's own thread)
+                errors.append((i, repr(e)))
+            turn[i + 1].set()
+    threads = [threading.Thread(target=steps, args=(m,)) for m in ((0, 2), (1,))]
+    for t in threads:
+        t.start()
+    turn[0].set()
+    for t in threads:
+        t.join()
+    assert errors == []
+
+
 # --------------------------------------------------------------------------- full width: workloads 2, 3, 4
 @pytest.mark.parametrize("wl_index,lin", [(2, "q"), (2, "down"), (3, "down"), (4, "fc2")])
 def test_channel_statistics_full_width_full_calibration(wl_index, lin):
