@@ -1541,7 +1541,12 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
             if (images_room && bn == 0 && o.split_k <= 8 && M > 16 && M <= 256) {
                 const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
                 if (!pair) {
-                    const bool pays = M <= 32 ? weight >= 200000000L : M <= 64 ? ((f_tiles >= 64 && weight >= 40000000L) || weight >= 64000000L) : M <= 128 ? weight >= 40000000L : weight >= 16000000L;
+                    // (33..64 tokens, 64 feature tiles or more: from 24 M elements -- 2472 x 11576 at 61 tokens 23.5 -> 17.9 us, 1792 x 19646 at 48 tokens
+                    // 26.9 -> 20.5, but 1824 x 10658 at 45 16.1 against 16.6 and 968 x 15484 at 46 10.5 against 14.1.  From 5 M where token-major X is transposed
+                    // by a launch that does not overlap, which the images save: 352 x 20560 at 42 tokens 16.2 -> 14.5, 1568 x 9158 at 38 18.6 -> 16.6, but
+                    // 280 x 13756 at 60 11.6 against 14.6)
+                    const long wide_from = o.x_layout == ESP_X_TOKEN_MAJOR && !o.static_weights ? 5000000L : 24000000L;
+                    const bool pays = M <= 32 ? weight >= 200000000L : M <= 64 ? ((f_tiles >= 64 && weight >= wide_from) || weight >= 64000000L) : M <= 128 ? weight >= 40000000L : weight >= 16000000L;
                     // (up to 32 tokens: 32-token images -- 36864 x 9216 at 32 tokens 67.5 -> 64.3 us, 9216 x 36864 76 -> 70)
                     if (pays) {
                         bn = M <= 32 ? 32 : (M > 128 && weight >= 64000000L) ? 128 : 64;

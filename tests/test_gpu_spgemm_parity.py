@@ -699,6 +699,22 @@ def test_form_chosen_for_small_weights(M, N, K, channel_major):
         check(Y.cpu().numpy(), Yref)
 
 
+@pytest.mark.parametrize("channel_major,static,M,N,K,kernel", [(False, 0, 38, 9158, 1568, 10), (False, 0, 60, 13756, 280, 4), (False, 1, 61, 11576, 2472, 10),
+                                                               (False, 1, 45, 8722, 1824, 4), (True, 1, 48, 19646, 1792, 10), (True, 0, 46, 8500, 968, 4)])
+def test_images_at_33_to_64_tokens(channel_major, static, M, N, K, kernel):
+    """Which form wide weights take at 33..64 tokens, on both sides of the sizes from which the image form measured faster (see the
+    rule), and its result."""
+    from paper_2310_15929_b200 import binding as b
+    from tests.gpu_util import pack_on_gpu, spgemm
+    o = b.esp_gemm_opts_default()
+    o.x_layout, o.static_weights = int(channel_major), static
+    assert b.esp_spgemm_plan(M, N, K, o, True)["kernel"] == kernel
+    vals, meta, theta = pruned(7700 + M, 260, K)
+    X = (np.random.default_rng(M).standard_normal((M, K))).astype(np.float16)
+    check(spgemm(X, pack_on_gpu(vals, meta), theta, 260, channel_major=channel_major, static_weights=static, kernel=kernel, token_tile=64),
+          ref_product(X, vals, meta, theta))
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
