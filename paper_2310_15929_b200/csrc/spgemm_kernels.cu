@@ -1461,7 +1461,11 @@ static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, bool image
             if (split > k_tiles || (long)ceil_div(k_tiles, split) * (split - 1) >= k_tiles) continue;
             if (!stream_shape(M, N, K, o, kernel, t.tokens, split, di, layer, &sh)) continue;
             const long ctas = tiles * split, waves = (ctas + sh.capacity - 1) / sh.capacity;
-            const long on_sm = waves * ((std::min<long>(ctas, sh.capacity) + di.sm_count - 1) / di.sm_count);
+            // (CTAs on an SM: by how many clusters find SMs of their own, not by the SM count -- 48 clusters of three CTAs are 144 CTAs, but the GPCs
+            // hold 45 such clusters with one CTA per SM, and the rest double up.  Counted by SMs, 2904 x 2980 at 204 tokens took the 128-token tile
+            // in three slices, 22.2 us, for 18.7 in the 256-token tile in five; 8136 x 1420 at 212 tokens 27.4 for 22.3)
+            const long alone = (long)std::max(1, layer[split]) * split;
+            const long on_sm = waves * ((std::min<long>(ctas, sh.capacity) + alone - 1) / alone);
             const int steps = ceil_div(k_tiles, split);
             const double mb = 1e-6 * (double)ctas * steps * (kTileBytes + 256.0 * t.tokens);
             take(t.start + waves * (t.wave + t.step * steps) + on_sm * (t.wave_sm + t.step_sm * steps) + t.per_mb * mb + t.slice * split + t.image * x_elems,
