@@ -1296,13 +1296,21 @@ struct PairTile { int tokens, feature_tiles; double step_us, fixed_us; };
 static const PairTile kPairTiles[] = {{240, 4, 0.83, 13.0}, {224, 4, 0.82, 12.5}, {192, 4, 0.80, 12.0}, {256, 2, 0.585, 9.7}, {128, 4, 0.66, 10.5}};
 
 // The pair kernel's tile and K-slices of least time (us, as measured) for these sizes; *tile != 0 and split_k != 0 are requests.
-static double best_pair_tile(int M, int f_tiles, int k_tiles, int split_k, bool wide_only, const DeviceInfo &di, int *tile, int *split) {
+// image_room: workspace bytes for X images.  A form that needs them takes a tile whose images have room; a tile without room runs in the gather form, whose step
+// costs kGatherStep more (0.66 -> 0.83 us and 0.585 -> 0.78 measured).  Counted as tiled, 5104 x 15382 at 67 tokens without room for images took the
+// 256-token tile, 47.2 us, for 42.7 in two slices of the 128-token tile.
+constexpr double kGatherStep = 0.18;
+static double best_pair_tile(int M, int K, int f_tiles, int k_tiles, int force_kernel, int split_k, bool wide_only, size_t image_room, const DeviceInfo &di, int *tile, int *split) {
     const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
     const bool requested = *tile != 0;
     const int request = *tile;
     double best = -1.0;
     for (const PairTile &t : kPairTiles) {
         if (requested ? t.tokens != request : (wide_only && (t.tokens == 128 || t.tokens == 256))) continue;
+        const bool tiled = wide_only || force_kernel == ESP_KERNEL_PAIR_TILED;
+        const bool room = image_room >= ximg_bytes(M, K, t.tokens);
+        if (!requested && tiled && !room) continue;
+        const double step_us = t.step_us + (force_kernel == ESP_KERNEL_PAIR || !room ? kGatherStep : 0.0);
         // waves x time of one wave.  Waves: a grid of up to two waves runs as whole waves (equal tiles end together); over many
         // waves the clusters drift apart and the last, partial wave costs less and less of a whole one.
         // K-slices (128- and 256-token tiles: the pushed partial rows of all slices must fit the ring), each of at least four
@@ -1324,7 +1332,7 @@ static double best_pair_tile(int M, int f_tiles, int k_tiles, int split_k, bool 
             if (sp > 1 && wanted == 0 && pairs > cap) continue;
             const double w = (double)pairs / (double)cap, whole = (double)ceil_div(pairs, cap);
             const double waves = w <= 2.0 ? whole : w + (whole - w) * (2.0 / w);
-            const double cost = waves * (t.step_us * ceil_div(k_tiles, sp) + t.fixed_us) + (sp > 1 ? 10.0 : 0.0);
+            const double cost = waves * (step_us * ceil_div(k_tiles, sp) + t.fixed_us) + (sp > 1 ? 10.0 : 0.0);
             if (log_plans()) fprintf(stderr, "esparse plan M=%d f_tiles=%d k_tiles=%d pair tile=%d split=%d pairs=%ld waves=%.2f cost=%.1f\n", M, f_tiles, k_tiles, t.tokens, sp, pairs, waves, cost);
             if (best < 0.0 || cost < best) { best = cost; *tile = t.tokens; *split = sp; }
         }
@@ -1437,7 +1445,7 @@ static const PairTime kPairTimes[] = {
 };
 
 // The form of least estimated time.
-static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, bool images_room, const DeviceInfo &di, const int *layer, GemmPlan *g) {
+static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, size_t image_room, const DeviceInfo &di, const int *layer, GemmPlan *g) {
     const int k_tiles = ceil_div(K, kTileK), f_tiles = ceil_div(N, kTileFeat);
     const double x_elems = 1e-6 * (double)K * M;
     double best = 1e30;
@@ -1453,7 +1461,7 @@ static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, bool image
         g->x_area = sh.x_area;
     };
     for (const StreamTime &t : kStreamTimes) {
-        if ((t.images && !images_room) || t.tokens >= 2 * M) continue;
+        if ((t.images && image_room < (t.tokens < 64 ? xtile_narrow_bytes(M, K, t.tokens) : ximg_bytes(M, K, 128))) || t.tokens >= 2 * M) continue;
         const int kernel = t.images ? ESP_KERNEL_STREAM_IMAGES : ESP_KERNEL_STREAM;
         const long tiles = (long)f_tiles * ceil_div(M, t.tokens);
         for (int split : {1, 2, 3, 4, 6, 8}) {
@@ -1474,7 +1482,7 @@ static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, bool image
     }
     const long per_wave = std::max(1, di.sm_count / 2);
     for (const PairTime &t : kPairTimes) {
-        if (t.tiled && !images_room) continue;
+        if (t.tiled && image_room < ximg_bytes(M, K, t.tokens)) continue;
         const bool sliced = t.tokens == 128 || t.tokens == 256;             // (as in best_pair_tile)
         const long pairs = (long)ceil_div(f_tiles, t.tokens == 256 ? 2 : 4) * ceil_div(M, t.tokens);
         for (int split = 1; split <= (sliced ? (M > 256 ? 2 : 4) : 1); ++split) {
@@ -1501,6 +1509,7 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
     const int k_tiles = ceil_div(K, kTileK);
     const int f_tiles = ceil_div(N, kTileFeat);
     const bool channel_major_available = (o.x_layout == ESP_X_CHANNEL_MAJOR) || have_workspace;
+    const size_t image_room = have_workspace ? workspace_bytes - transpose_bytes(M, K, o) : 0;      // behind the transposed copy
     int bn = o.token_tile;
     int layer[9] = {};
     for (int split = 1; split <= 8; ++split) layer[split] = stream_clusters_one_per_sm(di.device, split);
@@ -1522,7 +1531,7 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
             // default, as callers that ask for the plan expect; the others would gain up to 7 us of 15 there.)
             const bool narrow = M <= 256 && (long)f_tiles * k_tiles <= 64 && (long)f_tiles * ceil_div(M, 64) * std::min(k_tiles, 8) <= 2L * di.sm_count;
             if (M > 64 && bn == 0 && o.split_k == 0 && o.pipeline_stages == 0 && !narrow && (M <= 256 || k_tiles >= 16) && weight < (M > 1000 ? 15000000L : 40000000L) &&
-                fastest_form(M, N, K, o, workspace_bytes >= gemm_workspace_bytes(M, K, o), di, layer, &g)) {
+                fastest_form(M, N, K, o, image_room, di, layer, &g)) {
                 *plan = g;
                 return ESP_OK;
             }
@@ -1541,7 +1550,7 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
             // 78 -> 67 / 118 -> 68 us; 9216 x 9216 at 64 / 128 tokens 41 -> 28 / 47 -> 37 us; but 9216 x 9216 at 32 tokens
             // 22.5 -> 28.4, 4096 x 4096 at 128 tokens 15.0 -> 17.1).  It also replaces the pair kernel's gather form where that
             // would run K-slices at 129..256 tokens (9216 x 9216 at 256 tokens: 95 -> 55 us).
-            const bool images_room = workspace_bytes >= transpose_bytes(M, K, o) + ximg_bytes(M, K, 128);
+            const bool images_room = image_room >= ximg_bytes(M, K, 128);
             if (images_room && bn == 0 && o.split_k <= 8 && M > 16 && M <= 256) {
                 const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
                 if (!pair) {
@@ -1559,7 +1568,7 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
                         // pair kernel's K-slices, whose larger tiles pull less (4096 x 11008 at 200 tokens: 41.5 -> 40.0 us)
                         int tile = 0, sp = 1;
                         const double bytes = (double)f_tiles * ceil_div(M, bn) * k_tiles * (kTileBytes + 256.0 * bn);
-                        if (M > 128 && o.split_k == 0 && best_pair_tile(M, f_tiles, k_tiles, 0, false, di, &tile, &sp) < bytes / 9e6 - 2.0) {
+                        if (M > 128 && o.split_k == 0 && best_pair_tile(M, K, f_tiles, k_tiles, ESP_KERNEL_AUTO, 0, false, image_room, di, &tile, &sp) < bytes / 9e6 - 2.0) {
                             g.kernel = ESP_KERNEL_PAIR;
                             bn = 0;
                         }
@@ -1575,11 +1584,15 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
                            g.kernel == ESP_KERNEL_QUAD_MULTICAST;                                      // no 128-token form
     if (g.kernel == ESP_KERNEL_PAIR || g.kernel == ESP_KERNEL_PAIR_TILED || wide_only) {
         int split = 1;
-        if (best_pair_tile(M, f_tiles, k_tiles, o.split_k, wide_only, di, &bn, &split) < 0.0) return ESP_ERR_INVALID_ARG;
+        if (best_pair_tile(M, K, f_tiles, k_tiles, o.force_kernel, o.split_k, wide_only, image_room, di, &bn, &split) < 0.0) {
+            // (no tile at all, or none whose images have room)
+            const bool without_room = best_pair_tile(M, K, f_tiles, k_tiles, o.force_kernel, o.split_k, wide_only, SIZE_MAX, di, &bn, &split) >= 0.0;
+            return without_room ? ESP_ERR_WORKSPACE : ESP_ERR_INVALID_ARG;
+        }
         // the tiled form needs room for the X images behind the transposed copy; without it the gather form runs.  Up to
         // 128 tokens the gather form is taken anyway: one launch instead of two, and X is small.
         // (on a large weight the gather's row copies cost more than that launch: 22016 x 8192 at 100 tokens 76 -> 61 us)
-        const bool room = workspace_bytes >= transpose_bytes(M, K, o) + ximg_bytes(M, K, bn);
+        const bool room = image_room >= ximg_bytes(M, K, bn);
         if ((g.kernel == ESP_KERNEL_PAIR_TILED || wide_only) && !room) return ESP_ERR_WORKSPACE;
         if (wide_only && (bn == 128 || bn == 256)) return ESP_ERR_INVALID_ARG;
         // (129..256 tokens in one K-slice: the tiled form too -- 11008 x 4096 at 256 tokens 37.4 -> 33.4 us, 13824 x 5120
@@ -1605,7 +1618,7 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
         }
     }
     if (g.kernel == ESP_KERNEL_TMA && bn < 64) bn = 64;
-    if (g.kernel == ESP_KERNEL_STREAM_IMAGES && workspace_bytes < transpose_bytes(M, K, o) + ximg_bytes(M, K, 128)) return ESP_ERR_WORKSPACE;
+    if (g.kernel == ESP_KERNEL_STREAM_IMAGES && image_room < ximg_bytes(M, K, 128)) return ESP_ERR_WORKSPACE;
     if (bn != 16 && bn != 32 && bn != 64 && bn != 128 && bn != 256) return ESP_ERR_INVALID_ARG;
     g.token_tile = bn;
     g.stages = 4;

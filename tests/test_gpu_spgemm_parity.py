@@ -730,6 +730,40 @@ def test_clusters_that_do_not_fit_the_gpcs_are_not_counted_as_one_per_sm(M, N, K
     check(spgemm(X, pack_on_gpu(vals, meta), theta, N, channel_major=True, static_weights=1), ref_product(X, vals, meta, theta))
 
 
+def image_bytes(M, K, tile):
+    """Workspace that the X images of one token tile take: images, a flag each, the inverse permutation, a counter per half tile."""
+    up = lambda n: (n + 255) // 256 * 256
+    halves, k_tiles = 2 * ((M + tile - 1) // tile), (K + 127) // 128
+    return halves * k_tiles * (16384 if tile == 128 else 32768) + up(halves * k_tiles * 4) + up(K * 4) + up(halves * 4)
+
+
+@pytest.mark.parametrize("M,N,K,tile", [(100, 1030, 1032, 128), (300, 514, 2056, 128), (390, 700, 2056, 128), (270, 1030, 520, 192)])
+@pytest.mark.parametrize("channel_major", [False, True])
+def test_workspace_with_room_for_one_image_form(M, N, K, tile, channel_major):
+    """A workspace that holds the images of one token tile and not of every tile: the tiled pair kernel takes a tile whose images fit,
+    the default form runs on any size, and nothing is written behind the workspace."""
+    import torch
+    from paper_2310_15929_b200 import binding as b
+    from tests.gpu_util import pack_on_gpu
+    dev = torch.device("cuda:0")
+    vals, meta, theta = pruned(8500 + M + K, N, K)
+    X = (np.random.default_rng(M + K).standard_normal((M, K))).astype(np.float16)
+    Yref = ref_product(X, vals, meta, theta)
+    packed, perm = pack_on_gpu(vals, meta), torch.from_numpy(theta).to(dev)
+    ldx = (M + 7) // 8 * 8
+    Xt = torch.from_numpy(X).to(dev) if not channel_major else torch.nn.functional.pad(torch.from_numpy(X.T.copy()), (0, ldx - M)).to(dev)[:, :M]
+    transposed = 0 if channel_major else (K * ((M + 15) // 16 * 16) * 2 + 255) // 256 * 256
+    full = transposed + image_bytes(M, K, tile)
+    for kernel, nbytes in ((6, full), (0, full), (0, full - 256), (0, transposed + 256), (0, transposed)):
+        o = b.esp_gemm_opts_default()
+        o.x_layout, o.force_kernel = int(channel_major), kernel
+        buf = torch.full((nbytes + 4096,), 0x5A, dtype=torch.uint8, device=dev)
+        Y = torch.full((M, N), float("nan"), dtype=torch.float16, device=dev)
+        b.esp_spgemm(Xt, packed, perm, Y, o, buf[:nbytes] if nbytes else None)
+        check(Y.cpu().numpy(), Yref)
+        assert bool((buf[nbytes:] == 0x5A).all())
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
