@@ -296,8 +296,9 @@ esp_status_t esp_spgemm(const void *X, int M, int K, long ldx,
  * own weight, permutation, input and output.  (The paper times a layer's Q/K/V as one GEMM, Table 5; this keeps the three
  * weights, and their three channel permutations, separate.)  M, K, ldx and the options are common, N[i] and ldy[i] are
  * per problem; X, packed, perm, N, Y, ldy are HOST arrays of `count` entries (perm[i] may be NULL; opts->bias is not
- * supported here and must be NULL).  Up to 256 tokens the problems share one launch of the streaming kernel -- what a
- * short launch loses to start-up and drain is paid once; for more tokens the call is the same as `count` calls of
+ * supported here and must be NULL).  Up to 64 tokens the problems share one launch of the streaming kernel -- what a
+ * short launch loses to start-up and drain is paid once --, and up to 256 tokens where that is estimated to take less time than
+ * the problems one after the other; else, and for more tokens, the call is the same as `count` calls of
  * esp_spgemm.  workspace: count * esp_spgemm_workspace_bytes(M, max N, K, opts) bytes.
  */
 #define ESP_MAX_GROUP 4

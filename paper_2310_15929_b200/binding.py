@@ -255,7 +255,8 @@ _group_types = [(c_void_p * n, c_int * n, c_long * n) for n in range(5)]      # 
 
 
 def esp_spgemm_grouped(Xs, packeds, perms, Ys, opts, workspace=None, stream=None):
-    """Ys[i] = Xs[i] . P[i] . W_s[i]^T for up to 4 problems with common M and K in one call (one launch up to 256 tokens)."""
+    """Ys[i] = Xs[i] . P[i] . W_s[i]^T for up to 4 problems with common M and K in one call (one launch up to 64 tokens, and up
+    to 256 where that is estimated faster than one after the other)."""
     n = len(Ys)
     M = Ys[0].shape[0]
     K = Xs[0].shape[0] if opts.x_layout == ESP_X_CHANNEL_MAJOR else Xs[0].shape[1]

@@ -1444,8 +1444,8 @@ static const PairTime kPairTimes[] = {
     {256, true, 0.520, 11.7, 6.9, 0.96},
 };
 
-// The form of least estimated time.
-static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, size_t image_room, const DeviceInfo &di, const int *layer, GemmPlan *g) {
+// The form of least estimated time and that time (us; negative: none runs).  `gather_only`: of the streaming kernel's gather forms.
+static double fastest_form(int M, int N, int K, const esp_gemm_opts &o, bool gather_only, size_t image_room, const DeviceInfo &di, const int *layer, GemmPlan *g) {
     const int k_tiles = ceil_div(K, kTileK), f_tiles = ceil_div(N, kTileFeat);
     const double x_elems = 1e-6 * (double)K * M;
     double best = 1e30;
@@ -1461,7 +1461,7 @@ static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, size_t ima
         g->x_area = sh.x_area;
     };
     for (const StreamTime &t : kStreamTimes) {
-        if ((t.images && image_room < (t.tokens < 64 ? xtile_narrow_bytes(M, K, t.tokens) : ximg_bytes(M, K, 128))) || t.tokens >= 2 * M) continue;
+        if ((t.images && gather_only) || (t.images && image_room < (t.tokens < 64 ? xtile_narrow_bytes(M, K, t.tokens) : ximg_bytes(M, K, 128))) || t.tokens >= 2 * M) continue;
         const int kernel = t.images ? ESP_KERNEL_STREAM_IMAGES : ESP_KERNEL_STREAM;
         const long tiles = (long)f_tiles * ceil_div(M, t.tokens);
         for (int split : {1, 2, 3, 4, 6, 8}) {
@@ -1482,6 +1482,7 @@ static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, size_t ima
     }
     const long per_wave = std::max(1, di.sm_count / 2);
     for (const PairTime &t : kPairTimes) {
+        if (gather_only) break;
         if (t.tiled && image_room < ximg_bytes(M, K, t.tokens)) continue;
         const bool sliced = t.tokens == 128 || t.tokens == 256;             // (as in best_pair_tile)
         const long pairs = (long)ceil_div(f_tiles, t.tokens == 256 ? 2 : 4) * ceil_div(M, t.tokens);
@@ -1495,7 +1496,7 @@ static bool fastest_form(int M, int N, int K, const esp_gemm_opts &o, size_t ima
                  t.tiled ? ESP_KERNEL_PAIR_TILED : ESP_KERNEL_PAIR, t.tokens, StreamShape{split, 0, kXChannelMajor, 0, 0});
         }
     }
-    return best < 1e30;
+    return best < 1e30 ? best : -1.0;
 }
 
 static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts &o, size_t workspace_bytes, GemmPlan *plan) {
@@ -1531,7 +1532,7 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
             // default, as callers that ask for the plan expect; the others would gain up to 7 us of 15 there.)
             const bool narrow = M <= 256 && (long)f_tiles * k_tiles <= 64 && (long)f_tiles * ceil_div(M, 64) * std::min(k_tiles, 8) <= 2L * di.sm_count;
             if (M > 64 && bn == 0 && o.split_k == 0 && o.pipeline_stages == 0 && !narrow && (M <= 256 || k_tiles >= 16) && weight < (M > 1000 ? 15000000L : 40000000L) &&
-                fastest_form(M, N, K, o, image_room, di, layer, &g)) {
+                fastest_form(M, N, K, o, false, image_room, di, layer, &g) >= 0.0) {
                 *plan = g;
                 return ESP_OK;
             }
@@ -1871,6 +1872,41 @@ esp_status_t launch_spgemm(const __half *X, int M, int K, long ldx, const void *
     }
 }
 
+// More than 64 tokens, and the group's weights as one would take a form that has no launch for groups: true if the streaming kernel, one launch for all, is still
+// estimated faster than the problems one after the other in their own forms (three of 5936 x 1792 at 125 tokens: 29 us, 56 apart; of 6880 x 722 at 239: 27
+// and 50; two of 2456 x 4594 at 90: 18 and 23).  Remembered per thread, like the plans.
+static bool group_in_one_launch(int count, int M, int K, const int *N, int f_total, const esp_gemm_opts &o, size_t workspace_bytes, GemmPlan *plan) {
+    if (o.force_kernel != ESP_KERNEL_AUTO || o.token_tile != 0 || o.split_k != 0 || o.pipeline_stages != 0) return false;
+    struct Entry { int dev, count, M, K, N[ESP_MAX_GROUP], x_layout, static_weights; size_t ws; bool one; GemmPlan plan; };
+    thread_local Entry cache[16];
+    thread_local int n = 0, next = 0;
+    DeviceInfo di;
+    if (device_info(&di) != ESP_OK) return false;
+    Entry e = {di.device, count, M, K, {}, o.x_layout, o.static_weights, workspace_bytes, false, GemmPlan{}};
+    for (int i = 0; i < count; ++i) e.N[i] = N[i];
+    for (int i = 0; i < n; ++i) {
+        const Entry &c = cache[i];
+        if (c.dev == e.dev && c.count == e.count && c.M == e.M && c.K == e.K && std::equal(c.N, c.N + ESP_MAX_GROUP, e.N) && c.x_layout == e.x_layout &&
+            c.static_weights == e.static_weights && c.ws == e.ws) {
+            if (c.one) *plan = c.plan;
+            return c.one;
+        }
+    }
+    int layer[9] = {};
+    for (int split = 1; split <= 8; ++split) layer[split] = stream_clusters_one_per_sm(di.device, split);
+    const size_t share = (workspace_bytes / (size_t)count) & ~(size_t)255, transposed = transpose_bytes(M, K, o);
+    const double together = fastest_form(M, f_total * kTileFeat, K, o, true, 0, di, layer, &e.plan);
+    double apart = 0.0;
+    GemmPlan ignored;
+    for (int i = 0; i < count; ++i) apart += fastest_form(M, N[i], K, o, false, share > transposed ? share - transposed : 0, di, layer, &ignored);
+    e.one = together >= 0.0 && together < apart;
+    if (e.one) *plan = e.plan;
+    cache[next] = e;
+    next = (next + 1) % 16;
+    if (n < 16) ++n;
+    return e.one;
+}
+
 esp_status_t launch_spgemm_group(int count, const void *const *X, int M, int K, long ldx, const void *const *packed,
                                  const int32_t *const *perm, const int *N, void *const *Y, const long *ldy,
                                  const esp_gemm_opts &o, void *workspace, size_t workspace_bytes, cudaStream_t stream) {
@@ -1884,7 +1920,7 @@ esp_status_t launch_spgemm_group(int count, const void *const *X, int M, int K, 
     if (og.force_kernel == ESP_KERNEL_AUTO && M <= 64) og.force_kernel = ESP_KERNEL_STREAM;
     esp_status_t st = plan_gemm(M, f_total * kTileFeat, K, og, workspace ? workspace_bytes : 0, &plan);
     if (st != ESP_OK) return st;
-    if (plan.kernel != ESP_KERNEL_STREAM) return ESP_ERR_UNSUPPORTED;
+    if (plan.kernel != ESP_KERNEL_STREAM && !(M > 64 && group_in_one_launch(count, M, K, N, f_total, og, workspace ? workspace_bytes : 0, &plan))) return ESP_ERR_UNSUPPORTED;
     GemmGroup grp;
     grp.count = count;
     int ft = 0;
@@ -1905,7 +1941,7 @@ esp_status_t launch_spgemm_group(int count, const void *const *X, int M, int K, 
         p.xflags = nullptr;
         p.raster_panel = 0;
         p.x_mode = plan.x_mode;
-    p.x_area = plan.x_area;
+        p.x_area = plan.x_area;
         grp.ft_start[i] = ft;
         if (i < count) {
             if (o.x_layout != ESP_X_CHANNEL_MAJOR && plan.x_mode == kXChannelMajor) {      // token-major: a transposed copy per distinct input, one after the other

@@ -764,6 +764,35 @@ def test_workspace_with_room_for_one_image_form(M, N, K, tile, channel_major):
         assert bool((buf[nbytes:] == 0x5A).all())
 
 
+@pytest.mark.parametrize("M,K,Ns,launches", [(125, 5936, (1792, 1792, 1792), 1), (239, 6880, (722, 722, 722), 1), (90, 2456, (4594, 4594), 1), (64, 1160, (384, 200), 1),
+                                             (257, 1160, (384, 200), 4)])
+def test_grouped_products_in_one_launch(M, K, Ns, launches):
+    """Middle groups that measured faster in one launch of the streaming kernel get one, counted in a captured graph; more than 256 tokens
+    run one after the other (images and product each)."""
+    import torch
+    from cuda.bindings import runtime
+    from paper_2310_15929_b200 import binding as b
+    from tests.gpu_util import pack_on_gpu
+    dev = torch.device("cuda:0")
+    X = np.random.default_rng(3).standard_normal((M, K)).astype(np.float16)
+    Xt = torch.nn.functional.pad(torch.from_numpy(X.T.copy()), (0, -M % 8)).to(dev)[:, :M]
+    probs = [pruned(N + 19 + i, N, K) for i, N in enumerate(Ns)]
+    packed, perms = [pack_on_gpu(p[0], p[1]) for p in probs], [torch.from_numpy(p[2]).to(dev) for p in probs]
+    Ys = [torch.full((M, N), float("nan"), dtype=torch.float16, device=dev) for N in Ns]
+    o = b.esp_gemm_opts_default()
+    o.x_layout = b.ESP_X_CHANNEL_MAJOR
+    ws = torch.empty(len(Ns) * b.esp_spgemm_workspace_bytes(M, max(Ns), K, o) + 16, dtype=torch.uint8, device=dev)
+    call = lambda: b.esp_spgemm_grouped([Xt] * len(Ns), packed, perms, Ys, o, ws)
+    call()
+    for Y, p in zip(Ys, probs):
+        check(Y.cpu().numpy(), ref_product(X, *p))
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    err, _, n = runtime.cudaGraphGetNodes(graph.raw_cuda_graph())
+    assert int(err) == 0 and n == launches
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
