@@ -1368,7 +1368,12 @@ static bool stream_shape(int M, int N, int K, const esp_gemm_opts &o, int kernel
         if (kernel == ESP_KERNEL_STREAM && o.x_layout == ESP_X_TOKEN_MAJOR) {
             const long weight = (long)N * K;
             if (bn == 16 && (M == 1 || (M <= kXDirectTokens && K <= 8192))) x_mode = kXDirect;
-            else if (bn <= 32 && weight <= (M <= 16 ? 4500000L : 1200000L) && stream_x_area_bytes(bn, M, kts) <= kXAreaMax) {
+            // (with static_weights the transposing launch overlaps the product before it and costs the GPU little; reading a CTA's share of X at the
+            // start of the product then pays for shares that the producers read in about one go.  us per call in a queue, transposed -> through the
+            // cluster: 1600 x 818 at 12 tokens, shares of 3 steps, 6.8 -> 6.9 on the GPU and 8.2 -> 6.3 from the host; 5488 x 128 at 46, 6 steps of 16 tokens,
+            // 8.2 -> 9.2 and 8.6 -> 8.4; 9696 x 158 at 15 10.4 -> 12.2 and 9.8 -> 11.5; 32-token tiles, 2392 x 438 at 35 7.4 -> 8.4 and 8.6 -> 7.9)
+            else if (bn <= 32 && weight <= (M <= 16 ? 4500000L : 1200000L) && stream_x_area_bytes(bn, M, kts) <= kXAreaMax &&
+                     (!o.static_weights || kts * ((std::min(M, bn) + 7) / 8) <= (bn == 16 ? 10 : 6))) {
                 x_mode = kXCluster;
                 x_area = stream_x_area_bytes(bn, M, kts);
             }

@@ -793,6 +793,32 @@ def test_grouped_products_in_one_launch(M, K, Ns, launches):
     assert int(err) == 0 and n == launches
 
 
+@pytest.mark.parametrize("M,N,K,static,launches", [(16, 2048, 2048, 1, 1), (49, 156, 5472, 1, 2), (49, 156, 5472, 0, 1), (15, 158, 9696, 1, 2), (35, 438, 2392, 1, 2),
+                                                   (28, 5426, 216, 1, 1), (8, 158, 9696, 1, 1), (1, 158, 9696, 1, 1)])
+def test_small_token_major_products_in_one_launch(M, N, K, static, launches):
+    """Token-major X with and without a transposing launch, on both sides of the rule for launches that overlap; counted in a captured
+    graph."""
+    import torch
+    from cuda.bindings import runtime
+    from paper_2310_15929_b200 import binding as b
+    from tests.gpu_util import pack_on_gpu
+    dev = torch.device("cuda:0")
+    vals, meta, theta = pruned(7950 + M, N, K)
+    X = np.random.default_rng(M).standard_normal((M, K)).astype(np.float16)
+    Xd, packed, perm = torch.from_numpy(X).to(dev), pack_on_gpu(vals, meta), torch.from_numpy(theta).to(dev)
+    Y = torch.full((M, N), float("nan"), dtype=torch.float16, device=dev)
+    o = b.esp_gemm_opts_default()
+    o.static_weights = static
+    ws = torch.empty(b.esp_spgemm_workspace_bytes(M, N, K, o), dtype=torch.uint8, device=dev)
+    b.esp_spgemm(Xd, packed, perm, Y, o, ws)
+    check(Y.cpu().numpy(), ref_product(X, vals, meta, theta))
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        b.esp_spgemm(Xd, packed, perm, Y, o, ws)
+    err, _, n = runtime.cudaGraphGetNodes(graph.raw_cuda_graph())
+    assert int(err) == 0 and n == launches
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
