@@ -503,9 +503,11 @@ inline size_t stream_smem_bytes(int bn, int stages, int split, int x_area) {
 // XMODE: kernels of their own, so that the registers of the token-major producers cost the channel-major form no residency.
 // (Registers: two CTAs of 576 threads share an SM, 56 each; a 256-token tile has an SM to itself; of the narrow tiles, whose shared memory lets
 // two to four CTAs share one, four and three.  Bounded to 56 as well, a narrow tile's X loop lost up to 10 %: 4096 x 4096 at 16 tokens,
-// device-bound, 6.9 -> 6.45 us, 2208 x 6528 at 37 tokens 10.4 -> 9.7.)
-template <int BN, int XMODE>
-__global__ void __launch_bounds__(StreamCfg<BN>::kThreads, BN == 256 ? 1 : BN >= 64 ? 2 : XMODE == kXChannelMajor ? 4 : 3) spgemm_stream_kernel(const GemmGroup grp, const int stages) {
+// device-bound, 6.9 -> 6.45 us, 2208 x 6528 at 37 tokens 10.4 -> 9.7.  OVERLAP: launched as a dependent of the kernel before, whose tail then hides the start-up.
+// The 32-token tile launched in plain stream order is left unbounded, 56 registers by the compiler's own choice: with 80 its start-up showed, 680 x 9668
+// at 32 tokens 8.6 -> 9.6 us, 744 x 4408 at 60 8.6 -> 9.5; in dependent launches 80 are 1 % ahead, and for 16 tokens the two are even.)
+template <int BN, int XMODE, bool OVERLAP>
+__global__ void __launch_bounds__(StreamCfg<BN>::kThreads, BN == 256 ? 1 : BN >= 64 ? 2 : XMODE != kXChannelMajor ? 3 : OVERLAP ? 4 : 0) spgemm_stream_kernel(const GemmGroup grp, const int stages) {
     constexpr bool TM = XMODE != kXChannelMajor, xcluster = XMODE == kXCluster;
     using L = StreamCfg<BN>;
     // this CTA's problem: selected with constant indices so that the parameters stay in registers
@@ -1022,18 +1024,20 @@ esp_status_t launch_xtile_narrow(const GemmParams &p, uint8_t *img, uint32_t *fl
 
 // The kernel for these parameters.
 template <int BN>
-auto stream_kernel_for(int x_mode) {
+auto stream_kernel_for(int x_mode, bool dependent) {
     if constexpr (BN == 16)
-        if (x_mode == kXDirect) return spgemm_stream_kernel<BN, kXDirect>;
+        if (x_mode == kXDirect) return spgemm_stream_kernel<BN, kXDirect, true>;
     if constexpr (BN <= 32)
-        if (x_mode == kXCluster) return spgemm_stream_kernel<BN, kXCluster>;
-    return spgemm_stream_kernel<BN, kXChannelMajor>;
+        if (x_mode == kXCluster) return spgemm_stream_kernel<BN, kXCluster, true>;
+    if constexpr (BN == 32)
+        if (!dependent) return spgemm_stream_kernel<BN, kXChannelMajor, false>;
+    return spgemm_stream_kernel<BN, kXChannelMajor, true>;
 }
 
 template <int BN>
 esp_status_t launch_stream(const GemmParams &p, int f_tiles, int t_tiles, int split, int stages, bool dependent,
                            cudaStream_t stream) {
-    auto kern = stream_kernel_for<BN>(p.x_mode);
+    auto kern = stream_kernel_for<BN>(p.x_mode, dependent);
     const size_t smem = stream_smem_bytes(BN, stages, split, p.x_area);
     ESP_CUDA_OK(ensure_dynamic_smem((const void *)kern, (int)smem));
     cudaLaunchConfig_t cfg = {};
@@ -1061,7 +1065,7 @@ esp_status_t launch_stream(const GemmParams &p, int f_tiles, int t_tiles, int sp
 // The same launch for a group of problems (feature tiles concatenated along grid.x).
 template <int BN>
 esp_status_t launch_stream_group(const GemmGroup &grp, int t_tiles, int split, int stages, bool dependent, cudaStream_t stream) {
-    auto kern = stream_kernel_for<BN>(grp.p[0].x_mode);
+    auto kern = stream_kernel_for<BN>(grp.p[0].x_mode, dependent);
     const size_t smem = stream_smem_bytes(BN, stages, split, grp.p[0].x_area);
     ESP_CUDA_OK(ensure_dynamic_smem((const void *)kern, (int)smem));
     cudaLaunchConfig_t cfg = {};
@@ -1091,7 +1095,7 @@ static int stream_clusters_one_per_sm(int device, int split) {
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(device * 16 + split);
     if (it != cache.end()) return it->second;
-    auto kern = stream_kernel_for<128>(kXChannelMajor);
+    auto kern = stream_kernel_for<128>(kXChannelMajor, true);
     const size_t smem = stream_smem_bytes(128, 4, split, 0);
     int n = 0;
     if (ensure_dynamic_smem((const void *)kern, (int)smem) == cudaSuccess) {

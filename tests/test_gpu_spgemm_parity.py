@@ -819,6 +819,20 @@ def test_small_token_major_products_in_one_launch(M, N, K, static, launches):
     assert int(err) == 0 and n == launches
 
 
+@pytest.mark.parametrize("M,N,K,split", [(17, 130, 1032, 1), (32, 9668, 680, 3), (60, 250, 2056, 8), (33, 128, 8, 1)])
+@pytest.mark.parametrize("out_f32", [False, True])
+def test_32_token_tile_in_plain_stream_order(M, N, K, split, out_f32):
+    """The 32-token tile's kernel for launches in plain stream order: right values, the same bits as the one for dependent launches."""
+    from tests.gpu_util import pack_on_gpu, spgemm
+    vals, meta, theta = pruned(8600 + M + K, N, K)
+    X = (np.random.default_rng(M + K).standard_normal((M, K))).astype(np.float16)
+    kw = dict(channel_major=True, kernel=4, token_tile=32, split_k=split, out_f32=out_f32)
+    packed = pack_on_gpu(vals, meta)
+    Y = spgemm(X, packed, theta, N, **kw)
+    check(Y, ref_product(X, vals, meta, theta), out_f32)
+    assert np.array_equal(Y, spgemm(X, packed, theta, N, static_weights=1, **kw))
+
+
 def test_grouped_products_sharing_one_input():
     """q, k, v style: three weights on the SAME token-major X (one transposed copy serves all three)."""
     import torch
