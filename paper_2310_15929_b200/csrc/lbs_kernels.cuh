@@ -578,11 +578,12 @@ __device__ __forceinline__ void lbs_load_scores(const double *__restrict__ score
     __syncthreads();
 }
 
-// Ascending bitonic sort of a warp's 256 non-negative values, eight per lane.
-__device__ __forceinline__ void lbs_sort256(float (&v)[8]) {
+// Ascending bitonic sort of the first WIDTH (a power of two, 8 or more) of a warp's 256 non-negative values, eight per lane; the others are zero.
+template <int WIDTH>
+__device__ __forceinline__ void lbs_sort(float (&v)[8]) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 2; k <= 256; k <<= 1) {
+    for (int k = 2; k <= WIDTH; k <<= 1) {
 #pragma unroll
         for (int j = k >> 1; j > 0; j >>= 1) {
             if (j >= 8) {
@@ -609,8 +610,9 @@ __device__ __forceinline__ void lbs_sort256(float (&v)[8]) {
 // Wb[b][row][x] = |W[row, channel x of block b]| bits, `stride` (lbs_block rounded up to 8) per row, zeros beyond the block: one
 // pass over W, permuted through shared memory, so that everything below reads whole contiguous rows.  irregular[b][row] is set where
 // the row holds a magnitude of 0.5 or more, or two products that fp32 cannot tell apart (found by sorting the row's products: about
-// 700 instructions per row and block, two per cent of the table kernel), or the block a score that is no ordinary positive number.
-// A warp per (row, block).
+// 700 instructions per row of a 256-channel block, two per cent of the table kernel; a narrow block sorts no wider than it is -- 512 blocks of
+// 8 channels of a 4096 x 4096 weight 2.8 -> 0.77 ms), or the block a score that is no ordinary positive number.  A warp per (row, block).
+template <int WIDTH>                                              // lbs_block or more
 __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restrict__ W, int No, int C, long ldw, const double *__restrict__ score,
                                                          const int32_t *__restrict__ theta0, int lbs_block, int stride, int nblocks,
                                                          int rows_per_cta, uint16_t *__restrict__ Wb, uint8_t *__restrict__ irregular) {
@@ -655,7 +657,7 @@ __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restric
                     make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16), h[4] | ((uint32_t)h[5] << 16), h[6] | ((uint32_t)h[7] << 16));
             bool irr = bad || __any_sync(0xFFFFFFFFu, top >= kWideBits);
             if (!irr) {
-                lbs_sort256(p);
+                lbs_sort<WIDTH>(p);
                 float above = __shfl_down_sync(0xFFFFFFFFu, p[0], 1);
                 if (lane == 31) above = INFINITY;
                 bool close = false;
@@ -696,7 +698,7 @@ __global__ void __launch_bounds__(256) lbs_transpose_kernel(const __half *__rest
 }
 
 // table[b][g][slot][x] = V(group g of block b with its slot replaced by block channel x); base[G] = V(g).
-// One CTA per (block, group), all rows in chunks.  Two CTAs per SM (128 registers), so that one's sort runs under the other's
+// One CTA per (block, group of a full block), all rows in chunks.  Two CTAs per SM (128 registers), so that one's sort runs under the other's
 // candidates.
 constexpr int kTableRows = 1024, kTableThreads = 256;
 struct LbsTableSmem {
@@ -716,7 +718,7 @@ __global__ void __launch_bounds__(kTableThreads, 2) lbs_table_kernel(const uint1
                                                                      int lbs_block, double *__restrict__ table, double *__restrict__ base) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsTableSmem &S = *reinterpret_cast<LbsTableSmem *>(s_dyn);
-    const int g = blockIdx.x % kLbsGroups, b = blockIdx.x / kLbsGroups;
+    const int groups = lbs_block / 4, g = blockIdx.x % groups, b = blockIdx.x / groups;
     const int p0 = b * lbs_block, m = min(lbs_block, C - p0);
     if (g * 4 >= m) return;
     const int tid = threadIdx.x;

@@ -149,6 +149,26 @@ def test_block_shuffle_narrow_blocks(No, C, block):
     assert_identical_to_oracle(g, ref)
 
 
+@pytest.mark.parametrize("block", [12, 28, 32, 36, 128])
+def test_block_shuffle_rows_told_apart_in_blocks_of_every_width(block):
+    """Rows whose products fp32 cannot order are found by a sort as wide as the block: ties between the first and the last channels of
+    a block, at the widths where the sort changes."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8400 + block)
+    No, C = 90, 264
+    W = (g0.standard_normal((No, C)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(C)
+    perm = g0.permutation(C).astype(np.int32)                 # the order the shuffle starts from
+    for b0 in range(0, C, block):
+        first, last = perm[b0], perm[min(C, b0 + block) - 1]
+        s[last] = s[first]
+        W[::3, last] = W[::3, first]
+    theta, info = orc.local_block_shuffle(W, s, perm, block)
+    g = GpuPrune(W, None, 1.0, score=s, perm=perm, lbs_block=block)
+    assert np.array_equal(g.host()[2], theta)
+    assert g.stats.lbs_swaps_total == info.swaps_total and g.stats.near_tie_swaps == info.near_tie_swaps
+
+
 def test_llama7b_q_projection_full_size_block_shuffle():
     """Workload 1's q projection whole (4096 x 4096, 16 shuffle blocks, Student-t rows): global shuffle, block shuffle
     capped at 4 swaps per block on both sides (the oracle's table alone is 4.3e9 row evaluations), selection and
