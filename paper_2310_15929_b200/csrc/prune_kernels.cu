@@ -451,8 +451,12 @@ __global__ void __launch_bounds__(256) entropy_score_kernel(int C, int T, int bi
     if (counts) {
         for (int i = threadIdx.x; i < nc * bins; i += 256) {
             const unsigned int n = counts[(long)c0 * bins + i];
-            const double p = __ddiv_rn((double)n, (double)T);
-            s_term[(i / bins) * ld + i % bins] = n ? __dmul_rn(p, log(p)) : 0.0;
+            double term = 0.0;
+            if (n) {                         // (few tokens leave most bins empty: dividing for those too, 36864 channels of 512 bins took 190 us, not 149)
+                const double p = __ddiv_rn((double)n, (double)T);
+                term = __dmul_rn(p, log(p));
+            }
+            s_term[(i / bins) * ld + i % bins] = term;
         }
     }
     __syncthreads();
