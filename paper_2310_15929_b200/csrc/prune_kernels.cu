@@ -993,10 +993,11 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
     if (st != ESP_OK) return st;
     const int cthreads = 256;
     const int cblocks = ceil_div(C, cthreads);
-    ESP_CUDA_OK(cudaMemsetAsync(w.counters, 0, w.cleared_bytes, stream));
+    // (the counts, last of what is cleared, are only used by a statistics pass: 36864 channels of 512 bins without one, 1024 rows selected: 0.210 -> 0.199 ms)
+    const bool stats_pass = Xcal && (o.score_override == nullptr || chan_norm || chan_entropy);
+    ESP_CUDA_OK(cudaMemsetAsync(w.counters, 0, stats_pass ? w.cleared_bytes : (size_t)((char *)w.counts - (char *)w.counters), stream));
 
-    const bool need_stats_pass = (o.score_override == nullptr) || chan_norm || chan_entropy;
-    if (need_stats_pass && Xcal) {
+    if (stats_pass) {
         // K1
         st = launch_colstats(Xcal, T, C, ldx, ColStatsOut{nullptr, w.norm, w.lo, w.hi}, di.sm_count, stream);
         if (st != ESP_OK) return st;
