@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(kTableThreads, 2) lbs_table_kernel(const uint1
                                                                      int lbs_block, double *__restrict__ table, double *__restrict__ base) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsTableSmem &S = *reinterpret_cast<LbsTableSmem *>(s_dyn);
-    const int groups = lbs_block / 4, g = blockIdx.x % groups, b = blockIdx.x / groups;
+    const int g = blockIdx.x, b = blockIdx.y;
     const int p0 = b * lbs_block, m = min(lbs_block, C - p0);
     if (g * 4 >= m) return;
     const int tid = threadIdx.x;

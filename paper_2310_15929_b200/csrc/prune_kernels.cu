@@ -1047,7 +1047,7 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
                                                                                     gather_rows, w.wb, w.irregular);
         lbs_transpose_kernel<<<dim3(ceil_div(C, 64), ceil_div(No, 64)), 256, 0, stream>>>(W, No, C, ldw, w.wt, w.ldt);
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_table_kernel, (int)sizeof(LbsTableSmem)));
-        lbs_table_kernel<<<nblocks * (o.lbs_block / 4), kTableThreads, sizeof(LbsTableSmem), stream>>>(w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score,
+        lbs_table_kernel<<<dim3(o.lbs_block / 4, nblocks), kTableThreads, sizeof(LbsTableSmem), stream>>>(w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score,
                                                                                                 w.theta0, C, o.lbs_block, w.table, w.base[0]);
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_greedy_kernel, (int)lbs_greedy_smem(kGreedyMinCluster)));
         ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
