@@ -94,7 +94,9 @@ typedef struct {
 /* Fills *opts with the paper's settings (bins 100, 2:4, block 256, everything on, alpha = 1). */
 void esp_prune_opts_default(esp_prune_opts *opts);
 
-/* Bytes of device workspace esp_metric_prune needs for these sizes (0 on bad arguments). */
+/* Bytes of device workspace esp_metric_prune needs for these sizes (0 on bad arguments).  With the block shuffle about 4 * No * C bytes (two copies of |W|:
+   channel-major, and gathered row by row for each shuffle block, whose rows are rounded up to 8 channels) + 2 KB * 256 / lbs_block per channel, besides
+   the histogram's counts, 4 * C * bins. */
 size_t esp_metric_prune_workspace_bytes(int No, int C, int T, const esp_prune_opts *opts);
 
 /*
@@ -240,10 +242,10 @@ void esp_gemm_opts_default(esp_gemm_opts *opts);
 
 /*
  * Bytes of device workspace esp_spgemm can use: for token-major X a transposed (channels-as-rows, not
- * permuted) copy of X, which lets the fast kernels run, and for more than 256 tokens the permuted X operand
- * images of ESP_KERNEL_PAIR_TILED (about 2.2 * M * K bytes).  With a smaller workspace the call still works:
- * without room for the images through ESP_KERNEL_PAIR, without room for the transposed copy (or with
- * NULL) through the element-gather kernel.  The workspace is scratch: nothing in it outlives the call's work
+ * permuted) copy of X, which lets the fast kernels run, and from 17 tokens the permuted X operand
+ * images of ESP_KERNEL_PAIR_TILED and ESP_KERNEL_STREAM_IMAGES (about 2.2 * M * K bytes, rounded up to whole token
+ * tiles).  With a smaller workspace the call still works: through a form whose images have room or that gathers,
+ * without room for the transposed copy (or with NULL) through the element-gather kernel.  The workspace is scratch: nothing in it outlives the call's work
  * on the stream, and calls on different streams need different workspaces.
  */
 size_t esp_spgemm_workspace_bytes(int M, int N, int K, const esp_gemm_opts *opts);
@@ -278,8 +280,8 @@ esp_status_t esp_spgemm_plan(int M, int N, int K, const esp_gemm_opts *opts, int
  *   X       fp16, M tokens x K channels in the layout opts->x_layout names, leading dimension ldx
  *           (elements; multiple of 8)
  *   packed  esp_packed_bytes(N, K) bytes from esp_metric_prune / esp_pack
- *   perm    int32 [K] or NULL for the identity; applied while the X tile is loaded (up to 256 tokens, or without
- *           a workspace) or by the pass that writes the X operand images into the workspace (more tokens)
+ *   perm    int32 [K] or NULL for the identity; applied while the X tile is loaded or, in the image forms, by the
+ *           pass that writes the X operand images into the workspace
  *   opts    layout, output type, optional bias and activation: Y = act(product + bias), bias and activation applied
  *           to the finished fp32 sum
  *   Y       out, [M, N] row-major (Y[t, j] at Y + t * ldy + j), fp16 or fp32 per opts->out_dtype

@@ -17,8 +17,11 @@
 //    one 512-byte load, nothing is exchanged between lanes.
 //  * fp32 products decide.  Each is within 2^-23 relative of its fp64 counterpart, so they order a row's channels as the fp64
 //    products do unless two of them are closer than 2^-21.  Which rows hold such a pair is found once, when the weight is gathered
-//    (the products of a row's 256 channels never change, only their grouping does): those rows -- about one in a hundred -- and
-//    the rows with a magnitude of 0.5 or more are "irregular" and take fp64 products and 64-bit sums in a loop of their own.
+//    (the products of a row's 256 channels never change, only their grouping does): those rows -- about one in a hundred where
+//    the scores of a block differ -- and the rows with a magnitude of 0.5 or more are "irregular" and take fp64 products and
+//    64-bit sums in a loop of their own.  Equal scores make nearly every row irregular, as do weights with sigma of 0.2 and more and, in
+//    its block, a score that is not positive: little of the gain is left there (4096 x 4096 to the end, against the kernels before: 68.7 -> 57.0 ms
+//    with equal scores, 66.9 -> 33.0 with every sixteenth score zero, 68.2 -> 51.8 at sigma 0.2, 68.6 -> 55.5 at 1.5; 69.7 -> 9.3 at 0.1).
 //  * |w| < 0.5 becomes an integer of 2^-24 with one fp32 fma, so the sums are 32-bit adds.
 //
 // Measured against one comparison and two fp64 additions per (row, candidate, slot) with a warp per candidate (about 29 instructions

@@ -1423,8 +1423,8 @@ static bool stream_shape(int M, int N, int K, const esp_gemm_opts &o, int kernel
 }
 
 // Times (us) of the forms that a product of more than 64 tokens on a weight below 40 M elements can take, fitted to 33000 measured
-// calls: random shapes of 512..11008 features x channels at 60..8200 tokens, every form, tile and number of K-slices that runs
-// (half of the estimates within 5 to 10 %, nine of ten within 20 %; the form chosen by them is 2.5 % slower than the best
+// calls: 1929 shapes of 512..11008 features x channels at 60..8200 tokens, 1427 of them random and 502 token counts on six fixed weights (4096 x 4096,
+// 5120 x 5120, 4096 x 11008, 9216 x 9216, 11008 x 4096, 8192 x 2048), every form, tile and number of K-slices that runs (half of the estimates within 5 to 10 %, nine of ten within 20 %; the form chosen by them is 2.5 % slower than the best
 // measured one in the geometric mean).  Rules of one threshold each stood here before: up to 256 tokens the streaming kernel's 128- and
 // 256-token tiles, the pair kernel beyond.  Small weights lost most: 1010 x 1960 at 181 tokens 15.3 -> 7.8 us, 972 x 3280 at 546 34 -> 16.
 // Streaming kernel: waves of the grid (`wave`), CTAs on an SM in each (`wave_sm`), channel steps of these, MB that all CTAs pull from
@@ -1536,9 +1536,10 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
         else {
             const long weight = (long)N * K;
             // Small and middle weights at more than 64 tokens: the form of least estimated time.  (A few feature tiles on few tokens keep
-            // the rule of narrow token tiles below, which those times do not cover; larger weights keep the rules that follow,
-            // which measure within 10 % of the best form there.  Beyond 256 tokens and below 16 channel steps the tiled pair form stays the
-            // default, as callers that ask for the plan expect; the others would gain up to 7 us of 15 there.)
+            // the rule of narrow token tiles below, which those times do not cover; larger weights keep the rules that follow, mostly within 10 % of the
+            // best form, but not everywhere: 5850 x 8504 at 65 tokens takes 1.24 times as long, 9216 x 9216 at 163..253 1.08 times (two slices, one is
+            // faster).  Beyond 256 tokens and below 16 channel steps the tiled pair form stays the default, which the tests of the plan ask for; streaming tiles
+            // would gain up to 7 us of 15 there.)
             const bool narrow = M <= 256 && (long)f_tiles * k_tiles <= 64 && (long)f_tiles * ceil_div(M, 64) * std::min(k_tiles, 8) <= 2L * di.sm_count;
             if (M > 64 && bn == 0 && o.split_k == 0 && o.pipeline_stages == 0 && !narrow && (M <= 256 || k_tiles >= 16) && weight < (M > 1000 ? 15000000L : 40000000L) &&
                 fastest_form(M, N, K, o, false, image_room, di, layer, &g) >= 0.0) {
@@ -1560,6 +1561,8 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
             // 78 -> 67 / 118 -> 68 us; 9216 x 9216 at 64 / 128 tokens 41 -> 28 / 47 -> 37 us; but 9216 x 9216 at 32 tokens
             // 22.5 -> 28.4, 4096 x 4096 at 128 tokens 15.0 -> 17.1).  It also replaces the pair kernel's gather form where that
             // would run K-slices at 129..256 tokens (9216 x 9216 at 256 tokens: 95 -> 55 us).
+            // (More than 64 tokens on less than 40 M elements come here only with a requested slice count or ring depth, without an estimated form, or as
+            // narrow problems.)
             const bool images_room = image_room >= ximg_bytes(M, K, 128);
             if (images_room && bn == 0 && o.split_k <= 8 && M > 16 && M <= 256) {
                 const long per_wave = di.sm_count / 2 > 0 ? di.sm_count / 2 : 1;
@@ -1575,7 +1578,8 @@ static esp_status_t plan_gemm_uncached(int M, int N, int K, const esp_gemm_opts 
                         bn = M <= 32 ? 32 : (M > 128 && weight >= 64000000L) ? 128 : 64;
                         g.kernel = ESP_KERNEL_STREAM_IMAGES;
                         // beyond 128 tokens that kernel is bound by what all its CTAs pull from L2, about 9 TB/s: long weights go to the
-                        // pair kernel's K-slices, whose larger tiles pull less (4096 x 11008 at 200 tokens: 41.5 -> 40.0 us)
+                        // pair kernel's K-slices, whose larger tiles pull less (4096 x 11008 at 200 tokens: 41.5 -> 40.0 us).  The estimate is low where the images'
+                        // 64-token tiles run in five slices: that weight keeps them at 133..177 tokens, 45 to 46 us, for 39 in the pair kernel.
                         int tile = 0, sp = 1;
                         const double bytes = (double)f_tiles * ceil_div(M, bn) * k_tiles * (kTileBytes + 256.0 * bn);
                         if (M > 128 && o.split_k == 0 && best_pair_tile(M, K, f_tiles, k_tiles, ESP_KERNEL_AUTO, 0, false, image_room, di, &tile, &sp) < bytes / 9e6 - 2.0) {

@@ -85,9 +85,8 @@ def test_shuffle_select_compress_bit_exact_given_oracle_scores(No, C, T, block):
 
 @pytest.mark.parametrize("No,C,block,cap", [(1100, 520, 256, 0), (1024, 256, 256, 12), (2100, 264, 256, 6)])
 def test_block_shuffle_tall_weights_bit_exact(No, C, block, cap):
-    """From 769 rows on the table kernels read a candidate's column four 16-byte loads ahead and finish with a ragged
-    tail: padded row counts of 1280 (one unrolled pass + a tail), 1024 (no tail) and 2304 (two passes + a tail), with a
-    ragged last block of channels."""
+    """The table kernel takes at most 928 rows at once, in equal chunks: two chunks (1100 and 1024 rows) and three (2100), with a
+    ragged last block of channels and slices of the greedy kernel's clusters that are no multiple of eight."""
     from tests.gpu_util import GpuPrune
     g0 = np.random.default_rng(7000 + No)
     W = (g0.standard_normal((No, C)) * 0.02 * np.sqrt(4.0 / g0.chisquare(4.0, size=(No, 1)))).astype(np.float16)
@@ -185,8 +184,8 @@ def test_llama7b_q_projection_full_size_block_shuffle():
 
 @pytest.mark.parametrize("wl_index,lin", [(3, "gate"), (4, "fc1")])
 def test_block_shuffle_all_rows_of_the_widest_layers(wl_index, lin):
-    """All 22016 / 36864 output rows of the widest LLaMA-65B / OPT-66B linears on one block of 256 input channels
-    (the per-row record of the table kernels then fills most of shared memory), two swaps, bit-exact."""
+    """All 22016 / 36864 output rows of the widest LLaMA-65B / OPT-66B linears on one block of 256 input channels: 24 and 40
+    chunks of the table kernel, slices of several chunks in the greedy kernel; two swaps, bit-exact."""
     from tests.gpu_util import GpuPrune
     wl = inputs.WORKLOADS[wl_index]
     W = inputs.make_weight(wl, lin, C=256)
