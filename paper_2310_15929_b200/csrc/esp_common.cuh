@@ -54,6 +54,9 @@ struct PruneWorkspace {
     uint16_t *wb;                                            // [nblocks][No][stride] |W| bits, gathered per shuffle block
     uint8_t *irregular;                                      // [nblocks][No] the row needs fp64 products in the block shuffle
     double *table;                                           // [nblocks][64][4][256]
+    int *handed, *handed_swaps;                              // [nblocks] the exact kernels (re)start this block; swaps it has had
+    int *widest;                                             // [nblocks] bits of the block's largest |W|
+    int32_t *handed_pos;                                     // [C] the order it is in: position -> channel of the block
     long ldt;                                                // No rounded up to 8
     int stride;                                              // lbs_block rounded up to 8
     size_t total_bytes;

@@ -1,4 +1,5 @@
-// Local block shuffle (Algorithm 1 lines 3-14, Eq. 5).  Included by prune_kernels.cu inside namespace esp { namespace { ... } }.
+// Local block shuffle (Algorithm 1 lines 3-14, Eq. 5): the exact kernels.  Included by prune_kernels.cu inside namespace esp { namespace { ... } }.
+// lbs_bounds.cuh, included at the end, finds the same swaps from bounds; the kernels here take the blocks that it cannot decide, from the first swap or from where it stopped.
 //
 // Algorithm 1 needs, for every group g of a block, every slot k of g and every channel x of the block, the value
 //   V(g, k <- x) = retained metric sum of g with slot k replaced by x
@@ -611,14 +612,12 @@ __device__ __forceinline__ void lbs_sort(float (&v)[8]) {
 }
 
 // Wb[b][row][x] = |W[row, channel x of block b]| bits, `stride` (lbs_block rounded up to 8) per row, zeros beyond the block: one
-// pass over W, permuted through shared memory, so that everything below reads whole contiguous rows.  irregular[b][row] is set where
-// the row holds a magnitude of 0.5 or more, or two products that fp32 cannot tell apart (found by sorting the row's products: about
-// 700 instructions per row of a 256-channel block, two per cent of the table kernel; a narrow block sorts no wider than it is -- 512 blocks of
-// 8 channels of a 4096 x 4096 weight 2.8 -> 0.77 ms), or the block a score that is no ordinary positive number.  A warp per (row, block).
-template <int WIDTH>                                              // lbs_block or more
+// pass over W, permuted through shared memory, so that everything below reads whole contiguous rows.  A warp per (row, block).
+// widest[b] becomes the bits of the block's largest magnitude; handed[b] is set where the bounds of lbs_bounds.cuh do not hold: a weight that is not finite, a score that is no ordinary positive number, scores more
+// than 2^60 apart.
 __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restrict__ W, int No, int C, long ldw, const double *__restrict__ score,
                                                          const int32_t *__restrict__ theta0, int lbs_block, int stride, int nblocks,
-                                                         int rows_per_cta, uint16_t *__restrict__ Wb, uint8_t *__restrict__ irregular) {
+                                                         int rows_per_cta, uint16_t *__restrict__ Wb, int *__restrict__ handed, int *__restrict__ widest) {
     extern __shared__ __align__(16) uint16_t s_rows[];            // [rows_per_cta][C]
     const int j0 = blockIdx.x * rows_per_cta;
     const int nrows = min(rows_per_cta, No - j0);
@@ -634,45 +633,85 @@ __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restric
     for (int b = threadIdx.x >> 5; b < nblocks; b += 8) {
         const int p0 = b * lbs_block, m = min(lbs_block, C - p0);
         int ch[8];
-        float s32[8];
         bool bad = false;
+        int top = -100000, low = 100000;                          // exponents of the scores
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             ch[e] = x0 + e < m ? theta0[p0 + x0 + e] : -1;
-            const double s = ch[e] >= 0 ? score[ch[e]] : 1.0;
-            s32[e] = (float)s;
-            bad = bad || !(s >= 0x1p-80 && s <= 0x1p80);
+            if (ch[e] >= 0) {
+                const double s = score[ch[e]];
+                const bool ordinary = s >= 0x1p-80 && s <= 0x1p80;
+                bad = bad || !ordinary;
+                if (ordinary) { top = max(top, ilogb(s)); low = min(low, ilogb(s)); }
+            }
         }
-        bad = __any_sync(0xFFFFFFFFu, bad);
+        top = __reduce_max_sync(0xFFFFFFFFu, top);                // (all lanes, whatever they have found)
+        low = __reduce_min_sync(0xFFFFFFFFu, low);
+        bad = bad || top - low > 60;
+        uint32_t wide = 0;
         for (int r = 0; r < nrows; ++r) {
             uint16_t h[8];
-            uint16_t top = 0;
-            float p[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 h[e] = ch[e] >= 0 ? s_rows[(size_t)r * C + ch[e]] : (uint16_t)0;
-                top = max(top, h[e]);
-                p[e] = __half2float(__ushort_as_half(h[e])) * s32[e];
+                wide = max(wide, (uint32_t)h[e]);
             }
-            const size_t row = (size_t)b * No + j0 + r;
             if (x0 < stride)
-                *reinterpret_cast<uint4 *>(Wb + row * stride + x0) =
+                *reinterpret_cast<uint4 *>(Wb + ((size_t)b * No + j0 + r) * stride + x0) =
                     make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16), h[4] | ((uint32_t)h[5] << 16), h[6] | ((uint32_t)h[7] << 16));
-            bool irr = bad || __any_sync(0xFFFFFFFFu, top >= kWideBits);
-            if (!irr) {
-                lbs_sort<WIDTH>(p);
-                float above = __shfl_down_sync(0xFFFFFFFFu, p[0], 1);
-                if (lane == 31) above = INFINITY;
-                bool close = false;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const float hi = e < 7 ? p[e + 1] : above;
-                    close = close || (hi > 0.f && !(hi - p[e] > hi * kLbsMargin) && hi < INFINITY);
-                }
-                irr = __any_sync(0xFFFFFFFFu, close);
-            }
-            if (lane == 0) irregular[row] = irr ? 1 : 0;
         }
+        wide = __reduce_max_sync(0xFFFFFFFFu, wide);
+        if (lane == 0) atomicMax(&widest[b], (int)wide);
+        if (bad || wide >= 0x7C00u) handed[b] = 1;
+    }
+}
+
+// For the exact kernels: irregular[b][row] is set where
+// the row holds a magnitude of 0.5 or more, or two products that fp32 cannot tell apart (found by sorting the row's products: about
+// 700 instructions per row of a 256-channel block; a narrow block sorts no wider than it is -- 512 blocks of
+// 8 channels of a 4096 x 4096 weight 2.8 -> 0.77 ms), or the block a score that is no ordinary positive number.  A warp per row of a block.
+template <int WIDTH>                                              // lbs_block or more
+__global__ void __launch_bounds__(256) lbs_mark_kernel(const uint16_t *__restrict__ Wb, int No, int stride, const double *__restrict__ score,
+                                                       const int32_t *__restrict__ theta0, int C, int lbs_block, const int *__restrict__ handed,
+                                                       uint8_t *__restrict__ irregular) {
+    const int b = blockIdx.y, p0 = b * lbs_block, m = min(lbs_block, C - p0);
+    if (!handed[b]) return;
+    const int lane = threadIdx.x & 31, x0 = lane * 8;
+    float s32[8];
+    bool bad = false;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const double s = x0 + e < m ? score[theta0[p0 + x0 + e]] : 1.0;
+        s32[e] = (float)s;
+        bad = bad || !(s >= 0x1p-80 && s <= 0x1p80);
+    }
+    bad = __any_sync(0xFFFFFFFFu, bad);
+    for (int j = blockIdx.x * 8 + (threadIdx.x >> 5); j < No; j += gridDim.x * 8) {
+        const size_t row = (size_t)b * No + j;
+        const uint4 v = x0 < stride ? __ldg(reinterpret_cast<const uint4 *>(Wb + row * stride + x0)) : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        uint16_t top = 0;
+        float p[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const uint16_t h = (uint16_t)(w[e >> 1] >> (16 * (e & 1)));
+            top = max(top, h);
+            p[e] = __half2float(__ushort_as_half(h)) * s32[e];
+        }
+        bool irr = bad || __any_sync(0xFFFFFFFFu, top >= kWideBits);
+        if (!irr) {
+            lbs_sort<WIDTH>(p);
+            float above = __shfl_down_sync(0xFFFFFFFFu, p[0], 1);
+            if (lane == 31) above = INFINITY;
+            bool close = false;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float hi = e < 7 ? p[e + 1] : above;
+                close = close || (hi > 0.f && !(hi - p[e] > hi * kLbsMargin) && hi < INFINITY);
+            }
+            irr = __any_sync(0xFFFFFFFFu, close);
+        }
+        if (lane == 0) irregular[row] = irr ? 1 : 0;
     }
 }
 
@@ -718,21 +757,23 @@ struct LbsTableSmem {
 __global__ void __launch_bounds__(kTableThreads, 2) lbs_table_kernel(const uint16_t *__restrict__ Wb, const uint16_t *__restrict__ Wt, long ldt,
                                                                      const uint8_t *__restrict__ irregular, int No, int stride,
                                                                      const double *__restrict__ score, const int32_t *__restrict__ theta0, int C,
-                                                                     int lbs_block, double *__restrict__ table, double *__restrict__ base) {
+                                                                     int lbs_block, const int *__restrict__ handed, const int32_t *__restrict__ handed_pos,
+                                                                     double *__restrict__ table, double *__restrict__ base) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsTableSmem &S = *reinterpret_cast<LbsTableSmem *>(s_dyn);
     const int g = blockIdx.x, b = blockIdx.y;
     const int p0 = b * lbs_block, m = min(lbs_block, C - p0);
-    if (g * 4 >= m) return;
+    if (g * 4 >= m || !handed[b]) return;
     const int tid = threadIdx.x;
     for (int i = tid; i < 2 * LbsCells<4>::kWords; i += kTableThreads) S.cells[i] = 0u;
     if (tid < 2 * kLbsGroupSums) S.sums[tid] = 0u;
     if (tid < 32) S.rows.cnt[tid] = 0;
     lbs_load_scores(score, theta0, p0, m, S.s64, S.s32);
     if (tid < 4) {
-        S.grp.channel[tid] = theta0[p0 + g * 4 + tid];
-        S.grp.s[tid] = S.s64[g * 4 + tid];
-        S.grp.s32[tid] = S.s32[g * 4 + tid];
+        const int x = handed_pos[p0 + g * 4 + tid];
+        S.grp.channel[tid] = theta0[p0 + x];
+        S.grp.s[tid] = S.s64[x];
+        S.grp.s32[tid] = S.s32[x];
     }
     if (tid == 0) S.skip = -1;
     __syncthreads();
@@ -850,8 +891,9 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
                                                                        const uint8_t *__restrict__ irregular, int No, int stride,
                                                                        const double *__restrict__ score, const int32_t *__restrict__ theta0, int C,
                                                                        int lbs_block, int max_swaps, double *__restrict__ table,
-                                                                       const double *__restrict__ base0, double *__restrict__ base,
-                                                                       int32_t *__restrict__ theta, unsigned long long *__restrict__ counters, int nc) {
+                                                                       const double *__restrict__ base0, int32_t *__restrict__ theta,
+                                                                       unsigned long long *__restrict__ counters, const int *__restrict__ handed,
+                                                                       const int *__restrict__ handed_swaps, const int32_t *__restrict__ handed_pos, int nc) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsGreedySmem &S = *reinterpret_cast<LbsGreedySmem *>(s_dyn);
     using Cells = LbsCells<3>;
@@ -859,6 +901,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
     const int p0 = b * lbs_block, m = min(lbs_block, C - p0), G = m / 4;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr int kWarps = kGreedyThreads / 32;
+    if (!handed[b]) return;
     double *tb = table + (long)b * kLbsGroups * 4 * kLbsMax;      // row of position i: group i / 4, slot i % 4
     auto clear_sums = [&]() {
         for (int i = tid; i < (int)(sizeof(S.cells) / 16); i += kGreedyThreads) reinterpret_cast<uint4 *>(S.cells)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -866,7 +909,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
     };
     clear_sums();
     if (tid < 64) S.rows[tid >> 5].cnt[tid & 31] = 0;
-    for (int x = tid; x < m; x += kGreedyThreads) { S.pos2x[x] = x; S.chan[x] = theta0[p0 + x]; }
+    for (int x = tid; x < m; x += kGreedyThreads) { S.pos2x[x] = handed_pos[p0 + x]; S.chan[x] = theta0[p0 + x]; }
     for (int g = tid; g < G; g += kGreedyThreads) S.base[g] = base0[p0 / 4 + g];
     lbs_load_scores(score, theta0, p0, m, S.s64, S.s32);          // (ends with a barrier: everything above is visible)
     const int per_cta = (No + nc - 1) / nc, row0 = min(No, rank * per_cta), nrows_all = min(No, row0 + per_cta) - row0, chunk_rows = lbs_chunk_rows(nrows_all, kGreedyRows);
@@ -880,7 +923,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
         double *gr = S.gains + lbs_gain_offset(r, m, rank, nc);
 #pragma unroll 4
         for (int j = i + 1 + lane; j < m; j += 32) {
-            const double after = __dadd_rn(__ldcg(&tb[i * kLbsMax + j]), __ldcg(&tb[j * kLbsMax + i]));
+            const double after = __dadd_rn(__ldcg(&tb[i * kLbsMax + S.pos2x[j]]), __ldcg(&tb[j * kLbsMax + S.pos2x[i]]));
             gr[j - i - 1] = (i >> 2) == (j >> 2) ? -INFINITY : __dsub_rn(after, __dadd_rn(S.base[i >> 2], S.base[j >> 2]));
         }
     }
@@ -888,7 +931,8 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
     // running by then)
     cluster_arrive();
     cluster_wait();
-    int swaps = 0, near_swaps = 0;
+    const int swaps0 = handed_swaps[b];
+    int swaps = swaps0, near_swaps = 0;
     for (;;) {
         double best = -INFINITY, second = -INFINITY;              // second: largest gain once one instance of the best is set aside
         int at = 0x7FFFFFFF;
@@ -1019,8 +1063,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
     }
     if (rank != 0) return;
     for (int x = tid; x < m; x += kGreedyThreads) theta[p0 + x] = S.chan[S.pos2x[x]];
-    for (int g = tid; g < G; g += kGreedyThreads) base[p0 / 4 + g] = S.base[g];
-    if (tid == 0 && swaps) atomicAdd(&counters[1], (unsigned long long)swaps);
+    if (tid == 0 && swaps > swaps0) atomicAdd(&counters[1], (unsigned long long)(swaps - swaps0));
     if (tid == 0 && near_swaps) atomicAdd(&counters[3], (unsigned long long)near_swaps);
 }
 
@@ -1038,33 +1081,4 @@ inline void lbs_greedy_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr
     cfg.numAttrs = 1;
 }
 
-// CTAs per block: the size that ends soonest.  A swap costs about 10 us of barriers, search and exchange and 55 ns per output row of a
-// CTA's slice; the blocks run in waves of as many clusters as the device holds (asked once per size and device).
-inline int lbs_cluster_size(int nblocks, int No, int device) {
-    static std::mutex mu;
-    static std::map<int, int> cache;
-    const int sizes[] = {16, 14, 12, 10, 9, 8, 7, 6, 5, 4, kGreedyMinCluster};
-    int best = kGreedyMinCluster;
-    double best_cost = -1.0;
-    for (int nc : sizes) {
-        int cap = 0;
-        {
-            std::lock_guard<std::mutex> lock(mu);
-            auto it = cache.find(device * 64 + nc);
-            if (it != cache.end()) cap = it->second;
-            else {
-                cudaLaunchConfig_t cfg;
-                cudaLaunchAttribute attr;
-                lbs_greedy_config(cfg, attr, 1, nc, nullptr);
-                if (cudaOccupancyMaxActiveClusters(&cap, lbs_greedy_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); cap = 0; }
-                cache[device * 64 + nc] = cap;
-            }
-        }
-        if (cap <= 0) continue;
-        const double w = (double)nblocks / cap, whole = std::ceil(w), waves = w <= 2.0 ? whole : w + (whole - w) * (2.0 / w);
-        const double cost = waves * (10.0 + 0.055 * (double)((No + nc - 1) / nc));
-        if (log_plans()) fprintf(stderr, "esparse block shuffle: blocks=%d rows=%d cluster=%d capacity=%d cost=%.1f\n", nblocks, No, nc, cap, cost);
-        if (best_cost < 0.0 || cost < best_cost) { best_cost = cost; best = nc; }
-    }
-    return best;
-}
+#include "lbs_bounds.cuh"

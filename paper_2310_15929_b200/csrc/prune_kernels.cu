@@ -912,6 +912,11 @@ PruneWorkspace carve_prune_workspace(void *ws, int No, int C, int T, const esp_p
     w.objective = (double *)take(sizeof(double) * 4);
     w.colsum = (unsigned long long *)take(sizeof(unsigned long long) * C);
     w.kept = (unsigned long long *)take(sizeof(unsigned long long) * C);
+    if (o.use_lbs) {
+        w.handed = (int *)take(sizeof(int) * (size_t)ceil_div(C, o.lbs_block));
+        w.handed_swaps = (int *)take(sizeof(int) * (size_t)ceil_div(C, o.lbs_block));
+        w.widest = (int *)take(sizeof(int) * (size_t)ceil_div(C, o.lbs_block));
+    }
     w.counts = (unsigned int *)take(sizeof(unsigned int) * (size_t)C * o.bins);
     w.cleared_bytes = w.counts ? (size_t)((char *)w.counts - (char *)w.counters) + sizeof(unsigned int) * (size_t)C * o.bins : 0;
     w.theta0 = (int32_t *)take(sizeof(int32_t) * C);
@@ -922,8 +927,9 @@ PruneWorkspace carve_prune_workspace(void *ws, int No, int C, int T, const esp_p
         w.ldt = (long)align_up((size_t)No, 8);
         w.stride = (int)align_up((size_t)o.lbs_block, 8);
         w.wt = (uint16_t *)take(sizeof(uint16_t) * (size_t)C * w.ldt);
-        w.wb = (uint16_t *)take(sizeof(uint16_t) * (size_t)nblocks * No * w.stride);
+        w.wb = (uint16_t *)take(sizeof(uint16_t) * ((size_t)nblocks * No + kBoundOver) * w.stride);
         w.irregular = (uint8_t *)take((size_t)nblocks * No);
+        w.handed_pos = (int32_t *)take(sizeof(int32_t) * C);
         w.table = (double *)take(sizeof(double) * (size_t)nblocks * kLbsGroups * 4 * kLbsMax);
     }
     w.total_bytes = off;
@@ -1042,24 +1048,46 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
         // rows per CTA: about 96 KB of shared memory (two CTAs per SM), and a grid of two CTAs per SM at least
         int gather_rows = (int)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / row_bytes));
         gather_rows = std::max(1, std::min(gather_rows, No / (2 * std::max(1, di.sm_count))));
-        auto gather = o.lbs_block <= 8 ? lbs_gather_kernel<8> : o.lbs_block <= 32 ? lbs_gather_kernel<32> : lbs_gather_kernel<kLbsMax>;
-        ESP_CUDA_OK(ensure_dynamic_smem((const void *)gather, (int)(row_bytes * gather_rows)));
-        gather<<<ceil_div(No, gather_rows), 256, row_bytes * gather_rows, stream>>>(W, No, C, ldw, w.score, w.theta0, o.lbs_block, w.stride, nblocks,
-                                                                                    gather_rows, w.wb, w.irregular);
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_gather_kernel, (int)(row_bytes * gather_rows)));
+        lbs_gather_kernel<<<ceil_div(No, gather_rows), 256, row_bytes * gather_rows, stream>>>(W, No, C, ldw, w.score, w.theta0, o.lbs_block, w.stride, nblocks,
+                                                                                               gather_rows, w.wb, w.handed, w.widest);
         lbs_transpose_kernel<<<dim3(ceil_div(C, 64), ceil_div(No, 64)), 256, 0, stream>>>(W, No, C, ldw, w.wt, w.ldt);
-        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_table_kernel, (int)sizeof(LbsTableSmem)));
-        lbs_table_kernel<<<dim3(o.lbs_block / 4, nblocks), kTableThreads, sizeof(LbsTableSmem), stream>>>(w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score,
-                                                                                                w.theta0, C, o.lbs_block, w.table, w.base[0]);
-        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_greedy_kernel, (int)lbs_greedy_smem(kGreedyMinCluster)));
-        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        const int nc = lbs_cluster_size(nblocks, No, di.device);
+        // the swaps by bounds
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_table_kernel, (int)sizeof(LbsBoundTableSmem)));
+        lbs_bound_table_kernel<<<dim3(ceil_div(o.lbs_block, 8), nblocks), kBoundTableThreads, sizeof(LbsBoundTableSmem), stream>>>(
+            w.wb, w.wt, w.ldt, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.widest, w.table);
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_greedy_kernel, (int)lbs_bound_smem(kBoundMinCluster)));
+        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_bound_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        int nc = lbs_cluster_size(lbs_bound_greedy_kernel, lbs_bound_config, kBoundMinCluster, 10.0, 0.022, nblocks, No, di.device);
+        lbs_bound_config(cfg, attr, nblocks, nc, stream);
+        ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_bound_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, No, w.stride,
+                                       (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters, (const int *)w.widest, w.handed, w.handed_swaps, w.handed_pos, nc));
+        // the exact kernels, on the blocks that were handed to them (without any, 8 us)
+        auto mark = o.lbs_block <= 8 ? lbs_mark_kernel<8> : o.lbs_block <= 32 ? lbs_mark_kernel<32> : lbs_mark_kernel<kLbsMax>;
+        mark<<<dim3(ceil_div(No, 64), nblocks), 256, 0, stream>>>(w.wb, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.irregular);
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_table_kernel, (int)sizeof(LbsTableSmem)));
+        lbs_table_kernel<<<dim3(o.lbs_block / 4, nblocks), kTableThreads, sizeof(LbsTableSmem), stream>>>(
+            w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.handed_pos, w.table, w.base[1]);
+        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_greedy_kernel, (int)lbs_greedy_smem(kGreedyMinCluster)));
+        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        nc = lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, 10.0, 0.055, nblocks, No, di.device);
         lbs_greedy_config(cfg, attr, nblocks, nc, stream);
         ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, (const uint8_t *)w.irregular, No,
                                        w.stride, (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table,
-                                       (const double *)w.base[0], w.base[1], perm, w.counters, nc));
-        if (stats) objective_kernel<<<3, 256, 0, stream>>>(G, w.base[0], w.base[1], w.base[2], w.objective);
+                                       (const double *)w.base[1], perm, w.counters, (const int *)w.handed, (const int *)w.handed_swaps,
+                                       (const int32_t *)w.handed_pos, nc));
+        if (stats) {
+            // the objectives before and after (colabs_kernel, which gathers the permuted channels from W, took 47 us for each of the orders of a 4096 x 4096 weight)
+            const int rows = 2048;
+            ESP_CUDA_OK(cudaMemsetAsync(w.kept, 0, sizeof(unsigned long long) * C, stream));
+            ESP_CUDA_OK(cudaMemsetAsync(w.colsum, 0, sizeof(unsigned long long) * C, stream));       // (free by now)
+            lbs_kept_kernel<<<dim3(ceil_div(G, 8), ceil_div(No, rows), 2), 256, 0, stream>>>(w.wt, w.ldt, No, G, rows, w.score, w.theta0, perm, w.kept, w.colsum);
+            group_values_kernel<<<ceil_div(G, 256), 256, 0, stream>>>(w.kept, w.score, w.theta0, G, w.base[0]);
+            group_values_kernel<<<ceil_div(G, 256), 256, 0, stream>>>(w.colsum, w.score, perm, G, w.base[1]);
+            objective_kernel<<<3, 256, 0, stream>>>(G, w.base[0], w.base[1], w.base[2], w.objective);
+        }
     } else if (stats) {
         ESP_CUDA_OK(cudaMemsetAsync(w.kept, 0, sizeof(unsigned long long) * C, stream));
         colabs_kernel<false, true><<<wgrid, 256, 0, stream>>>(W, No, C, ldw, wrows, w.score, w.theta0, w.colsum, w.kept);

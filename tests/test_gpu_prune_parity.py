@@ -168,6 +168,49 @@ def test_block_shuffle_rows_told_apart_in_blocks_of_every_width(block):
     assert g.stats.lbs_swaps_total == info.swaps_total and g.stats.near_tie_swaps == info.near_tie_swaps
 
 
+@pytest.mark.parametrize("No", [16 * 512, 16 * 512 + 1, 16 * 1024 + 8 * 16 + 1])
+def test_block_shuffle_bound_sums_at_the_edges_of_folds_and_chunks(No):
+    """Slices of one fold (512 rows of a CTA), of a row more, of a chunk (1024) and some rows."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8500 + No)
+    W = (g0.standard_normal((No, 64)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(64)
+    ref = orc.metric_prune(W, None, 1.0, score=s, lbs_max_swaps=6)
+    g = GpuPrune(W, None, 1.0, score=s, lbs_max_swaps=6)
+    assert_identical_to_oracle(g, ref)
+    assert ref.lbs.swaps_total == 6
+
+
+@pytest.mark.parametrize("kind", ["tied_from_the_start", "tied_later", "few_ties", "far_apart"])
+@pytest.mark.parametrize("cap", [0, 9])
+def test_block_shuffle_handed_to_the_exact_kernels(kind, cap):
+    """Blocks that bounds cannot decide: dozens of tied pairs at the first swap, or only once the wide channels have found their places; a
+    tie that is settled by itself (two equal channels); scores too far apart for bounds.  One block among others that need no help."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8600)
+    No, C, block = 120, 264, 64
+    W = (g0.standard_normal((No, C)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(C)
+    perm = g0.permutation(C).astype(np.int32)
+    first = perm[:block]                                      # the channels of the first block
+    if kind == "tied_from_the_start":
+        W[:, first] = W[:, first[np.arange(block) % 6]]
+        s[first] = 2.0
+    elif kind == "tied_later":
+        small = first[block // 2:]
+        W[:, small] = (W[:, small[np.arange(block // 2) % 5]].astype(np.float32) / 64).astype(np.float16)
+        s[small] = 1.0
+    elif kind == "few_ties":
+        W[:, first[9]], s[first[9]] = W[:, first[40]], s[first[40]]
+    else:
+        s[first[7]] = 2.0 ** -70
+    theta, info = orc.local_block_shuffle(W, s, perm, block, cap)
+    g = GpuPrune(W, None, 1.0, score=s, perm=perm, lbs_block=block, lbs_max_swaps=cap)
+    assert np.array_equal(g.host()[2], theta)
+    assert g.stats.lbs_swaps_total == info.swaps_total and g.stats.near_tie_swaps == info.near_tie_swaps
+    assert g.stats.obj_after_lbs == orc.objective(W, s, theta)
+
+
 def test_llama7b_q_projection_full_size_block_shuffle():
     """Workload 1's q projection whole (4096 x 4096, 16 shuffle blocks, Student-t rows): global shuffle, block shuffle
     capped at 4 swaps per block on both sides (the oracle's table alone is 4.3e9 row evaluations), selection and
