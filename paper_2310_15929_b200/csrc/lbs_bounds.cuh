@@ -52,7 +52,7 @@ __device__ __forceinline__ float2 bound_gain(double there, double back) {
 }
 // An entry of a group whose value has moved by the gain `by`.
 __device__ __forceinline__ double bound_shift(double entry, double by) {
-    return bound_pack(bound_value(entry) - bound_value(by), __double2float_ru((bound_error(entry) + bound_error(by)) * (1.0 + 0x1p-20)));
+    return bound_pack(bound_value(entry) - bound_value(by), __double2float_ru((bound_error(entry) + bound_error(by)) * (1.0 + 0x1p-9)));
 }
 
 __device__ __forceinline__ float relu_fma(float a, float b, float c) {       // min(1, max(0, a b + c))
