@@ -20,8 +20,8 @@
 // is off by at most x + f2 + d = 2 d + 2 f2 (2 f2 where only the computed value is positive), one of D_k by 2 d + 2 p3.  Together 2 R + 2 D + 4 S with S the sum over rows of
 // p2.  An addition rounds by at most one unit of the partial sum, so R takes one unit per
 // addition on its way: up to kBoundFold in a register, one per fold in shared memory, four in the tree over the warps; D one per row of a thread, five in a warp, one
-// per chunk, four over the warps.  Sums over CTAs are fp64; they, the packing and the exact
-// kernels' own roundings add less than 2^-50 of the group's value, and with products of at most 1 that is at most twice the number of rows.
+// per chunk, six over the warps; both five over the CTAs.  The packing and the exact kernels' own roundings add less than 2^-50 of the group's value, and with
+// products of at most 1 that is at most twice the number of rows.
 //
 // What bounds it: on long slices instruction issue -- a row costs a warp 48 fma, 48 additions, 8 conversions and some 30 others for both groups (256
 // candidates, 6 slots), about 20 ns of an SM's time where the exact kernels take 55 --, on short ones the latency of a swap (search, three cluster barriers,
@@ -305,7 +305,7 @@ struct LbsBoundSmem {
     };
     float4 best[kBoundWarps], won[kBoundMaxCluster];              // (the latter written by the CTAs of the cluster)
     float D[kBoundWarps][8];                                      // of the six live slots, S of the two groups
-    double D_of[kBoundMaxCluster][8];                             // written by the CTAs of the cluster
+    float D_of[kBoundMaxCluster][8];                              // written by the CTAs of the cluster
     unsigned long long exact[kBoundCand * 4][4];                  // this CTA's rows' sums
     double value[kBoundCand * 4];
     int list[kBoundMaxCluster][kBoundCand], list_n[kBoundMaxCluster];       // written by the CTAs of the cluster
@@ -539,8 +539,8 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
     bound_load_scores(score, theta0, p0, m, widest[b], S.s64, S.s32, &S.top);           // (ends with a barrier: everything above is visible)
     for (int x = tid; x < m; x += kBoundThreads) S.split[x] = bound_split(S.s64[x]);          // (visible after the barrier below)
     const int per_cta = ((No + nc - 1) / nc + 7) & ~7, row0 = min(No, rank * per_cta), nrows_all = min(No, row0 + per_cta) - row0;
-    const int add_r = min(kBoundFold, per_cta / kBoundWarps + 1) + per_cta / (kBoundWarps * kBoundFold) + 2 + 4;
-    const int add_d = kBoundChunk / kBoundThreads + 5 + per_cta / kBoundChunk + 1 + 4;
+    const int add_r = min(kBoundFold, per_cta / kBoundWarps + 1) + per_cta / (kBoundWarps * kBoundFold) + 2 + 4 + 5;
+    const int add_d = kBoundChunk / kBoundThreads + 5 + per_cta / kBoundChunk + 1 + 4 + 5;
     const uint16_t *wt_rows = Wt + row0;
     BoundSums<6> sums;
     BoundFeed feed;
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
                 for (int w = 0; w < kBoundWarps / 4; ++w) t += S.D[(lane >> 3) * (kBoundWarps / 4) + w][lane & 7];
                 t += __shfl_xor_sync(0xFFFFFFFFu, t, 8);
                 t += __shfl_xor_sync(0xFFFFFFFFu, t, 16);
-                for (int c = lane >> 3; c < nc; c += 4) st_remote_f64(map_to_rank(smem_u32(&S.D_of[rank][lane & 7]), (uint32_t)c), (double)t);
+                for (int c = lane >> 3; c < nc; c += 4) st_remote_f32(map_to_rank(smem_u32(&S.D_of[rank][lane & 7]), (uint32_t)c), t);
             }
         }
         cluster_arrive();
@@ -733,19 +733,21 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
         if (tid < share && c < kBoundCells) {
             const int t = c >> 8, x = bound_cell_candidate(c), g = t >= 3 ? 1 : 0, l = t - 3 * g, k = l + (l >= (g ? skip_b : skip_a) ? 1 : 0);
             const uint32_t cell = smem_u32(reinterpret_cast<const float *>(S.part) + c), to = smem_u32(&S.fresh[t][x]);
-            double D = 0.0, T = 0.0, R = 0.0;
+            float D = 0.f, T = 0.f, R = 0.f;
+            auto tree = [](const float (&v)[8]) { return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])); };
             for (int c0 = 0; c0 < nc; c0 += 8) {                  // (eight loads in flight)
-                float v[8];
-#pragma unroll
-                for (int r = 0; r < 8; ++r) v[r] = c0 + r < nc ? ld_dsmem_f32(cell, (uint32_t)(c0 + r)) : 0.f;
+                float v[8], d[8], u[8];
 #pragma unroll
                 for (int r = 0; r < 8; ++r) {
-                    D += c0 + r < nc ? S.D_of[c0 + r][t] : 0.0;
-                    T += c0 + r < nc ? S.D_of[c0 + r][6 + g] : 0.0;
-                    R += (double)v[r];
+                    v[r] = c0 + r < nc ? ld_dsmem_f32(cell, (uint32_t)(c0 + r)) : 0.f;
+                    d[r] = c0 + r < nc ? S.D_of[c0 + r][t] : 0.f;
+                    u[r] = c0 + r < nc ? S.D_of[c0 + r][6 + g] : 0.f;
                 }
+                D += tree(d);
+                T += tree(u);
+                R += tree(v);
             }
-            const double packed = bound_pack(R - D, bound_of(__double2float_ru(R), add_r, __double2float_ru(D), add_d, __double2float_ru(T), No));
+            const double packed = bound_pack((double)R - (double)D, bound_of(R, add_r, D, add_d, T, No));
             for (int r = 0; r < nc; ++r) st_remote_f64(map_to_rank(to, (uint32_t)r), packed);
             if (x < m) tb[((g ? gb : ga) * 4 + k) * kLbsMax + x] = packed;
         }
