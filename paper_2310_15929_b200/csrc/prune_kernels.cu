@@ -408,7 +408,8 @@ __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restr
     }
 }
 
-// Counter replicas for a bin count: as many as keep three CTAs on an SM (about 75 KB each), none beyond.
+// Counter replicas for a bin count: as many as keep three CTAs on an SM (about 75 KB each), none beyond; a second one of 100 bins is cleared and
+// added up for nothing where a CTA has few rows (8 chunks of 795 x 568, 32 rows each: 89.2 us with one, 90.8 with two; 2048 x 8192, 683 rows: 263 and 258).
 // Token splits: whole waves of three CTAs per SM (the counting is bound by the shared-memory atomics, about 17 ns per token row of a CTA
 // at that residency, so a partial wave is lost time; 2048 x 8192: 640 CTAs 30 us, 384 CTAs 20.5); a CTA's set-up and the addition of its counters to the global ones take as long
 // as some 250 rows.
@@ -416,8 +417,6 @@ inline esp_status_t launch_histogram(const __half *X, int T, int C, long ldx, in
                                      int sm_count, cudaStream_t stream) {
     const size_t per_replica = sizeof(unsigned int) * 64 * (size_t)bins;
     const size_t ring = (size_t)(kHistAhead + 1) * 256 * 16;
-    const int R = per_replica * 4 + ring <= 75 * 1024 ? 4 : per_replica * 2 + ring <= 75 * 1024 ? 2 : 1;
-    const size_t smem = per_replica * R + ring;
     const int cols = ceil_div(C, 64), most = std::max(1, std::min(64, ceil_div(T, 32)));
     int splits = 1;
     long best = -1;
@@ -426,6 +425,9 @@ inline esp_status_t launch_histogram(const __half *X, int T, int C, long ldx, in
         if (best < 0 || cost < best) { best = cost; splits = s; }
     }
     const int rows = ceil_div(T, splits);
+    const size_t room = (rows >= 256 ? 75 : 59) * 1024 - ring;
+    const int R = per_replica * 4 <= room ? 4 : per_replica * 2 <= room ? 2 : 1;
+    const size_t smem = per_replica * R + ring;
     auto kern = R == 4 ? histogram_kernel<4> : R == 2 ? histogram_kernel<2> : histogram_kernel<1>;
     ESP_CUDA_OK(ensure_dynamic_smem((const void *)kern, (int)smem));
     ESP_CUDA_OK(launch_overlapped(kern, dim3(cols, splits), 1, 256, smem, stream, X, T, C, ldx, rows, bins, lo, hi, counts));
