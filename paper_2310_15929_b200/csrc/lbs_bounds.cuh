@@ -14,7 +14,7 @@
 // near-tie distance, it is the exact kernels' choice; if no u is positive, the block is done.  Otherwise (about one swap in ten on a LLaMA-7B-shaped
 // projection, with two pairs in question) the pairs that may be the best or nearly tied with it are evaluated exactly, from integer sums.  More of them than
 // kBoundCand (ties by the dozen: equal columns, scores that leave nothing to choose) and the block is handed to the exact kernels as it stands; so are, from the
-// start, blocks with weights that are not finite or with scores that are not ordinary positive numbers of similar size.
+// start, blocks with weights that are not finite or with scores that are not ordinary positive numbers of similar size (or zero).
 //
 // E, in units of 2^-24: a product that stays is rounded once (bound_split), a candidate's takes the rounding of its score; the fma rounds once.  A clamped term of R, d = x - f2 > 0,
 // is off by at most x + f2 + d = 2 d + 2 f2 (2 f2 where only the computed value is positive), one of D_k by 2 d + 2 p3.  Together 2 R + 2 D + 4 S with S the sum over rows of
@@ -22,6 +22,9 @@
 // addition on its way: up to kBoundFold in a register, one per fold in shared memory, four in the tree over the warps; D one per row of a thread, five in a warp, one
 // per chunk, six over the warps; both five over the CTAs.  The packing and the exact kernels' own roundings add less than 2^-50 of the group's value, and with
 // products of at most 1 that is at most twice the number of rows.
+//
+// Two channels of score zero (dead inputs) exchange for nothing: exactly 0 on both sides, so such entries carry no bound; otherwise dozens of them would stay in question to
+// the end.
 //
 // What bounds it: on long slices instruction issue -- a row costs a warp 48 fma, 48 additions, 8 conversions and some 30 others for both groups (256
 // candidates, 6 slots), about 20 ns of an SM's time where the exact kernels take 55 --, on short ones the latency of a swap (search, three cluster barriers,
@@ -288,8 +291,9 @@ __global__ void __launch_bounds__(kBoundTableThreads, 2) lbs_bound_table_kernel(
 #pragma unroll
             for (int w = 0; w < n; ++w) v[w] += v[w + n];
         const double D = S.total[t >> 2][t & 3];
+        const bool idle = S.s64[x] == 0.0 && S.s64[q0 + t] == 0.0;
         table[((long)b * kLbsGroups * 4 + q0 + t) * kLbsMax + x] =
-            bound_pack((double)v[0] - D, bound_of(v[0], add_r, __double2float_ru(D), add_d, __double2float_ru(S.total[t >> 2][4]), No));
+            idle ? 0.0 : bound_pack((double)v[0] - D, bound_of(v[0], add_r, __double2float_ru(D), add_d, __double2float_ru(S.total[t >> 2][4]), No));
     }
 }
 
@@ -687,6 +691,7 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
         double skip_entry = skip_x ? __ldcg(skip_at) : 0.0;
         auto old_entry = [&](int p, int x) { return (p >> 2) != ga && (p >> 2) != gb || p == bi || p == bj ? __ldcg(&tb[p * kLbsMax + x]) : (double)NAN; };
         auto moved = [&](double e, int p, int x) {
+            if ((p == bi || p == bj) && S.s64[x] == 0.0 && S.s64[p == bi ? xj : xi] == 0.0) return 0.0;
             return p == bi ? bound_shift(x == xi ? 0.0 : e, by_a) : p == bj ? bound_shift(x == xj ? 0.0 : e, by_b) : e;
         };
 #pragma unroll
@@ -747,7 +752,8 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
                 T += tree(u);
                 R += tree(v);
             }
-            const double packed = bound_pack((double)R - (double)D, bound_of(R, add_r, D, add_d, T, No));
+            const bool idle = S.s64[x] == 0.0 && S.grp_s[4 * g + k].x == 0.f;
+            const double packed = idle ? 0.0 : bound_pack((double)R - (double)D, bound_of(R, add_r, D, add_d, T, No));
             for (int r = 0; r < nc; ++r) st_remote_f64(map_to_rank(to, (uint32_t)r), packed);
             if (x < m) tb[((g ? gb : ga) * 4 + k) * kLbsMax + x] = packed;
         }
