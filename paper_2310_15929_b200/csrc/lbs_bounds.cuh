@@ -11,7 +11,7 @@
 //
 // An entry G carries a bound E on its distance from the exact gain (the exact kernels' fp64 roundings, some 2^-50 of a group's value, included), and a pair's gain is
 // kept as the interval [l, u] in directed rounding.  If the pair with the largest l leaves every other pair's u behind by more than the
-// near-tie distance, it is the exact kernels' choice; if no u is positive, the block is done.  Otherwise (about one swap in ten on a LLaMA-7B-shaped
+// near-tie distance, it is the exact kernels' choice; if no u is positive, the block is done.  Otherwise (three swaps in a hundred on a LLaMA-7B-shaped
 // projection, with two pairs in question) the pairs that may be the best or nearly tied with it are evaluated exactly, from integer sums.  More of them than
 // kBoundCand (ties by the dozen: equal columns, scores that leave nothing to choose) and the block is handed to the exact kernels as it stands; so are, from the
 // start, blocks with weights that are not finite or with scores that are not ordinary positive numbers of similar size (or zero).
