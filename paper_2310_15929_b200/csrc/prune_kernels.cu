@@ -272,7 +272,9 @@ __device__ __noinline__ int histogram_exact_bin(float xf, int c, int bins, const
 // of a group meet only through the low bits of their bins.  R = 4 gives each of them a counter row of its own (no conflict
 // at all), R = 2 one per two, R = 1 none (expected 1.0 / 1.5 / 2.1 passes per counting instruction; the plain
 // [channel][bin] layout needed 3.3).  R is chosen so that three CTAs still fit an SM.
-constexpr int kHistAhead = 4;                 // rows each thread keeps in flight (eight left room for one replica of 100 bins, not two: 8 chunks of 2048 x 8192 263 -> 258 us)
+constexpr int kHistAhead = 4;                 // rows each thread keeps in flight (eight are never faster, and beyond 150 bins cost the third CTA: 200 bins of 2048 x 8192 33 us against 23)
+constexpr int kHistStatic = 768;              // bytes of the kernel's fixed arrays
+constexpr size_t kHistRoom = (228 * 1024 / 3 - 1024 - kHistStatic) / 256 * 256;     // dynamic shared memory of one of three CTAs on an SM (1 KB is set aside for each)
 template <int R>
 __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restrict__ X, int T, int C, long ldx,
                                                            int rows_per_split, int bins, const double *__restrict__ lo,
@@ -280,6 +282,7 @@ __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restr
     extern __shared__ __align__(16) unsigned int s_cnt[];   // [8][bins][8][R] | the threads' load rings: [kHistAhead + 1][256] x 16 bytes
     __shared__ float s_neg_lo[64], s_r[64];
     __shared__ __half s_lo[64], s_hi[64];
+    static_assert(sizeof(s_neg_lo) + sizeof(s_r) + sizeof(s_lo) + sizeof(s_hi) == kHistStatic, "counted in kHistRoom");
     for (int i = threadIdx.x; i < 64 * R * bins; i += 256) s_cnt[i] = 0;
     grid_dependency_wait();
     grid_launch_dependents();
@@ -408,8 +411,10 @@ __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restr
     }
 }
 
-// Counter replicas for a bin count: as many as keep three CTAs on an SM (about 75 KB each), none beyond; a second one of 100 bins is cleared and
-// added up for nothing where a CTA has few rows (8 chunks of 795 x 568, 32 rows each: 89.2 us with one, 90.8 with two; 2048 x 8192, 683 rows: 263 and 258).
+// Counter replicas for a bin count: one where a CTA has fewer than 1024 rows, beyond as many as keep three CTAs on an SM (kHistRoom; with 109 or 110
+// bins a limit of 75 KB let only two on: 2048 x 8192 of 110 bins 32 us, one replica 22).  Replicas are cleared and added up whatever the rows, and what they
+// spare is small: 100 bins of N(0, 1), one against two, 683 rows 19.8 / 20.1 us, 1366 rows 29.8 / 29.5, 2521 rows 47.4 / 45.5; 50 bins, one against four,
+// 1366 rows 28.1 / 27.2, 2521 rows 45.8 / 42.4; all but a few elements in one or two bins: within 4 % either way.
 // Token splits: whole waves of three CTAs per SM (the counting is bound by the shared-memory atomics, about 17 ns per token row of a CTA
 // at that residency, so a partial wave is lost time; 2048 x 8192: 640 CTAs 30 us, 384 CTAs 20.5); a CTA's set-up and the addition of its counters to the global ones take as long
 // as some 250 rows.
@@ -425,8 +430,7 @@ inline esp_status_t launch_histogram(const __half *X, int T, int C, long ldx, in
         if (best < 0 || cost < best) { best = cost; splits = s; }
     }
     const int rows = ceil_div(T, splits);
-    const size_t room = (rows >= 256 ? 75 : 59) * 1024 - ring;
-    const int R = per_replica * 4 <= room ? 4 : per_replica * 2 <= room ? 2 : 1;
+    const int R = rows < 1024 ? 1 : per_replica * 4 + ring <= kHistRoom ? 4 : per_replica * 2 + ring <= kHistRoom ? 2 : 1;
     const size_t smem = per_replica * R + ring;
     auto kern = R == 4 ? histogram_kernel<4> : R == 2 ? histogram_kernel<2> : histogram_kernel<1>;
     ESP_CUDA_OK(ensure_dynamic_smem((const void *)kern, (int)smem));

@@ -366,6 +366,21 @@ def test_streaming_calibration_equals_one_shot(C, splits):
     assert_identical_to_oracle(g, ref)
 
 
+@pytest.mark.parametrize("T", [300, 6600])
+@pytest.mark.parametrize("bins", [2, 54, 55, 108, 109, 110, 512])
+def test_histogram_counter_replicas(T, bins):
+    """Counts at the bin counts where the number of counter replicas changes, with few and with more than 1024 rows per CTA (4096
+    channels are dealt to six row slices)."""
+    from tests.gpu_util import calibrate_in_chunks
+    g0 = np.random.default_rng(1000 + bins)
+    C = 4096
+    X = (g0.standard_normal((T, C), dtype=np.float32) * np.where(np.arange(C) % 7, 1.0, 20.0).astype(np.float32)).astype(np.float16)
+    counts = calibrate_in_chunks([X], 0.1, bins=bins)[3]
+    cols = np.unique(np.concatenate([[0, 7, 63, 64, C - 1], g0.choice(C, 60, replace=False)]))
+    assert np.array_equal(counts[cols], orc.channel_histogram(np.ascontiguousarray(X[:, cols]), bins))
+    assert counts.sum(axis=1).tolist() == [T] * C
+
+
 @pytest.mark.parametrize("No,C,T", [(128, 264, 333), (96, 1024, 200)])
 def test_global_bin_range_variant(No, C, T):
     """Layer-wide bin range (the other reading of Eq. 1): entropy and score to the statistics bar, everything downstream
