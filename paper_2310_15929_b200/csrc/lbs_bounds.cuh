@@ -418,13 +418,16 @@ __device__ __forceinline__ void bound_exact_sums(const uint16_t *__restrict__ Wt
     }
 }
 
-// kept[o][4 g + k] += the exact sum that slot k of group g retains under order o (theta0, theta).  A warp per (group, rows).
-__global__ void __launch_bounds__(256) lbs_kept_kernel(const uint16_t *__restrict__ Wt, long ldt, int No, int G, int rows, const double *__restrict__ score,
-                                                       const int32_t *__restrict__ theta0, const int32_t *__restrict__ theta,
-                                                       unsigned long long *__restrict__ kept0, unsigned long long *__restrict__ kept) {
-    const int g = blockIdx.x * 8 + (threadIdx.x >> 5), lo = blockIdx.y * rows;
-    if (g >= G) return;
-    const int32_t *order = blockIdx.z ? theta : theta0;
+// value[o][g] = V(g) under order o (theta0, theta), for the objectives.  A CTA per (group, order), one launch that needs nothing cleared and adds nothing up
+// in memory: sums per slot in memory, cleared before and turned into values behind, were four launches more, which a weight with two swaps to make
+// noticed (512 x 512, two swaps: 165 -> 155 us a call; by the exact kernels, which have the values at hand, 158).
+constexpr int kValueThreads = 256;
+__global__ void __launch_bounds__(kValueThreads) lbs_value_kernel(const uint16_t *__restrict__ Wt, long ldt, int No, const double *__restrict__ score,
+                                                                  const int32_t *__restrict__ theta0, const int32_t *__restrict__ theta,
+                                                                  double *__restrict__ value0, double *__restrict__ value) {
+    __shared__ unsigned long long s_sum[4];
+    const int g = blockIdx.x;
+    const int32_t *order = blockIdx.y ? theta : theta0;
     int channel[4];
     double s[4];
 #pragma unroll
@@ -432,7 +435,14 @@ __global__ void __launch_bounds__(256) lbs_kept_kernel(const uint16_t *__restric
         channel[k] = order[4 * g + k];
         s[k] = score[channel[k]];
     }
-    bound_exact_sums(Wt, ldt, lo / 8, 32, min(No, lo + rows), channel, s, (blockIdx.z ? kept : kept0) + 4 * g);
+    if (threadIdx.x < 4) s_sum[threadIdx.x] = 0;
+    __syncthreads();
+    bound_exact_sums(Wt, ldt, threadIdx.x & ~31, blockDim.x, No, channel, s, s_sum);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned long long A[4] = {s_sum[0], s_sum[1], s_sum[2], s_sum[3]};
+        (blockIdx.y ? value : value0)[g] = lbs_group_value(A, s);
+    }
 }
 
 // The exact choice among the pairs whose u reaches `reach` (all threads of all CTAs, three barriers of the cluster): 1 with the pair and whether it is nearly tied, 0 if it

@@ -1085,13 +1085,10 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
                                        (const double *)w.base[1], perm, w.counters, (const int *)w.handed, (const int *)w.handed_swaps,
                                        (const int32_t *)w.handed_pos, nc));
         if (stats) {
-            // the objectives before and after (colabs_kernel, which gathers the permuted channels from W, took 47 us for each of the orders of a 4096 x 4096 weight)
-            const int rows = 2048;
-            ESP_CUDA_OK(cudaMemsetAsync(w.kept, 0, sizeof(unsigned long long) * C, stream));
-            ESP_CUDA_OK(cudaMemsetAsync(w.colsum, 0, sizeof(unsigned long long) * C, stream));       // (free by now)
-            lbs_kept_kernel<<<dim3(ceil_div(G, 8), ceil_div(No, rows), 2), 256, 0, stream>>>(w.wt, w.ldt, No, G, rows, w.score, w.theta0, perm, w.kept, w.colsum);
-            group_values_kernel<<<ceil_div(G, 256), 256, 0, stream>>>(w.kept, w.score, w.theta0, G, w.base[0]);
-            group_values_kernel<<<ceil_div(G, 256), 256, 0, stream>>>(w.colsum, w.score, perm, G, w.base[1]);
+            // the objectives before and after (colabs_kernel, which gathers the permuted channels from W, took 47 us for each of the orders of a 4096 x 4096 weight);
+            // a warp's lanes take eight rows each
+            lbs_value_kernel<<<dim3(G, 2), 32 * std::min(kValueThreads / 32, ceil_div(No, 256)), 0, stream>>>(w.wt, w.ldt, No, w.score, w.theta0, perm, w.base[0],
+                                                                                                              w.base[1]);
             objective_kernel<<<3, 256, 0, stream>>>(G, w.base[0], w.base[1], w.base[2], w.objective);
         }
     } else if (stats) {

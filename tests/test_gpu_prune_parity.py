@@ -211,6 +211,17 @@ def test_block_shuffle_handed_to_the_exact_kernels(kind, cap):
     assert g.stats.obj_after_lbs == orc.objective(W, s, theta)
 
 
+@pytest.mark.parametrize("No", [1, 255, 256, 257, 2048, 2049])
+def test_objectives_at_the_edges_of_a_warps_rows(No):
+    """Group values of both orders: a warp's lanes take 256 rows at a time, a CTA has up to eight warps (2048 rows)."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8700 + No)
+    W = (g0.standard_normal((No, 40)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(40)
+    ref = orc.metric_prune(W, None, 1.0, score=s, lbs_block=16, lbs_max_swaps=2)
+    assert_identical_to_oracle(GpuPrune(W, None, 1.0, score=s, lbs_block=16, lbs_max_swaps=2), ref)
+
+
 def test_llama7b_q_projection_full_size_block_shuffle():
     """Workload 1's q projection whole (4096 x 4096, 16 shuffle blocks, Student-t rows): global shuffle, block shuffle
     capped at 4 swaps per block on both sides (the oracle's table alone is 4.3e9 row evaluations), selection and
