@@ -56,6 +56,7 @@ struct PruneWorkspace {
     double *table;                                           // [nblocks][64][4][256]
     int *handed, *handed_swaps;                              // [nblocks] the exact kernels (re)start this block; swaps it has had
     int *widest;                                             // [nblocks] bits of the block's largest |W|
+    uint8_t *live;                                           // [nblocks][stride] the channel's column holds anything but zeros
     int32_t *handed_pos;                                     // [C] the order it is in: position -> channel of the block
     long ldt;                                                // No rounded up to 8
     int stride;                                              // lbs_block rounded up to 8

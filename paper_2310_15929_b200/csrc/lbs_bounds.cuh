@@ -23,8 +23,8 @@
 // per chunk, six over the warps; both five over the CTAs.  The packing and the exact kernels' own roundings add less than 2^-50 of the group's value, and with
 // products of at most 1 that is at most twice the number of rows.
 //
-// Two channels of score zero (dead inputs) exchange for nothing: exactly 0 on both sides, so such entries carry no bound; otherwise dozens of them would stay in question to
-// the end.
+// Two channels whose products are all zero (score zero: dead inputs; column zero: pruned before) exchange for nothing: exactly 0 on both sides, so such entries carry no bound;
+// otherwise dozens of them would stay in question to the end.  Columns of zeros count as scores of zero, which changes no product.
 //
 // What bounds it: on long slices instruction issue -- a row costs a warp 48 fma, 48 additions, 8 conversions and some 30 others for both groups (256
 // candidates, 6 slots), about 20 ns of an SM's time where the exact kernels take 55 --, on short ones the latency of a swap (search, three cluster barriers,
@@ -187,16 +187,17 @@ struct BoundFeed {
     }
 };
 
-// Scores of a block scaled by a power of two so that its products |w| s come close to 1 and not beyond (`widest`: the bits of its largest |w|).  Then a barrier.
+// Scores of a block scaled by a power of two so that its products |w| s come close to 1 and not beyond (`widest`: the bits of its largest |w|), zero for
+// channels without a live weight.  Then a barrier.
 __device__ __forceinline__ void bound_load_scores(const double *__restrict__ score, const int32_t *__restrict__ theta0, int p0, int m, int widest,
-                                                  double *s64, float *s32, int *top) {
+                                                  const uint8_t *__restrict__ live, double *s64, float *s32, int *top) {
     if (threadIdx.x == 0) *top = -100000;
     __syncthreads();
     for (int x = threadIdx.x; x < m; x += blockDim.x) atomicMax(top, ilogb(score[theta0[p0 + x]]));
     __syncthreads();
     const int e = *top + 2 + (widest ? ilogbf(__half2float(__ushort_as_half((unsigned short)widest))) : 0);
     for (int x = threadIdx.x; x < kLbsMax; x += blockDim.x) {
-        const double s = x < m ? scalbn(score[theta0[p0 + x]], -e) : 0.0;
+        const double s = x < m && live[x] ? scalbn(score[theta0[p0 + x]], -e) : 0.0;
         s64[x] = s;
         s32[x] = (float)s;
     }
@@ -218,7 +219,7 @@ __global__ void __launch_bounds__(kBoundTableThreads, 2) lbs_bound_table_kernel(
                                                                                 int No, int stride, const double *__restrict__ score,
                                                                                 const int32_t *__restrict__ theta0, int C, int lbs_block,
                                                                                 const int *__restrict__ handed, const int *__restrict__ widest,
-                                                                                double *__restrict__ table) {
+                                                                                const uint8_t *__restrict__ live, double *__restrict__ table) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsBoundTableSmem &S = *reinterpret_cast<LbsBoundTableSmem *>(s_dyn);
     const int b = blockIdx.y, p0 = b * lbs_block, m = min(lbs_block, C - p0), q0 = blockIdx.x * 8;
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(kBoundTableThreads, 2) lbs_bound_table_kernel(
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, x0 = lane * 8;
     BoundFeed feed;
     feed.step = (uint32_t)(kBoundTableWarps * stride);
-    bound_load_scores(score, theta0, p0, m, widest[b], S.s64, S.s32, &S.top);
+    bound_load_scores(score, theta0, p0, m, widest[b], live + (size_t)b * stride, S.s64, S.s32, &S.top);
     BoundSums<8> sums;
 #pragma unroll
     for (int e = 0; e < 8; ++e) sums.s[e] = S.s32[x0 + e];
@@ -533,7 +534,7 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
                                                                             int stride, const double *__restrict__ score,
                                                                             const int32_t *__restrict__ theta0, int C, int lbs_block, int max_swaps,
                                                                             double *__restrict__ table, int32_t *__restrict__ theta, unsigned long long *__restrict__ counters,
-                                                                            const int *__restrict__ widest, int *__restrict__ handed, int *__restrict__ handed_swaps,
+                                                                            const int *__restrict__ widest, const uint8_t *__restrict__ live, int *__restrict__ handed, int *__restrict__ handed_swaps,
                                                                             int32_t *__restrict__ handed_pos, int nc) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsBoundSmem &S = *reinterpret_cast<LbsBoundSmem *>(s_dyn);
@@ -550,7 +551,7 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
         S.chan[x] = theta0[p0 + x];
         S.own_row[x] = x % nc == rank ? (uint8_t)(x / nc) : (uint8_t)255;
     }
-    bound_load_scores(score, theta0, p0, m, widest[b], S.s64, S.s32, &S.top);           // (ends with a barrier: everything above is visible)
+    bound_load_scores(score, theta0, p0, m, widest[b], live + (size_t)b * stride, S.s64, S.s32, &S.top);           // (ends with a barrier: everything above is visible)
     for (int x = tid; x < m; x += kBoundThreads) S.split[x] = bound_split(S.s64[x]);          // (visible after the barrier below)
     const int per_cta = ((No + nc - 1) / nc + 7) & ~7, row0 = min(No, rank * per_cta), nrows_all = min(No, row0 + per_cta) - row0;
     const int add_r = min(kBoundFold, per_cta / kBoundWarps + 1) + per_cta / (kBoundWarps * kBoundFold) + 2 + 4 + 5;

@@ -613,11 +613,12 @@ __device__ __forceinline__ void lbs_sort(float (&v)[8]) {
 
 // Wb[b][row][x] = |W[row, channel x of block b]| bits, `stride` (lbs_block rounded up to 8) per row, zeros beyond the block: one
 // pass over W, permuted through shared memory, so that everything below reads whole contiguous rows.  A warp per (row, block).
-// widest[b] becomes the bits of the block's largest magnitude; handed[b] is set where the bounds of lbs_bounds.cuh do not hold: a weight that is not finite, a score that is neither zero nor an ordinary positive number,
-// scores more than 2^60 apart.
+// widest[b] becomes the bits of the block's largest magnitude, live[b][x] is set where the column of channel x holds anything but zeros; handed[b] is set where the bounds of
+// lbs_bounds.cuh do not hold: a weight that is not finite, a score that is neither zero nor an ordinary positive number, scores more than 2^60 apart.
 __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restrict__ W, int No, int C, long ldw, const double *__restrict__ score,
                                                          const int32_t *__restrict__ theta0, int lbs_block, int stride, int nblocks,
-                                                         int rows_per_cta, uint16_t *__restrict__ Wb, int *__restrict__ handed, int *__restrict__ widest) {
+                                                         int rows_per_cta, uint16_t *__restrict__ Wb, int *__restrict__ handed, int *__restrict__ widest,
+                                                         uint8_t *__restrict__ live) {
     extern __shared__ __align__(16) uint16_t s_rows[];            // [rows_per_cta][C]
     const int j0 = blockIdx.x * rows_per_cta;
     const int nrows = min(rows_per_cta, No - j0);
@@ -648,17 +649,30 @@ __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restric
         top = __reduce_max_sync(0xFFFFFFFFu, top);                // (all lanes, whatever they have found)
         low = __reduce_min_sync(0xFFFFFFFFu, low);
         bad = bad || top - low > 60;
-        uint32_t wide = 0;
+        uint16_t most[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         for (int r = 0; r < nrows; ++r) {
             uint16_t h[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 h[e] = ch[e] >= 0 ? s_rows[(size_t)r * C + ch[e]] : (uint16_t)0;
-                wide = max(wide, (uint32_t)h[e]);
+                most[e] = max(most[e], h[e]);
             }
             if (x0 < stride)
                 *reinterpret_cast<uint4 *>(Wb + ((size_t)b * No + j0 + r) * stride + x0) =
                     make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16), h[4] | ((uint32_t)h[5] << 16), h[6] | ((uint32_t)h[7] << 16));
+        }
+        uint32_t wide = 0, on[2] = {0, 0};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            wide = max(wide, (uint32_t)most[e]);
+            on[e >> 2] |= (most[e] ? 1u : 0u) << (8 * (e & 3));
+        }
+        uint2 *live_at = reinterpret_cast<uint2 *>(live + (size_t)b * stride + x0);
+        if (on[0] == 0x01010101u && on[1] == 0x01010101u) *live_at = make_uint2(on[0], on[1]);      // (every CTA that writes a byte writes a one)
+        else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (most[e]) reinterpret_cast<uint8_t *>(live_at)[e] = 1;
         }
         wide = __reduce_max_sync(0xFFFFFFFFu, wide);
         if (lane == 0) atomicMax(&widest[b], (int)wide);

@@ -919,6 +919,8 @@ PruneWorkspace carve_prune_workspace(void *ws, int No, int C, int T, const esp_p
     w.colsum = (unsigned long long *)take(sizeof(unsigned long long) * C);
     w.kept = (unsigned long long *)take(sizeof(unsigned long long) * C);
     if (o.use_lbs) {
+        w.stride = (int)align_up((size_t)o.lbs_block, 8);
+        w.live = (uint8_t *)take((size_t)ceil_div(C, o.lbs_block) * w.stride);
         w.handed = (int *)take(sizeof(int) * (size_t)ceil_div(C, o.lbs_block));
         w.handed_swaps = (int *)take(sizeof(int) * (size_t)ceil_div(C, o.lbs_block));
         w.widest = (int *)take(sizeof(int) * (size_t)ceil_div(C, o.lbs_block));
@@ -931,7 +933,6 @@ PruneWorkspace carve_prune_workspace(void *ws, int No, int C, int T, const esp_p
     if (o.use_lbs) {
         const int nblocks = ceil_div(C, o.lbs_block);
         w.ldt = (long)align_up((size_t)No, 8);
-        w.stride = (int)align_up((size_t)o.lbs_block, 8);
         w.wt = (uint16_t *)take(sizeof(uint16_t) * (size_t)C * w.ldt);
         w.wb = (uint16_t *)take(sizeof(uint16_t) * ((size_t)nblocks * No + kBoundOver) * w.stride);
         w.irregular = (uint8_t *)take((size_t)nblocks * No);
@@ -1056,12 +1057,12 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
         gather_rows = std::max(1, std::min(gather_rows, No / (2 * std::max(1, di.sm_count))));
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_gather_kernel, (int)(row_bytes * gather_rows)));
         lbs_gather_kernel<<<ceil_div(No, gather_rows), 256, row_bytes * gather_rows, stream>>>(W, No, C, ldw, w.score, w.theta0, o.lbs_block, w.stride, nblocks,
-                                                                                               gather_rows, w.wb, w.handed, w.widest);
+                                                                                               gather_rows, w.wb, w.handed, w.widest, w.live);
         lbs_transpose_kernel<<<dim3(ceil_div(C, 64), ceil_div(No, 64)), 256, 0, stream>>>(W, No, C, ldw, w.wt, w.ldt);
         // the swaps by bounds
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_table_kernel, (int)sizeof(LbsBoundTableSmem)));
         lbs_bound_table_kernel<<<dim3(ceil_div(o.lbs_block, 8), nblocks), kBoundTableThreads, sizeof(LbsBoundTableSmem), stream>>>(
-            w.wb, w.wt, w.ldt, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.widest, w.table);
+            w.wb, w.wt, w.ldt, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.widest, w.live, w.table);
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_greedy_kernel, (int)lbs_bound_smem(kBoundMinCluster)));
@@ -1069,7 +1070,8 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
         int nc = lbs_cluster_size(lbs_bound_greedy_kernel, lbs_bound_config, kBoundMinCluster, 10.0, 0.022, nblocks, No, di.device);
         lbs_bound_config(cfg, attr, nblocks, nc, stream);
         ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_bound_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, No, w.stride,
-                                       (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters, (const int *)w.widest, w.handed, w.handed_swaps, w.handed_pos, nc));
+                                       (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters,
+                                       (const int *)w.widest, (const uint8_t *)w.live, w.handed, w.handed_swaps, w.handed_pos, nc));
         // the exact kernels, on the blocks that were handed to them (without any, 8 us)
         auto mark = o.lbs_block <= 8 ? lbs_mark_kernel<8> : o.lbs_block <= 32 ? lbs_mark_kernel<32> : lbs_mark_kernel<kLbsMax>;
         mark<<<dim3(ceil_div(No, 64), nblocks), 256, 0, stream>>>(w.wb, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.irregular);

@@ -18,6 +18,7 @@ class GpuPrune:
         o.alpha = alpha
         for k, v in opts.items():
             setattr(o, k, v)
+        self.lbs_block = o.lbs_block
         self.Wd = torch.from_numpy(np.ascontiguousarray(W)).to(dev)
         self.Xd = None if Xcal is None else torch.from_numpy(np.ascontiguousarray(Xcal)).to(dev)
         T = 0 if Xcal is None else Xcal.shape[0]
@@ -47,6 +48,14 @@ class GpuPrune:
 
     def host(self):
         return (self.vals.cpu().numpy(), self.meta.cpu().numpy(), self.perm.cpu().numpy())
+
+    def handed(self):
+        """Per shuffle block, from the workspace: whether the exact kernels took it, and the swaps it had had by then."""
+        blocks, stride = -(-self.C // self.lbs_block), -(-self.lbs_block // 8) * 8
+        up = lambda n: -(-n // 256) * 256
+        at = 7 * up(8 * self.C) + up(64) + up(32) + up(blocks * stride)
+        words = [self.ws[a: a + 4 * blocks].view(torch.int32).tolist() for a in (at, at + up(4 * blocks))]
+        return words[0], words[1]
 
 
 def pack_on_gpu(vals, meta):

@@ -211,6 +211,22 @@ def test_block_shuffle_handed_to_the_exact_kernels(kind, cap):
     assert g.stats.obj_after_lbs == orc.objective(W, s, theta)
 
 
+@pytest.mark.parametrize("block", [12, 64, 256])
+@pytest.mark.parametrize("every", [1, 4, 10])
+def test_block_shuffle_zero_columns_are_decided_by_bounds(every, block):
+    """Columns of zeros (a weight that was pruned before) exchange for exactly nothing: no block needs the exact kernels for them.
+    (Every second one would: groups that keep both of their other channels in every row tie with each other.)"""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8650 + every)
+    W = (g0.standard_normal((150, 264)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(264)
+    W[:, ::every] = 0.0
+    ref = orc.metric_prune(W, None, 1.0, score=s, lbs_block=block)
+    g = GpuPrune(W, None, 1.0, score=s, lbs_block=block)
+    assert_identical_to_oracle(g, ref)
+    assert not any(g.handed()[0])
+
+
 @pytest.mark.parametrize("No", [1, 255, 256, 257, 2048, 2049])
 def test_objectives_at_the_edges_of_a_warps_rows(No):
     """Group values of both orders: a warp's lanes take 256 rows at a time, a CTA has up to eight warps (2048 rows)."""
