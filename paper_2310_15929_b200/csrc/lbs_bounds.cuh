@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(kValueThreads) lbs_value_kernel(const uint16_t
 
 // The exact choice among the pairs whose u reaches `reach` (all threads of all CTAs, three barriers of the cluster): 1 with the pair and whether it is nearly tied, 0 if it
 // gains nothing, -1 if there are too many.
-__device__ __noinline__ int bound_settle(LbsBoundSmem &S, float reach, int my_pairs, int my_rows, int m, int rank, int nc, const uint16_t *__restrict__ Wt,
+__device__ __noinline__ int bound_settle(LbsBoundSmem &S, float reach, int my_rows, int m, int rank, int nc, const uint16_t *__restrict__ Wt,
                                          long ldt, int nrows, int &pair, bool &near_tie) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) S.found = 0;
@@ -460,7 +460,7 @@ __device__ __noinline__ int bound_settle(LbsBoundSmem &S, float reach, int my_pa
         const float2 *gr = S.gains + lbs_gain_offset(r, m, rank, nc);
         for (int j = i + 1 + lane; j < m; j += 32) {
             const float2 g = gr[j - i - 1];
-            if (g.y >= reach && g.y > -INFINITY) {
+            if (g.y >= reach && g.y > 0.f) {                      // (a pair that cannot gain is neither the best nor nearly tied with one that does)
                 const int at = atomicAdd(&S.found, 1);
                 if (at < kBoundCand)
                     for (int c = 0; c < nc; ++c) st_remote_s32(map_to_rank(smem_u32(&S.list[rank][at]), (uint32_t)c), i * kLbsMax + j);
@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
         else {                                                    // a near tie (1e-6) or closer than the bounds
             bool near_tie = false;
             const float reach = __fsub_rd(best.l, __fmul_ru(2e-6f, fmaxf(best.u, best.rest)));
-            const int found = bound_settle(S, reach, my_pairs, my_rows, m, rank, nc, wt_rows, ldt, nrows_all, pair, near_tie);
+            const int found = bound_settle(S, reach, my_rows, m, rank, nc, wt_rows, ldt, nrows_all, pair, near_tie);
             hand_over = found < 0;
             if (found <= 0) break;
             near_swaps += near_tie ? 1 : 0;                       // counted, not acted on

@@ -227,6 +227,23 @@ def test_block_shuffle_zero_columns_are_decided_by_bounds(every, block):
     assert not any(g.handed()[0])
 
 
+def test_block_shuffle_settles_only_pairs_that_may_gain():
+    """Nine channels of score zero in nine groups (36 pairs that exchange for exactly nothing) and two equal channels, whose exchange
+    bounds cannot tell from a gain: the last question is about one pair, and is settled without the exact kernels."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8660)
+    W = (g0.standard_normal((150, 64)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(64)
+    s[0:36:4] = 0.0
+    W[:, 41], s[41] = W[:, 50], s[50]
+    perm = np.arange(64, dtype=np.int32)
+    theta, info = orc.local_block_shuffle(W, s, perm, 64)
+    g = GpuPrune(W, None, 1.0, score=s, perm=perm, lbs_block=64)
+    assert np.array_equal(g.host()[2], theta)
+    assert g.stats.lbs_swaps_total == info.swaps_total and g.stats.near_tie_swaps == info.near_tie_swaps
+    assert g.handed()[0] == [0]
+
+
 @pytest.mark.parametrize("No", [1, 255, 256, 257, 2048, 2049])
 def test_objectives_at_the_edges_of_a_warps_rows(No):
     """Group values of both orders: a warp's lanes take 256 rows at a time, a CTA has up to eight warps (2048 rows)."""
