@@ -6,22 +6,27 @@
 // f1 + max(f2, x).  So what the group gains by it is
 //     G(g, k <- x) = R - D_k,     R = sum over rows of max(0, |w_x| s_x - f2),     D_k = sum over rows of max(0, |w_k| s_k - p3),
 // and a pair gains the sum of its two entries.  R costs ONE saturating fp32 fma and one addition per (row, candidate, slot): products are
-// scaled to at most 1, so that the clamp at 0 is the fma's own, and the clamp at 1 never acts.  No ranks, no sort, no branch, no case for products
-// that fp32 cannot tell apart: the sums are continuous where they cross.
+// scaled to at most 1/2 in magnitude, so that the clamp at 0 is the fma's own, and the clamp at 1 never acts.  No ranks, no sort, no branch, no case for
+// products that fp32 cannot tell apart: the sums are continuous where they cross.  Nothing here asks for scores of one sign.
 //
-// An entry G carries a bound E on its distance from the exact gain (the exact kernels' fp64 roundings, some 2^-50 of a group's value, included), and a pair's gain is
+// An entry G carries a bound E on its distance from the exact kernels' gain (their fp64 roundings included), and a pair's gain is
 // kept as the interval [l, u] in directed rounding.  If the pair with the largest l leaves every other pair's u behind by more than the
 // near-tie distance, it is the exact kernels' choice; if no u is positive, the block is done.  Otherwise (three swaps in a hundred on a LLaMA-7B-shaped
 // projection, with two pairs in question) the pairs that may be the best or nearly tied with it are evaluated exactly, from integer sums.  More of them than
 // kBoundCand (ties by the dozen: equal columns, scores that leave nothing to choose) and the block is handed to the exact kernels as it stands; so are, from the
-// start, blocks with weights that are not finite or with scores that are not ordinary positive numbers of similar size (or zero).
+// start, blocks with weights that are not finite or with scores beyond 2^+-300 or 2^200 apart (fp64 products of scaled scores are then no longer the scaled
+// products).
 //
-// E, in units of 2^-24: a product that stays is rounded once (bound_split), a candidate's takes the rounding of its score; the fma rounds once.  A clamped term of R, d = x - f2 > 0,
-// is off by at most x + f2 + d = 2 d + 2 f2 (2 f2 where only the computed value is positive), one of D_k by 2 d + 2 p3.  Together 2 R + 2 D + 4 S with S the sum over rows of
-// p2.  An addition rounds by at most one unit of the partial sum, so R takes one unit per
-// addition on its way: up to kBoundFold in a register, one per fold in shared memory, four in the tree over the warps; D one per row of a thread, five in a warp, one
-// per chunk, six over the warps; both five over the CTAs.  The packing and the exact kernels' own roundings add less than 2^-50 of the group's value, and with
-// products of at most 1 that is at most twice the number of rows.
+// E, in units of 2^-24.  A product that stays is rounded once (bound_split), a candidate's takes the rounding of its score; the fma rounds once.  Rounding
+// preserves order, so the computed p2 and p3 are within one unit of theirs.  A clamped term of R, d = x - f2 > 0, is off by at most
+// |x| + |f2| + d <= 2 d + 2 |f2| (2 |f2| where only the computed value is positive), one of D_k by 2 d + 2 |p3|.  Together 2 R + 2 D + 4 S with S the sum over
+// rows of max(|p2|, |p3|) = max(p2, -p3).  An addition rounds by at most one unit of the partial sum, so R takes one unit per addition on its way (add_r): up to
+// kBoundFold in a register, one per fold in shared memory, four in the tree over the warps; D (add_d) one per row of a thread, five in a warp, one per chunk, five
+// over the warps; both five over the CTAs.  bound_of takes one unit more of R and two of D than that, and 1/85 of the whole: there second-order terms find room,
+// and the 16 bits of mantissa that an entry gives up (bound_pack), 2^-36 of |R - D| = 2^-12 units of it.  (bound_shift makes room for them once more: E is at
+// least five units of the entry, 2^-9 of it 2^-31.)  The last term, rows * 2^-49, is for the exact kernels' roundings: a group's value is at most the number of
+// rows (two products of 1/2 in each), five roundings of 2^-53 in each of the four values of a gain and three in adding them make less than 26 * 2^-53 rows a
+// pair; two entries have 32.  What is left of it (2^-51 rows a pair) is more than the underflow of products down to 2^-200 in fp32, 2^-132 a row, adds.
 //
 // Two channels whose products are all zero (score zero: dead inputs; column zero: pruned before) exchange for nothing: exactly 0 on both sides, so such entries carry no bound;
 // otherwise dozens of them would stay in question to the end.  Columns of zeros count as scores of zero, which changes no product.
@@ -46,7 +51,7 @@ __device__ __forceinline__ double bound_error(double p) { return (double)__uint_
 // The bound of an entry R - D: additions on the way of R and of D, S (above), output rows.
 __device__ __forceinline__ float bound_of(float R, int add_r, float D, int add_d, float S, int No) {
     const float units = __fadd_ru(__fadd_ru(__fmul_ru((float)(add_r + 3), R), __fmul_ru((float)(add_d + 4), D)), __fmul_ru(4.f, S));
-    return __fmaf_ru(0x1.03p-24f, units, (float)No * 0x1p-48f);
+    return __fmaf_ru(0x1.03p-24f, units, (float)No * 0x1p-49f);
 }
 // [l, u] of the gain of exchanging the channels behind two table entries.
 __device__ __forceinline__ float2 bound_gain(double there, double back) {
@@ -69,8 +74,8 @@ __device__ __forceinline__ float2 bound_split(double s) {
     const float hi = __uint_as_float(__float_as_uint((float)s) & 0xFFFFF000u);
     return make_float2(hi, (float)(s - (double)hi));
 }
-// Per row of a group: for each slot the threshold f2 its candidates have to pass (negated) and the row's term of D; p2.
-__device__ __forceinline__ void bound_row(const uint16_t (&h)[4], const float2 *s, float (&neg)[4], float (&D)[4], float &p2) {
+// Per row of a group: for each slot the threshold f2 its candidates have to pass (negated) and the row's term of D; the row's term of S.
+__device__ __forceinline__ void bound_row(const uint16_t (&h)[4], const float2 *s, float (&neg)[4], float (&D)[4], float &size) {
     float a[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {                                 // (rounded once)
@@ -78,8 +83,8 @@ __device__ __forceinline__ void bound_row(const uint16_t (&h)[4], const float2 *
         a[k] = __fmaf_rn(w, s[k].y, __fmul_rn(w, s[k].x));
     }
     const float h0 = fmaxf(a[0], a[1]), l0 = fminf(a[0], a[1]), h1 = fmaxf(a[2], a[3]), l1 = fminf(a[2], a[3]);
-    const float y = fminf(h0, h1), z = fmaxf(l0, l1), p3 = fminf(y, z);
-    p2 = fmaxf(y, z);
+    const float y = fminf(h0, h1), z = fmaxf(l0, l1), p3 = fminf(y, z), p2 = fmaxf(y, z);
+    size = fmaxf(p2, -p3);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         neg[k] = a[k] >= p2 ? -p3 : -p2;
@@ -187,7 +192,7 @@ struct BoundFeed {
     }
 };
 
-// Scores of a block scaled by a power of two so that its products |w| s come close to 1 and not beyond (`widest`: the bits of its largest |w|), zero for
+// Scores of a block scaled by a power of two so that its products |w| s come close to 1/2 and not beyond (`widest`: the bits of its largest |w|), zero for
 // channels without a live weight.  Then a barrier.
 __device__ __forceinline__ void bound_load_scores(const double *__restrict__ score, const int32_t *__restrict__ theta0, int p0, int m, int widest,
                                                   const uint8_t *__restrict__ live, double *s64, float *s32, int *top) {
@@ -195,7 +200,7 @@ __device__ __forceinline__ void bound_load_scores(const double *__restrict__ sco
     __syncthreads();
     for (int x = threadIdx.x; x < m; x += blockDim.x) atomicMax(top, ilogb(score[theta0[p0 + x]]));
     __syncthreads();
-    const int e = *top + 2 + (widest ? ilogbf(__half2float(__ushort_as_half((unsigned short)widest))) : 0);
+    const int e = *top + 3 + (widest ? ilogbf(__half2float(__ushort_as_half((unsigned short)widest))) : 0);
     for (int x = threadIdx.x; x < kLbsMax; x += blockDim.x) {
         const double s = x < m && live[x] ? scalbn(score[theta0[p0 + x]], -e) : 0.0;
         s64[x] = s;
@@ -654,10 +659,10 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
                     const uint16_t hg[4] = {h[u][4 * g], h[u][4 * g + 1], h[u][4 * g + 2], h[u][4 * g + 3]};
-                    float t[4], D[4], p2;
+                    float t[4], D[4], size;
                     const int skip = g ? skip_b : skip_a;
-                    bound_row(hg, S.grp_s + 4 * g, t, D, p2);     // (a row beyond the slice has zeros everywhere)
-                    total[6 + g] += p2;
+                    bound_row(hg, S.grp_s + 4 * g, t, D, size);   // (a row beyond the slice has zeros everywhere)
+                    total[6 + g] += size;
 #pragma unroll
                     for (int l = 0; l < 3; ++l) {
                         neg[3 * g + l] = l >= skip ? t[l + 1] : t[l];

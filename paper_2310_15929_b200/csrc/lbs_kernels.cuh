@@ -614,7 +614,7 @@ __device__ __forceinline__ void lbs_sort(float (&v)[8]) {
 // Wb[b][row][x] = |W[row, channel x of block b]| bits, `stride` (lbs_block rounded up to 8) per row, zeros beyond the block: one
 // pass over W, permuted through shared memory, so that everything below reads whole contiguous rows.  A warp per (row, block).
 // widest[b] becomes the bits of the block's largest magnitude, live[b][x] is set where the column of channel x holds anything but zeros; handed[b] is set where the bounds of
-// lbs_bounds.cuh do not hold: a weight that is not finite, a score that is neither zero nor an ordinary positive number, scores more than 2^60 apart.
+// lbs_bounds.cuh do not hold: a weight that is not finite, a score that is neither zero nor of ordinary magnitude, scores more than 2^200 apart.
 __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restrict__ W, int No, int C, long ldw, const double *__restrict__ score,
                                                          const int32_t *__restrict__ theta0, int lbs_block, int stride, int nblocks,
                                                          int rows_per_cta, uint16_t *__restrict__ Wb, int *__restrict__ handed, int *__restrict__ widest,
@@ -641,14 +641,14 @@ __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restric
             ch[e] = x0 + e < m ? theta0[p0 + x0 + e] : -1;
             if (ch[e] >= 0) {
                 const double s = score[ch[e]];
-                const bool ordinary = s >= 0x1p-80 && s <= 0x1p80;
+                const bool ordinary = fabs(s) >= 0x1p-300 && fabs(s) <= 0x1p300;
                 bad = bad || !(ordinary || s == 0.0);
                 if (ordinary) { top = max(top, ilogb(s)); low = min(low, ilogb(s)); }
             }
         }
         top = __reduce_max_sync(0xFFFFFFFFu, top);                // (all lanes, whatever they have found)
         low = __reduce_min_sync(0xFFFFFFFFu, low);
-        bad = bad || top - low > 60;
+        bad = bad || top - low > 200;
         uint16_t most[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         for (int r = 0; r < nrows; ++r) {
             uint16_t h[8];

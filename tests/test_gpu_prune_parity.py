@@ -181,11 +181,12 @@ def test_block_shuffle_bound_sums_at_the_edges_of_folds_and_chunks(No):
     assert ref.lbs.swaps_total == 6
 
 
-@pytest.mark.parametrize("kind", ["tied_from_the_start", "tied_later", "few_ties", "far_apart"])
+@pytest.mark.parametrize("kind", ["tied_from_the_start", "tied_later", "few_ties", "far_apart", "negative", "very_far_apart", "not_finite"])
 @pytest.mark.parametrize("cap", [0, 9])
 def test_block_shuffle_handed_to_the_exact_kernels(kind, cap):
-    """Blocks that bounds cannot decide: dozens of tied pairs at the first swap, or only once the wide channels have found their places; a
-    tie that is settled by itself (two equal channels); scores too far apart for bounds.  One block among others that need no help."""
+    """Blocks that bounds cannot decide: dozens of tied pairs at the first swap, or only once the wide channels have found their places; scores
+    too far apart, a weight that is not finite.  One block among others that need no help.  And what needs none: a tie that is settled by
+    itself (two equal channels), one score far below the others, a negative one."""
     from tests.gpu_util import GpuPrune
     g0 = np.random.default_rng(8600)
     No, C, block = 120, 264, 64
@@ -202,13 +203,19 @@ def test_block_shuffle_handed_to_the_exact_kernels(kind, cap):
         s[small] = 1.0
     elif kind == "few_ties":
         W[:, first[9]], s[first[9]] = W[:, first[40]], s[first[40]]
+    elif kind == "not_finite":
+        W[17, first[23]] = np.inf
     else:
-        s[first[7]] = 2.0 ** -70
+        s[first[7]] = {"far_apart": 2.0 ** -70, "negative": -3.0, "very_far_apart": 2.0 ** -220}[kind]
     theta, info = orc.local_block_shuffle(W, s, perm, block, cap)
     g = GpuPrune(W, None, 1.0, score=s, perm=perm, lbs_block=block, lbs_max_swaps=cap)
     assert np.array_equal(g.host()[2], theta)
     assert g.stats.lbs_swaps_total == info.swaps_total and g.stats.near_tie_swaps == info.near_tie_swaps
     assert g.stats.obj_after_lbs == orc.objective(W, s, theta)
+    handed, swaps = g.handed()
+    assert handed[1:] == [0, 0, 0, 0]
+    assert bool(handed[0]) == (kind not in ("few_ties", "far_apart", "negative") and not (kind == "tied_later" and cap))
+    assert (swaps[0] > 0) == (kind == "tied_later" and cap == 0)
 
 
 @pytest.mark.parametrize("block", [12, 64, 256])
