@@ -614,11 +614,12 @@ __device__ __forceinline__ void lbs_sort(float (&v)[8]) {
 // Wb[b][row][x] = |W[row, channel x of block b]| bits, `stride` (lbs_block rounded up to 8) per row, zeros beyond the block: one
 // pass over W, permuted through shared memory, so that everything below reads whole contiguous rows.  A warp per (row, block).
 // widest[b] becomes the bits of the block's largest magnitude, live[b][x] is set where the column of channel x holds anything but zeros; handed[b] is set where the bounds of
-// lbs_bounds.cuh do not hold: a weight that is not finite, a score that is neither zero nor of ordinary magnitude, scores more than 2^200 apart.
+// lbs_bounds.cuh do not hold: a weight that is not finite, a score that is neither zero nor of ordinary magnitude, scores more than 2^200 apart;
+// in all of them if `all` says so.
 __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restrict__ W, int No, int C, long ldw, const double *__restrict__ score,
                                                          const int32_t *__restrict__ theta0, int lbs_block, int stride, int nblocks,
                                                          int rows_per_cta, uint16_t *__restrict__ Wb, int *__restrict__ handed, int *__restrict__ widest,
-                                                         uint8_t *__restrict__ live) {
+                                                         uint8_t *__restrict__ live, bool all) {
     extern __shared__ __align__(16) uint16_t s_rows[];            // [rows_per_cta][C]
     const int j0 = blockIdx.x * rows_per_cta;
     const int nrows = min(rows_per_cta, No - j0);
@@ -676,7 +677,7 @@ __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restric
         }
         wide = __reduce_max_sync(0xFFFFFFFFu, wide);
         if (lane == 0) atomicMax(&widest[b], (int)wide);
-        if (bad || wide >= 0x7C00u) handed[b] = 1;
+        if (all || bad || wide >= 0x7C00u) handed[b] = 1;
     }
 }
 
@@ -753,7 +754,7 @@ __global__ void __launch_bounds__(256) lbs_transpose_kernel(const __half *__rest
     }
 }
 
-// table[b][g][slot][x] = V(group g of block b with its slot replaced by block channel x); base[G] = V(g).
+// table[b][g][slot][x] = V(group g of block b with its slot replaced by block channel x); base[G] = V(g).  handed_pos: null = the order theta0.
 // One CTA per (block, group of a full block), all rows in chunks.  Two CTAs per SM (128 registers), so that one's sort runs under the other's
 // candidates.
 constexpr int kTableRows = 1024, kTableThreads = 256;
@@ -784,7 +785,7 @@ __global__ void __launch_bounds__(kTableThreads, 2) lbs_table_kernel(const uint1
     if (tid < 32) S.rows.cnt[tid] = 0;
     lbs_load_scores(score, theta0, p0, m, S.s64, S.s32);
     if (tid < 4) {
-        const int x = handed_pos[p0 + g * 4 + tid];
+        const int x = handed_pos ? handed_pos[p0 + g * 4 + tid] : g * 4 + tid;
         S.grp.channel[tid] = theta0[p0 + x];
         S.grp.s[tid] = S.s64[x];
         S.grp.s32[tid] = S.s32[x];
@@ -923,7 +924,7 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
     };
     clear_sums();
     if (tid < 64) S.rows[tid >> 5].cnt[tid & 31] = 0;
-    for (int x = tid; x < m; x += kGreedyThreads) { S.pos2x[x] = handed_pos[p0 + x]; S.chan[x] = theta0[p0 + x]; }
+    for (int x = tid; x < m; x += kGreedyThreads) { S.pos2x[x] = handed_pos ? handed_pos[p0 + x] : x; S.chan[x] = theta0[p0 + x]; }
     for (int g = tid; g < G; g += kGreedyThreads) S.base[g] = base0[p0 / 4 + g];
     lbs_load_scores(score, theta0, p0, m, S.s64, S.s32);          // (ends with a barrier: everything above is visible)
     const int per_cta = (No + nc - 1) / nc, row0 = min(No, rank * per_cta), nrows_all = min(No, row0 + per_cta) - row0, chunk_rows = lbs_chunk_rows(nrows_all, kGreedyRows);

@@ -1052,40 +1052,45 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
     if (lbs) {
         const int nblocks = ceil_div(C, o.lbs_block);
         const size_t row_bytes = sizeof(uint16_t) * (size_t)C;
+        const bool few = No < 4;                                  // (see below)
         // rows per CTA: about 96 KB of shared memory (two CTAs per SM), and a grid of two CTAs per SM at least
         int gather_rows = (int)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / row_bytes));
         gather_rows = std::max(1, std::min(gather_rows, No / (2 * std::max(1, di.sm_count))));
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_gather_kernel, (int)(row_bytes * gather_rows)));
         lbs_gather_kernel<<<ceil_div(No, gather_rows), 256, row_bytes * gather_rows, stream>>>(W, No, C, ldw, w.score, w.theta0, o.lbs_block, w.stride, nblocks,
-                                                                                               gather_rows, w.wb, w.handed, w.widest, w.live);
+                                                                                               gather_rows, w.wb, w.handed, w.widest, w.live, few);
         lbs_transpose_kernel<<<dim3(ceil_div(C, 64), ceil_div(No, 64)), 256, 0, stream>>>(W, No, C, ldw, w.wt, w.ldt);
-        // the swaps by bounds
-        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_table_kernel, (int)sizeof(LbsBoundTableSmem)));
-        lbs_bound_table_kernel<<<dim3(ceil_div(o.lbs_block, 8), nblocks), kBoundTableThreads, sizeof(LbsBoundTableSmem), stream>>>(
-            w.wb, w.wt, w.ldt, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.widest, w.live, w.table);
+        // the swaps by bounds, but for one to three rows: their last question is about exchanges that move a kept product to another group, dozens of gains of rounding
+        // noise, so every block would end in the exact kernels all the same (256..4096 channels, by bounds and to the end / exactly from the start: 1 row 0.64 / 0.60 ms,
+        // 2 rows 1.28 / 1.04, 3 rows 1.39 / 1.18, 4 rows 1.43 / 1.43, 5 rows 1.39 / 1.55)
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
-        ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_greedy_kernel, (int)lbs_bound_smem(kBoundMinCluster)));
-        ESP_CUDA_OK(cudaFuncSetAttribute(lbs_bound_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        int nc = lbs_cluster_size(lbs_bound_greedy_kernel, lbs_bound_config, kBoundMinCluster, 10.0, 0.022, nblocks, No, di.device);
-        lbs_bound_config(cfg, attr, nblocks, nc, stream);
-        ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_bound_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, No, w.stride,
-                                       (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters,
-                                       (const int *)w.widest, (const uint8_t *)w.live, w.handed, w.handed_swaps, w.handed_pos, nc));
+        if (!few) {
+            ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_table_kernel, (int)sizeof(LbsBoundTableSmem)));
+            lbs_bound_table_kernel<<<dim3(ceil_div(o.lbs_block, 8), nblocks), kBoundTableThreads, sizeof(LbsBoundTableSmem), stream>>>(
+                w.wb, w.wt, w.ldt, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.widest, w.live, w.table);
+            ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_greedy_kernel, (int)lbs_bound_smem(kBoundMinCluster)));
+            ESP_CUDA_OK(cudaFuncSetAttribute(lbs_bound_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            const int nc = lbs_cluster_size(lbs_bound_greedy_kernel, lbs_bound_config, kBoundMinCluster, 10.0, 0.022, nblocks, No, di.device);
+            lbs_bound_config(cfg, attr, nblocks, nc, stream);
+            ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_bound_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, No, w.stride,
+                                           (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters,
+                                           (const int *)w.widest, (const uint8_t *)w.live, w.handed, w.handed_swaps, w.handed_pos, nc));
+        }
         // the exact kernels, on the blocks that were handed to them (without any, 8 us)
         auto mark = o.lbs_block <= 8 ? lbs_mark_kernel<8> : o.lbs_block <= 32 ? lbs_mark_kernel<32> : lbs_mark_kernel<kLbsMax>;
         mark<<<dim3(ceil_div(No, 64), nblocks), 256, 0, stream>>>(w.wb, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.irregular);
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_table_kernel, (int)sizeof(LbsTableSmem)));
         lbs_table_kernel<<<dim3(o.lbs_block / 4, nblocks), kTableThreads, sizeof(LbsTableSmem), stream>>>(
-            w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.handed_pos, w.table, w.base[1]);
+            w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, few ? nullptr : w.handed_pos, w.table, w.base[1]);
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_greedy_kernel, (int)lbs_greedy_smem(kGreedyMinCluster)));
         ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        nc = lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, 10.0, 0.055, nblocks, No, di.device);
+        const int nc = lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, 10.0, 0.055, nblocks, No, di.device);
         lbs_greedy_config(cfg, attr, nblocks, nc, stream);
         ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, (const uint8_t *)w.irregular, No,
                                        w.stride, (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table,
                                        (const double *)w.base[1], perm, w.counters, (const int *)w.handed, (const int *)w.handed_swaps,
-                                       (const int32_t *)w.handed_pos, nc));
+                                       (const int32_t *)(few ? nullptr : w.handed_pos), nc));
         if (stats) {
             // the objectives before and after (colabs_kernel, which gathers the permuted channels from W, took 47 us for each of the orders of a 4096 x 4096 weight);
             // a warp's lanes take eight rows each

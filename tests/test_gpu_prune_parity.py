@@ -218,6 +218,21 @@ def test_block_shuffle_handed_to_the_exact_kernels(kind, cap):
     assert (swaps[0] > 0) == (kind == "tied_later" and cap == 0)
 
 
+@pytest.mark.parametrize("No", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("block,equal", [(12, False), (256, False), (256, True)])
+def test_block_shuffle_few_rows(No, block, equal):
+    """One to three rows are shuffled by the exact kernels from the start, more by bounds first."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8640 + No)
+    W = (g0.standard_normal((No, 520)) * 0.02).astype(np.float16)
+    s = np.full(520, 2.5) if equal else 1.0 + 3.0 * g0.random(520)
+    g = GpuPrune(W, None, 1.0, score=s, lbs_block=block)
+    assert_identical_to_oracle(g, orc.metric_prune(W, None, 1.0, score=s, lbs_block=block))
+    handed, swaps = g.handed()
+    if No < 4:
+        assert all(handed) and not any(swaps)
+
+
 @pytest.mark.parametrize("block", [12, 64, 256])
 @pytest.mark.parametrize("every", [1, 4, 10])
 def test_block_shuffle_zero_columns_are_decided_by_bounds(every, block):
