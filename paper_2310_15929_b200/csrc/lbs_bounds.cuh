@@ -821,33 +821,38 @@ inline void lbs_bound_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr,
 // A swap costs `fixed` us of barriers, search and exchange and `per_row` us per output row of a CTA's slice: about 10 and 0.055 by the exact kernel,
 // 10 and 0.022 by bounds.
 template <typename Kernel, typename Config>
-inline int lbs_cluster_size(Kernel kernel, Config config, int smallest, double fixed, double per_row, int nblocks, int No, int device) {
+inline int lbs_cluster_capacity(Kernel kernel, Config config, int nc, int device) {
     static std::mutex mu;
     static std::map<std::pair<const void *, int>, int> cache;
+    std::lock_guard<std::mutex> lock(mu);
+    const std::pair<const void *, int> key((const void *)kernel, device * 64 + nc);
+    auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    int cap = 0;
+    config(cfg, attr, 1, nc, nullptr);
+    if (cudaOccupancyMaxActiveClusters(&cap, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); cap = 0; }
+    return cache[key] = cap;
+}
+struct LbsSwapCost {
+    double fixed, per_row;
+    double of(int nc, int capacity, int nblocks, int No) const {
+        const double w = (double)nblocks / capacity, whole = std::ceil(w), waves = w <= 2.0 ? whole : w + (whole - w) * (2.0 / w);
+        return waves * (fixed + per_row * (double)((No + nc - 1) / nc));
+    }
+};
+template <typename Kernel, typename Config>
+inline int lbs_cluster_size(Kernel kernel, Config config, int smallest, LbsSwapCost cost, int nblocks, int No, int device) {
     const int sizes[] = {16, 14, 12, 10, 9, 8, 7, 6, 5, 4, 3};
     int best = smallest;
     double best_cost = -1.0;
     for (int nc : sizes) {
-        if (nc < smallest) continue;
-        int cap = 0;
-        {
-            std::lock_guard<std::mutex> lock(mu);
-            const std::pair<const void *, int> key((const void *)kernel, device * 64 + nc);
-            auto it = cache.find(key);
-            if (it != cache.end()) cap = it->second;
-            else {
-                cudaLaunchConfig_t cfg;
-                cudaLaunchAttribute attr;
-                config(cfg, attr, 1, nc, nullptr);
-                if (cudaOccupancyMaxActiveClusters(&cap, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); cap = 0; }
-                cache[key] = cap;
-            }
-        }
+        const int cap = nc < smallest ? 0 : lbs_cluster_capacity(kernel, config, nc, device);
         if (cap <= 0) continue;
-        const double w = (double)nblocks / cap, whole = std::ceil(w), waves = w <= 2.0 ? whole : w + (whole - w) * (2.0 / w);
-        const double cost = waves * (fixed + per_row * (double)((No + nc - 1) / nc));
-        if (log_plans()) fprintf(stderr, "esparse block shuffle: blocks=%d rows=%d cluster=%d capacity=%d cost=%.1f\n", nblocks, No, nc, cap, cost);
-        if (best_cost < 0.0 || cost < best_cost) { best_cost = cost; best = nc; }
+        const double c = cost.of(nc, cap, nblocks, No);
+        if (log_plans()) fprintf(stderr, "esparse block shuffle: blocks=%d rows=%d cluster=%d capacity=%d cost=%.1f\n", nblocks, No, nc, cap, c);
+        if (best_cost < 0.0 || c < best_cost) { best_cost = c; best = nc; }
     }
     return best;
 }

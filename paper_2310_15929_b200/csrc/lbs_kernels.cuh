@@ -827,6 +827,7 @@ __global__ void __launch_bounds__(kTableThreads, 2) lbs_table_kernel(const uint1
 //     gains of 8 of the 256 positions, so about 2000 pairs are looked up again in the table (L2) and the search itself reads
 //     shared memory only.
 // Every CTA takes the same decision from the exchanged winners; all cluster barriers are reached by all threads.
+// Does nothing unless more than `from` and at most `to` blocks were handed over.
 constexpr int kGreedyRows = 1024, kGreedyThreads = 512, kGreedyMaxCluster = 16, kGreedyMinCluster = 3;
 constexpr int kLbsSwapLimit = 1 << 16;                            // far above any block's swaps; beyond it the kernel reports a timeout
 struct LbsGreedySmem {
@@ -908,7 +909,8 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
                                                                        int lbs_block, int max_swaps, double *__restrict__ table,
                                                                        const double *__restrict__ base0, int32_t *__restrict__ theta,
                                                                        unsigned long long *__restrict__ counters, const int *__restrict__ handed,
-                                                                       const int *__restrict__ handed_swaps, const int32_t *__restrict__ handed_pos, int nc) {
+                                                                       const int *__restrict__ handed_swaps, const int32_t *__restrict__ handed_pos, int nc,
+                                                                       int nblocks, int from, int to) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsGreedySmem &S = *reinterpret_cast<LbsGreedySmem *>(s_dyn);
     using Cells = LbsCells<3>;
@@ -917,6 +919,17 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr int kWarps = kGreedyThreads / 32;
     if (!handed[b]) return;
+    if (from > 0 || to < nblocks) {                               // (all CTAs find the same)
+        int *number = reinterpret_cast<int *>(s_dyn), n = 0;
+        if (tid == 0) *number = 0;
+        __syncthreads();
+        for (int i = tid; i < nblocks; i += kGreedyThreads) n += handed[i] ? 1 : 0;
+        if (n) atomicAdd(number, n);
+        __syncthreads();
+        n = *number;
+        __syncthreads();                                          // (the place is used for other things from here on)
+        if (n <= from || n > to) return;
+    }
     double *tb = table + (long)b * kLbsGroups * 4 * kLbsMax;      // row of position i: group i / 4, slot i % 4
     auto clear_sums = [&]() {
         for (int i = tid; i < (int)(sizeof(S.cells) / 16); i += kGreedyThreads) reinterpret_cast<uint4 *>(S.cells)[i] = make_uint4(0u, 0u, 0u, 0u);

@@ -1071,7 +1071,7 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
                 w.wb, w.wt, w.ldt, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.widest, w.live, w.table);
             ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_bound_greedy_kernel, (int)lbs_bound_smem(kBoundMinCluster)));
             ESP_CUDA_OK(cudaFuncSetAttribute(lbs_bound_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            const int nc = lbs_cluster_size(lbs_bound_greedy_kernel, lbs_bound_config, kBoundMinCluster, 10.0, 0.022, nblocks, No, di.device);
+            const int nc = lbs_cluster_size(lbs_bound_greedy_kernel, lbs_bound_config, kBoundMinCluster, {10.0, 0.022}, nblocks, No, di.device);
             lbs_bound_config(cfg, attr, nblocks, nc, stream);
             ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_bound_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, No, w.stride,
                                            (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters,
@@ -1085,12 +1085,24 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
             w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, few ? nullptr : w.handed_pos, w.table, w.base[1]);
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_greedy_kernel, (int)lbs_greedy_smem(kGreedyMinCluster)));
         ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        const int nc = lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, 10.0, 0.055, nblocks, No, di.device);
-        lbs_greedy_config(cfg, attr, nblocks, nc, stream);
-        ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, (const uint8_t *)w.irregular, No,
-                                       w.stride, (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table,
-                                       (const double *)w.base[1], perm, w.counters, (const int *)w.handed, (const int *)w.handed_swaps,
-                                       (const int32_t *)(few ? nullptr : w.handed_pos), nc));
+        // How many blocks there is work in is not known here: none as a rule, one now and then, all of a weight made of ties.  Up to as many as large clusters serve sooner
+        // they are launched in those, beyond that in the size for all blocks; the other launch's clusters leave at once (2 us).  One block of the 16 of 4096 x 4096 (a weight that
+        // is not finite) 11.5 -> 8.6 ms for the whole call, 9.3 by the exact kernels alone; all sixteen handed over before their first swap 3.72 ms as before (4.5 in large clusters).
+        const LbsSwapCost cost{10.0, 0.055};
+        const int sizes[2] = {lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, cost, few ? nblocks : 1, No, di.device),
+                              lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, cost, nblocks, No, di.device)};
+        const int caps[2] = {lbs_cluster_capacity(lbs_greedy_kernel, lbs_greedy_config, sizes[0], di.device),
+                             lbs_cluster_capacity(lbs_greedy_kernel, lbs_greedy_config, sizes[1], di.device)};
+        if (caps[0] <= 0 || caps[1] <= 0) return ESP_ERR_CUDA;
+        int most = sizes[0] == sizes[1] ? nblocks : 1;
+        while (most < nblocks && cost.of(sizes[0], caps[0], most + 1, No) <= cost.of(sizes[1], caps[1], most + 1, No)) ++most;
+        for (int all = 0; all < (most < nblocks ? 2 : 1); ++all) {
+            lbs_greedy_config(cfg, attr, nblocks, sizes[all], stream);
+            ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, (const uint8_t *)w.irregular, No,
+                                           w.stride, (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table,
+                                           (const double *)w.base[1], perm, w.counters, (const int *)w.handed, (const int *)w.handed_swaps,
+                                           (const int32_t *)(few ? nullptr : w.handed_pos), sizes[all], nblocks, all ? most : 0, all ? nblocks : most));
+        }
         if (stats) {
             // the objectives before and after (colabs_kernel, which gathers the permuted channels from W, took 47 us for each of the orders of a 4096 x 4096 weight);
             // a warp's lanes take eight rows each

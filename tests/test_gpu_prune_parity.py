@@ -218,6 +218,24 @@ def test_block_shuffle_handed_to_the_exact_kernels(kind, cap):
     assert (swaps[0] > 0) == (kind == "tied_later" and cap == 0)
 
 
+@pytest.mark.parametrize("number", [1, 9, 64])
+def test_block_shuffle_number_of_blocks_handed_over(number):
+    """One block of 64, nine (more than there is room for clusters of 16), all: in large clusters, or in the size for all blocks."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8630)
+    No, C, block = 300, 2048, 32
+    W = (g0.standard_normal((No, C)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(C)
+    perm = g0.permutation(C).astype(np.int32)
+    chosen = g0.choice(C // block, number, replace=False)
+    W[17, perm[chosen * block]] = np.inf
+    theta, info = orc.local_block_shuffle(W, s, perm, block)
+    g = GpuPrune(W, None, 1.0, score=s, perm=perm, lbs_block=block)
+    assert np.array_equal(g.host()[2], theta)
+    assert g.stats.lbs_swaps_total == info.swaps_total and g.stats.near_tie_swaps == info.near_tie_swaps
+    assert np.flatnonzero(g.handed()[0]).tolist() == sorted(chosen.tolist())
+
+
 @pytest.mark.parametrize("No", [1, 2, 3, 4, 5])
 @pytest.mark.parametrize("block,equal", [(12, False), (256, False), (256, True)])
 def test_block_shuffle_few_rows(No, block, equal):
