@@ -85,8 +85,8 @@ def test_shuffle_select_compress_bit_exact_given_oracle_scores(No, C, T, block):
 
 @pytest.mark.parametrize("No,C,block,cap", [(1100, 520, 256, 0), (1024, 256, 256, 12), (2100, 264, 256, 6)])
 def test_block_shuffle_tall_weights_bit_exact(No, C, block, cap):
-    """The table kernel takes at most 928 rows at once, in equal chunks: two chunks (1100 and 1024 rows) and three (2100), with a
-    ragged last block of channels and slices of the greedy kernel's clusters that are no multiple of eight."""
+    """Several chunks of the bounds' table (256 rows each), with a ragged last block of channels and slices of the clusters that end in a
+    ragged eight rows.  (The exact kernels' chunks: test_block_shuffle_exact_kernels_on_tall_weights.)"""
     from tests.gpu_util import GpuPrune
     g0 = np.random.default_rng(7000 + No)
     W = (g0.standard_normal((No, C)) * 0.02 * np.sqrt(4.0 / g0.chisquare(4.0, size=(No, 1)))).astype(np.float16)
@@ -100,8 +100,8 @@ def test_block_shuffle_tall_weights_bit_exact(No, C, block, cap):
 @pytest.mark.parametrize("kind", ["equal_scores", "zero_scores", "negative_scores", "large_weights", "ties_in_some_rows"])
 @pytest.mark.parametrize("No,C,block,cap", [(40, 264, 256, 0), (1100, 256, 256, 5), (67, 48, 12, 0)])
 def test_block_shuffle_rows_that_fp32_cannot_decide(kind, No, C, block, cap):
-    """The block shuffle's fp64 path: rows with equal products (settled by position), rows with |w| >= 0.5, blocks with scores
-    that are zero or negative -- all rows of a weight or a few among regular ones, in slices shorter and longer than a chunk."""
+    """Rows with equal products (settled by position), rows with |w| >= 0.5, blocks with scores that are zero or negative -- all rows of a
+    weight or a few among regular ones, in short and long slices: whichever kernels decide them."""
     from tests.gpu_util import GpuPrune
     g0 = np.random.default_rng(8100 + No)
     W = (g0.standard_normal((No, C)) * (1.5 if kind == "large_weights" else 0.02)).astype(np.float16)
@@ -123,8 +123,7 @@ def test_block_shuffle_rows_that_fp32_cannot_decide(kind, No, C, block, cap):
 
 @pytest.mark.parametrize("No", [1, 3, 192 * 16, 192 * 16 + 1, 1024 * 16 + 5])
 def test_block_shuffle_row_slices(No):
-    """Rows dealt to the CTAs of one block's cluster: fewer rows than CTAs, slices at the edge between the two row loops,
-    slices of more than one chunk."""
+    """Rows dealt to the CTAs of one block's cluster: fewer rows than CTAs, slices of a chunk and of more than one."""
     from tests.gpu_util import GpuPrune
     g0 = np.random.default_rng(8200 + No)
     W = (g0.standard_normal((No, 64)) * 0.02).astype(np.float16)
@@ -150,8 +149,8 @@ def test_block_shuffle_narrow_blocks(No, C, block):
 
 @pytest.mark.parametrize("block", [12, 28, 32, 36, 128])
 def test_block_shuffle_rows_told_apart_in_blocks_of_every_width(block):
-    """Rows whose products fp32 cannot order are found by a sort as wide as the block: ties between the first and the last channels of
-    a block, at the widths where the sort changes."""
+    """Two channels of a block that tie in every third row, at the widths where kernels and layouts change.  (The sort that finds such rows
+    for the exact kernels: test_block_shuffle_exact_kernels_in_blocks_of_every_width.)"""
     from tests.gpu_util import GpuPrune
     g0 = np.random.default_rng(8400 + block)
     No, C = 90, 264
@@ -267,6 +266,58 @@ def test_block_shuffle_zero_columns_are_decided_by_bounds(every, block):
     assert not any(g.handed()[0])
 
 
+def handed_over(kind, No, C, block, seed):
+    """A weight whose first block the exact kernels take: from the start, by an infinite weight (all rows but that one have products that fp32
+    can order), or after some swaps, by ties among narrow channels."""
+    g0 = np.random.default_rng(seed)
+    W = (g0.standard_normal((No, C)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(C)
+    perm = g0.permutation(C).astype(np.int32)
+    if kind == "not_finite":
+        W[No // 2, perm[min(block, C) - 1]] = np.inf
+    else:
+        small = perm[block // 2: block]
+        W[:, small] = (W[:, small[np.arange(len(small)) % 5]].astype(np.float32) / 64).astype(np.float16)
+        s[small] = 1.0
+    return W, s, perm
+
+
+@pytest.mark.parametrize("kind", ["not_finite", "tied_later"])
+@pytest.mark.parametrize("No", [192, 193, 1100, 2100, 192 * 16, 192 * 16 + 1, 1024 * 16 + 5])
+def test_block_shuffle_exact_kernels_on_tall_weights(kind, No):
+    """The exact kernels on the edge between their two row loops (192 rows of the table kernel, of a CTA of the cluster), on one to
+    eighteen chunks of the table kernel (928 rows at most) and on slices of more than one chunk; from the start and from where bounds stopped."""
+    from tests.gpu_util import GpuPrune
+    W, s, perm = handed_over(kind, No, 128, 64, 8670 + No)
+    cap = 6 if kind == "not_finite" else 0
+    theta, info = orc.local_block_shuffle(W, s, perm, 64, cap)
+    g = GpuPrune(W, None, 1.0, score=s, perm=perm, lbs_block=64, lbs_max_swaps=cap)
+    assert np.array_equal(g.host()[2], theta)
+    assert g.stats.lbs_swaps_total == info.swaps_total and g.stats.near_tie_swaps == info.near_tie_swaps
+    assert g.stats.obj_after_lbs == orc.objective(W, s, theta)
+    handed, swaps = g.handed()
+    assert [bool(h) for h in handed] == [True, False]
+    assert (swaps[0] > 0) == (kind == "tied_later")
+
+
+@pytest.mark.parametrize("block", [8, 12, 28, 32, 36, 64, 128, 256])
+@pytest.mark.parametrize("ties", [False, True])
+def test_block_shuffle_exact_kernels_in_blocks_of_every_width(block, ties):
+    """Rows whose products fp32 cannot order are found by a sort as wide as the block: none (but the infinite one), or ties between the
+    first and the last channels of the block in every third row, at the widths where the sort changes."""
+    from tests.gpu_util import GpuPrune
+    W, s, perm = handed_over("not_finite", 250, 264, block, 8680 + block)
+    if ties:
+        first, last = perm[0], perm[block - 2]
+        s[last] = s[first]
+        W[::3, last] = W[::3, first]
+    theta, info = orc.local_block_shuffle(W, s, perm, block)
+    g = GpuPrune(W, None, 1.0, score=s, perm=perm, lbs_block=block)
+    assert np.array_equal(g.host()[2], theta)
+    assert g.stats.lbs_swaps_total == info.swaps_total and g.stats.near_tie_swaps == info.near_tie_swaps
+    assert g.handed()[0][0] == 1
+
+
 def test_block_shuffle_settles_only_pairs_that_may_gain():
     """Nine channels of score zero in nine groups (36 pairs that exchange for exactly nothing) and two equal channels, whose exchange
     bounds cannot tell from a gain: the last question is about one pair, and is settled without the exact kernels."""
@@ -311,8 +362,8 @@ def test_llama7b_q_projection_full_size_block_shuffle():
 
 @pytest.mark.parametrize("wl_index,lin", [(3, "gate"), (4, "fc1")])
 def test_block_shuffle_all_rows_of_the_widest_layers(wl_index, lin):
-    """All 22016 / 36864 output rows of the widest LLaMA-65B / OPT-66B linears on one block of 256 input channels: 24 and 40
-    chunks of the table kernel, slices of several chunks in the greedy kernel; two swaps, bit-exact."""
+    """All 22016 / 36864 output rows of the widest LLaMA-65B / OPT-66B linears on one block of 256 input channels: 86 and
+    144 chunks of the bounds' table, slices of several chunks in the clusters; two swaps, bit-exact."""
     from tests.gpu_util import GpuPrune
     wl = inputs.WORKLOADS[wl_index]
     W = inputs.make_weight(wl, lin, C=256)
