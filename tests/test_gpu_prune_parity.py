@@ -266,6 +266,46 @@ def test_block_shuffle_zero_columns_are_decided_by_bounds(every, block):
     assert not any(g.handed()[0])
 
 
+@pytest.mark.parametrize("kind", ["ordinary", "zero_scores", "negative_scores", "far_apart", "zero_columns", "equal"])
+@pytest.mark.parametrize("No,cap", [(100, 1), (700, 7), (17 * 1024, 3)])
+def test_block_shuffle_bounds_hold(kind, No, cap):
+    """Every entry of the bounds' table, as `cap` swaps have left it (untouched, formed anew, shifted): its distance from the exact gain is at
+    most the bound that it carries, and the bound is small against the sums of the block's products."""
+    from tests.gpu_util import GpuPrune
+    g0 = np.random.default_rng(8690 + No)
+    m = 64
+    W = (g0.standard_normal((No, m)) * 0.02).astype(np.float16)
+    s = 1.0 + 3.0 * g0.random(m)
+    if kind == "zero_scores":
+        s[::7] = 0.0
+    elif kind == "negative_scores":
+        s[::3] *= -1.0
+    elif kind == "far_apart":
+        s[::9] *= 2.0 ** -70
+    elif kind == "zero_columns":
+        W[:, ::7] = 0.0
+    elif kind == "equal":
+        s[:] = 2.5
+    perm = g0.permutation(m).astype(np.int32)
+    g = GpuPrune(W, None, 1.0, score=s, perm=perm, lbs_block=m, lbs_max_swaps=cap)
+    assert g.stats.lbs_swaps_total == cap and g.handed()[0] == [0]
+    theta = g.host()[2]
+    bits = g.ws[g.ws.numel() - 256 * 256 * 8:].cpu().numpy().view(np.uint64).reshape(256, 256)[:m, :m]
+    value = (bits & ~np.uint64(0xFFFF)).view(np.float64)
+    error = (bits.astype(np.uint32) << np.uint32(16)).view(np.float32).astype(np.float64)
+    # products scaled to 1/2 by a power of two
+    a = np.abs(W.astype(np.float64))
+    p = a * s * 2.0 ** -(np.frexp(np.abs(s).max())[1] - 1 + 3 + np.frexp(a.max())[1] - 1)
+    for pos in range(m):
+        mine = theta[pos // 4 * 4: pos // 4 * 4 + 4]
+        f2 = np.sort(p[:, [c for c in mine if c != theta[pos]]], axis=1)[:, 1]
+        exact = np.maximum(p[:, perm] - f2[:, None], 0.0).sum(0) - np.maximum(p[:, theta[pos]] - f2, 0.0).sum()
+        others = ~np.isin(perm, mine)
+        assert np.all(np.abs(value[pos] - exact)[others] <= error[pos, others] + 1e-13 * No * (error[pos, others] > 0))
+        # (an entry's R, D and S are column sums at most; below 100 additions and 4 S; shifted once per swap)
+        assert error[pos, others].max() <= (1 + cap) * 2.0 ** -16 * np.abs(p).sum(0).max()
+
+
 def handed_over(kind, No, C, block, seed):
     """A weight whose first block the exact kernels take: from the start, by an infinite weight (all rows but that one have products that fp32
     can order), or after some swaps, by ties among narrow channels."""
