@@ -690,6 +690,7 @@ __global__ void __launch_bounds__(256) lbs_mark_kernel(const uint16_t *__restric
                                                        const int32_t *__restrict__ theta0, int C, int lbs_block, const int *__restrict__ handed,
                                                        uint8_t *__restrict__ irregular) {
     const int b = blockIdx.y, p0 = b * lbs_block, m = min(lbs_block, C - p0);
+    grid_dependency_wait();
     if (!handed[b]) return;
     const int lane = threadIdx.x & 31, x0 = lane * 8;
     float s32[8];
@@ -778,6 +779,7 @@ __global__ void __launch_bounds__(kTableThreads, 2) lbs_table_kernel(const uint1
     LbsTableSmem &S = *reinterpret_cast<LbsTableSmem *>(s_dyn);
     const int g = blockIdx.x, b = blockIdx.y;
     const int p0 = b * lbs_block, m = min(lbs_block, C - p0);
+    grid_dependency_wait();
     if (g * 4 >= m || !handed[b]) return;
     const int tid = threadIdx.x;
     for (int i = tid; i < 2 * LbsCells<4>::kWords; i += kTableThreads) S.cells[i] = 0u;

@@ -1077,12 +1077,14 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
                                            (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters,
                                            (const int *)w.widest, (const uint8_t *)w.live, w.handed, w.handed_swaps, w.handed_pos, nc));
         }
-        // the exact kernels, on the blocks that were handed to them (without any, 8 us)
+        // the exact kernels, on the blocks that were handed to them (without any, 4 us for the first two set up under their predecessors, 8 otherwise; it is the smallest calls
+        // that notice: 8 x 8 112 -> 108 us, by the exact kernels alone 107)
         auto mark = o.lbs_block <= 8 ? lbs_mark_kernel<8> : o.lbs_block <= 32 ? lbs_mark_kernel<32> : lbs_mark_kernel<kLbsMax>;
-        mark<<<dim3(ceil_div(No, 64), nblocks), 256, 0, stream>>>(w.wb, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, w.irregular);
+        ESP_CUDA_OK(launch_overlapped(mark, dim3(ceil_div(No, 64), nblocks), 1, 256, 0, stream, w.wb, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed,
+                                      w.irregular));
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_table_kernel, (int)sizeof(LbsTableSmem)));
-        lbs_table_kernel<<<dim3(o.lbs_block / 4, nblocks), kTableThreads, sizeof(LbsTableSmem), stream>>>(
-            w.wb, w.wt, w.ldt, w.irregular, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, few ? nullptr : w.handed_pos, w.table, w.base[1]);
+        ESP_CUDA_OK(launch_overlapped(lbs_table_kernel, dim3(o.lbs_block / 4, nblocks), 1, kTableThreads, sizeof(LbsTableSmem), stream, w.wb, w.wt, w.ldt, w.irregular, No,
+                                      w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, (few ? (int32_t *)nullptr : w.handed_pos), w.table, w.base[1]));
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_greedy_kernel, (int)lbs_greedy_smem(kGreedyMinCluster)));
         ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         // How many blocks there is work in is not known here: none as a rule, one now and then, all of a weight made of ties.  Up to as many as large clusters serve sooner
