@@ -1095,9 +1095,9 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
                               lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, cost, nblocks, No, di.device)};
         const int caps[2] = {lbs_cluster_capacity(lbs_greedy_kernel, lbs_greedy_config, sizes[0], di.device),
                              lbs_cluster_capacity(lbs_greedy_kernel, lbs_greedy_config, sizes[1], di.device)};
-        if (caps[0] <= 0 || caps[1] <= 0) return ESP_ERR_CUDA;
-        int most = sizes[0] == sizes[1] ? nblocks : 1;
-        while (most < nblocks && cost.of(sizes[0], caps[0], most + 1, No) <= cost.of(sizes[1], caps[1], most + 1, No)) ++most;
+        int most = nblocks;
+        if (sizes[0] != sizes[1])                                 // (both then come from a capacity)
+            for (most = 1; most < nblocks && cost.of(sizes[0], caps[0], most + 1, No) <= cost.of(sizes[1], caps[1], most + 1, No);) ++most;
         for (int all = 0; all < (most < nblocks ? 2 : 1); ++all) {
             lbs_greedy_config(cfg, attr, nblocks, sizes[all], stream);
             ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, (const uint8_t *)w.irregular, No,
