@@ -28,8 +28,8 @@
 // rows (two products of 1/2 in each), five roundings of 2^-53 in each of the four values of a gain and three in adding them make less than 26 * 2^-53 rows a
 // pair; two entries have 32.  What is left of it (2^-51 rows a pair) is more than the underflow of products down to 2^-200 in fp32, 2^-132 a row, adds.
 //
-// Two channels whose products are all zero (score zero: dead inputs; column zero: pruned before) exchange for nothing: exactly 0 on both sides, so such entries carry no bound;
-// otherwise dozens of them would stay in question to the end.  Columns of zeros count as scores of zero, which changes no product.
+// Two channels whose products are all zero (score zero: dead inputs; column zero: pruned before) exchange for nothing: exactly 0 on both sides, so such
+// entries carry no bound; otherwise dozens of them would stay in question to the end.  Columns of zeros count as scores of zero, which changes no product.
 //
 // What bounds it: on long slices instruction issue -- a row costs a warp 48 fma, 48 additions, 8 conversions and some 30 others for both groups (256
 // candidates, 6 slots), about 20 ns of an SM's time where the exact kernels take 55 --, on short ones the latency of a swap (search, three cluster barriers,
@@ -305,8 +305,8 @@ __global__ void __launch_bounds__(kBoundTableThreads, 2) lbs_bound_table_kernel(
 
 // ---- The swaps.  One cluster of CTAs per block of positions; the output rows are dealt to its CTAs, and so are the pairs, (i, j) to rank
 // i mod cluster size.  Three cluster barriers per swap: after every CTA's best pair has been sent to all, when the sums of all CTAs are
-// complete, and when the 6 x 256 new entries, each formed by one of the CTAs, are in all; the table in L2 is only for the columns that a swap looks up (entries of other groups, asked for while
-// the sums are being added).
+// complete, and when the 6 x 256 new entries, each formed by one of the CTAs, are in all; the table in L2 is only for the columns that a swap looks up
+// (entries of other groups, asked for while the sums are being added).
 struct LbsBoundSmem {
     float4 part[kBoundWarps][6 * 64];                             // the warps' sums; the CTA's end up in the first warp's
     union {
@@ -314,7 +314,7 @@ struct LbsBoundSmem {
         double fresh[6][kLbsMax];                                 // the new entries, written by the CTAs of the cluster (the thresholds are used up)
     };
     float4 best[kBoundWarps], won[kBoundMaxCluster];              // (the latter written by the CTAs of the cluster)
-    float D[kBoundWarps][8];                                      // of the six live slots, S of the two groups
+    float D[kBoundWarps][8];                                      // of the six live slots; S of the two groups
     float D_of[kBoundMaxCluster][8];                              // written by the CTAs of the cluster
     unsigned long long exact[kBoundCand * 4][4];                  // this CTA's rows' sums
     double value[kBoundCand * 4];
@@ -465,7 +465,7 @@ __device__ __noinline__ int bound_settle(LbsBoundSmem &S, float reach, int my_ro
         const float2 *gr = S.gains + lbs_gain_offset(r, m, rank, nc);
         for (int j = i + 1 + lane; j < m; j += 32) {
             const float2 g = gr[j - i - 1];
-            if (g.y >= reach && g.y > 0.f) {                      // (a pair that cannot gain is neither the best nor nearly tied with one that does)
+            if (g.y >= reach && g.y > 0.f) {                      // (who cannot gain is neither the best nor nearly tied with it)
                 const int at = atomicAdd(&S.found, 1);
                 if (at < kBoundCand)
                     for (int c = 0; c < nc; ++c) st_remote_s32(map_to_rank(smem_u32(&S.list[rank][at]), (uint32_t)c), i * kLbsMax + j);

@@ -1,5 +1,6 @@
 // Local block shuffle (Algorithm 1 lines 3-14, Eq. 5): the exact kernels.  Included by prune_kernels.cu inside namespace esp { namespace { ... } }.
-// lbs_bounds.cuh, included at the end, finds the same swaps from bounds; the kernels here take the blocks that it cannot decide, from the first swap or from where it stopped.
+// lbs_bounds.cuh, included at the end, finds the same swaps from bounds; the kernels here take the blocks that it cannot decide, from the first swap or
+// from where it stopped.
 //
 // Algorithm 1 needs, for every group g of a block, every slot k of g and every channel x of the block, the value
 //   V(g, k <- x) = retained metric sum of g with slot k replaced by x
@@ -17,17 +18,17 @@
 //  * A lane owns 8 candidates and a warp one row at a time: the row's record is uniform, a row of the block's gathered copy is
 //    one 512-byte load, nothing is exchanged between lanes.
 //  * fp32 products decide.  Each is within 2^-23 relative of its fp64 counterpart, so they order a row's channels as the fp64
-//    products do unless two of them are closer than 2^-21.  Which rows hold such a pair is found once, when the weight is gathered
-//    (the products of a row's 256 channels never change, only their grouping does): those rows -- about one in a hundred where
+//    products do unless two of them are closer than 2^-21.  Which rows hold such a pair is found once, in the blocks that come here (lbs_mark_kernel;
+//    the products of a row's 256 channels never change, only their grouping does): those rows -- about one in a hundred where
 //    the scores of a block differ -- and the rows with a magnitude of 0.5 or more are "irregular" and take fp64 products and
 //    64-bit sums in a loop of their own.  Equal scores make nearly every row irregular, as do weights with sigma of 0.2 and more and, in
-//    its block, a score that is not positive: little of the gain is left there (4096 x 4096 to the end, against the kernels before: 68.7 -> 57.0 ms
-//    with equal scores, 66.9 -> 33.0 with every sixteenth score zero, 68.2 -> 51.8 at sigma 0.2, 68.6 -> 55.5 at 1.5; 69.7 -> 9.3 at 0.1).
+//    its block, a score that is not positive: little of the gain is left there.
 //  * |w| < 0.5 becomes an integer of 2^-24 with one fp32 fma, so the sums are 32-bit adds.
 //
-// Measured against one comparison and two fp64 additions per (row, candidate, slot) with a warp per candidate (about 29 instructions
-// each): table of a 4096 x 4096 weight 6.94 -> 0.92 ms, greedy kernel 67.7 -> 8.7 ms; 13824 x 5120: 29.1 -> 3.8 ms and 223 -> 24.4 ms;
-// 512 x 512 (two blocks): 15.6 -> 2.6 ms.
+// Measured, all blocks by these kernels, against one comparison and two fp64 additions per (row, candidate, slot) with a warp per candidate (about 29
+// instructions each): table of a 4096 x 4096 weight 6.94 -> 0.92 ms, greedy kernel 67.7 -> 8.7 ms; 13824 x 5120: 29.1 -> 3.8 ms and 223 -> 24.4 ms; 512 x 512
+// (two blocks): 15.6 -> 2.6 ms; to the end, 4096 x 4096 of irregular rows: 68.7 -> 57.0 ms with equal scores, 68.2 -> 51.8 at sigma 0.2.  (By bounds 4 ms,
+// all of those.)
 
 constexpr int kLbsMax = 256;       // widest local-shuffle block
 constexpr int kLbsGroups = kLbsMax / 4;
@@ -611,11 +612,10 @@ __device__ __forceinline__ void lbs_sort(float (&v)[8]) {
     }
 }
 
-// Wb[b][row][x] = |W[row, channel x of block b]| bits, `stride` (lbs_block rounded up to 8) per row, zeros beyond the block: one
-// pass over W, permuted through shared memory, so that everything below reads whole contiguous rows.  A warp per (row, block).
-// widest[b] becomes the bits of the block's largest magnitude, live[b][x] is set where the column of channel x holds anything but zeros; handed[b] is set where the bounds of
-// lbs_bounds.cuh do not hold: a weight that is not finite, a score that is neither zero nor of ordinary magnitude, scores more than 2^200 apart;
-// in all of them if `all` says so.
+// Wb[b][row][x] = |W[row, channel x of block b]| bits, `stride` (lbs_block rounded up to 8) per row, zeros beyond the block: one pass over W, permuted
+// through shared memory, so that everything below reads whole contiguous rows.  A warp per (row, block). widest[b] becomes the bits of the block's largest
+// magnitude, live[b][x] is set where the column of channel x holds anything but zeros; handed[b] is set where the bounds of lbs_bounds.cuh do not hold: a
+// weight that is not finite, a score that is neither zero nor of ordinary magnitude, scores more than 2^200 apart; in all of them if `all` says so.
 __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restrict__ W, int No, int C, long ldw, const double *__restrict__ score,
                                                          const int32_t *__restrict__ theta0, int lbs_block, int stride, int nblocks,
                                                          int rows_per_cta, uint16_t *__restrict__ Wb, int *__restrict__ handed, int *__restrict__ widest,
@@ -681,9 +681,8 @@ __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restric
     }
 }
 
-// For the exact kernels: irregular[b][row] is set where
-// the row holds a magnitude of 0.5 or more, or two products that fp32 cannot tell apart (found by sorting the row's products: about
-// 700 instructions per row of a 256-channel block; a narrow block sorts no wider than it is -- 512 blocks of
+// For the exact kernels: irregular[b][row] is set where the row holds a magnitude of 0.5 or more, or two products that fp32 cannot tell apart (found by
+// sorting the row's products: about 700 instructions per row of a 256-channel block; a narrow block sorts no wider than it is -- 512 blocks of
 // 8 channels of a 4096 x 4096 weight 2.8 -> 0.77 ms), or the block a score that is no ordinary positive number.  A warp per row of a block.
 template <int WIDTH>                                              // lbs_block or more
 __global__ void __launch_bounds__(256) lbs_mark_kernel(const uint16_t *__restrict__ Wb, int No, int stride, const double *__restrict__ score,

@@ -2,9 +2,10 @@
 // naive shuffle, local block shuffle (Algorithm 1, Eq. 5), 2-of-4 selection and compression.
 //
 // All of these stream fp16 matrices once or twice; they are bound by HBM and by instruction issue, the block shuffle by
-// instruction issue and, on short weights, by the latency of a swap.  Every quantity that feeds a discrete decision is fp64 with explicit round-to-nearest
-// multiplies/adds (no FMA contraction), and every sum over rows of |W| is taken exactly in 64-bit
-// integers of 2^-24, so results do not depend on the order in which threads visit rows.
+// instruction issue and, on short weights, by the latency of a swap.  Every discrete decision is the one that fp64 quantities with explicit round-to-nearest
+// multiplies/adds (no FMA contraction) give, over sums of |W| taken exactly in 64-bit integers of 2^-24, so results do not depend on the order in which
+// threads visit rows.  The block shuffle need not form those sums for most of its swaps: fp32 sums with proven bounds tell which pair they would choose
+// (lbs_bounds.cuh), and where the bounds leave a choice the pairs in question are evaluated exactly.
 #include "esp_common.cuh"
 
 #include <math.h>
@@ -272,7 +273,8 @@ __device__ __noinline__ int histogram_exact_bin(float xf, int c, int bins, const
 // of a group meet only through the low bits of their bins.  R = 4 gives each of them a counter row of its own (no conflict
 // at all), R = 2 one per two, R = 1 none (expected 1.0 / 1.5 / 2.1 passes per counting instruction; the plain
 // [channel][bin] layout needed 3.3).  R is chosen so that three CTAs still fit an SM.
-constexpr int kHistAhead = 4;                 // rows each thread keeps in flight (eight are never faster, and beyond 150 bins cost the third CTA: 200 bins of 2048 x 8192 33 us against 23)
+// Rows each thread keeps in flight (eight are never faster, and beyond 150 bins cost the third CTA: 200 bins of 2048 x 8192 33 us against 23).
+constexpr int kHistAhead = 4;
 constexpr int kHistStatic = 768;              // bytes of the kernel's fixed arrays
 constexpr size_t kHistRoom = (228 * 1024 / 3 - 1024 - kHistStatic) / 256 * 256;     // dynamic shared memory of one of three CTAs on an SM (1 KB is set aside for each)
 template <int R>
@@ -411,13 +413,14 @@ __global__ void __launch_bounds__(256, 3) histogram_kernel(const __half *__restr
     }
 }
 
-// Counter replicas for a bin count: one where a CTA has fewer than 1024 rows, beyond as many as keep three CTAs on an SM (kHistRoom; with 109 or 110
+// Counter replicas for a bin count: one where a CTA has fewer than 512 rows, beyond as many as keep three CTAs on an SM (kHistRoom; with 109 or 110
 // bins a limit of 75 KB let only two on: 2048 x 8192 of 110 bins 32 us, one replica 22).  Replicas are cleared and added up whatever the rows, and what they
-// spare is small: 100 bins of N(0, 1), one against two, 683 rows 19.8 / 20.1 us, 1366 rows 29.8 / 29.5, 2521 rows 47.4 / 45.5; 50 bins, one against four,
-// 1366 rows 28.1 / 27.2, 2521 rows 45.8 / 42.4; all but a few elements in one or two bins: within 4 % either way.
+// spare is small: 100 bins of N(0, 1), one against two, 342 rows 13.6 / 13.8 us, 683 rows 19.8 / 20.1 by itself but eight chunks of a calibration 259.6 / 258.9,
+// 1366 rows 29.8 / 29.5, 2521 rows 47.4 / 45.5; 50 bins, one against four, 1366 rows 28.1 / 27.2, 2521 rows 45.8 / 42.4; all but a few elements in one or
+// two bins: within 4 % either way.
 // Token splits: whole waves of three CTAs per SM (the counting is bound by the shared-memory atomics, about 17 ns per token row of a CTA
-// at that residency, so a partial wave is lost time; 2048 x 8192: 640 CTAs 30 us, 384 CTAs 20.5); a CTA's set-up and the addition of its counters to the global ones take as long
-// as some 250 rows.
+// at that residency, so a partial wave is lost time; 2048 x 8192: 640 CTAs 30 us, 384 CTAs 20.5); a CTA's set-up and the addition of its counters to the
+// global ones take as long as some 250 rows.
 inline esp_status_t launch_histogram(const __half *X, int T, int C, long ldx, int bins, const double *lo, const double *hi, unsigned int *counts,
                                      int sm_count, cudaStream_t stream) {
     const size_t per_replica = sizeof(unsigned int) * 64 * (size_t)bins;
@@ -430,7 +433,7 @@ inline esp_status_t launch_histogram(const __half *X, int T, int C, long ldx, in
         if (best < 0 || cost < best) { best = cost; splits = s; }
     }
     const int rows = ceil_div(T, splits);
-    const int R = rows < 1024 ? 1 : per_replica * 4 + ring <= kHistRoom ? 4 : per_replica * 2 + ring <= kHistRoom ? 2 : 1;
+    const int R = rows < 512 ? 1 : per_replica * 4 + ring <= kHistRoom ? 4 : per_replica * 2 + ring <= kHistRoom ? 2 : 1;
     const size_t smem = per_replica * R + ring;
     auto kern = R == 4 ? histogram_kernel<4> : R == 2 ? histogram_kernel<2> : histogram_kernel<1>;
     ESP_CUDA_OK(ensure_dynamic_smem((const void *)kern, (int)smem));
@@ -1077,8 +1080,8 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
                                            (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters,
                                            (const int *)w.widest, (const uint8_t *)w.live, w.handed, w.handed_swaps, w.handed_pos, nc));
         }
-        // the exact kernels, on the blocks that were handed to them (without any, 4 us for the first two set up under their predecessors, 8 otherwise; it is the smallest calls
-        // that notice: 8 x 8 112 -> 108 us, by the exact kernels alone 107)
+        // the exact kernels, on the blocks that were handed to them (without any, 8 us of empty launches, 4 with the first two set up under their
+        // predecessors, which the smallest calls notice: 8 x 8 112 -> 108 us, by the exact kernels alone 107)
         auto mark = o.lbs_block <= 8 ? lbs_mark_kernel<8> : o.lbs_block <= 32 ? lbs_mark_kernel<32> : lbs_mark_kernel<kLbsMax>;
         ESP_CUDA_OK(launch_overlapped(mark, dim3(ceil_div(No, 64), nblocks), 1, 256, 0, stream, w.wb, No, w.stride, w.score, w.theta0, C, o.lbs_block, w.handed,
                                       w.irregular));
@@ -1087,9 +1090,10 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
                                       w.stride, w.score, w.theta0, C, o.lbs_block, w.handed, (few ? (int32_t *)nullptr : w.handed_pos), w.table, w.base[1]));
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_greedy_kernel, (int)lbs_greedy_smem(kGreedyMinCluster)));
         ESP_CUDA_OK(cudaFuncSetAttribute(lbs_greedy_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        // How many blocks there is work in is not known here: none as a rule, one now and then, all of a weight made of ties.  Up to as many as large clusters serve sooner
-        // they are launched in those, beyond that in the size for all blocks; the other launch's clusters leave at once (2 us).  One block of the 16 of 4096 x 4096 (a weight that
-        // is not finite) 11.5 -> 8.6 ms for the whole call, 9.3 by the exact kernels alone; all sixteen handed over before their first swap 3.72 ms as before (4.5 in large clusters).
+        // How many blocks there is work in is not known here: none as a rule, one now and then, all of a weight made of ties.  Up to as many as large
+        // clusters serve sooner they are launched in those, beyond that in the size for all blocks; the other launch's clusters leave at once (2 us).  One
+        // block of the 16 of 4096 x 4096 (a weight that is not finite) 11.5 -> 8.6 ms for the whole call, 9.3 by the exact kernels alone; all sixteen handed
+        // over before their first swap 3.72 ms as before (4.5 in large clusters).
         const LbsSwapCost cost{10.0, 0.055};
         const int sizes[2] = {lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, cost, few ? nblocks : 1, No, di.device),
                               lbs_cluster_size(lbs_greedy_kernel, lbs_greedy_config, kGreedyMinCluster, cost, nblocks, No, di.device)};

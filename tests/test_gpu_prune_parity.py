@@ -544,7 +544,7 @@ def test_streaming_calibration_equals_one_shot(C, splits):
 @pytest.mark.parametrize("T", [300, 6600])
 @pytest.mark.parametrize("bins", [2, 54, 55, 108, 109, 110, 512])
 def test_histogram_counter_replicas(T, bins):
-    """Counts at the bin counts where the number of counter replicas changes, with few and with more than 1024 rows per CTA (4096
+    """Counts at the bin counts where the number of counter replicas changes, with few and with more than 512 rows per CTA (4096
     channels are dealt to six row slices)."""
     from tests.gpu_util import calibrate_in_chunks
     g0 = np.random.default_rng(1000 + bins)
