@@ -45,7 +45,7 @@ struct PruneWorkspace {
     unsigned long long *colsum;                              // [C]
     int32_t *theta0;                                         // [C]
     size_t cleared_bytes;                                    // from counters to the end of counts: zeroed at the start of a call
-    unsigned long long *counters;                            // [8]: 0 near-tie groups, 1 lbs swaps, 2 near-ties of the sort, 3 of the swaps
+    unsigned long long *counters;                            // [8]: 0 near-tie groups, 1 lbs swaps, 2 near-ties of the sort, 3 of the swaps, 4 blocks handed over
     double *objective;                                       // [4]: after gns, after lbs, identity order
     double *sorted_mean;                                     // [C] channel means in rank order
     unsigned long long *kept;                                // [C] retained sums of |W| per position of an order
@@ -57,6 +57,7 @@ struct PruneWorkspace {
     int *handed, *handed_swaps;                              // [nblocks] the exact kernels (re)start this block; swaps it has had
     int *widest;                                             // [nblocks] bits of the block's largest |W|
     uint8_t *live;                                           // [nblocks][stride] the channel's column holds anything but zeros
+    int *handed_list;                                        // [nblocks] the blocks handed over, counters[4] of them
     int32_t *handed_pos;                                     // [C] the order it is in: position -> channel of the block
     long ldt;                                                // No rounded up to 8
     int stride;                                              // lbs_block rounded up to 8

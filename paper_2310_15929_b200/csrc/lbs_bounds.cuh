@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
                                                                             const int32_t *__restrict__ theta0, int C, int lbs_block, int max_swaps,
                                                                             double *__restrict__ table, int32_t *__restrict__ theta, unsigned long long *__restrict__ counters,
                                                                             const int *__restrict__ widest, const uint8_t *__restrict__ live, int *__restrict__ handed, int *__restrict__ handed_swaps,
-                                                                            int32_t *__restrict__ handed_pos, int nc) {
+                                                                            int32_t *__restrict__ handed_pos, int *__restrict__ handed_list, int nc) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsBoundSmem &S = *reinterpret_cast<LbsBoundSmem *>(s_dyn);
     const int b = blockIdx.x / nc, rank = (int)cluster_ctarank();
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(kBoundThreads, 1) lbs_bound_greedy_kernel(cons
         handed_pos[p0 + x] = S.pos2x[x];
     }
     if (tid == 0) {
-        if (hand_over) { handed_swaps[b] = swaps; handed[b] = 1; }
+        if (hand_over) { handed_swaps[b] = swaps; lbs_hand_over(b, handed, handed_list, counters); }
         if (swaps) atomicAdd(&counters[1], (unsigned long long)swaps);
         if (near_swaps) atomicAdd(&counters[3], (unsigned long long)near_swaps);
     }

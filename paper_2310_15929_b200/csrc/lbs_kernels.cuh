@@ -612,6 +612,11 @@ __device__ __forceinline__ void lbs_sort(float (&v)[8]) {
     }
 }
 
+// Hands block b to the exact kernels (again: nothing happens).
+__device__ __forceinline__ void lbs_hand_over(int b, int *handed, int *handed_list, unsigned long long *counters) {
+    if (atomicExch(&handed[b], 1) == 0) handed_list[atomicAdd(&counters[4], 1ULL)] = b;
+}
+
 // Wb[b][row][x] = |W[row, channel x of block b]| bits, `stride` (lbs_block rounded up to 8) per row, zeros beyond the block: one pass over W, permuted
 // through shared memory, so that everything below reads whole contiguous rows.  A warp per (row, block). widest[b] becomes the bits of the block's largest
 // magnitude, live[b][x] is set where the column of channel x holds anything but zeros; handed[b] is set where the bounds of lbs_bounds.cuh do not hold: a
@@ -619,7 +624,8 @@ __device__ __forceinline__ void lbs_sort(float (&v)[8]) {
 __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restrict__ W, int No, int C, long ldw, const double *__restrict__ score,
                                                          const int32_t *__restrict__ theta0, int lbs_block, int stride, int nblocks,
                                                          int rows_per_cta, uint16_t *__restrict__ Wb, int *__restrict__ handed, int *__restrict__ widest,
-                                                         uint8_t *__restrict__ live, bool all) {
+                                                         uint8_t *__restrict__ live, bool all, int *__restrict__ handed_list,
+                                                         unsigned long long *__restrict__ counters) {
     extern __shared__ __align__(16) uint16_t s_rows[];            // [rows_per_cta][C]
     const int j0 = blockIdx.x * rows_per_cta;
     const int nrows = min(rows_per_cta, No - j0);
@@ -677,7 +683,8 @@ __global__ void __launch_bounds__(256) lbs_gather_kernel(const __half *__restric
         }
         wide = __reduce_max_sync(0xFFFFFFFFu, wide);
         if (lane == 0) atomicMax(&widest[b], (int)wide);
-        if (all || bad || wide >= 0x7C00u) handed[b] = 1;
+        bad = __any_sync(0xFFFFFFFFu, bad);
+        if ((all || bad || wide >= 0x7C00u) && lane == 0) lbs_hand_over(b, handed, handed_list, counters);
     }
 }
 
@@ -828,7 +835,7 @@ __global__ void __launch_bounds__(kTableThreads, 2) lbs_table_kernel(const uint1
 //     gains of 8 of the 256 positions, so about 2000 pairs are looked up again in the table (L2) and the search itself reads
 //     shared memory only.
 // Every CTA takes the same decision from the exchanged winners; all cluster barriers are reached by all threads.
-// Does nothing unless more than `from` and at most `to` blocks were handed over.
+// The i-th cluster takes the i-th block that was handed over, if these are more than `from` and at most `to`.
 constexpr int kGreedyRows = 1024, kGreedyThreads = 512, kGreedyMaxCluster = 16, kGreedyMinCluster = 3;
 constexpr int kLbsSwapLimit = 1 << 16;                            // far above any block's swaps; beyond it the kernel reports a timeout
 struct LbsGreedySmem {
@@ -909,28 +916,18 @@ __global__ void __launch_bounds__(kGreedyThreads, 1) lbs_greedy_kernel(const uin
                                                                        const double *__restrict__ score, const int32_t *__restrict__ theta0, int C,
                                                                        int lbs_block, int max_swaps, double *__restrict__ table,
                                                                        const double *__restrict__ base0, int32_t *__restrict__ theta,
-                                                                       unsigned long long *__restrict__ counters, const int *__restrict__ handed,
+                                                                       unsigned long long *__restrict__ counters, const int *__restrict__ handed_list,
                                                                        const int *__restrict__ handed_swaps, const int32_t *__restrict__ handed_pos, int nc,
-                                                                       int nblocks, int from, int to) {
+                                                                       int from, int to) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     LbsGreedySmem &S = *reinterpret_cast<LbsGreedySmem *>(s_dyn);
     using Cells = LbsCells<3>;
-    const int b = blockIdx.x / nc, rank = (int)cluster_ctarank();
+    const int number = (int)counters[4], at_list = blockIdx.x / nc;
+    if (number <= from || number > to || at_list >= number) return;
+    const int b = handed_list[at_list], rank = (int)cluster_ctarank();
     const int p0 = b * lbs_block, m = min(lbs_block, C - p0), G = m / 4;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr int kWarps = kGreedyThreads / 32;
-    if (!handed[b]) return;
-    if (from > 0 || to < nblocks) {                               // (all CTAs find the same)
-        int *number = reinterpret_cast<int *>(s_dyn), n = 0;
-        if (tid == 0) *number = 0;
-        __syncthreads();
-        for (int i = tid; i < nblocks; i += kGreedyThreads) n += handed[i] ? 1 : 0;
-        if (n) atomicAdd(number, n);
-        __syncthreads();
-        n = *number;
-        __syncthreads();                                          // (the place is used for other things from here on)
-        if (n <= from || n > to) return;
-    }
     double *tb = table + (long)b * kLbsGroups * 4 * kLbsMax;      // row of position i: group i / 4, slot i % 4
     auto clear_sums = [&]() {
         for (int i = tid; i < (int)(sizeof(S.cells) / 16); i += kGreedyThreads) reinterpret_cast<uint4 *>(S.cells)[i] = make_uint4(0u, 0u, 0u, 0u);

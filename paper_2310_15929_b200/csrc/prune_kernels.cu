@@ -940,6 +940,7 @@ PruneWorkspace carve_prune_workspace(void *ws, int No, int C, int T, const esp_p
         w.wb = (uint16_t *)take(sizeof(uint16_t) * ((size_t)nblocks * No + kBoundOver) * w.stride);
         w.irregular = (uint8_t *)take((size_t)nblocks * No);
         w.handed_pos = (int32_t *)take(sizeof(int32_t) * C);
+        w.handed_list = (int *)take(sizeof(int) * (size_t)nblocks);
         w.table = (double *)take(sizeof(double) * (size_t)nblocks * kLbsGroups * 4 * kLbsMax);
     }
     w.total_bytes = off;
@@ -1061,7 +1062,7 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
         gather_rows = std::max(1, std::min(gather_rows, No / (2 * std::max(1, di.sm_count))));
         ESP_CUDA_OK(ensure_dynamic_smem((const void *)lbs_gather_kernel, (int)(row_bytes * gather_rows)));
         lbs_gather_kernel<<<ceil_div(No, gather_rows), 256, row_bytes * gather_rows, stream>>>(W, No, C, ldw, w.score, w.theta0, o.lbs_block, w.stride, nblocks,
-                                                                                               gather_rows, w.wb, w.handed, w.widest, w.live, few);
+                                                                                               gather_rows, w.wb, w.handed, w.widest, w.live, few, w.handed_list, w.counters);
         lbs_transpose_kernel<<<dim3(ceil_div(C, 64), ceil_div(No, 64)), 256, 0, stream>>>(W, No, C, ldw, w.wt, w.ldt);
         // the swaps by bounds, but for one to three rows: their last question is about exchanges that move a kept product to another group, dozens of gains of rounding
         // noise, so every block would end in the exact kernels all the same (256..4096 channels, by bounds and to the end / exactly from the start: 1 row 0.64 / 0.60 ms,
@@ -1078,7 +1079,7 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
             lbs_bound_config(cfg, attr, nblocks, nc, stream);
             ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_bound_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, No, w.stride,
                                            (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table, perm, w.counters,
-                                           (const int *)w.widest, (const uint8_t *)w.live, w.handed, w.handed_swaps, w.handed_pos, nc));
+                                           (const int *)w.widest, (const uint8_t *)w.live, w.handed, w.handed_swaps, w.handed_pos, w.handed_list, nc));
         }
         // the exact kernels, on the blocks that were handed to them (without any, 8 us of empty launches, 4 with the first two set up under their
         // predecessors, which the smallest calls notice: 8 x 8 112 -> 108 us, by the exact kernels alone 107)
@@ -1103,11 +1104,11 @@ esp_status_t launch_prune(const __half *W, int No, int C, long ldw, const __half
         if (sizes[0] != sizes[1])                                 // (both then come from a capacity)
             for (most = 1; most < nblocks && cost.of(sizes[0], caps[0], most + 1, No) <= cost.of(sizes[1], caps[1], most + 1, No);) ++most;
         for (int all = 0; all < (most < nblocks ? 2 : 1); ++all) {
-            lbs_greedy_config(cfg, attr, nblocks, sizes[all], stream);
+            lbs_greedy_config(cfg, attr, all ? nblocks : most, sizes[all], stream);
             ESP_CUDA_OK(cudaLaunchKernelEx(&cfg, lbs_greedy_kernel, (const uint16_t *)w.wb, (const uint16_t *)w.wt, w.ldt, (const uint8_t *)w.irregular, No,
                                            w.stride, (const double *)w.score, (const int32_t *)w.theta0, C, o.lbs_block, o.lbs_max_swaps, w.table,
-                                           (const double *)w.base[1], perm, w.counters, (const int *)w.handed, (const int *)w.handed_swaps,
-                                           (const int32_t *)(few ? nullptr : w.handed_pos), sizes[all], nblocks, all ? most : 0, all ? nblocks : most));
+                                           (const double *)w.base[1], perm, w.counters, (const int *)w.handed_list, (const int *)w.handed_swaps,
+                                           (const int32_t *)(few ? nullptr : w.handed_pos), sizes[all], all ? most : 0, all ? nblocks : most));
         }
         if (stats) {
             // the objectives before and after (colabs_kernel, which gathers the permuted channels from W, took 47 us for each of the orders of a 4096 x 4096 weight);
